@@ -83,6 +83,8 @@ struct DevStatus {
   unsigned long long nnzb_K;       // 3x3 blocks of the linearisation
   unsigned long long over_K;       // linearisation block buffer too small
   unsigned long long nonfinite;    // elements with a non-finite node coordinate
+  unsigned long long work_ctr4;    // work counter of the quadrature kernels
+  unsigned long long work_ctr5;    // work counter of the pair sort
   double J;
 };
 

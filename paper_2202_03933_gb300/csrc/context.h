@@ -73,6 +73,7 @@ struct mortar_ctx {
   mortar::DevBuf pairs_s, pairs_m;          // int32 (pair_cap)
   int64_t pair_cap = 0;
   mortar::DevBuf Mblk, Dblk, flag;          // FP64 16/pair (quadratic slaves 32), uint8/pair
+  mortar::DevBuf rec, order;                // fixed-point pair records (groups of 32), sorted pair order (int32)
   mortar::DevBuf Qunit, Qflag;              // quadratic slaves: per (pair, sub-element) 32 FP64, uint8
   mortar::DevBuf row_cnt, row_cnt2;         // int32 (max(Ns, Nm)), int32 (Ns)
   mortar::DevBuf rowptr_D, col_D, val_D;
@@ -169,6 +170,7 @@ RunParams run_params(const mortar_ctx* c);
 
 // Quadratic slave elements (tri6, quad8): forward path only, 8 x 4 pair blocks.
 inline bool quadratic_slave(const mortar_ctx* c) { return c->nen_s > 4; }
+constexpr size_t kRecordGroupBytes = 32 * 45 * 8;   // FxRecord::kWords words of 32 pairs
 inline int mblk_stride(const mortar_ctx* c) { return quadratic_slave(c) ? 32 : 16; }
 
 // k_quadratic.cu
@@ -203,6 +205,8 @@ struct IntegrateArgs {
   DevStatus* st;
   cudaStream_t stream;
   unsigned long long* cta_t = nullptr;   // per-CTA busy interval (timing only)
+  long long* rec = nullptr;              // pair records and sorted order; null: the one-kernel form
+  int32_t* order = nullptr;
   int* grid_out = nullptr;               // receives the grid size used
 };
 void launch_slave_precompute_raw(const double* xs, const int32_t* conn_s, int64_t Es, int nen_s,

@@ -12,35 +12,52 @@
 // coefficients A (Phi_a = sum_c A[a][c] N_c, Eq. AnsatzDiscretizationLagrangeMult).
 //
 // GB300 has two FP64 lanes per SM and clock, and a warp-wide FP64 instruction
-// costs the same with 1 or 32 active lanes, so the kernels are written to
-// issue few FP64 instructions with full warps:
+// costs the same with 1 or 32 active lanes, so the FP64 work is kept small and
+// in full warps:
 //
-//  * variant 0 (default): each warp takes a batch of up to 32 R pairs
-//    (guided self-scheduling).  Phase A clips one pair per lane in FP32 for
-//    a sort key (cell count and edge intersections); the warp sorts its
-//    pairs by key (ballot counting sort) and phase B clips in FP64 and
-//    integrates them in rounds of 32 lanes of similar cost.  Affine element
-//    maps are inverted with
-//    one precomputed 2x2 inverse; bilinear ones by Newton in FP32 on
-//    power-of-two-scaled coordinates, then one Newton step with an FP64
-//    residual and the FP32 Jacobian inverse (the converged xi agrees with a
-//    full FP64 Newton to rounding; MapInverse in clip.cuh).
+//  * variant 0 (default): three kernels.  k_pair_sort orders batches of pairs
+//    by the cell count and edge intersections of an FP32 clip; k_pair_clip clips
+//    in FP64 (which decides what a pair contributes) and turns the polygon, the
+//    element maps and the cell weights into a fixed-point record;
+//    k_pair_quadrature integrates the records on the integer pipe, one cell of
+//    a pair per lane (fixed.cuh, quadrature.cuh).
+//    planar_600x520 (1.35 M pairs, dual LMs): 0.20 + 1.16 + 1.65 ms, against
+//    6.2 ms (batches of 64 pairs, the former default) and 5.6 ms (1024) of the
+//    one-kernel FP64 form.  The clip kernel is bound by the FP64 pipe (50 %
+//    busy, 400 instructions a pair) and instruction fetch, the quadrature
+//    kernel by issue (0.52 per scheduler and clock) over the multiply-add and
+//    integer pipes.
+//  * one kernel with everything in FP64 (k_integrate_batched): for callers
+//    without workspace, and pairs that do not fit the fixed-point frame.  Each
+//    warp sorts a batch of up to 32 R pairs and runs rounds of 32; affine maps
+//    are inverted with one precomputed 2x2 inverse, bilinear ones by Newton in
+//    FP32, then one step with an FP64 residual (MapInverse in clip.cuh).
 //  * variant 1: one pair per thread, FP64 Newton from xi = 0 at every point
 //    (the oracle's iteration), kept as the reference schedule.
 //
-// Both are persistent grids taking work from a global counter; the loops are
+// All are persistent grids taking work from a global counter; the loops are
 // bounded by the pair count.
-#include <type_traits>
-
 #include "clip.cuh"
 #include "context.h"
+#include "pair_sort.cuh"
+#include "quadrature.cuh"
 
 namespace mortar {
+
+static_assert(kRecordGroupBytes == 32 * FxRecord::kWords * 8, "record size");
 
 namespace {
 
 struct PairCounters {
   unsigned long long nonempty = 0, gp = 0, cells = 0, newton_fail = 0, xi_oor = 0, clip_over = 0;
+  __device__ __forceinline__ void add(DevStatus* st) const {
+    block_count_add(&st->nonempty, nonempty);
+    block_count_add(&st->gauss_points, gp);
+    block_count_add(&st->cells, cells);
+    block_count_add(&st->newton_fail, newton_fail);
+    block_count_add(&st->xi_oor, xi_oor);
+    block_count_add(&st->clip_overflow, clip_over);
+  }
 };
 
 // Writes M = A G (and D = A H) for pair p.
@@ -201,28 +218,17 @@ __global__ void __launch_bounds__(kMaxPairBlock) k_integrate(const int32_t* __re
     for (int64_t p = base + lane; p < end; p += 32)
       integrate_one<NS, NM, SEG>(p, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, ctr);
   }
-  block_count_add(&st->nonempty, ctr.nonempty);
-  block_count_add(&st->gauss_points, ctr.gp);
-  block_count_add(&st->cells, ctr.cells);
-  block_count_add(&st->newton_fail, ctr.newton_fail);
-  block_count_add(&st->xi_oor, ctr.xi_oor);
-  block_count_add(&st->clip_overflow, ctr.clip_over);
+  ctr.add(st);
 }
 
 // ---------------------------------------------------------------- variant 0
-// Shared memory of a warp: the sort keys of its batch, the sorted order and
-// the set of key values present.
-template <int R>
-struct BatchSmem {
-  static constexpr int B = 32 * R;
-  using PermT = typename std::conditional<(B > 256), uint16_t, uint8_t>::type;
-  static constexpr int kBytes = B * (1 + (int)sizeof(PermT)) + 8 * 4;
-};
+constexpr int kPtsBytes = 28 * 8;   // back-projections of a cell's seven points
 
-// One pair of a sorted round: FP64 clip, then the 7-point rule on the
+// One pair in FP64 (the one-kernel form, and pairs whose geometry does not fit
+// the fixed-point frame of the two-kernel form): FP64 clip, then the 7-point rule on the
 // centroid fan with the map inversions of MapInverse.
 template <int NS, int NM, bool SEG>
-__device__ __forceinline__ void integrate_pair_sorted(int64_t p, const int32_t* __restrict__ ps,
+__device__ __noinline__ void integrate_pair_fp64(int64_t p, const int32_t* __restrict__ ps,
                                                       const int32_t* __restrict__ pm,
                                                       const double* __restrict__ srec, const double* __restrict__ xm,
                                                       const int32_t* __restrict__ conn_m, const RunParams& rp,
@@ -324,128 +330,280 @@ __device__ __forceinline__ void integrate_pair_sorted(int64_t p, const int32_t* 
   flag[p] = 1;
 }
 
-template <int NS, int NM, bool SEG, int R>
+
+template <int NS, int NM, bool SEG>
 __global__ void __launch_bounds__(kMaxPairBlock) k_integrate_batched(
     const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
     const double* __restrict__ xm, const int32_t* __restrict__ conn_m, RunParams rp, double* __restrict__ Mblk,
-    double* __restrict__ Dblk, uint8_t* __restrict__ flag, int64_t pair_cap, DevStatus* st,
+    double* __restrict__ Dblk, uint8_t* __restrict__ flag, int64_t pair_cap, int B, DevStatus* st,
     unsigned long long* cta_t) {
   cta_mark(cta_t, 0);
-  using L = BatchSmem<R>;
-  using PermT = typename L::PermT;
-  constexpr int B = L::B;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned char* my = smem_raw + (size_t)warp * L::kBytes;
-  unsigned* pres = reinterpret_cast<unsigned*>(my);
-  PermT* perm = reinterpret_cast<PermT*>(my + 32);
-  uint8_t* keys = reinterpret_cast<uint8_t*>(perm + B);
+  unsigned char* my = smem_raw + (size_t)warp * batch_smem_bytes(B);
+  uint16_t* perm = reinterpret_cast<uint16_t*>(my + 32);
 
   PairCounters ctr;
   const bool ok = st->over_pairs == 0 && st->over_bins == 0;
   const int64_t n = ok ? (int64_t)min((unsigned long long)pair_cap, st->n_pairs) : 0;
-  const unsigned lt_mask = (1u << lane) - 1u;
   const Watchdog wd(rp.watchdog_us);
-  // guided self-scheduling: a warp takes half an even share of the pairs
-  // left (at most B, at least 32, a multiple of 32)
   const int64_t share = 2 * (int64_t)gridDim.x * (blockDim.x >> 5);
   for (;;) {   // bounded: the shared counter only grows
     if (wd.expired(&st->timeout)) break;
-    int64_t base = 0;
-    int fetch = B;
-    if (lane == 0) {
-      const unsigned long long seen = *reinterpret_cast<volatile unsigned long long*>(&st->work_ctr);
-      const int64_t f = (n - (int64_t)seen) / share;
-      fetch = f >= B ? B : (f < 32 ? 32 : (int)(f & ~31ll));
-      base = (int64_t)atomicAdd(&st->work_ctr, (unsigned long long)fetch);
-    }
-    base = __shfl_sync(0xffffffffu, base, 0);
-    fetch = __shfl_sync(0xffffffffu, fetch, 0);
-    if (base >= n) break;
-    const int64_t lim = min(n, base + (int64_t)fetch);
-    const int rounds = (fetch + 31) >> 5;
-    // ---- phase A: sort key of each pair from an FP32 clip: 1 + 16 x its
-    //      cell count + its edge intersections (0 = no pair); a cost
-    //      estimate only, the FP64 clip of phase B decides
-    if (lane < 8) pres[lane] = 0u;
-    __syncwarp();
-#pragma unroll 1
-    for (int rr = 0; rr < rounds; ++rr) {
-      const int64_t p = base + rr * 32 + lane;
-      int key = 0;
-      if (p < lim) {
-        int n_int = 0;
-        const int nr = clip_count_f32<NS, NM>(srec + (int64_t)SR_STRIDE * ps[p], xm, conn_m, pm[p], n_int);
-        key = 1 + 16 * (nr == 0 ? 0 : (nr == 3 ? 1 : min(nr, kPolyS))) + min(n_int, 15);
-        atomicOr(&pres[key >> 5], 1u << (key & 31));
-      }
-      keys[rr * 32 + lane] = (uint8_t)key;
-    }
-    __syncwarp();
-    // ---- sort by key, descending, over the key values present (ballots)
-    int basecnt = 0;
-#pragma unroll 1
-    for (int w = 7; w >= 0; --w) {
-      unsigned bits = pres[w];
-      while (bits != 0u) {   // uniform across the warp
-        const int b = 31 - __clz(bits);
-        bits &= ~(1u << b);
-        const int v = 32 * w + b;
-        int before = 0;
-#pragma unroll 1
-        for (int rr = 0; rr < rounds; ++rr) {
-          const int slot = rr * 32 + lane;
-          const bool hit = keys[slot] == v;
-          const unsigned mk = __ballot_sync(0xffffffffu, hit);
-          if (hit) perm[basecnt + before + __popc(mk & lt_mask)] = (PermT)slot;
-          before += __popc(mk);
-        }
-        basecnt += before;
-      }
-    }
-    const int n_live = basecnt;
-    __syncwarp();
+    int64_t base;
+    int fetch;
+    if (!fetch_batch(&st->work_ctr, n, share, B, base, fetch)) break;
+    const int n_live = sort_batch<NS, NM>(my, B, base, min(n, base + (int64_t)fetch), (fetch + 31) >> 5, ps, pm, srec,
+                                          xm, conn_m);
     // ---- phase B: one pair per lane, rounds of similar cost
     for (int i0 = 0; i0 < n_live; i0 += 32) {
       const int i = i0 + lane;
       if (i < n_live)
-        integrate_pair_sorted<NS, NM, SEG>(base + perm[i], ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, ctr);
+        integrate_pair_fp64<NS, NM, SEG>(base + perm[i], ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, ctr);
     }
     __syncwarp();
   }
-  block_count_add(&st->nonempty, ctr.nonempty);
-  block_count_add(&st->gauss_points, ctr.gp);
-  block_count_add(&st->cells, ctr.cells);
-  block_count_add(&st->newton_fail, ctr.newton_fail);
-  block_count_add(&st->xi_oor, ctr.xi_oor);
-  block_count_add(&st->clip_overflow, ctr.clip_over);
+  ctr.add(st);
   __syncthreads();
   cta_mark(cta_t, 1);
 }
 
+// ------------------------------------------- three-kernel form (default)
+// The batched kernel's work, split where its character changes: a sort kernel
+// (FP32 keys, k_pair_sort), a clip kernel (FP64 clip, and the polygon's
+// conversion to fixed point) that leaves one record per pair in sorted order,
+// and a quadrature kernel on the integer pipe.  One kernel with all of it does
+// not fit the instruction cache (about 2,300 instructions run at full rate,
+// measured with straight-line loops; IPC 0.75 -> 0.35 beyond that): its warps,
+// each in another phase, issued 0.24 instructions per scheduler and clock at 8
+// and at 16 warps per SM alike.
+template <int NS, int NM, bool SEG>
+__global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_clip(
+    const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
+    const double* __restrict__ xm, const int32_t* __restrict__ conn_m, RunParams rp, double* __restrict__ Mblk,
+    double* __restrict__ Dblk, uint8_t* __restrict__ flag, int64_t pair_cap, const int32_t* __restrict__ order,
+    long long* __restrict__ rec, DevStatus* st, unsigned long long* cta_t) {
+  cta_mark(cta_t, 0);
+  const int lane = threadIdx.x & 31;
+  PairCounters ctr;
+  const bool ok = st->over_pairs == 0 && st->over_bins == 0;
+  const int64_t n = ok ? (int64_t)min((unsigned long long)pair_cap, st->n_pairs) : 0;
+  const Watchdog wd(rp.watchdog_us);
+  for (;;) {   // bounded: the shared counter only grows; one group of 32 pairs per turn
+    if (wd.expired(&st->timeout)) break;
+    unsigned long long g = 0;
+    if (lane == 0) g = atomicAdd(&st->work_ctr, 1ull);
+    g = __shfl_sync(0xffffffffu, g, 0);
+    const int64_t i = 32 * (int64_t)g + lane;
+    if (32 * (int64_t)g >= n) break;
+    long long* o = rec + (int64_t)g * (32 * FxRecord::kWords) + lane;
+    bool stored = false;
+    if (i < n) {
+      const int64_t p = order[i];
+      const double* r = srec + (int64_t)SR_STRIDE * ps[p];
+      PlaneMap mmap;
+      double pu[kPolyS], pv[kPolyS];
+      const int nr = clip_polygon<NS, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
+      if (nr == 0) {
+        write_zero_blocks(p, SEG, Mblk, Dblk);
+        flag[p] = 0;
+      } else {
+        FxPolygon f;
+        stored = f.setup<NS, NM>(r, mmap, pu, pv, nr);
+        if (stored) {
+          FxRecord::store<NS, NM>(o, f, p);
+          ctr.cells += f.ncell;
+          ctr.gp += 7 * f.ncell;
+          ctr.nonempty++;
+        } else {
+          integrate_pair_fp64<NS, NM, SEG>(p, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, ctr);
+        }
+      }
+    }
+    if (!stored) o[32 * FxRecord::kInfo] = 0;   // nr = 0: nothing left for the quadrature kernel
+    __syncwarp();
+  }
+  ctr.add(st);
+  __syncthreads();
+  cta_mark(cta_t, 1);
+}
+
+// Adds up the cells' sums g of every pair of the warp and writes the pair's
+// 4x4 block M = A G (standard LMs: G).  The lanes of a pair take its entries in
+// turn: sum over the cells, conversion, product with A.  buf: this thread's
+// slice of shared memory (entry i at buf[i * stride], lane L's at buf - lane +
+// L), free to use by the whole warp.
+template <int NS, int NC>
+__device__ __forceinline__ void write_block(const FxAcc g[4][4], const CellSlot& cs, bool ok, int ke,
+                                            const FxScales& ss, const FxScales& sc, bool dual,
+                                            const double* __restrict__ r, double* __restrict__ out,
+                                            long long* __restrict__ buf, int stride) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+#pragma unroll
+  for (int a = 0; a < NS; ++a)
+#pragma unroll
+    for (int l = 0; l < NC; ++l) {
+      buf[(NC * a + l) * stride] = g[a][l].hh + (g[a][l].cr >> 32);
+      reinterpret_cast<unsigned*>(buf + (16 + ((NC * a + l) >> 1)) * stride)[l + NC * a & 1] = (unsigned)g[a][l].cr;
+    }
+  __syncwarp();
+  const long long* pair = buf - lane + cs.first;
+  double G[16];
+  int n = 0;
+  if (ok) {
+#pragma unroll 1
+    for (int e = cs.cell; e < NS * NC; e += cs.cells) {
+      const int a = e / NC, l = e - NC * a;
+      long long hh = 0, cr = 0;
+      for (int k = 0; k < cs.cells; ++k) {
+        hh += pair[e * stride + k];
+        cr += reinterpret_cast<const unsigned*>(pair + (16 + (e >> 1)) * stride + k)[e & 1];
+      }
+      const double v = fx_to_double(hh, cr, ke - ss.shape<NS>(a) - sc.shape<NC>(l));
+      if (dual) G[n++] = v;
+      else __stcs(out + 4 * a + l, v);
+    }
+    if (NS * NC < 16 || !dual) {   // the block is padded with zeros
+      for (int e = cs.cell; e < 16 && NS * NC < 16; e += cs.cells)
+        if ((e >> 2) >= NS || (e & 3) >= NC) __stcs(out + e, 0.0);
+    }
+  }
+  if (dual) {
+    __syncwarp();
+    double* Gs = reinterpret_cast<double*>(const_cast<long long*>(pair));
+    if (ok) {
+      n = 0;
+      for (int e = cs.cell; e < NS * NC; e += cs.cells) Gs[e * stride] = G[n++];
+    }
+    __syncwarp();
+    if (ok)
+#pragma unroll 1
+      for (int e = cs.cell; e < NS * NC; e += cs.cells) {
+        const int a = e / NC, l = e - NC * a;
+        double v = 0.0;
+#pragma unroll
+        for (int c = 0; c < NS; ++c) v = fma(r[SR_A + 4 * a + c], Gs[(NC * c + l) * stride], v);
+        __stcs(out + 4 * a + l, v);
+      }
+  }
+}
+
+// Quadrature of the clip kernel's records, one cell of a pair per lane (all
+// cells cost the same, so lanes idle only at the ends of warps): the cell's
+// back-projections, then its products, then the pair's sums through shared
+// memory.  A turn is up to `turn` groups of 32 records.
+template <int NS, int NM, bool SEG>
+__global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_quadrature(
+    const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
+    const double* __restrict__ xm, const int32_t* __restrict__ conn_m, RunParams rp, double* __restrict__ Mblk,
+    double* __restrict__ Dblk, uint8_t* __restrict__ flag, int64_t pair_cap, const long long* __restrict__ rec,
+    DevStatus* st) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  long long* pts = reinterpret_cast<long long*>(smem_raw) + threadIdx.x;
+  const int stride = (int)blockDim.x;
+  const int lane = threadIdx.x & 31;
+  const bool run = st->over_pairs == 0 && st->over_bins == 0;
+  const int64_t n = run ? (int64_t)min((unsigned long long)pair_cap, st->n_pairs) : 0;
+  const int64_t groups = (n + 31) >> 5;
+  // enough turns for every warp, at most 8 groups each
+  const int turn = (int)max((int64_t)1, min((int64_t)8, groups / (4 * (int64_t)gridDim.x * (blockDim.x >> 5))));
+  const Watchdog wd(rp.watchdog_us);
+  PairCounters slow;
+  for (;;) {   // bounded: the shared counter only grows
+    if (wd.expired(&st->timeout)) break;
+    unsigned long long g0 = 0;
+    if (lane == 0) g0 = atomicAdd(&st->work_ctr4, (unsigned long long)turn);
+    g0 = __shfl_sync(0xffffffffu, g0, 0);
+    if ((int64_t)g0 >= groups) break;
+    const int64_t r0 = 32 * (int64_t)g0;
+    const int records = 32 * (int)min((int64_t)turn, groups - (int64_t)g0);
+    for (int w = 0; w < records;) {
+      int ncell = 0;
+      if (w + lane < records) {
+        const int64_t i = r0 + w + lane;
+        const int nr = (int)(rec[((i >> 5) * FxRecord::kWords + FxRecord::kInfo) * 32 + (i & 31)] & 0xff);
+        ncell = nr > 3 ? nr : (nr == 3 ? 1 : 0);
+      }
+      const CellSlot cs = assign_cells(ncell);
+      const int64_t i = r0 + w + cs.rec;
+      w += cs.taken;
+      bool ok = cs.cell >= 0;
+      int64_t p = 0;
+      int32_t m = 0;
+      const double* r = srec;
+      FxScales ss, sm;
+      int ke = 0;
+      long long weight = 0;
+      if (ok) {
+        const long long* o = rec + (i >> 5) * (32 * FxRecord::kWords) + (i & 31);
+        FxView f;
+        f.load<NS, NM>(o);
+        p = o[32 * FxRecord::kPair];
+        r = srec + (int64_t)SR_STRIDE * ps[p];
+        m = pm[p];
+        weight = f.weight(cs.cell);
+        ss = f.ss;
+        sm = f.sm;
+        ke = f.ke;
+        ok = fx_back_project<NS, NM>(f, cs.cell, r, xm, conn_m, m, pts, stride);
+      }
+      const unsigned bad = __ballot_sync(0xffffffffu, cs.cell >= 0 && !ok);
+      const bool slow_pair = cs.cell >= 0 && (bad >> cs.first & ((1u << cs.cells) - 1u)) != 0;
+      ok &= !slow_pair;
+      FxAcc g[4][4];
+      if (SEG) {   // first, while the points are in shared memory: D in the lane's registers, then M
+        FxAcc h[4][4];
+        fx_cell_products<NS, NS, true>(ss, ss, weight, pts, stride, h);
+        fx_cell_products<NS, NM, false>(ss, sm, weight, pts, stride, g);
+        write_block<NS, NS>(h, cs, ok, ke, ss, ss, rp.lm == 1, r, Dblk + 16 * p, pts, stride);
+      } else {
+        fx_cell_products<NS, NM, false>(ss, sm, weight, pts, stride, g);
+      }
+      write_block<NS, NM>(g, cs, ok, ke, ss, sm, rp.lm == 1, r, Mblk + 16 * p, pts, stride);
+      if (cs.cell == 0) {
+        if (ok) flag[p] = 1;
+        else integrate_pair_fp64<NS, NM, SEG>(p, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, slow);
+      }
+      __syncwarp();
+    }
+  }
+  // pairs, cells and points were counted by the clip kernel
+  block_count_add(&st->newton_fail, slow.newton_fail);
+  block_count_add(&st->xi_oor, slow.xi_oor);
+}
+
 #ifdef MORTAR_PAIR_NS
-template <int NS, int NM, bool SEG, int R>
-void launch_batched_t(const IntegrateArgs& a, const RunParams& rp, int n_sm, int kWarps) {
-  const size_t shm = (size_t)kWarps * BatchSmem<R>::kBytes;
-  auto kern = k_integrate_batched<NS, NM, SEG, R>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+template <int NS, int NM, bool SEG>
+void launch_split(const IntegrateArgs& a, const RunParams& rp, int n_sm, int rounds, int warps) {
+  launch_pair_sort<NS, NM>(a, rp, n_sm, 32 * rounds);
+  auto clip = k_pair_clip<NS, NM, SEG>;
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, shm);
-  if (per_sm < 1) per_sm = 1;
-  const unsigned grid = (unsigned)(n_sm * per_sm);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, clip, warps * 32, 0);
+  const unsigned grid = (unsigned)(n_sm * (per_sm < 1 ? 1 : per_sm));
   if (a.grid_out) *a.grid_out = (int)grid;
-  kern<<<grid, kWarps * 32, shm, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag,
-                                             a.pair_cap, a.st, a.cta_t);
+  clip<<<grid, warps * 32, 0, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag, a.pair_cap,
+                                          a.order, a.rec, a.st, a.cta_t);
+  auto quad = k_pair_quadrature<NS, NM, SEG>;
+  const size_t shq = (size_t)warps * 32 * kPtsBytes;
+  cudaFuncSetAttribute(quad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shq);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quad, warps * 32, shq);
+  quad<<<(unsigned)(n_sm * (per_sm < 1 ? 1 : per_sm)), warps * 32, shq, a.stream>>>(
+      a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag, a.pair_cap, a.rec, a.st);
 }
 
 template <int NS, int NM, bool SEG>
-void launch_batched_r(const IntegrateArgs& a, const RunParams& rp, int n_sm, int rounds, int warps) {
-  if (rounds <= 1) launch_batched_t<NS, NM, SEG, 1>(a, rp, n_sm, warps);
-  else if (rounds == 2) launch_batched_t<NS, NM, SEG, 2>(a, rp, n_sm, warps);
-  else if (rounds == 4) launch_batched_t<NS, NM, SEG, 4>(a, rp, n_sm, warps);
-  else if (rounds == 8) launch_batched_t<NS, NM, SEG, 8>(a, rp, n_sm, warps);
-  else if (rounds == 16) launch_batched_t<NS, NM, SEG, 16>(a, rp, n_sm, warps);
-  else launch_batched_t<NS, NM, SEG, 32>(a, rp, n_sm, warps);
+void launch_batched(const IntegrateArgs& a, const RunParams& rp, int n_sm, int rounds, int warps) {
+  const size_t shm = (size_t)warps * batch_smem_bytes(32 * rounds);
+  auto kern = k_integrate_batched<NS, NM, SEG>;
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+  int per_sm = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, shm);
+  if (per_sm < 1) per_sm = 1;
+  const unsigned grid = (unsigned)(n_sm * per_sm);
+  if (a.grid_out) *a.grid_out = (int)grid;
+  kern<<<grid, warps * 32, shm, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag,
+                                             a.pair_cap, 32 * rounds, a.st, a.cta_t);
 }
 
 template <int NS, int NM, bool SEG>
@@ -469,8 +627,13 @@ void integrate_nsnm(const IntegrateArgs& a, const RunParams& rp, int n_sm, int v
     else launch_one_pair_per_thread<NS, NM, false>(a, rp, n_sm, block, chunk);
     return;
   }
-  if (seg) launch_batched_r<NS, NM, true>(a, rp, n_sm, rounds, block / 32);
-  else launch_batched_r<NS, NM, false>(a, rp, n_sm, rounds, block / 32);
+  if (a.rec) {
+    if (seg) launch_split<NS, NM, true>(a, rp, n_sm, rounds, block / 32);
+    else launch_split<NS, NM, false>(a, rp, n_sm, rounds, block / 32);
+    return;
+  }
+  if (seg) launch_batched<NS, NM, true>(a, rp, n_sm, rounds, block / 32);
+  else launch_batched<NS, NM, false>(a, rp, n_sm, rounds, block / 32);
 }
 template void integrate_nsnm<MORTAR_PAIR_NS, MORTAR_PAIR_NM>(const IntegrateArgs&, const RunParams&, int, int, int,
                                                               int, int);
@@ -487,9 +650,7 @@ void launch_dispatch(const IntegrateArgs& a, const RunParams& rp, int nen_s, int
 }  // namespace
 
 bool integrate_batched_fits(int rounds, int block) {
-  const size_t per_warp = (size_t)BatchSmem<32>::kBytes;   // the largest batch
-  (void)rounds;
-  return block >= 32 && block <= kMaxPairBlock && (size_t)(block / 32) * per_warp <= kMaxDynSmem;
+  return block >= 32 && block <= kMaxPairBlock && (size_t)(block / 32) * batch_smem_bytes(32 * rounds) <= kMaxDynSmem;
 }
 
 int integrate_rounds(int rounds, int block) {
@@ -514,6 +675,8 @@ void launch_integrate(mortar_ctx* c, const RunParams& rp) {
   IntegrateArgs a{c->pairs_s.as<int32_t>(), c->pairs_m.as<int32_t>(), c->srec.as<double>(), c->xm.as<double>(),
                   c->conn_m.as<int32_t>(), c->Mblk.as<double>(), c->Dblk.as<double>(), c->flag.as<uint8_t>(),
                   c->pair_cap, c->dstat.as<DevStatus>(), c->stream};
+  a.rec = c->rec.as<long long>();
+  a.order = c->order.as<int32_t>();
   c->pair_grid = 0;
   if (c->timing && c->cta_t.p) {
     a.cta_t = c->cta_t.as<unsigned long long>();
@@ -521,7 +684,7 @@ void launch_integrate(mortar_ctx* c, const RunParams& rp) {
   }
   const int block = c->block_size > 0 ? c->block_size : 128;
   const int chunk = c->chunk_pairs > 0 ? c->chunk_pairs : 32;
-  const int rounds = integrate_rounds(c->rounds > 0 ? c->rounds : 2, block);
+  const int rounds = integrate_rounds(c->rounds > 0 ? c->rounds : kSortBatch / 32, block);
   launch_dispatch(a, rp, c->nen_s, c->nen_m, c->n_sm, c->variant, block, chunk, rounds);
 }
 #endif  // MORTAR_PAIR_NS
