@@ -85,6 +85,7 @@ struct DevStatus {
   unsigned long long nonfinite;    // elements with a non-finite node coordinate
   unsigned long long work_ctr4;    // work counter of the quadrature kernels
   unsigned long long work_ctr5;    // work counter of the pair sort
+  unsigned long long work_ctr6;    // work counter of the adjoint's last kernel
   double J;
 };
 

@@ -49,6 +49,7 @@ __device__ __forceinline__ long long mul_wide(int a, int b) {
   asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
   return d;
 }
+__device__ __forceinline__ int mul_hi(int a, int b) { return __mulhi(a, b); }
 __device__ __forceinline__ float rcp_f32(float x) {   // about 1 ulp; seeds only
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -57,6 +58,7 @@ __device__ __forceinline__ float rcp_f32(float x) {   // about 1 ulp; seeds only
 #else
 inline long long mad_wide(int a, int b, long long c) { return (long long)a * b + c; }
 inline long long mul_wide(int a, int b) { return (long long)a * b; }
+inline int mul_hi(int a, int b) { return (int)(((long long)a * b) >> 32); }
 inline float rcp_f32(float x) { return 1.0f / x; }
 #endif
 
@@ -80,6 +82,8 @@ struct FxAcc {
   __device__ __forceinline__ long long get(int k) const {
     return (long long)((unsigned long long)hh << k) + (cr >> (32 - k));
   }
+  // the low digits' product of the last mul or mac, where 2^-2 unit matters
+  __device__ __forceinline__ void low(Dg a, Dg b) { cr += mul_hi(a.l, b.l); }
   // moves the whole units of the cross sum into hh (keeps the fraction): bounds cr between runs of products
   __device__ __forceinline__ void carry() {
     hh += cr >> 32;

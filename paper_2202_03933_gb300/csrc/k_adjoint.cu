@@ -26,8 +26,10 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "adjoint_fixed.cuh"
 #include "clip.cuh"
 #include "context.h"
+#include "pair_sort.cuh"
 #include "reverse.cuh"
 
 namespace mortar {
@@ -276,6 +278,163 @@ __global__ void __launch_bounds__(kMaxPairBlock) k_adjoint_pairs(
   block_count_add(&st->newton_fail, ctr.newton_fail);
 }
 
+// Node coordinates and multipliers of a pair.  Read for the set-up and again
+// (from L1/L2) after the quadrature: keeping them in registers would spill.
+template <int NS, int NM>
+__device__ __forceinline__ void load_pair_nodes(const int32_t* __restrict__ cs, const int32_t* __restrict__ cm,
+                                                const double* __restrict__ xs, const double* __restrict__ xm,
+                                                const double* __restrict__ lambda, V3* X, V3* Y, V3* lam) {
+  for (int a = 0; a < NS; ++a) {
+    const int64_t n = cs[a];
+    X[a] = v3(xs[3 * n], xs[3 * n + 1], xs[3 * n + 2]);
+    lam[a] = v3(lambda[3 * n], lambda[3 * n + 1], lambda[3 * n + 2]);
+  }
+  for (int l = 0; l < NM; ++l) {
+    const int64_t n = cm[l];
+    Y[l] = v3(xm[3 * n], xm[3 * n + 1], xm[3 * n + 2]);
+  }
+}
+
+// Lambda_c = sum_a A[a][c] lambda_a (dual LMs), lambda_c (standard)
+template <int NS, bool DUAL>
+__device__ __forceinline__ void lm_weights(const double* __restrict__ r, const V3* lam, V3* Lam) {
+  for (int c = 0; c < NS; ++c) {
+    if (DUAL) {
+      V3 acc = v3(0, 0, 0);
+      for (int a = 0; a < NS; ++a) acc = acc + r[SR_A + 4 * a + c] * lam[a];
+      Lam[c] = acc;
+    } else {
+      Lam[c] = lam[c];
+    }
+  }
+}
+
+// From a pair's sums (G, H, map-coefficient adjoints smb and mmb, adjoints Bu,
+// Bv of the polygon's vertices at their pool slots): the reverse of clip,
+// projection and plane, the direct terms and J; and the forward blocks if
+// `blocks`.  Outputs go out with streaming (evict-first) stores: each is
+// written once and read by a later kernel, and L2 keeps the threads' stack
+// lines instead.
+template <int NS, int NM, bool SEG, bool DUAL>
+__device__ __forceinline__ void adjoint_finish(int64_t p, int32_t s, int32_t m, const double* __restrict__ r,
+                                               const double* __restrict__ xs, const double* __restrict__ xm,
+                                               const int32_t* __restrict__ conn_s,
+                                               const int32_t* __restrict__ conn_m, const double* __restrict__ lambda,
+                                               const ClipPool<NS, NM>& cp, double* Bu, double* Bv, bool mrev,
+                                               const double* smb, const double* mmb, const double G[4][4],
+                                               const double H[4][4], bool blocks, double* __restrict__ gs_out,
+                                               double* __restrict__ gm_out, double* __restrict__ ab_out,
+                                               double* __restrict__ J_out, const FwdOut& fo) {
+  const int32_t* cs = conn_s + (int64_t)NS * s;
+  const int32_t* cm = conn_m + (int64_t)NM * m;
+  const V3 x0 = v3(r[SR_X0], r[SR_X0 + 1], r[SR_X0 + 2]);
+  const V3 t1 = v3(r[SR_T1], r[SR_T1 + 1], r[SR_T1 + 2]);
+  const V3 t2 = v3(r[SR_T2], r[SR_T2 + 1], r[SR_T2 + 2]);
+  const bool srev = r[SR_REV] != 0.0;
+  double Jp = 0.0;
+  V3 Lb[4];
+  if (blocks) {   // forward: M = A G, D = A H of this pair
+    double* mo = fo.Mblk + 16 * p;
+    for (int a = 0; a < 4; ++a)
+      for (int l = 0; l < 4; ++l) {
+        double v = 0.0;
+        if (a < NS && l < NM) {
+          if (DUAL)
+            for (int c = 0; c < NS; ++c) v += r[SR_A + 4 * a + c] * G[c][l];
+          else
+            v = G[a][l];
+        }
+        __stcs(mo + 4 * a + l, v);
+      }
+    if (SEG) {
+      double* dout = fo.Dblk + 16 * p;
+      for (int a = 0; a < 4; ++a)
+        for (int b = 0; b < 4; ++b) {
+          double v = 0.0;
+          if (a < NS && b < NS) {
+            if (DUAL)
+              for (int c = 0; c < NS; ++c) v += r[SR_A + 4 * a + c] * H[c][b];
+            else
+              v = H[a][b];
+          }
+          __stcs(dout + 4 * a + b, v);
+        }
+    }
+    __stcs(fo.flag + p, (uint8_t)1);
+  }
+  // ---- reverse merge and clipping (vertex pool) and the element maps
+  double sbu[4] = {0, 0, 0, 0}, sbv[4] = {0, 0, 0, 0}, mbu[4] = {0, 0, 0, 0}, mbv[4] = {0, 0, 0, 0};
+  cp.reverse(r, Bu, Bv, srev, mrev, sbu, sbv, mbu, mbv);
+  map_coeff_reverse<NS>(smb, sbu, sbv);
+  map_coeff_reverse<NM>(mmb, mbu, mbv);
+  // ---- direct terms and J from the forward accumulators, then the
+  //      reverse of the projection onto the auxiliary plane
+  V3 X[4], Y[4], lam[4], Lam[4];
+  load_pair_nodes<NS, NM>(cs, cm, xs, xm, lambda, X, Y, lam);
+  lm_weights<NS, DUAL>(r, lam, Lam);
+  double gX[4][3], gY[4][3];
+  for (int a = 0; a < 4; ++a)
+    for (int k = 0; k < 3; ++k) { gX[a][k] = 0.0; gY[a][k] = 0.0; }
+  for (int c = 0; c < NS; ++c) {
+    V3 acc = v3(0, 0, 0);
+    if (SEG)
+      for (int b = 0; b < NS; ++b) acc = acc + H[c][b] * X[b];
+    for (int l = 0; l < NM; ++l) acc = acc - G[c][l] * Y[l];
+    Lb[c] = acc;
+    Jp += dot(Lam[c], acc);
+  }
+  for (int l = 0; l < NM; ++l) {
+    V3 acc = v3(0, 0, 0);
+    for (int c = 0; c < NS; ++c) acc = acc + G[c][l] * Lam[c];
+    gY[l][0] -= acc.x; gY[l][1] -= acc.y; gY[l][2] -= acc.z;
+  }
+  if (SEG)
+    for (int b = 0; b < NS; ++b) {
+      V3 acc = v3(0, 0, 0);
+      for (int c = 0; c < NS; ++c) acc = acc + H[c][b] * Lam[c];
+      gX[b][0] += acc.x; gX[b][1] += acc.y; gX[b][2] += acc.z;
+    }
+  const V3 n0 = v3(r[SR_N0], r[SR_N0 + 1], r[SR_N0 + 2]);
+  plane_reverse<NS, NM>(X, Y, x0, t1, t2, n0, sbu, sbv, mbu, mbv, gX, gY);
+  double* go = gs_out + 12 * p;
+  double* gmo = gm_out + 12 * p;
+  for (int a = 0; a < 4; ++a)
+    for (int k = 0; k < 3; ++k) {
+      __stcs(go + 3 * a + k, gX[a][k]);
+      __stcs(gmo + 3 * a + k, gY[a][k]);
+    }
+  if (DUAL) {
+    double* ab = ab_out + 16 * p;
+    for (int a = 0; a < 4; ++a)
+      for (int c = 0; c < 4; ++c) __stcs(ab + 4 * a + c, (a < NS && c < NS) ? dot(lam[a], Lb[c]) : 0.0);
+  }
+  __stcs(J_out + p, Jp);
+}
+
+// Outputs of a pair without a polygon.
+template <bool SEG, bool DUAL>
+__device__ __forceinline__ void adjoint_empty(int64_t p, double* __restrict__ gs_out, double* __restrict__ gm_out,
+                                              double* __restrict__ ab_out, double* __restrict__ J_out,
+                                              const FwdOut& fo) {
+  double2* g1 = reinterpret_cast<double2*>(gs_out + 12 * p);
+  double2* g2 = reinterpret_cast<double2*>(gm_out + 12 * p);
+  for (int k = 0; k < 6; ++k) { __stcs(g1 + k, make_double2(0.0, 0.0)); __stcs(g2 + k, make_double2(0.0, 0.0)); }
+  if (DUAL) {
+    double2* a2 = reinterpret_cast<double2*>(ab_out + 16 * p);
+    for (int k = 0; k < 8; ++k) __stcs(a2 + k, make_double2(0.0, 0.0));
+  }
+  {
+    double2* mo = reinterpret_cast<double2*>(fo.Mblk + 16 * p);
+    for (int k = 0; k < 8; ++k) __stcs(mo + k, make_double2(0.0, 0.0));
+    if (SEG) {
+      double2* dd = reinterpret_cast<double2*>(fo.Dblk + 16 * p);
+      for (int k = 0; k < 8; ++k) __stcs(dd + k, make_double2(0.0, 0.0));
+    }
+    __stcs(fo.flag + p, (uint8_t)0);
+  }
+  __stcs(J_out + p, 0.0);
+}
+
 // ---------------------------------------------------------------- variant 0
 // Same functional, reorganised for the FP64 pipe:
 //  * the per-point work is written in the monomial basis of the shape
@@ -299,50 +458,22 @@ __global__ void __launch_bounds__(kMaxPairBlock) k_adjoint_pairs(
 //  * the clip is recorded as a compact vertex pool (ClipPool);
 //  * a warp sorts its batch of pairs by the cell count and edge
 //    intersections of an FP32 clip before the sweep.
-template <int NS, int NM, bool SEG, bool DUAL, bool FWD>
-__device__ void adjoint_pair_fast(int64_t p, const int32_t* __restrict__ ps, const int32_t* __restrict__ pm,
+template <int NS, int NM, bool SEG, bool DUAL>
+__device__ __noinline__ void adjoint_pair_fast(int64_t p, const int32_t* __restrict__ ps, const int32_t* __restrict__ pm,
                                   const double* __restrict__ srec, const double* __restrict__ xs,
                                   const double* __restrict__ xm, const int32_t* __restrict__ conn_s,
                                   const int32_t* __restrict__ conn_m, const double* __restrict__ lambda,
                                   double* __restrict__ gs_out, double* __restrict__ gm_out,
                                   double* __restrict__ ab_out, double* __restrict__ J_out,
-                                  const FwdOut& fo, AdjCounters& ctr, double* __restrict__ csh, int cstride) {
+                                  const FwdOut& fo, AdjCounters& ctr) {
   constexpr int KS = NS, KM = NM;   // monomials per side (quad4: 4, tri3: 3)
-  // CY (and [seg] SX) live in this thread's slice of shared memory, entry k
-  // at csh[k * cstride] (interleaved across the block's threads: no bank
-  // conflicts); they are read at every quadrature point and would otherwise
-  // hold 32 (64) registers through the loop
-  auto CYs = [&](int i, int j) -> double& { return csh[(4 * i + j) * cstride]; };
-  auto SXs = [&](int i, int j) -> double& { return csh[(16 + 4 * i + j) * cstride]; };
+  double CYv[16], SXv[SEG ? 16 : 1];
+  auto CYs = [&](int i, int j) -> double& { return CYv[4 * i + j]; };
+  auto SXs = [&](int i, int j) -> double& { return SXv[4 * i + j]; };
   const int32_t s = ps[p], m = pm[p];
   const double* r = srec + (int64_t)SR_STRIDE * s;
   const int32_t* cs = conn_s + (int64_t)NS * s;
   const int32_t* cm = conn_m + (int64_t)NM * m;
-  // Node coordinates and multipliers are read here for the set-up and read
-  // again (from L1/L2) after the quadrature loop: keeping them in registers
-  // across the loop would spill.
-  auto load_nodes = [&](V3* X, V3* Y, V3* lam) {
-    for (int a = 0; a < NS; ++a) {
-      const int64_t n = cs[a];
-      X[a] = v3(xs[3 * n], xs[3 * n + 1], xs[3 * n + 2]);
-      lam[a] = v3(lambda[3 * n], lambda[3 * n + 1], lambda[3 * n + 2]);
-    }
-    for (int l = 0; l < NM; ++l) {
-      const int64_t n = cm[l];
-      Y[l] = v3(xm[3 * n], xm[3 * n + 1], xm[3 * n + 2]);
-    }
-  };
-  auto lm_weights = [&](const V3* lam, V3* Lam) {   // Lambda_c = sum_a A[a][c] lambda_a (dual), lambda_c
-    for (int c = 0; c < NS; ++c) {
-      if (DUAL) {
-        V3 acc = v3(0, 0, 0);
-        for (int a = 0; a < NS; ++a) acc = acc + r[SR_A + 4 * a + c] * lam[a];
-        Lam[c] = acc;
-      } else {
-        Lam[c] = lam[c];
-      }
-    }
-  };
   const V3 x0 = v3(r[SR_X0], r[SR_X0 + 1], r[SR_X0 + 2]);
   const V3 t1 = v3(r[SR_T1], r[SR_T1 + 1], r[SR_T1 + 2]);
   const V3 t2 = v3(r[SR_T2], r[SR_T2 + 1], r[SR_T2 + 2]);
@@ -360,19 +491,16 @@ __device__ void adjoint_pair_fast(int64_t p, const int32_t* __restrict__ ps, con
   double ma2 = 0.0;
   for (int l = 0; l < NM; ++l) ma2 += cross2(mu[l], mv[l], mu[(l + 1) % NM], mv[(l + 1) % NM]);
   const bool mrev = ma2 < 0.0;
-  const bool srev = r[SR_REV] != 0.0;
   // ---- forward clip recorded as a vertex pool, and merge (same decisions as clip_polygon)
   ClipPool<NS, NM> cp;
   const bool nonempty = cp.run(r, mu, mv, mrev, ctr.clip_over);
   const int nr = cp.nr;
-  double Jp = 0.0;
-  V3 Lb[4];
   if (nonempty) {
     // monomial coefficients and the pair's bilinear forms
     {
       V3 X[4], Y[4], lam[4], Lam[4], LM[4], YM[4];
-      load_nodes(X, Y, lam);
-      lm_weights(lam, Lam);
+      load_pair_nodes<NS, NM>(cs, cm, xs, xm, lambda, X, Y, lam);
+      lm_weights<NS, DUAL>(r, lam, Lam);
       nodal_to_mono<NS>(Lam, LM);
       nodal_to_mono<NM>(Y, YM);
 #pragma unroll
@@ -435,7 +563,7 @@ __device__ void adjoint_pair_fast(int64_t p, const int32_t* __restrict__ ps, con
       const double cr = cross2(e1u, e1v, e2u, e2v);
       const double area = 0.5 * fabs(cr);
       double area_b = 0.0, e1bu = 0.0, e1bv = 0.0, e2bu = 0.0, e2bv = 0.0, abu = 0.0, abv = 0.0;
-      if (FWD) { ctr.cells++; ctr.gp += 7; }
+ctr.cells++; ctr.gp += 7;
 #pragma unroll 1
       for (int q = 0; q < 7; ++q) {
         double l1, l2, w;
@@ -572,214 +700,452 @@ __device__ void adjoint_pair_fast(int64_t p, const int32_t* __restrict__ ps, con
       const double inv = kInvCount[nr];
       for (int k = 0; k < nr; ++k) { const int sk = cp.id(k); Bu[sk] += cbu * inv; Bv[sk] += cbv * inv; }
     }
-    // Outputs go out with streaming (evict-first) stores: each is written once
-    // and read by a later kernel, and L2 keeps the threads' stack lines instead.
-    if (FWD) {   // fused forward: M = A G, D = A H of this pair
-      ctr.nonempty++;
-      double* mo = fo.Mblk + 16 * p;
-      for (int a = 0; a < 4; ++a)
-        for (int l = 0; l < 4; ++l) {
-          double v = 0.0;
-          if (a < NS && l < NM) {
-            if (DUAL)
-              for (int c = 0; c < NS; ++c) v += r[SR_A + 4 * a + c] * G[c][l];
-            else
-              v = G[a][l];
-          }
-          __stcs(mo + 4 * a + l, v);
-        }
-      if (SEG) {
-        double* dout = fo.Dblk + 16 * p;
-        for (int a = 0; a < 4; ++a)
-          for (int b = 0; b < 4; ++b) {
-            double v = 0.0;
-            if (a < NS && b < NS) {
-              if (DUAL)
-                for (int c = 0; c < NS; ++c) v += r[SR_A + 4 * a + c] * H[c][b];
-              else
-                v = H[a][b];
-            }
-            __stcs(dout + 4 * a + b, v);
-          }
-      }
-      __stcs(fo.flag + p, (uint8_t)1);
-    }
-    // ---- reverse merge and clipping (vertex pool) and the element maps
-    double sbu[4] = {0, 0, 0, 0}, sbv[4] = {0, 0, 0, 0}, mbu[4] = {0, 0, 0, 0}, mbv[4] = {0, 0, 0, 0};
-    cp.reverse(r, Bu, Bv, srev, mrev, sbu, sbv, mbu, mbv);
-    map_coeff_reverse<NS>(smb, sbu, sbv);
-    map_coeff_reverse<NM>(mmb, mbu, mbv);
-    // ---- direct terms and J from the forward accumulators, then the
-    //      reverse of the projection onto the auxiliary plane
-    V3 X[4], Y[4], lam[4], Lam[4];
-    load_nodes(X, Y, lam);
-    lm_weights(lam, Lam);
-    double gX[4][3], gY[4][3];
-    for (int a = 0; a < 4; ++a)
-      for (int k = 0; k < 3; ++k) { gX[a][k] = 0.0; gY[a][k] = 0.0; }
-    for (int c = 0; c < NS; ++c) {
-      V3 acc = v3(0, 0, 0);
-      if (SEG)
-        for (int b = 0; b < NS; ++b) acc = acc + H[c][b] * X[b];
-      for (int l = 0; l < NM; ++l) acc = acc - G[c][l] * Y[l];
-      Lb[c] = acc;
-      Jp += dot(Lam[c], acc);
-    }
-    for (int l = 0; l < NM; ++l) {
-      V3 acc = v3(0, 0, 0);
-      for (int c = 0; c < NS; ++c) acc = acc + G[c][l] * Lam[c];
-      gY[l][0] -= acc.x; gY[l][1] -= acc.y; gY[l][2] -= acc.z;
-    }
-    if (SEG)
-      for (int b = 0; b < NS; ++b) {
-        V3 acc = v3(0, 0, 0);
-        for (int c = 0; c < NS; ++c) acc = acc + H[c][b] * Lam[c];
-        gX[b][0] += acc.x; gX[b][1] += acc.y; gX[b][2] += acc.z;
-      }
-    const V3 n0 = v3(r[SR_N0], r[SR_N0 + 1], r[SR_N0 + 2]);
-    plane_reverse<NS, NM>(X, Y, x0, t1, t2, n0, sbu, sbv, mbu, mbv, gX, gY);
-    double* go = gs_out + 12 * p;
-    double* gmo = gm_out + 12 * p;
-    for (int a = 0; a < 4; ++a)
-      for (int k = 0; k < 3; ++k) {
-        __stcs(go + 3 * a + k, gX[a][k]);
-        __stcs(gmo + 3 * a + k, gY[a][k]);
-      }
-    if (DUAL) {
-      double* ab = ab_out + 16 * p;
-      for (int a = 0; a < 4; ++a)
-        for (int c = 0; c < 4; ++c) __stcs(ab + 4 * a + c, (a < NS && c < NS) ? dot(lam[a], Lb[c]) : 0.0);
-    }
+    adjoint_finish<NS, NM, SEG, DUAL>(p, s, m, r, xs, xm, conn_s, conn_m, lambda, cp, Bu, Bv, mrev, smb, mmb, G, H, true,
+                                      gs_out, gm_out, ab_out, J_out, fo);
+    ctr.nonempty++;
   } else {
-    double2* g1 = reinterpret_cast<double2*>(gs_out + 12 * p);
-    double2* g2 = reinterpret_cast<double2*>(gm_out + 12 * p);
-    for (int k = 0; k < 6; ++k) { __stcs(g1 + k, make_double2(0.0, 0.0)); __stcs(g2 + k, make_double2(0.0, 0.0)); }
-    if (DUAL) {
-      double2* a2 = reinterpret_cast<double2*>(ab_out + 16 * p);
-      for (int k = 0; k < 8; ++k) __stcs(a2 + k, make_double2(0.0, 0.0));
-    }
-    if (FWD) {
-      double2* mo = reinterpret_cast<double2*>(fo.Mblk + 16 * p);
-      for (int k = 0; k < 8; ++k) __stcs(mo + k, make_double2(0.0, 0.0));
-      if (SEG) {
-        double2* dd = reinterpret_cast<double2*>(fo.Dblk + 16 * p);
-        for (int k = 0; k < 8; ++k) __stcs(dd + k, make_double2(0.0, 0.0));
-      }
-      __stcs(fo.flag + p, (uint8_t)0);
-    }
+    adjoint_empty<SEG, DUAL>(p, gs_out, gm_out, ab_out, J_out, fo);
   }
-  __stcs(J_out + p, Jp);
 }
 
-// shared-memory coefficients per thread of the batched adjoint kernel: CY and [seg] SX
-template <bool SEG>
-constexpr int kAdjCoef = SEG ? 32 : 16;
+// Words of the clip record in a pair's adjoint record.
+template <int NS, int NM>
+__device__ __forceinline__ void store_pool(long long* o, const ClipPool<NS, NM>& cp, bool mrev) {
+  constexpr int K = ClipPool<NS, NM>::kSlots;
+  static_assert(K == 12, "record layout");
+  o += 32 * AdjRecord::kPool;
+  for (int k = 0; k < cp.nv; ++k) {
+    o[32 * k] = __double_as_longlong(cp.pu[k]);
+    o[32 * (K + k)] = __double_as_longlong(cp.pv[k]);
+    if (k >= NM) o[32 * (2 * K + k)] = __double_as_longlong(cp.tt[k]);
+  }
+#pragma unroll
+  for (int w = 0; w < 3; ++w) {
+    unsigned long long v = 0;
+    for (int k = 0; k < 4; ++k)
+      if (4 * w + k >= NM && 4 * w + k < cp.nv) v |= (unsigned long long)cp.meta[4 * w + k] << (16 * k);
+    o[32 * (3 * K + w)] = (long long)v;
+  }
+  o[32 * (3 * K + 3)] = (long long)cp.poly;
+  o[32 * (3 * K + 4)] = cp.nv | cp.nr << 8 | (mrev ? 1 : 0) << 16;
+}
+template <int NS, int NM>
+__device__ __forceinline__ bool load_pool(const long long* o, ClipPool<NS, NM>& cp) {
+  constexpr int K = ClipPool<NS, NM>::kSlots;
+  o += 32 * AdjRecord::kPool;
+  const int n = (int)o[32 * (3 * K + 4)];
+  cp.nv = n & 0xff;
+  cp.nr = n >> 8 & 0xff;
+  cp.poly = (uint64_t)o[32 * (3 * K + 3)];
+  for (int k = 0; k < cp.nv; ++k) {
+    cp.pu[k] = __longlong_as_double(o[32 * k]);
+    cp.pv[k] = __longlong_as_double(o[32 * (K + k)]);
+    if (k >= NM) {
+      cp.tt[k] = __longlong_as_double(o[32 * (2 * K + k)]);
+      cp.meta[k] = (uint16_t)(o[32 * (3 * K + (k >> 2))] >> (16 * (k & 3)));
+    }
+  }
+  return (n >> 16 & 1) != 0;
+}
 
-template <int NS, int NM, bool SEG, bool DUAL, bool FWD, int R>
-__global__ void __launch_bounds__(kMaxPairBlock) k_adjoint_batched(
-    const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
-    const double* __restrict__ xs, const double* __restrict__ xm, const int32_t* __restrict__ conn_s,
-    const int32_t* __restrict__ conn_m, const double* __restrict__ lambda, int64_t pair_cap,
-    double* __restrict__ gs_out, double* __restrict__ gm_out, double* __restrict__ ab_out,
-    double* __restrict__ J_out, FwdOut fo, DevStatus* st, unsigned long long* cta_t, int32_t watchdog_us) {
+constexpr int kSlowPair = 0xff;   // nr of a record whose pair the finish kernel runs in FP64
+
+struct AdjArgs {
+  const int32_t* ps;
+  const int32_t* pm;
+  const double* srec;
+  const double* xs;
+  const double* xm;
+  const int32_t* conn_s;
+  const int32_t* conn_m;
+  const double* lambda;
+  int64_t pair_cap;
+  const int32_t* order;
+  long long* rec;
+  double* gs;
+  double* gm;
+  double* ab;
+  double* J;
+  FwdOut fo;
+  DevStatus* st;
+  int32_t watchdog_us;
+};
+
+// Group of 32 pairs for a warp; false when none are left.
+__device__ __forceinline__ bool next_group(unsigned long long* ctr, int64_t n, int64_t& g) {
+  unsigned long long v = 0;
+  if ((threadIdx.x & 31) == 0) v = atomicAdd(ctr, 1ull);
+  g = (int64_t)__shfl_sync(0xffffffffu, v, 0);
+  return 32 * g < n;
+}
+
+// First kernel of the default adjoint (variant 0; the forward blocks come with
+// it): FP64 clip with its record, the pair's bilinear forms CY [and SX], and
+// the conversion to fixed point.  One record per pair, in sorted order.
+template <int NS, int NM, bool SEG, bool DUAL>
+__global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, unsigned long long* cta_t) {
   cta_mark(cta_t, 0);
-  constexpr int B = 32 * R;
-  using PermT = typename std::conditional<(B > 256), uint16_t, uint8_t>::type;
-  __shared__ PermT perm_s[kMaxPairBlock / 32][B];
-  __shared__ uint8_t key_s[kMaxPairBlock / 32][B];
-  __shared__ unsigned pres_s[kMaxPairBlock / 32][8];   // key values present in the batch (256 bits)
-  extern __shared__ double adj_coef[];   // kAdjCoef doubles per thread, interleaved
-  PermT* perm = perm_s[threadIdx.x >> 5];
-  uint8_t* keys = key_s[threadIdx.x >> 5];
-  unsigned* pres = pres_s[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31;
-  const unsigned lt_mask = (1u << lane) - 1u;
+  constexpr int W = SEG ? AdjRecord::kWordsSeg : AdjRecord::kWords;
   AdjCounters ctr;
-  const bool ok = st->over_pairs == 0 && st->over_bins == 0;
-  const int64_t n = ok ? (int64_t)min((unsigned long long)pair_cap, st->n_pairs) : 0;
-  // guided self-scheduling: a warp takes half an even share of the pairs
-  // left (at most B, at least 32, a multiple of 32), so batches are full
-  // while there is plenty of work and shrink towards the end of the queue
-  const int64_t share = 2 * (int64_t)gridDim.x * (blockDim.x >> 5);
-  const Watchdog wd(watchdog_us);
-  for (;;) {   // bounded: the shared counter only grows
-    if (wd.expired(&st->timeout)) break;
-    int64_t base = 0;
-    int fetch = B;
-    if (lane == 0) {
-      const unsigned long long seen = *reinterpret_cast<volatile unsigned long long*>(&st->work_ctr2);
-      const int64_t f = (n - (int64_t)seen) / share;
-      fetch = f >= B ? B : (f < 32 ? 32 : (int)(f & ~31ll));
-      base = (int64_t)atomicAdd(&st->work_ctr2, (unsigned long long)fetch);
-    }
-    base = __shfl_sync(0xffffffffu, base, 0);
-    fetch = __shfl_sync(0xffffffffu, fetch, 0);
-    if (base >= n) break;
-    const int64_t lim = min(n, base + (int64_t)fetch);
-    const int rounds = (fetch + 31) >> 5;
-    // phase A: sort key of each pair from an FP32 clip: 1 + 16 x its cell
-    // count + its edge intersections (cells 0 = empty in FP32; key 0 = no
-    // pair).  The cell count sets the quadrature work, the intersections the
-    // divergent clip and reverse-clip work.  Every pair goes through phase B,
-    // where the FP64 clip decides what it contributes.
-    if (lane < 8) pres[lane] = 0u;
-    __syncwarp();
-#pragma unroll 1
-    for (int rr = 0; rr < rounds; ++rr) {
-      const int64_t p = base + rr * 32 + lane;
-      int key = 0;
-      if (p < lim) {
-        int n_int = 0;
-        const int nr = clip_count_f32<NS, NM>(srec + (int64_t)SR_STRIDE * ps[p], xm, conn_m, pm[p], n_int);
-        key = 1 + 16 * (nr == 0 ? 0 : (nr == 3 ? 1 : min(nr, kPolyS))) + min(n_int, 15);
-        atomicOr(&pres[key >> 5], 1u << (key & 31));
+  DevStatus* st = g.st;
+  const bool run = st->over_pairs == 0 && st->over_bins == 0;
+  const int64_t n = run ? (int64_t)min((unsigned long long)g.pair_cap, st->n_pairs) : 0;
+  const Watchdog wd(g.watchdog_us);
+  int64_t grp;
+  while (!wd.expired(&st->timeout) && next_group(&st->work_ctr2, n, grp)) {   // bounded: the counter only grows
+    const int64_t i = 32 * grp + (threadIdx.x & 31);
+    long long* o = g.rec + grp * (32 * W) + (threadIdx.x & 31);
+    int mark = 0;   // nr of a record with nothing for the cell kernel
+    if (i < n) {
+      const int64_t p = g.order[i];
+      const int32_t s = g.ps[p], m = g.pm[p];
+      const double* r = g.srec + (int64_t)SR_STRIDE * s;
+      const int32_t* cm = g.conn_m + (int64_t)NM * m;
+      o[32 * FxRecord::kPair] = p;
+      double mu[4], mv[4];
+      for (int l = 0; l < NM; ++l) {
+        const int64_t nd = cm[l];
+        const double dx = g.xm[3 * nd] - r[SR_X0], dy = g.xm[3 * nd + 1] - r[SR_X0 + 1],
+                     dz = g.xm[3 * nd + 2] - r[SR_X0 + 2];
+        mu[l] = dx * r[SR_T1] + dy * r[SR_T1 + 1] + dz * r[SR_T1 + 2];
+        mv[l] = dx * r[SR_T2] + dy * r[SR_T2 + 1] + dz * r[SR_T2 + 2];
       }
-      keys[rr * 32 + lane] = (uint8_t)key;
-    }
-    __syncwarp();
-    // counting sort of the batch by key, descending, over the key values
-    // present (ballots per value)
-    int basecnt = 0;
-#pragma unroll 1
-    for (int w = 7; w >= 0; --w) {
-      unsigned bits = pres[w];
-      while (bits != 0u) {   // uniform across the warp
-        const int b = 31 - __clz(bits);
-        bits &= ~(1u << b);
-        const int v = 32 * w + b;
-        int before = 0;
-#pragma unroll 1
-        for (int rr = 0; rr < rounds; ++rr) {
-          const int slot = rr * 32 + lane;
-          const bool hit = keys[slot] == v;
-          const unsigned mk = __ballot_sync(0xffffffffu, hit);
-          if (hit) perm[basecnt + before + __popc(mk & lt_mask)] = (PermT)slot;
-          before += __popc(mk);
+      const PlaneMap mmap = plane_map<NM>(mu, mv);
+      double ma2 = 0.0;
+      for (int l = 0; l < NM; ++l) ma2 += cross2(mu[l], mv[l], mu[(l + 1) % NM], mv[(l + 1) % NM]);
+      const bool mrev = ma2 < 0.0;
+      ClipPool<NS, NM> cp;
+      if (!cp.run(r, mu, mv, mrev, ctr.clip_over)) {
+        adjoint_empty<SEG, DUAL>(p, g.gs, g.gm, g.ab, g.J, g.fo);
+      } else {
+        store_pool(o, cp, mrev);
+        double pu[FxPolygon::kCap], pv[FxPolygon::kCap];
+        for (int k = 0; k < min(cp.nr, FxPolygon::kCap); ++k) {
+          pu[k] = cp.u(k);
+          pv[k] = cp.v(k);
         }
-        basecnt += before;
+        FxPolygon f;
+        mark = kSlowPair;
+        if (f.setup<NS, NM>(r, mmap, pu, pv, cp.nr)) {
+          // bilinear forms of the pair, and their scales
+          V3 X[4], Y[4], lam[4], LM[4], YM[4];
+          load_pair_nodes<NS, NM>(g.conn_s + (int64_t)NS * s, cm, g.xs, g.xm, g.lambda, X, Y, lam);
+          {
+            V3 Lam[4];
+            lm_weights<NS, DUAL>(r, lam, Lam);
+            nodal_to_mono<NS>(Lam, LM);
+          }
+          nodal_to_mono<NM>(Y, YM);
+          double C[4][4], S[4][4];
+#pragma unroll
+          for (int a = 0; a < NS; ++a)
+#pragma unroll
+            for (int b = 0; b < NM; ++b) C[a][b] = dot(LM[a], YM[b]);
+          if (SEG) {
+            V3 XM[4];
+            nodal_to_mono<NS>(X, XM);
+#pragma unroll
+            for (int a = 0; a < NS; ++a)
+#pragma unroll
+              for (int b = 0; b < NS; ++b) S[a][b] = dot(LM[a], XM[b]);
+#pragma unroll
+            for (int a = 0; a < NS; ++a)
+#pragma unroll
+              for (int b = 0; b <= a; ++b) {
+                S[a][b] += S[b][a];   // a == b: doubled
+                S[b][a] = S[a][b];
+              }
+          }
+          AdjScale sc;
+          sc.kys = fx_inverse_exponent(f.s);
+          sc.kym = fx_inverse_exponent(f.m);
+          sc.eu = f.su;
+          sc.ev = f.sv;
+          // out of range: multipliers beyond FP32, or nearly singular maps
+          if (sc.set<NS, NM, SEG>(C, S) && sc.kys < 20 && sc.kym < 20) {
+            FxRecord::store<NS, NM>(o, f, p);
+            auto put = [&](int w, double v, int sc) {
+              const Dg d = fx_split(fx_of_double(v, 62 - sc));
+              o[32 * w] = (long long)(((unsigned long long)(unsigned)d.h << 32) | (unsigned)d.l);
+            };
+#pragma unroll
+            for (int a = 0; a < NS; ++a) {
+              put(AdjRecord::kC0 + a, C[a][0], a == 0 ? sc.s0 : sc.sv);
+#pragma unroll
+              for (int b = 1; b < NM; ++b) put(AdjRecord::kC1 + 3 * a + b - 1, C[a][b], a == 0 ? sc.s1 : sc.s11);
+              if (SEG)
+#pragma unroll
+                for (int b = 0; b < NS; ++b) put(AdjRecord::kSX + 4 * a + b, S[a][b], a == 0 ? sc.s0 : sc.sv);
+            }
+            o[32 * AdjRecord::kScales] = sc.word1();
+            o[32 * AdjRecord::kScales2] = sc.word2();
+            mark = -1;
+            ctr.cells += f.ncell;
+            ctr.gp += 7 * f.ncell;
+            ctr.nonempty++;
+          }
+        }
       }
     }
-    const int n_live = basecnt;
-    __syncwarp();
-    // phase B: full adjoint of each pair, rounds of similar cost
-    for (int i0 = 0; i0 < n_live; i0 += 32) {
-      const int i = i0 + lane;
-      if (i < n_live)
-        adjoint_pair_fast<NS, NM, SEG, DUAL, FWD>(base + perm[i], ps, pm, srec, xs, xm, conn_s, conn_m, lambda,
-                                                  gs_out, gm_out, ab_out, J_out, fo, ctr, adj_coef + threadIdx.x,
-                                                  (int)blockDim.x);
-    }
+    if (mark >= 0) o[32 * FxRecord::kInfo] = mark;
     __syncwarp();
   }
   block_count_add(&st->clip_overflow, ctr.clip_over);
-  block_count_add(&st->newton_fail, ctr.newton_fail);
-  if (FWD) {
-    block_count_add(&st->nonempty, ctr.nonempty);
-    block_count_add(&st->cells, ctr.cells);
-    block_count_add(&st->gauss_points, ctr.gp);
-  }
+  block_count_add(&st->nonempty, ctr.nonempty);
+  block_count_add(&st->cells, ctr.cells);
+  block_count_add(&st->gauss_points, ctr.gp);
   __syncthreads();
   cta_mark(cta_t, 1);
+}
+
+// Sums g of every pair's cells, entry by entry by the pair's lanes in turn,
+// into record words w0 + 4 a + l as FP64.  buf as in the quadrature kernel.
+template <int NS, int NC>
+__device__ __forceinline__ void pair_products(const FxAcc g[4][4], const CellSlot& cs, bool ok, int ke,
+                                              const FxScales& ss, const FxScales& sc, long long* __restrict__ o,
+                                              int w0, long long* __restrict__ buf, int stride) {
+  __syncwarp();
+#pragma unroll
+  for (int a = 0; a < NS; ++a)
+#pragma unroll
+    for (int l = 0; l < NC; ++l) {
+      const int e = NC * a + l;
+      buf[e * stride] = g[a][l].hh + (g[a][l].cr >> 32);
+      reinterpret_cast<unsigned*>(buf + (16 + (e >> 1)) * stride)[e & 1] = (unsigned)g[a][l].cr;
+    }
+  __syncwarp();
+  const long long* pair = buf - (threadIdx.x & 31) + cs.first;
+  if (ok)
+#pragma unroll 1
+    for (int e = cs.cell; e < NS * NC; e += cs.cells) {
+      const int a = e / NC, l = e - NC * a;
+      long long hh = 0, cr = 0;
+      for (int k = 0; k < cs.cells; ++k) {
+        hh += pair[e * stride + k];
+        cr += reinterpret_cast<const unsigned*>(pair + (16 + (e >> 1)) * stride + k)[e & 1];
+      }
+      o[32 * (w0 + 4 * a + l)] = __double_as_longlong(fx_to_double(hh, cr, ke - ss.shape<NS>(a) - sc.shape<NC>(l)));
+    }
+}
+
+constexpr int kAdjSlots = 58;      // shared 64-bit words per thread of the cell kernel: points, W y or sums
+constexpr int kCellThreads = 384;  // the registers of an SM at 168 a thread
+
+// Second kernel: one cell of a pair per lane, as k_pair_quadrature.  Leaves G
+// [and H], the map-coefficient adjoints and the polygon vertices' adjoints in
+// the record.
+template <int NS, int NM, bool SEG>
+__global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
+  constexpr int W = SEG ? AdjRecord::kWordsSeg : AdjRecord::kWords;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  long long* pts = reinterpret_cast<long long*>(smem_raw) + threadIdx.x;
+  const int stride = (int)blockDim.x;
+  long long* sums = pts + 28 * stride;
+  const int lane = threadIdx.x & 31;
+  DevStatus* st = ar.st;
+  const bool run = st->over_pairs == 0 && st->over_bins == 0;
+  const int64_t n = run ? (int64_t)min((unsigned long long)ar.pair_cap, st->n_pairs) : 0;
+  const int64_t groups = (n + 31) >> 5;
+  const int turn = (int)max((int64_t)1, min((int64_t)8, groups / (4 * (int64_t)gridDim.x * (blockDim.x >> 5))));
+  const Watchdog wd(ar.watchdog_us);
+  // The warps of a block run their rounds in step: every round costs the same
+  // (one cell per lane), and the round's code, about 3,000 instructions, does not
+  // fit the instruction cache that all warps of an SM share unless they are in
+  // the same part of it.  A warp takes a new turn when its last is used up.
+  int64_t r0 = 0;
+  int records = 0, w = 0;
+  bool more = true;
+  for (;;) {   // bounded: the shared counter only grows
+    if (w >= records && more) {
+      unsigned long long g0 = ~0ull;
+      if (!wd.expired(&st->timeout)) {
+        if (lane == 0) g0 = atomicAdd(&st->work_ctr4, (unsigned long long)turn);
+        g0 = __shfl_sync(0xffffffffu, g0, 0);
+      }
+      more = g0 < (unsigned long long)groups;
+      r0 = 32 * (int64_t)g0;
+      records = more ? 32 * (int)min((int64_t)turn, groups - (int64_t)g0) : 0;
+      w = 0;
+    }
+    if (!__syncthreads_or(w < records)) break;
+    int ncell = 0;
+    if (w + lane < records) {
+      const int64_t i = r0 + w + lane;
+      const int nr = (int)(ar.rec[((i >> 5) * W + FxRecord::kInfo) * 32 + (i & 31)] & 0xff);
+      ncell = nr == kSlowPair ? 0 : (nr > 3 ? nr : (nr == 3 ? 1 : 0));
+    }
+    const CellSlot cs = assign_cells(ncell);
+    const int64_t i = w < records ? r0 + w + cs.rec : 0;
+    w += cs.taken;
+    long long* o = ar.rec + (i >> 5) * (32 * W) + (i & 31);
+    bool ok = cs.cell >= 0;
+    FxView f;
+    AdjScale sc;
+    long long weight = 0, e1u = 0, e1v = 0, e2u = 0, e2v = 0;
+    if (ok) {
+      const int64_t p = o[32 * FxRecord::kPair];
+      f.load<NS, NM>(o);
+      sc.load(o[32 * AdjRecord::kScales], o[32 * AdjRecord::kScales2], f.ke, f.E);
+      weight = f.weight(cs.cell);
+      const int ib = f.ib(cs.cell), iw = f.iw(cs.cell);
+      e1u = f.x(ib) - f.cu; e1v = f.y(ib) - f.cv;
+      e2u = f.x(iw) - f.cu; e2v = f.y(iw) - f.cv;
+      ok = fx_back_project<NS, NM>(f, cs.cell, ar.srec + (int64_t)SR_STRIDE * ar.ps[p], ar.xm, ar.conn_m, ar.pm[p],
+                                   pts, stride);
+    }
+    __syncthreads();
+    long long area = 0;
+    if (ok) ok = fx_cell_sweep<NS, NM, SEG>(f.s, f.m, sc, o, weight, pts, stride, area);
+    const unsigned bad = __ballot_sync(0xffffffffu, cs.cell >= 0 && !ok);
+    const bool slow = cs.cell >= 0 && (bad >> cs.first & (cs.cells < 32 ? (1u << cs.cells) - 1u : ~0u)) != 0;
+    ok &= !slow;
+    // every lane of the pair has read the record by now: results take its words' places
+    __syncthreads();
+    {
+      AdjSums r;
+      fx_cell_moments<NS, NM>(pts, stride, r);
+      // map-coefficient adjoints: minus the sums of W y (x) (1, xi, eta, xi eta), units of 2^64 of Q61 x Q61
+      __syncwarp();
+      if (ok) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          const int c = e & 1, k = (e & 7) >> 1;
+          long long hh, cr;
+          if (k == 0) {
+            const long long v = e < 8 ? r.s1[c] : r.m1[c];
+            hh = v >> 3;
+            cr = (v & 7) << 29;
+          } else {
+            const FxAcc& a = e < 8 ? r.sx[k - 1][c] : r.mx[k - 1][c];
+            hh = a.hh + (a.cr >> 32);
+            cr = (long long)(unsigned)a.cr;
+          }
+          sums[e * stride] = hh;
+          reinterpret_cast<unsigned*>(sums + (16 + (e >> 1)) * stride)[e & 1] = (unsigned)cr;
+        }
+        // vertex adjoints of the cell: moments of both sides and the area's part,
+        // d area = +-(1/2)(e2v de1u - e2u de1v + e1u de2v - e1v de2u)
+        FxAcc a;
+        a.mul(fx_split(e1u), fx_split(e2v));
+        FxAcc b;
+        b.mul(fx_split(e1v), fx_split(e2u));
+        const bool neg = (a.hh - b.hh) + ((a.cr - b.cr) >> 32) < 0;
+        const Dg ar2 = fx_split(neg ? -area : area);
+        // one component of a vertex: the moments, and the area with the other component of an edge
+        auto part = [&](long long s, long long mv, long long e, int es, int xa, int xv) {
+          a.mul(ar2, fx_split(e << es));
+          return fx_down(s, xv - sc.xs) + fx_down(mv, xv - sc.xm) + fx_down(a.hh + (a.cr >> 32), xv - xa);
+        };
+        const long long v1u = part(r.es1[0], r.em1[0], e2v, sc.ev, sc.xav, sc.xvu);
+        const long long v1v = part(r.es1[1], r.em1[1], -e2u, sc.eu, sc.xau, sc.xvv);
+        const long long v2u = part(r.es2[0], r.em2[0], -e1v, sc.ev, sc.xav, sc.xvu);
+        const long long v2v = part(r.es2[1], r.em2[1], e1u, sc.eu, sc.xau, sc.xvv);
+        sums[24 * stride] = v1u; sums[25 * stride] = v1v;
+        sums[26 * stride] = v2u; sums[27 * stride] = v2v;
+        sums[28 * stride] = fx_down(r.s1[0], sc.xvu - sc.xs) + fx_down(r.m1[0], sc.xvu - sc.xm) - v1u - v2u;
+        sums[29 * stride] = fx_down(r.s1[1], sc.xvv - sc.xs) + fx_down(r.m1[1], sc.xvv - sc.xm) - v1v - v2v;
+      }
+      __syncwarp();
+      if (ok) {
+        const long long* pair = sums - lane + cs.first;
+#pragma unroll 1
+        for (int e = cs.cell; e < 16; e += cs.cells) {
+          long long hh = 0, cr = 0;
+          for (int k = 0; k < cs.cells; ++k) {
+            hh += pair[e * stride + k];
+            cr += reinterpret_cast<const unsigned*>(pair + (16 + (e >> 1)) * stride + k)[e & 1];
+          }
+          const double v = -fx_to_double(hh, cr, 3 + (e < 8 ? sc.xs : sc.xm));
+          o[32 * (AdjRecord::kMapS + e)] = __double_as_longlong(v);
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          long long* ov = o + 32 * (AdjRecord::kVertex + c);
+          const int xv = c == 0 ? sc.xvu : sc.xvv;
+          if (f.nr == 3) {   // one cell: its corner, then the two vertices
+            ov[0] = __double_as_longlong(fx_to_double(pair[(28 + c) * stride], 0, xv));
+            ov[64] = __double_as_longlong(fx_to_double(pair[(24 + c) * stride], 0, xv));
+            ov[128] = __double_as_longlong(fx_to_double(pair[(26 + c) * stride], 0, xv));
+          } else {   // vertex k: cell k's first, cell k - 1's second, 1 / nr of the centre's
+            long long centre = 0;
+            for (int k = 0; k < cs.cells; ++k) centre += pair[(28 + c) * stride + k];
+            FxAcc a;
+            a.mul(fx_split(centre), kInvCountFx.d[f.nr]);
+            const int prev = cs.cell == 0 ? cs.cells - 1 : cs.cell - 1;
+            const long long v = a.get<2>() + pair[(24 + c) * stride + cs.cell] + pair[(26 + c) * stride + prev];
+            ov[64 * cs.cell] = __double_as_longlong(fx_to_double(v, 0, xv));
+          }
+        }
+      }
+    }
+    __syncthreads();
+    {
+      FxAcc g[4][4];
+      FxAcc h[4][4];
+      if (SEG) fx_cell_products<NS, NS, true>(f.ss, f.ss, weight, pts, stride, h);
+      fx_cell_products<NS, NM, false>(f.ss, f.sm, weight, pts, stride, g);
+      if (SEG) pair_products<NS, NS>(h, cs, ok, f.ke, f.ss, f.ss, o, AdjRecord::kH, pts, stride);
+      pair_products<NS, NM>(g, cs, ok, f.ke, f.ss, f.sm, o, AdjRecord::kG, pts, stride);
+    }
+    if (slow && cs.cell == 0) o[32 * FxRecord::kInfo] = kSlowPair;
+  }
+}
+
+// Third kernel: per pair, the forward blocks, the reverse of clip, projection
+// and plane, the direct terms and J.
+template <int NS, int NM, bool SEG, bool DUAL>
+__global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_finish(AdjArgs g) {
+  constexpr int W = SEG ? AdjRecord::kWordsSeg : AdjRecord::kWords;
+  AdjCounters ctr;
+  DevStatus* st = g.st;
+  const bool run = st->over_pairs == 0 && st->over_bins == 0;
+  const int64_t n = run ? (int64_t)min((unsigned long long)g.pair_cap, st->n_pairs) : 0;
+  const Watchdog wd(g.watchdog_us);
+  int64_t grp;
+  while (!wd.expired(&st->timeout) && next_group(&st->work_ctr6, n, grp)) {   // bounded: the counter only grows
+    const long long* o = g.rec + grp * (32 * W) + (threadIdx.x & 31);
+    const int nr = (int)(o[32 * FxRecord::kInfo] & 0xff);
+    if (nr == kSlowPair) {
+      adjoint_pair_fast<NS, NM, SEG, DUAL>(o[32 * FxRecord::kPair], g.ps, g.pm, g.srec, g.xs, g.xm, g.conn_s, g.conn_m,
+                                           g.lambda, g.gs, g.gm, g.ab, g.J, g.fo, ctr);
+    } else if (nr != 0) {
+      const int64_t p = o[32 * FxRecord::kPair];
+      const int32_t s = g.ps[p], m = g.pm[p];
+      ClipPool<NS, NM> cp;
+      const bool mrev = load_pool(o, cp);
+      auto word = [&](int w) { return __longlong_as_double(o[32 * w]); };
+      double G[4][4], H[4][4], smb[8], mmb[8];
+#pragma unroll
+      for (int a = 0; a < NS; ++a) {
+#pragma unroll
+        for (int l = 0; l < NM; ++l) G[a][l] = word(AdjRecord::kG + 4 * a + l);
+        if (SEG)
+#pragma unroll
+          for (int b = 0; b < NS; ++b) H[a][b] = word(AdjRecord::kH + 4 * a + b);
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        smb[k] = word(AdjRecord::kMapS + k);
+        mmb[k] = word(AdjRecord::kMapM + k);
+      }
+      double Bu[ClipPool<NS, NM>::kSlots], Bv[ClipPool<NS, NM>::kSlots];
+      for (int k = 0; k < cp.nv; ++k) { Bu[k] = 0.0; Bv[k] = 0.0; }
+      for (int k = 0; k < cp.nr; ++k) {
+        const int id = cp.id(k);
+        Bu[id] += word(AdjRecord::kVertex + 2 * k);
+        Bv[id] += word(AdjRecord::kVertex + 2 * k + 1);
+      }
+      adjoint_finish<NS, NM, SEG, DUAL>(p, s, m, g.srec + (int64_t)SR_STRIDE * s, g.xs, g.xm, g.conn_s, g.conn_m,
+                                        g.lambda, cp, Bu, Bv, mrev, smb, mmb, G, H, true, g.gs, g.gm, g.ab, g.J, g.fo);
+    }
+    __syncwarp();
+  }
+  // pairs run here in FP64; the others were counted by the clip kernel
+  block_count_add(&st->clip_overflow, ctr.clip_over);
+  block_count_add(&st->newton_fail, ctr.newton_fail);
+  block_count_add(&st->nonempty, ctr.nonempty);
+  block_count_add(&st->cells, ctr.cells);
+  block_count_add(&st->gauss_points, ctr.gp);
 }
 
 // Constant tables of a flat element with dual LMs.  There Dh_a = d for every
@@ -1217,39 +1583,35 @@ void launch_pairs_t(mortar_ctx* c, const RunParams& rp, unsigned grid, unsigned 
       c->dstat.as<DevStatus>());
 }
 
-template <int NS, int NM, bool SEG, bool DUAL, bool FWD>
-void launch_batched_f(mortar_ctx* c, int rounds) {
-  const FwdOut fo{c->Mblk.as<double>(), c->Dblk.as<double>(), c->flag.as<uint8_t>()};
-  unsigned long long* cta_t = (FWD && c->timing && c->cta_t.p) ? c->cta_t.as<unsigned long long>() : nullptr;
-  const int block = c->block_size > 0 ? c->block_size : 128;
-  const size_t shm = (size_t)block * kAdjCoef<SEG> * sizeof(double);
-  auto go = [&](auto kern) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);   // > 48 KB at 256 threads
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, shm);
-    if (per_sm < 1) per_sm = 1;
-    const unsigned grid = (unsigned)(c->n_sm * per_sm);
-    if (cta_t) c->pair_grid = (int)grid;
-    kern<<<grid, block, shm, c->stream>>>(
-        c->pairs_s.as<int32_t>(), c->pairs_m.as<int32_t>(), c->srec.as<double>(), c->xs.as<double>(),
-        c->xm.as<double>(), c->conn_s.as<int32_t>(), c->conn_m.as<int32_t>(), c->lambda.as<double>(), c->pair_cap,
-        c->gs_pair.as<double>(), c->gm_pair.as<double>(), c->abar_pair.as<double>(), c->J_pair.as<double>(), fo,
-        c->dstat.as<DevStatus>(), cta_t, c->watchdog_us);
-  };
-  if (rounds <= 1) go(k_adjoint_batched<NS, NM, SEG, DUAL, FWD, 1>);
-  else if (rounds == 2) go(k_adjoint_batched<NS, NM, SEG, DUAL, FWD, 2>);
-  else if (rounds == 4) go(k_adjoint_batched<NS, NM, SEG, DUAL, FWD, 4>);
-  else if (rounds == 8) go(k_adjoint_batched<NS, NM, SEG, DUAL, FWD, 8>);
-  else if (rounds == 16) go(k_adjoint_batched<NS, NM, SEG, DUAL, FWD, 16>);
-  else go(k_adjoint_batched<NS, NM, SEG, DUAL, FWD, 32>);
-}
-
-// The warp-batched adjoint always produces the forward blocks as well (the
-// run pipeline fuses the two whenever the batched schedule is selected); a
-// non-fused call only rewrites the same blocks.
+// The default adjoint always produces the forward blocks as well (the run
+// pipeline fuses the two); a non-fused call only rewrites the same blocks.
 template <int NS, int NM, bool SEG, bool DUAL>
-void launch_batched_t(mortar_ctx* c, int rounds, bool) {
-  launch_batched_f<NS, NM, SEG, DUAL, true>(c, rounds);
+void launch_fixed(mortar_ctx* c, const RunParams& rp, int block, int rounds) {
+  IntegrateArgs ia{c->pairs_s.as<int32_t>(), c->pairs_m.as<int32_t>(), c->srec.as<double>(), c->xm.as<double>(),
+                   c->conn_m.as<int32_t>(), nullptr, nullptr, nullptr, c->pair_cap, c->dstat.as<DevStatus>(),
+                   c->stream};
+  ia.order = c->order.as<int32_t>();
+  launch_pair_sort<NS, NM>(ia, rp, c->n_sm, 32 * rounds);
+  const AdjArgs a{ia.ps, ia.pm, ia.srec, c->xs.as<double>(), ia.xm, c->conn_s.as<int32_t>(), ia.conn_m,
+                  c->lambda.as<double>(), c->pair_cap, ia.order, c->rec.as<long long>(), c->gs_pair.as<double>(),
+                  c->gm_pair.as<double>(), c->abar_pair.as<double>(), c->J_pair.as<double>(),
+                  FwdOut{c->Mblk.as<double>(), c->Dblk.as<double>(), c->flag.as<uint8_t>()}, ia.st, c->watchdog_us};
+  auto grid = [&](auto kern, int threads, size_t shm) {
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, shm);
+    return (unsigned)(c->n_sm * (per_sm < 1 ? 1 : per_sm));
+  };
+  unsigned long long* cta_t = (c->timing && c->cta_t.p) ? c->cta_t.as<unsigned long long>() : nullptr;
+  auto clip = k_adjoint_clip<NS, NM, SEG, DUAL>;
+  const unsigned gc = grid(clip, block, 0);
+  if (cta_t) c->pair_grid = (int)gc;
+  clip<<<gc, block, 0, c->stream>>>(a, cta_t);
+  auto cells = k_adjoint_cells<NS, NM, SEG>;
+  const size_t shm = (size_t)kCellThreads * kAdjSlots * 8;
+  cudaFuncSetAttribute(cells, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+  cells<<<grid(cells, kCellThreads, shm), kCellThreads, shm, c->stream>>>(a);
+  auto fin = k_adjoint_finish<NS, NM, SEG, DUAL>;
+  fin<<<grid(fin, block, 0), block, 0, c->stream>>>(a);
 }
 
 }  // namespace
@@ -1265,11 +1627,12 @@ void adjoint_pairs_nsnm(mortar_ctx* c, const RunParams& rp, unsigned grid, unsig
     else launch_pairs_t<NS, NM, false, false>(c, rp, grid, block, chunk);
     return;
   }
-  const int rounds = c->rounds > 0 ? c->rounds : 2;
-  if (seg && dual) launch_batched_t<NS, NM, true, true>(c, rounds, fused);
-  else if (seg) launch_batched_t<NS, NM, true, false>(c, rounds, fused);
-  else if (dual) launch_batched_t<NS, NM, false, true>(c, rounds, fused);
-  else launch_batched_t<NS, NM, false, false>(c, rounds, fused);
+  (void)fused;
+  const int rounds = c->rounds > 0 ? c->rounds : kSortBatch / 32;
+  if (seg && dual) launch_fixed<NS, NM, true, true>(c, rp, (int)block, rounds);
+  else if (seg) launch_fixed<NS, NM, true, false>(c, rp, (int)block, rounds);
+  else if (dual) launch_fixed<NS, NM, false, true>(c, rp, (int)block, rounds);
+  else launch_fixed<NS, NM, false, false>(c, rp, (int)block, rounds);
 }
 template void adjoint_pairs_nsnm<MORTAR_PAIR_NS, MORTAR_PAIR_NM>(mortar_ctx*, const RunParams&, unsigned, unsigned,
                                                                   int32_t, bool);
@@ -1297,6 +1660,15 @@ void launch_elems_ns(mortar_ctx* c, const RunParams& rp) {
 int prepare_adjoint_buffers(mortar_ctx* c) {
   const size_t P = (size_t)std::max<int64_t>(c->pair_cap, 1);
   int r;
+  if (c->variant == 0) {
+    const size_t words = c->opt.d_domain == MORTAR_D_SEGMENT ? AdjRecord::kWordsSeg : AdjRecord::kWords;
+    const size_t need = (P + 31) / 32 * 32 * words * 8;
+    if (c->rec.bytes < need && c->graph_exec) {   // a captured forward run holds the records' address
+      cudaGraphExecDestroy(c->graph_exec);
+      c->graph_exec = nullptr;
+    }
+    if ((r = buf_reserve(c->rec, need)) != MORTAR_OK) return r;
+  }
   if ((r = buf_reserve(c->gs_pair, P * 12 * 8)) != MORTAR_OK) return r;
   if ((r = buf_reserve(c->gm_pair, P * 12 * 8)) != MORTAR_OK) return r;
   if ((r = buf_reserve(c->J_pair, P * 8)) != MORTAR_OK) return r;

@@ -10,6 +10,7 @@ struct FxPolygon {
   static constexpr int kCap = 8;
   long long X[kCap], Y[kCap], A[kCap];   // vertices (Q62), cell weights omega
   long long cu, cv;                      // fan centre
+  int su, sv;                            // shifts that bring the fan's edges to 2^61 .. 2^62
   int nr, ncell, E, ke;                  // 2^ke: unit of sums of omega w N_s N_m / 2^64 with N Q61
   FxScales ss, sm;
   FxMap s, m;
@@ -75,7 +76,8 @@ struct FxPolygon {
       mu |= (unsigned long long)(a < 0 ? ~a : a);
       mv |= (unsigned long long)(b < 0 ? ~b : b);
     }
-    const int su = min(max(__clzll((long long)mu) - 2, 0), 60), sv = min(max(__clzll((long long)mv) - 2, 0), 60);
+    su = min(max(__clzll((long long)mu) - 2, 0), 60);
+    sv = min(max(__clzll((long long)mv) - 2, 0), 60);
     unsigned long long sum = 0;
     for (int c = 0; c < ncell; ++c) {
       const int b = ib(c), w = iw(c);
@@ -121,10 +123,10 @@ __device__ __forceinline__ void fx_shape(const FxScales& s, long long xi, long l
 // memory.  Records are stored in groups of 32, word w of lane i of group g at
 // rec[(g kWords + w) 32 + i]: a warp reads or writes 256 contiguous bytes.
 struct FxRecord {
-  static constexpr int kPair = 26, kInfo = 27, kScale = 28, kMapS = 29, kMapM = 37, kWords = 45;
+  static constexpr int kScale = 26, kMapS = 27, kMapM = 35, kPair = 43, kInfo = 44, kWords = 45;
   // words: 2k, 2k + 1: vertex k; 16 + c: weight of cell c; 24, 25: centre;
-  // 26: pair id; 27: nr | kb_s << 8 | kb_m << 16 | affine_s << 24 | affine_m << 25 | ke << 32 | E << 48;
-  // 28: the eight factor scales; 29.., 37..: maps (c0, then the digits k1 k2 k3)
+  // 26: the eight factor scales; 27.., 35..: maps (c0, then the digits k1 k2 k3); 43: pair id;
+  // 44: nr | kb_s << 8 | kb_m << 16 | affine_s << 24 | affine_m << 25 | ke << 32 | E << 48
   static __device__ __forceinline__ void store_map(long long* o, const FxMap& m, bool bilinear_possible) {
     auto put = [&](int w, Dg d) { o[32 * w] = (long long)(((unsigned long long)(unsigned)d.h << 32) | (unsigned)d.l); };
     o[0] = m.c0u;
