@@ -115,9 +115,9 @@ int alloc_pair_buffers(mortar_ctx* c, int64_t cap) {
   if (c->opt.d_domain == MORTAR_D_SEGMENT) MORTAR_TRY(buf_reserve(c->Dblk, n * 16 * 8));
   MORTAR_TRY(buf_reserve(c->flag, n));
   if (!quadratic_slave(c) && c->opt.integration == MORTAR_INTEGRATE_SEGMENT) {
-    const size_t groups = (n + 31) / 32;
-    MORTAR_TRY(buf_reserve(c->rec, groups * kRecordGroupBytes));
-    MORTAR_TRY(buf_reserve(c->order, n * 4));
+    const size_t chunk = std::min<size_t>(n, kPairChunk);   // records of one chunk of pairs
+    MORTAR_TRY(buf_reserve(c->rec, (chunk + 31) / 32 * kRecordGroupBytes));
+    MORTAR_TRY(buf_reserve(c->order, chunk * 4));
   }
   c->pair_cap = cap;
   return MORTAR_OK;
@@ -404,7 +404,7 @@ int set_common(mortar_ctx* c, int32_t n_if, const int64_t* sn_off, const int64_t
   if (c->pair_cap < 8 * c->Es + 1024 || c->Mblk.bytes < (size_t)c->pair_cap * mblk_stride(c) * 8 ||
       (quad_s && c->Qunit.bytes < (size_t)c->pair_cap * 4 * 32 * 8) ||
       (!quad_s && c->opt.integration == MORTAR_INTEGRATE_SEGMENT &&
-       c->rec.bytes < (size_t)((c->pair_cap + 31) / 32) * kRecordGroupBytes))
+       c->rec.bytes < (size_t)((std::min<int64_t>(c->pair_cap, kPairChunk) + 31) / 32) * kRecordGroupBytes))
     MORTAR_TRY(alloc_pair_buffers(c, std::max<int64_t>(c->pair_cap, 8 * c->Es + 1024)));
   if (c->nnz_cap_D < 9 * c->Ns + 64 || c->nnz_cap_M < 16 * c->Ns + 64)
     MORTAR_TRY(alloc_csr_buffers(c, std::max(c->nnz_cap_D, 9 * c->Ns + 64), std::max(c->nnz_cap_M, 16 * c->Ns + 64)));

@@ -83,11 +83,15 @@ struct DevStatus {
   unsigned long long nnzb_K;       // 3x3 blocks of the linearisation
   unsigned long long over_K;       // linearisation block buffer too small
   unsigned long long nonfinite;    // elements with a non-finite node coordinate
-  unsigned long long work_ctr4;    // work counter of the quadrature kernels
-  unsigned long long work_ctr5;    // work counter of the pair sort
-  unsigned long long work_ctr6;    // work counter of the adjoint's last kernel
+  unsigned long long pair_ctr[4];  // work counters of a chunk's sort, clip, quadrature and finish kernels
   double J;
 };
+
+// The fixed-point pair kernels run chunks of at most kPairChunk pairs, one
+// after the other, so that their records (0.4 to 1 KB a pair) take a bounded
+// workspace however many pairs there are: 4 GB, 4 M pairs, about 25 ms of
+// kernel time, beside which a chunk's tail and launches cost nothing.
+constexpr int64_t kPairChunk = int64_t(1) << 22;
 
 // Per-interface search grid.
 struct GridParams {

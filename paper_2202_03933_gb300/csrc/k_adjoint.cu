@@ -760,6 +760,7 @@ struct AdjArgs {
   const int32_t* conn_m;
   const double* lambda;
   int64_t pair_cap;
+  int64_t first;   // first pair of the chunk
   const int32_t* order;
   long long* rec;
   double* gs;
@@ -788,16 +789,15 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, un
   constexpr int W = SEG ? AdjRecord::kWordsSeg : AdjRecord::kWords;
   AdjCounters ctr;
   DevStatus* st = g.st;
-  const bool run = st->over_pairs == 0 && st->over_bins == 0;
-  const int64_t n = run ? (int64_t)min((unsigned long long)g.pair_cap, st->n_pairs) : 0;
+  const int64_t n = chunk_pairs(st, g.pair_cap, g.first, kPairChunk);
   const Watchdog wd(g.watchdog_us);
   int64_t grp;
-  while (!wd.expired(&st->timeout) && next_group(&st->work_ctr2, n, grp)) {   // bounded: the counter only grows
+  while (!wd.expired(&st->timeout) && next_group(&st->pair_ctr[1], n, grp)) {   // bounded: the counter only grows
     const int64_t i = 32 * grp + (threadIdx.x & 31);
     long long* o = g.rec + grp * (32 * W) + (threadIdx.x & 31);
     int mark = 0;   // nr of a record with nothing for the cell kernel
     if (i < n) {
-      const int64_t p = g.order[i];
+      const int64_t p = g.first + g.order[i];
       const int32_t s = g.ps[p], m = g.pm[p];
       const double* r = g.srec + (int64_t)SR_STRIDE * s;
       const int32_t* cm = g.conn_m + (int64_t)NM * m;
@@ -943,10 +943,8 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
   long long* sums = pts + 28 * stride;
   const int lane = threadIdx.x & 31;
   DevStatus* st = ar.st;
-  const bool run = st->over_pairs == 0 && st->over_bins == 0;
-  const int64_t n = run ? (int64_t)min((unsigned long long)ar.pair_cap, st->n_pairs) : 0;
-  const int64_t groups = (n + 31) >> 5;
-  const int turn = (int)max((int64_t)1, min((int64_t)8, groups / (4 * (int64_t)gridDim.x * (blockDim.x >> 5))));
+  const int64_t n = chunk_pairs(st, ar.pair_cap, ar.first, kPairChunk);
+  const int turn = cell_turn(n);
   const Watchdog wd(ar.watchdog_us);
   // The warps of a block run their rounds in step: every round costs the same
   // (one cell per lane), and the round's code, about 3,000 instructions, does not
@@ -957,14 +955,14 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
   bool more = true;
   for (;;) {   // bounded: the shared counter only grows
     if (w >= records && more) {
-      unsigned long long g0 = ~0ull;
+      unsigned long long g0 = ~0ull >> 1;
       if (!wd.expired(&st->timeout)) {
-        if (lane == 0) g0 = atomicAdd(&st->work_ctr4, (unsigned long long)turn);
+        if (lane == 0) g0 = atomicAdd(&st->pair_ctr[2], (unsigned long long)turn);
         g0 = __shfl_sync(0xffffffffu, g0, 0);
       }
-      more = g0 < (unsigned long long)groups;
-      r0 = 32 * (int64_t)g0;
-      records = more ? 32 * (int)min((int64_t)turn, groups - (int64_t)g0) : 0;
+      more = (int64_t)g0 < n;
+      r0 = (int64_t)g0;
+      records = more ? (int)min((int64_t)turn, n - r0) : 0;
       w = 0;
     }
     if (!__syncthreads_or(w < records)) break;
@@ -1098,11 +1096,10 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_finish(AdjArgs g) 
   constexpr int W = SEG ? AdjRecord::kWordsSeg : AdjRecord::kWords;
   AdjCounters ctr;
   DevStatus* st = g.st;
-  const bool run = st->over_pairs == 0 && st->over_bins == 0;
-  const int64_t n = run ? (int64_t)min((unsigned long long)g.pair_cap, st->n_pairs) : 0;
+  const int64_t n = chunk_pairs(st, g.pair_cap, g.first, kPairChunk);
   const Watchdog wd(g.watchdog_us);
   int64_t grp;
-  while (!wd.expired(&st->timeout) && next_group(&st->work_ctr6, n, grp)) {   // bounded: the counter only grows
+  while (!wd.expired(&st->timeout) && next_group(&st->pair_ctr[3], n, grp)) {   // bounded: the counter only grows
     const long long* o = g.rec + grp * (32 * W) + (threadIdx.x & 31);
     const int nr = (int)(o[32 * FxRecord::kInfo] & 0xff);
     if (nr == kSlowPair) {
@@ -1591,11 +1588,10 @@ void launch_fixed(mortar_ctx* c, const RunParams& rp, int block, int rounds) {
                    c->conn_m.as<int32_t>(), nullptr, nullptr, nullptr, c->pair_cap, c->dstat.as<DevStatus>(),
                    c->stream};
   ia.order = c->order.as<int32_t>();
-  launch_pair_sort<NS, NM>(ia, rp, c->n_sm, 32 * rounds);
-  const AdjArgs a{ia.ps, ia.pm, ia.srec, c->xs.as<double>(), ia.xm, c->conn_s.as<int32_t>(), ia.conn_m,
-                  c->lambda.as<double>(), c->pair_cap, ia.order, c->rec.as<long long>(), c->gs_pair.as<double>(),
-                  c->gm_pair.as<double>(), c->abar_pair.as<double>(), c->J_pair.as<double>(),
-                  FwdOut{c->Mblk.as<double>(), c->Dblk.as<double>(), c->flag.as<uint8_t>()}, ia.st, c->watchdog_us};
+  AdjArgs a{ia.ps, ia.pm, ia.srec, c->xs.as<double>(), ia.xm, c->conn_s.as<int32_t>(), ia.conn_m,
+            c->lambda.as<double>(), c->pair_cap, 0, ia.order, c->rec.as<long long>(), c->gs_pair.as<double>(),
+            c->gm_pair.as<double>(), c->abar_pair.as<double>(), c->J_pair.as<double>(),
+            FwdOut{c->Mblk.as<double>(), c->Dblk.as<double>(), c->flag.as<uint8_t>()}, ia.st, c->watchdog_us};
   auto grid = [&](auto kern, int threads, size_t shm) {
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, shm);
@@ -1603,15 +1599,18 @@ void launch_fixed(mortar_ctx* c, const RunParams& rp, int block, int rounds) {
   };
   unsigned long long* cta_t = (c->timing && c->cta_t.p) ? c->cta_t.as<unsigned long long>() : nullptr;
   auto clip = k_adjoint_clip<NS, NM, SEG, DUAL>;
-  const unsigned gc = grid(clip, block, 0);
-  if (cta_t) c->pair_grid = (int)gc;
-  clip<<<gc, block, 0, c->stream>>>(a, cta_t);
   auto cells = k_adjoint_cells<NS, NM, SEG>;
+  auto fin = k_adjoint_finish<NS, NM, SEG, DUAL>;
   const size_t shm = (size_t)kCellThreads * kAdjSlots * 8;
   cudaFuncSetAttribute(cells, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-  cells<<<grid(cells, kCellThreads, shm), kCellThreads, shm, c->stream>>>(a);
-  auto fin = k_adjoint_finish<NS, NM, SEG, DUAL>;
-  fin<<<grid(fin, block, 0), block, 0, c->stream>>>(a);
+  const unsigned gc = grid(clip, block, 0), gq = grid(cells, kCellThreads, shm), gf = grid(fin, block, 0);
+  if (cta_t) c->pair_grid = (int)gc;
+  for (; a.first < c->pair_cap; a.first += kPairChunk) {
+    launch_pair_sort<NS, NM>(ia, rp, c->n_sm, 32 * rounds, a.first);
+    clip<<<gc, block, 0, c->stream>>>(a, cta_t);
+    cells<<<gq, kCellThreads, shm, c->stream>>>(a);
+    fin<<<gf, block, 0, c->stream>>>(a);
+  }
 }
 
 }  // namespace
@@ -1662,7 +1661,7 @@ int prepare_adjoint_buffers(mortar_ctx* c) {
   int r;
   if (c->variant == 0) {
     const size_t words = c->opt.d_domain == MORTAR_D_SEGMENT ? AdjRecord::kWordsSeg : AdjRecord::kWords;
-    const size_t need = (P + 31) / 32 * 32 * words * 8;
+    const size_t need = (std::min<size_t>(P, kPairChunk) + 31) / 32 * 32 * words * 8;
     if (c->rec.bytes < need && c->graph_exec) {   // a captured forward run holds the records' address
       cudaGraphExecDestroy(c->graph_exec);
       c->graph_exec = nullptr;

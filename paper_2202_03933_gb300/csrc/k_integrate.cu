@@ -381,25 +381,24 @@ template <int NS, int NM, bool SEG>
 __global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_clip(
     const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
     const double* __restrict__ xm, const int32_t* __restrict__ conn_m, RunParams rp, double* __restrict__ Mblk,
-    double* __restrict__ Dblk, uint8_t* __restrict__ flag, int64_t pair_cap, const int32_t* __restrict__ order,
+    double* __restrict__ Dblk, uint8_t* __restrict__ flag, int64_t pair_cap, int64_t first, const int32_t* __restrict__ order,
     long long* __restrict__ rec, DevStatus* st, unsigned long long* cta_t) {
   cta_mark(cta_t, 0);
   const int lane = threadIdx.x & 31;
   PairCounters ctr;
-  const bool ok = st->over_pairs == 0 && st->over_bins == 0;
-  const int64_t n = ok ? (int64_t)min((unsigned long long)pair_cap, st->n_pairs) : 0;
+  const int64_t n = chunk_pairs(st, pair_cap, first, kPairChunk);
   const Watchdog wd(rp.watchdog_us);
   for (;;) {   // bounded: the shared counter only grows; one group of 32 pairs per turn
     if (wd.expired(&st->timeout)) break;
     unsigned long long g = 0;
-    if (lane == 0) g = atomicAdd(&st->work_ctr, 1ull);
+    if (lane == 0) g = atomicAdd(&st->pair_ctr[1], 1ull);
     g = __shfl_sync(0xffffffffu, g, 0);
     const int64_t i = 32 * (int64_t)g + lane;
     if (32 * (int64_t)g >= n) break;
     long long* o = rec + (int64_t)g * (32 * FxRecord::kWords) + lane;
     bool stored = false;
     if (i < n) {
-      const int64_t p = order[i];
+      const int64_t p = first + order[i];
       const double* r = srec + (int64_t)SR_STRIDE * ps[p];
       PlaneMap mmap;
       double pu[kPolyS], pv[kPolyS];
@@ -492,32 +491,28 @@ __device__ __forceinline__ void write_block(const FxAcc g[4][4], const CellSlot&
 // Quadrature of the clip kernel's records, one cell of a pair per lane (all
 // cells cost the same, so lanes idle only at the ends of warps): the cell's
 // back-projections, then its products, then the pair's sums through shared
-// memory.  A turn is up to `turn` groups of 32 records.
+// memory.
 template <int NS, int NM, bool SEG>
 __global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_quadrature(
     const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
     const double* __restrict__ xm, const int32_t* __restrict__ conn_m, RunParams rp, double* __restrict__ Mblk,
-    double* __restrict__ Dblk, uint8_t* __restrict__ flag, int64_t pair_cap, const long long* __restrict__ rec,
-    DevStatus* st) {
+    double* __restrict__ Dblk, uint8_t* __restrict__ flag, int64_t pair_cap, int64_t first,
+    const long long* __restrict__ rec, DevStatus* st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   long long* pts = reinterpret_cast<long long*>(smem_raw) + threadIdx.x;
   const int stride = (int)blockDim.x;
   const int lane = threadIdx.x & 31;
-  const bool run = st->over_pairs == 0 && st->over_bins == 0;
-  const int64_t n = run ? (int64_t)min((unsigned long long)pair_cap, st->n_pairs) : 0;
-  const int64_t groups = (n + 31) >> 5;
-  // enough turns for every warp, at most 8 groups each
-  const int turn = (int)max((int64_t)1, min((int64_t)8, groups / (4 * (int64_t)gridDim.x * (blockDim.x >> 5))));
+  const int64_t n = chunk_pairs(st, pair_cap, first, kPairChunk);
+  const int turn = cell_turn(n);
   const Watchdog wd(rp.watchdog_us);
   PairCounters slow;
   for (;;) {   // bounded: the shared counter only grows
     if (wd.expired(&st->timeout)) break;
     unsigned long long g0 = 0;
-    if (lane == 0) g0 = atomicAdd(&st->work_ctr4, (unsigned long long)turn);
-    g0 = __shfl_sync(0xffffffffu, g0, 0);
-    if ((int64_t)g0 >= groups) break;
-    const int64_t r0 = 32 * (int64_t)g0;
-    const int records = 32 * (int)min((int64_t)turn, groups - (int64_t)g0);
+    if (lane == 0) g0 = atomicAdd(&st->pair_ctr[2], (unsigned long long)turn);
+    const int64_t r0 = (int64_t)__shfl_sync(0xffffffffu, g0, 0);
+    if (r0 >= n) break;
+    const int records = (int)min((int64_t)turn, n - r0);
     for (int w = 0; w < records;) {
       int ncell = 0;
       if (w + lane < records) {
@@ -576,20 +571,22 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_quadrature(
 #ifdef MORTAR_PAIR_NS
 template <int NS, int NM, bool SEG>
 void launch_split(const IntegrateArgs& a, const RunParams& rp, int n_sm, int rounds, int warps) {
-  launch_pair_sort<NS, NM>(a, rp, n_sm, 32 * rounds);
   auto clip = k_pair_clip<NS, NM, SEG>;
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, clip, warps * 32, 0);
-  const unsigned grid = (unsigned)(n_sm * (per_sm < 1 ? 1 : per_sm));
-  if (a.grid_out) *a.grid_out = (int)grid;
-  clip<<<grid, warps * 32, 0, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag, a.pair_cap,
-                                          a.order, a.rec, a.st, a.cta_t);
   auto quad = k_pair_quadrature<NS, NM, SEG>;
   const size_t shq = (size_t)warps * 32 * kPtsBytes;
   cudaFuncSetAttribute(quad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shq);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quad, warps * 32, shq);
-  quad<<<(unsigned)(n_sm * (per_sm < 1 ? 1 : per_sm)), warps * 32, shq, a.stream>>>(
-      a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag, a.pair_cap, a.rec, a.st);
+  int clip_sm = 0, quad_sm = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&clip_sm, clip, warps * 32, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&quad_sm, quad, warps * 32, shq);
+  const unsigned gc = (unsigned)(n_sm * (clip_sm < 1 ? 1 : clip_sm)), gq = (unsigned)(n_sm * (quad_sm < 1 ? 1 : quad_sm));
+  if (a.grid_out) *a.grid_out = (int)gc;
+  for (int64_t first = 0; first < a.pair_cap; first += kPairChunk) {
+    launch_pair_sort<NS, NM>(a, rp, n_sm, 32 * rounds, first);
+    clip<<<gc, warps * 32, 0, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag, a.pair_cap,
+                                          first, a.order, a.rec, a.st, a.cta_t);
+    quad<<<gq, warps * 32, shq, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag,
+                                            a.pair_cap, first, a.rec, a.st);
+  }
 }
 
 template <int NS, int NM, bool SEG>

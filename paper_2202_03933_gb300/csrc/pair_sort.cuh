@@ -4,6 +4,7 @@
 
 #include "clip.cuh"
 #include "context.h"
+#include "quadrature.cuh"
 
 namespace mortar {
 
@@ -85,7 +86,8 @@ __device__ __forceinline__ int sort_batch(unsigned char* my, int B, int64_t base
   return basecnt;
 }
 
-// Writes the sorted order of every batch: order[base + i] = pair.  A kernel of
+// Writes the sorted order of every batch of the chunk that begins at pair
+// `first`: order[base + i] = pair, relative to it.  A kernel of
 // its own, so that the pair kernels' code stays within the instruction cache,
 // and because it is latency-bound where they are not: small batches' worth of
 // registers, many warps.
@@ -94,20 +96,22 @@ constexpr int kSortBatch = 1024;   // default pairs per warp batch, and the most
 template <int NS, int NM>
 __global__ void __launch_bounds__(kSortThreads) k_pair_sort(
     const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
-    const double* __restrict__ xm, const int32_t* __restrict__ conn_m, int64_t pair_cap, int B, int32_t watchdog_us,
+    const double* __restrict__ xm, const int32_t* __restrict__ conn_m, int64_t pair_cap, int64_t first, int B,
+    int32_t watchdog_us,
     int32_t* __restrict__ order, DevStatus* st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* my = smem_raw + (size_t)(threadIdx.x >> 5) * batch_smem_bytes(B);
   const uint16_t* perm = reinterpret_cast<const uint16_t*>(my + 32);
-  const bool ok = st->over_pairs == 0 && st->over_bins == 0;
-  const int64_t n = ok ? (int64_t)min((unsigned long long)pair_cap, st->n_pairs) : 0;
+  const int64_t n = chunk_pairs(st, pair_cap, first, kPairChunk);
+  ps += first;
+  pm += first;
   const int64_t share = 2 * (int64_t)gridDim.x * (blockDim.x >> 5);
   const Watchdog wd(watchdog_us);
   for (;;) {   // bounded: the shared counter only grows
     if (wd.expired(&st->timeout)) break;
     int64_t base;
     int fetch;
-    if (!fetch_batch(&st->work_ctr5, n, share, B, base, fetch)) break;
+    if (!fetch_batch(&st->pair_ctr[0], n, share, B, base, fetch)) break;
     const int64_t lim = min(n, base + (int64_t)fetch);
     const int live = sort_batch<NS, NM>(my, B, base, lim, (fetch + 31) >> 5, ps, pm, srec, xm, conn_m);
     for (int i = threadIdx.x & 31; i < live; i += 32) order[base + i] = (int32_t)(base + perm[i]);
@@ -116,13 +120,14 @@ __global__ void __launch_bounds__(kSortThreads) k_pair_sort(
 }
 
 template <int NS, int NM>
-void launch_pair_sort(const IntegrateArgs& a, const RunParams& rp, int n_sm, int B) {
+void launch_pair_sort(const IntegrateArgs& a, const RunParams& rp, int n_sm, int B, int64_t first) {
+  cudaMemsetAsync(&a.st->pair_ctr, 0, sizeof(a.st->pair_ctr), a.stream);   // the chunk's kernels
   auto kern = k_pair_sort<NS, NM>;
   const size_t shm = (size_t)(kSortThreads / 32) * batch_smem_bytes(B);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSortThreads, shm);
   kern<<<(unsigned)(n_sm * (per_sm < 1 ? 1 : per_sm)), kSortThreads, shm, a.stream>>>(
-      a.ps, a.pm, a.srec, a.xm, a.conn_m, a.pair_cap, B, rp.watchdog_us, a.order, a.st);
+      a.ps, a.pm, a.srec, a.xm, a.conn_m, a.pair_cap, first, B, rp.watchdog_us, a.order, a.st);
 }
 
 }  // namespace

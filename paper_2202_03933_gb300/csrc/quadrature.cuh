@@ -311,6 +311,20 @@ __device__ __forceinline__ void fx_cell_products(const FxScales& ss, const FxSca
   }
 }
 
+// Pairs [first, first + count) that the run has; 0 after an overflow.
+__device__ __forceinline__ int64_t chunk_pairs(const DevStatus* st, int64_t pair_cap, int64_t first, int64_t count) {
+  if (st->over_pairs != 0 || st->over_bins != 0) return 0;
+  const int64_t n = (int64_t)min((unsigned long long)pair_cap, st->n_pairs) - first;
+  return max((int64_t)0, min(n, count));
+}
+
+// Records per turn of a cell kernel's warp: about 16 turns a warp, 8 (a warp's
+// lanes) to 256 records.
+__device__ __forceinline__ int cell_turn(int64_t n) {
+  const int64_t t = n / (16 * (int64_t)gridDim.x * (blockDim.x >> 5));
+  return (int)max((int64_t)8, min((int64_t)256, t & ~(int64_t)7));
+}
+
 // Cells of consecutive records on consecutive lanes: each lane gets one cell
 // of one pair, whole pairs only, as many as fit in a warp.
 struct CellSlot {
