@@ -114,8 +114,8 @@ int alloc_pair_buffers(mortar_ctx* c, int64_t cap) {
   }
   if (c->opt.d_domain == MORTAR_D_SEGMENT) MORTAR_TRY(buf_reserve(c->Dblk, n * 16 * 8));
   MORTAR_TRY(buf_reserve(c->flag, n));
-  if (!quadratic_slave(c) && c->opt.integration == MORTAR_INTEGRATE_SEGMENT) {
-    const size_t chunk = std::min<size_t>(n, kPairChunk);   // records of one chunk of pairs
+  if (c->opt.integration == MORTAR_INTEGRATE_SEGMENT) {   // records of one chunk of pairs (units)
+    const size_t chunk = std::min<size_t>(quadratic_slave(c) ? 4 * n : n, kPairChunk);
     MORTAR_TRY(buf_reserve(c->rec, (chunk + 31) / 32 * kRecordGroupBytes));
     MORTAR_TRY(buf_reserve(c->order, chunk * 4));
   }
@@ -403,8 +403,9 @@ int set_common(mortar_ctx* c, int32_t n_if, const int64_t* sn_off, const int64_t
   MORTAR_TRY(buf_reserve(c->scan_tmp, (size_t)scan_temp_words(scan_n) * 8));
   if (c->pair_cap < 8 * c->Es + 1024 || c->Mblk.bytes < (size_t)c->pair_cap * mblk_stride(c) * 8 ||
       (quad_s && c->Qunit.bytes < (size_t)c->pair_cap * 4 * 32 * 8) ||
-      (!quad_s && c->opt.integration == MORTAR_INTEGRATE_SEGMENT &&
-       c->rec.bytes < (size_t)((std::min<int64_t>(c->pair_cap, kPairChunk) + 31) / 32) * kRecordGroupBytes))
+      (c->opt.integration == MORTAR_INTEGRATE_SEGMENT &&
+       c->rec.bytes <
+           (size_t)((std::min<int64_t>((quad_s ? 4 : 1) * c->pair_cap, kPairChunk) + 31) / 32) * kRecordGroupBytes))
     MORTAR_TRY(alloc_pair_buffers(c, std::max<int64_t>(c->pair_cap, 8 * c->Es + 1024)));
   if (c->nnz_cap_D < 9 * c->Ns + 64 || c->nnz_cap_M < 16 * c->Ns + 64)
     MORTAR_TRY(alloc_csr_buffers(c, std::max(c->nnz_cap_D, 9 * c->Ns + 64), std::max(c->nnz_cap_M, 16 * c->Ns + 64)));

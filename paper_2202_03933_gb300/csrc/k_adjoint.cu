@@ -898,36 +898,6 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, un
   cta_mark(cta_t, 1);
 }
 
-// Sums g of every pair's cells, entry by entry by the pair's lanes in turn,
-// into record words w0 + 4 a + l as FP64.  buf as in the quadrature kernel.
-template <int NS, int NC>
-__device__ __forceinline__ void pair_products(const FxAcc g[4][4], const CellSlot& cs, bool ok, int ke,
-                                              const FxScales& ss, const FxScales& sc, long long* __restrict__ o,
-                                              int w0, long long* __restrict__ buf, int stride) {
-  __syncwarp();
-#pragma unroll
-  for (int a = 0; a < NS; ++a)
-#pragma unroll
-    for (int l = 0; l < NC; ++l) {
-      const int e = NC * a + l;
-      buf[e * stride] = g[a][l].hh + (g[a][l].cr >> 32);
-      reinterpret_cast<unsigned*>(buf + (16 + (e >> 1)) * stride)[e & 1] = (unsigned)g[a][l].cr;
-    }
-  __syncwarp();
-  const long long* pair = buf - (threadIdx.x & 31) + cs.first;
-  if (ok)
-#pragma unroll 1
-    for (int e = cs.cell; e < NS * NC; e += cs.cells) {
-      const int a = e / NC, l = e - NC * a;
-      long long hh = 0, cr = 0;
-      for (int k = 0; k < cs.cells; ++k) {
-        hh += pair[e * stride + k];
-        cr += reinterpret_cast<const unsigned*>(pair + (16 + (e >> 1)) * stride + k)[e & 1];
-      }
-      o[32 * (w0 + 4 * a + l)] = __double_as_longlong(fx_to_double(hh, cr, ke - ss.shape<NS>(a) - sc.shape<NC>(l)));
-    }
-}
-
 constexpr int kAdjSlots = 58;      // shared 64-bit words per thread of the cell kernel: points, W y or sums
 constexpr int kCellThreads = 384;  // the registers of an SM at 168 a thread
 
@@ -1082,8 +1052,15 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
       FxAcc h[4][4];
       if (SEG) fx_cell_products<NS, NS, true>(f.ss, f.ss, weight, pts, stride, h);
       fx_cell_products<NS, NM, false>(f.ss, f.sm, weight, pts, stride, g);
-      if (SEG) pair_products<NS, NS>(h, cs, ok, f.ke, f.ss, f.ss, o, AdjRecord::kH, pts, stride);
-      pair_products<NS, NM>(g, cs, ok, f.ke, f.ss, f.sm, o, AdjRecord::kG, pts, stride);
+      if (SEG)
+        fx_sum_cells<NS, NS>(h, cs, ok, pts, stride, [&](int a, int b, long long hh, long long cr) {
+          o[32 * (AdjRecord::kH + 4 * a + b)] =
+              __double_as_longlong(fx_to_double(hh, cr, f.ke - f.ss.shape<NS>(a) - f.ss.shape<NS>(b)));
+        });
+      fx_sum_cells<NS, NM>(g, cs, ok, pts, stride, [&](int a, int l, long long hh, long long cr) {
+        o[32 * (AdjRecord::kG + 4 * a + l)] =
+            __double_as_longlong(fx_to_double(hh, cr, f.ke - f.ss.shape<NS>(a) - f.sm.shape<NM>(l)));
+      });
     }
     if (slow && cs.cell == 0) o[32 * FxRecord::kInfo] = kSlowPair;
   }

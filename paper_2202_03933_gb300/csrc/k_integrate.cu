@@ -222,7 +222,9 @@ __global__ void __launch_bounds__(kMaxPairBlock) k_integrate(const int32_t* __re
 }
 
 // ---------------------------------------------------------------- variant 0
-constexpr int kPtsBytes = 28 * 8;   // back-projections of a cell's seven points
+// shared memory per thread: a cell's seven back-projections [and, SEG, its sums apart from them]
+template <bool SEG>
+constexpr int kPtsBytes = (SEG ? 52 : 28) * 8;
 
 // One pair in FP64 (the one-kernel form, and pairs whose geometry does not fit
 // the fixed-point frame of the two-kernel form): FP64 clip, then the 7-point rule on the
@@ -353,7 +355,7 @@ __global__ void __launch_bounds__(kMaxPairBlock) k_integrate_batched(
     int64_t base;
     int fetch;
     if (!fetch_batch(&st->work_ctr, n, share, B, base, fetch)) break;
-    const int n_live = sort_batch<NS, NM>(my, B, base, min(n, base + (int64_t)fetch), (fetch + 31) >> 5, ps, pm, srec,
+    const int n_live = sort_batch<NS, NM, 1>(my, B, base, min(n, base + (int64_t)fetch), (fetch + 31) >> 5, ps, pm, srec,
                                           xm, conn_m);
     // ---- phase B: one pair per lane, rounds of similar cost
     for (int i0 = 0; i0 < n_live; i0 += 32) {
@@ -427,50 +429,26 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_clip(
   cta_mark(cta_t, 1);
 }
 
-// Adds up the cells' sums g of every pair of the warp and writes the pair's
-// 4x4 block M = A G (standard LMs: G).  The lanes of a pair take its entries in
-// turn: sum over the cells, conversion, product with A.  buf: this thread's
-// slice of shared memory (entry i at buf[i * stride], lane L's at buf - lane +
-// L), free to use by the whole warp.
+// Writes the 4x4 block M = A G (standard LMs: G) of every pair of the warp from
+// its cells' sums g (fx_sum_cells).
 template <int NS, int NC>
 __device__ __forceinline__ void write_block(const FxAcc g[4][4], const CellSlot& cs, bool ok, int ke,
                                             const FxScales& ss, const FxScales& sc, bool dual,
                                             const double* __restrict__ r, double* __restrict__ out,
                                             long long* __restrict__ buf, int stride) {
-  const int lane = threadIdx.x & 31;
-  __syncwarp();
-#pragma unroll
-  for (int a = 0; a < NS; ++a)
-#pragma unroll
-    for (int l = 0; l < NC; ++l) {
-      buf[(NC * a + l) * stride] = g[a][l].hh + (g[a][l].cr >> 32);
-      reinterpret_cast<unsigned*>(buf + (16 + ((NC * a + l) >> 1)) * stride)[l + NC * a & 1] = (unsigned)g[a][l].cr;
-    }
-  __syncwarp();
-  const long long* pair = buf - lane + cs.first;
-  double G[16];
+  double G[16];   // dual: this lane's entries, until every lane has read the sums
   int n = 0;
-  if (ok) {
-#pragma unroll 1
-    for (int e = cs.cell; e < NS * NC; e += cs.cells) {
-      const int a = e / NC, l = e - NC * a;
-      long long hh = 0, cr = 0;
-      for (int k = 0; k < cs.cells; ++k) {
-        hh += pair[e * stride + k];
-        cr += reinterpret_cast<const unsigned*>(pair + (16 + (e >> 1)) * stride + k)[e & 1];
-      }
-      const double v = fx_to_double(hh, cr, ke - ss.shape<NS>(a) - sc.shape<NC>(l));
-      if (dual) G[n++] = v;
-      else __stcs(out + 4 * a + l, v);
-    }
-    if (NS * NC < 16 || !dual) {   // the block is padded with zeros
-      for (int e = cs.cell; e < 16 && NS * NC < 16; e += cs.cells)
-        if ((e >> 2) >= NS || (e & 3) >= NC) __stcs(out + e, 0.0);
-    }
-  }
+  fx_sum_cells<NS, NC>(g, cs, ok, buf, stride, [&](int a, int l, long long hh, long long cr) {
+    const double v = fx_to_double(hh, cr, ke - ss.shape<NS>(a) - sc.shape<NC>(l));
+    if (dual) G[n++] = v;
+    else __stcs(out + 4 * a + l, v);
+  });
+  if (ok && NS * NC < 16)   // the block is padded with zeros
+    for (int e = cs.cell; e < 16; e += cs.cells)
+      if ((e >> 2) >= NS || (e & 3) >= NC) __stcs(out + e, 0.0);
   if (dual) {
     __syncwarp();
-    double* Gs = reinterpret_cast<double*>(const_cast<long long*>(pair));
+    double* Gs = reinterpret_cast<double*>(buf - (threadIdx.x & 31) + cs.first);
     if (ok) {
       n = 0;
       for (int e = cs.cell; e < NS * NC; e += cs.cells) Gs[e * stride] = G[n++];
@@ -547,15 +525,12 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_quadrature(
       const bool slow_pair = cs.cell >= 0 && (bad >> cs.first & ((1u << cs.cells) - 1u)) != 0;
       ok &= !slow_pair;
       FxAcc g[4][4];
-      if (SEG) {   // first, while the points are in shared memory: D in the lane's registers, then M
-        FxAcc h[4][4];
-        fx_cell_products<NS, NS, true>(ss, ss, weight, pts, stride, h);
-        fx_cell_products<NS, NM, false>(ss, sm, weight, pts, stride, g);
-        write_block<NS, NS>(h, cs, ok, ke, ss, ss, rp.lm == 1, r, Dblk + 16 * p, pts, stride);
-      } else {
-        fx_cell_products<NS, NM, false>(ss, sm, weight, pts, stride, g);
+      if (SEG) {   // the sums' memory is apart from the points', which M's products read again
+        fx_cell_products<NS, NS, true>(ss, ss, weight, pts, stride, g);
+        write_block<NS, NS>(g, cs, ok, ke, ss, ss, rp.lm == 1, r, Dblk + 16 * p, pts + 28 * stride, stride);
       }
-      write_block<NS, NM>(g, cs, ok, ke, ss, sm, rp.lm == 1, r, Mblk + 16 * p, pts, stride);
+      fx_cell_products<NS, NM, false>(ss, sm, weight, pts, stride, g);
+      write_block<NS, NM>(g, cs, ok, ke, ss, sm, rp.lm == 1, r, Mblk + 16 * p, SEG ? pts + 28 * stride : pts, stride);
       if (cs.cell == 0) {
         if (ok) flag[p] = 1;
         else integrate_pair_fp64<NS, NM, SEG>(p, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, slow);
@@ -573,7 +548,7 @@ template <int NS, int NM, bool SEG>
 void launch_split(const IntegrateArgs& a, const RunParams& rp, int n_sm, int rounds, int warps) {
   auto clip = k_pair_clip<NS, NM, SEG>;
   auto quad = k_pair_quadrature<NS, NM, SEG>;
-  const size_t shq = (size_t)warps * 32 * kPtsBytes;
+  const size_t shq = (size_t)warps * 32 * kPtsBytes<SEG>;
   cudaFuncSetAttribute(quad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shq);
   int clip_sm = 0, quad_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&clip_sm, clip, warps * 32, 0);

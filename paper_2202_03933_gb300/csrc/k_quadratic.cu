@@ -14,16 +14,17 @@
 //
 // Work unit = (pair, sub-element), u = 4 p + k: the four sub-elements of a
 // pair overlap the master element in different cell counts (often none), so
-// one pair per lane would leave most lanes idle.  A persistent grid takes
-// batches of units (guided self-scheduling), sorts each batch by the cell
-// count and edge intersections of an FP32 clip, and runs the units in rounds
-// of similar cost: FP64 clip, quadrature into the unit's 8 x 4 block.  A
-// second kernel sums the four unit blocks of every pair in the fixed order
-// k = 0..3 (bitwise reproducible) into the pair block and its flag.
-#include <type_traits>
-
+// one pair per lane would leave most lanes idle.  As for linear elements
+// (k_integrate.cu), three kernels: the units are sorted by an FP32 clip
+// (k_pair_sort), clipped in FP64 and turned into fixed-point records
+// (k_quadratic_clip), and integrated on the integer pipe with one cell of a unit
+// per lane (k_quadratic_cells).  A last kernel sums the non-empty unit blocks
+// of every pair in the fixed order k = 0..3 (bitwise reproducible) into the pair
+// block and its flag.
 #include "clip.cuh"
 #include "context.h"
+#include "pair_sort.cuh"
+#include "quadrature.cuh"
 #include "quadratic.cuh"
 
 namespace mortar {
@@ -31,15 +32,16 @@ namespace mortar {
 namespace {
 
 constexpr int kQThreads = 128;
-constexpr int kQRounds = 16;   // units per warp batch: 32 x 16
+constexpr int kQPtsBytes = 52 * 8;   // shared memory per thread: a cell's seven back-projections, and its sums
 
 struct QCounters {
   unsigned long long gp = 0, cells = 0, newton_fail = 0, clip_over = 0;
 };
 
-// One unit: sub-element k of pair p.  Writes the unit's 8 x 4 block and flag.
+// One unit in FP64, for those that do not fit the fixed-point frame:
+// sub-element k of pair p.  Writes the unit's 8 x 4 block and flag.
 template <int NP, int NM>
-__device__ void integrate_unit(int64_t u, const int32_t* __restrict__ ps, const int32_t* __restrict__ pm,
+__device__ __noinline__ void integrate_unit(int64_t u, const int32_t* __restrict__ ps, const int32_t* __restrict__ pm,
                                const double* __restrict__ srec, const double* __restrict__ xm,
                                const int32_t* __restrict__ conn_m, double* __restrict__ U,
                                uint8_t* __restrict__ uflag, QCounters& ctr) {
@@ -129,87 +131,140 @@ __device__ void integrate_unit(int64_t u, const int32_t* __restrict__ ps, const 
   uflag[u] = 1;
 }
 
+// Half of a quadratic element's shape functions in Q61 (HALF 0: corners, 1:
+// mid-sides) at the parent point of sub-element k's (xi, eta) (Q61).  quad8
+// with A, B = 1 -+ xi_p, C, D = 1 -+ eta_p:
+//   corners (AC (A + C - 3), BC (B + C - 3), BD (B + D - 3), AD (A + D - 3)) / 4,
+//   mid-sides (AB C, CD B, AB D, CD A) / 2.
+template <int NP, int HALF>
+__device__ __forceinline__ void fx_shape_quadratic(int k, long long xi, long long eta, Dg* N) {
+  FxAcc p;
+  const long long one = 1ll << 61;
+  if constexpr (NP == 8) {
+    const long long xp = (xi + (k == 1 || k == 2 ? one : -one)) >> 1, ep = (eta + (k >= 2 ? one : -one)) >> 1;
+    const long long A = one - xp, B = one + xp, C = one - ep, D = one + ep;
+    const Dg a = fx_split(A), b = fx_split(B), c = fx_split(C), d = fx_split(D);
+    if (HALF == 0) {
+      auto corner = [&](Dg u, Dg v, long long s) {
+        p.mul(u, v);
+        const Dg uv = fx_split(p.get<2>());   // Q60, at most 4
+        p.mul(uv, fx_split(s - 3 * one));
+        return fx_split(p.get<2>());
+      };
+      N[0] = corner(a, c, A + C);
+      N[1] = corner(b, c, B + C);
+      N[2] = corner(b, d, B + D);
+      N[3] = corner(a, d, A + D);
+    } else {
+      p.mul(a, b);
+      const Dg ab = fx_split(p.get<3>());   // at most 1
+      p.mul(c, d);
+      const Dg cd = fx_split(p.get<3>());
+      p.mul(ab, c);
+      N[0] = fx_split(p.get<2>());
+      p.mul(cd, b);
+      N[1] = fx_split(p.get<2>());
+      p.mul(ab, d);
+      N[2] = fx_split(p.get<2>());
+      p.mul(cd, a);
+      N[3] = fx_split(p.get<2>());
+    }
+  } else {
+    const long long hx = xi >> 1, he = eta >> 1, half = one >> 1;
+    const long long xp = k == 1 ? half + hx : (k == 3 ? half - he : hx);
+    const long long ep = k == 2 ? half + he : (k == 3 ? hx + he : he);
+    const long long L[3] = {one - xp - ep, xp, ep};
+    const Dg l0 = fx_split(L[0]), l1 = fx_split(L[1]), l2 = fx_split(L[2]);
+    if (HALF == 0) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        p.mul(i == 0 ? l0 : (i == 1 ? l1 : l2), fx_split(2 * L[i] - one));
+        N[i] = fx_split(p.get<3>());
+      }
+    } else {
+      p.mul(l0, l1);
+      N[0] = fx_split(p.get<5>());
+      p.mul(l1, l2);
+      N[1] = fx_split(p.get<5>());
+      p.mul(l2, l0);
+      N[2] = fx_split(p.get<5>());
+    }
+  }
+}
+
+// Sums over one cell's points of N_p (W N_m)^T for half of the parent's shape
+// functions (bounds as in fx_cell_products, with the roles exchanged).
+template <int NP, int NM, int HALF>
+__device__ __forceinline__ void fx_cell_quadratic(int k, const FxScales& sm, long long weight,
+                                                  const long long* __restrict__ pts, int stride, FxAcc g[4][4]) {
+  constexpr int NR = NP / 2;
+#pragma unroll
+  for (int a = 0; a < NR; ++a)
+#pragma unroll
+    for (int l = 0; l < NM; ++l) g[a][l].zero();
+  const Dg om = fx_split(weight);
+#pragma unroll 1
+  for (int q = 0; q < 7; ++q) {
+    Dg Nm[4], Np[4];
+    FxAcc a;
+    a.mul(om, kTri7Fx.w[q]);
+    const Dg W = fx_split(a.get<2>());
+    fx_shape<NM>(sm, pts[(4 * q + 2) * stride], pts[(4 * q + 3) * stride], Nm);
+#pragma unroll
+    for (int l = 0; l < NM; ++l) {
+      a.mul(W, Nm[l]);
+      Nm[l] = fx_split(a.get<3>());
+    }
+    fx_shape_quadratic<NP, HALF>(k, pts[(4 * q) * stride], pts[(4 * q + 1) * stride], Np);
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+#pragma unroll
+      for (int l = 0; l < NM; ++l) g[i][l].mac(Nm[l], Np[i]);
+  }
+}
+
+// Clip of the chunk's units in sorted order, one record each (see k_pair_clip).
 template <int NP, int NM>
-__global__ void __launch_bounds__(kQThreads) k_integrate_quadratic(
+__global__ void __launch_bounds__(kQThreads, 4) k_quadratic_clip(
     const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
     const double* __restrict__ xm, const int32_t* __restrict__ conn_m, RunParams rp, double* __restrict__ U,
-    uint8_t* __restrict__ uflag, int64_t pair_cap, DevStatus* st) {
+    uint8_t* __restrict__ uflag, int64_t pair_cap, int64_t first, const int32_t* __restrict__ order,
+    long long* __restrict__ rec, DevStatus* st) {
   constexpr int NSUB = NP == 8 ? 4 : 3;
-  constexpr int B = 32 * kQRounds;
-  using PermT = typename std::conditional<(B > 256), uint16_t, uint8_t>::type;
-  __shared__ PermT perm_s[kQThreads / 32][B];
-  __shared__ uint8_t key_s[kQThreads / 32][B];
-  __shared__ unsigned pres_s[kQThreads / 32][8];
-  PermT* perm = perm_s[threadIdx.x >> 5];
-  uint8_t* keys = key_s[threadIdx.x >> 5];
-  unsigned* pres = pres_s[threadIdx.x >> 5];
-  QCounters ctr;
   const int lane = threadIdx.x & 31;
-  const unsigned lt_mask = (1u << lane) - 1u;
-  const bool ok = st->over_pairs == 0 && st->over_bins == 0;
-  const int64_t n = ok ? 4 * (int64_t)min((unsigned long long)pair_cap, st->n_pairs) : 0;   // units
-  const int64_t share = 2 * (int64_t)gridDim.x * (blockDim.x >> 5);
+  QCounters ctr;
+  const int64_t n = 4 * chunk_pairs(st, pair_cap, first, kPairChunk / 4);   // units
   const Watchdog wd(rp.watchdog_us);
-  for (;;) {   // bounded: the shared counter only grows
+  for (;;) {   // bounded: the shared counter only grows; one group of 32 units per turn
     if (wd.expired(&st->timeout)) break;
-    int64_t base = 0;
-    int fetch = B;
-    if (lane == 0) {
-      const unsigned long long seen = *reinterpret_cast<volatile unsigned long long*>(&st->work_ctr);
-      const int64_t f = (n - (int64_t)seen) / share;
-      fetch = f >= B ? B : (f < 32 ? 32 : (int)(f & ~31ll));
-      base = (int64_t)atomicAdd(&st->work_ctr, (unsigned long long)fetch);
-    }
-    base = __shfl_sync(0xffffffffu, base, 0);
-    fetch = __shfl_sync(0xffffffffu, fetch, 0);
-    if (base >= n) break;
-    const int64_t lim = min(n, base + (int64_t)fetch);
-    const int rounds = (fetch + 31) >> 5;
-    // phase A: sort key of each unit from an FP32 clip of its sub-element
-    if (lane < 8) pres[lane] = 0u;
-    __syncwarp();
-#pragma unroll 1
-    for (int rr = 0; rr < rounds; ++rr) {
-      const int64_t u = base + rr * 32 + lane;
-      int key = 0;
-      if (u < lim) {
-        const int64_t p = u >> 2;
-        const double* r = srec + (int64_t)SR_STRIDE * (4 * (int64_t)ps[p] + (u & 3));
-        int n_int = 0;
-        const int nr = clip_count_f32<NSUB, NM>(r, xm, conn_m, pm[p], n_int);
-        key = 1 + 16 * (nr == 0 ? 0 : (nr == 3 ? 1 : min(nr, kPolyS))) + min(n_int, 15);
-        atomicOr(&pres[key >> 5], 1u << (key & 31));
-      }
-      keys[rr * 32 + lane] = (uint8_t)key;
-    }
-    __syncwarp();
-    int basecnt = 0;
-#pragma unroll 1
-    for (int w = 7; w >= 0; --w) {
-      unsigned bits = pres[w];
-      while (bits != 0u) {   // uniform across the warp
-        const int b = 31 - __clz(bits);
-        bits &= ~(1u << b);
-        const int v = 32 * w + b;
-        int before = 0;
-#pragma unroll 1
-        for (int rr = 0; rr < rounds; ++rr) {
-          const int slot = rr * 32 + lane;
-          const bool hit = keys[slot] == v;
-          const unsigned mk = __ballot_sync(0xffffffffu, hit);
-          if (hit) perm[basecnt + before + __popc(mk & lt_mask)] = (PermT)slot;
-          before += __popc(mk);
+    unsigned long long g = 0;
+    if (lane == 0) g = atomicAdd(&st->pair_ctr[1], 1ull);
+    g = __shfl_sync(0xffffffffu, g, 0);
+    const int64_t i = 32 * (int64_t)g + lane;
+    if (32 * (int64_t)g >= n) break;
+    long long* o = rec + (int64_t)g * (32 * FxRecord::kWords) + lane;
+    bool stored = false;
+    if (i < n) {
+      const int64_t u = 4 * first + order[i], p = u >> 2;
+      const double* r = srec + (int64_t)SR_STRIDE * (4 * (int64_t)ps[p] + (u & 3));
+      PlaneMap mmap;
+      double pu[kPolyS], pv[kPolyS];
+      const int nr = clip_polygon<NSUB, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
+      if (nr == 0) {
+        uflag[u] = 0;
+      } else {
+        FxPolygon f;
+        stored = f.setup<NSUB, NM>(r, mmap, pu, pv, nr);
+        if (stored) {
+          FxRecord::store<NSUB, NM>(o, f, u);
+          ctr.cells += f.ncell;
+          ctr.gp += 7 * f.ncell;
+        } else {
+          integrate_unit<NP, NM>(u, ps, pm, srec, xm, conn_m, U, uflag, ctr);
         }
-        basecnt += before;
       }
     }
-    const int n_live = basecnt;
-    __syncwarp();
-    // phase B: one unit per lane, rounds of similar cost
-    for (int i0 = 0; i0 < n_live; i0 += 32) {
-      const int i = i0 + lane;
-      if (i < n_live) integrate_unit<NP, NM>(base + perm[i], ps, pm, srec, xm, conn_m, U, uflag, ctr);
-    }
+    if (!stored) o[32 * FxRecord::kInfo] = 0;   // nr = 0: nothing left for the cell kernel
     __syncwarp();
   }
   block_count_add(&st->gauss_points, ctr.gp);
@@ -218,7 +273,84 @@ __global__ void __launch_bounds__(kQThreads) k_integrate_quadratic(
   block_count_add(&st->clip_overflow, ctr.clip_over);
 }
 
-// Pair block = sum of its four unit blocks in the order k = 0..3; flag = any.
+// Quadrature of the units' records, one cell per lane (see k_pair_quadrature);
+// the corner and the mid-side rows one after the other, so that each pass has
+// 16 sums.  Bound by issue over the integer pipes, as for linear elements.
+template <int NP, int NM>
+__global__ void __launch_bounds__(kQThreads, 4) k_quadratic_cells(
+    const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
+    const double* __restrict__ xm, const int32_t* __restrict__ conn_m, RunParams rp, double* __restrict__ U,
+    uint8_t* __restrict__ uflag, int64_t pair_cap, int64_t first, const long long* __restrict__ rec, DevStatus* st) {
+  constexpr int NSUB = NP == 8 ? 4 : 3, NR = NP / 2;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  long long* pts = reinterpret_cast<long long*>(smem_raw) + threadIdx.x;
+  const int stride = (int)blockDim.x;
+  const int lane = threadIdx.x & 31;
+  const int64_t n = 4 * chunk_pairs(st, pair_cap, first, kPairChunk / 4);
+  const int turn = cell_turn(n);
+  const Watchdog wd(rp.watchdog_us);
+  QCounters slow;
+  for (;;) {   // bounded: the shared counter only grows
+    if (wd.expired(&st->timeout)) break;
+    unsigned long long g0 = 0;
+    if (lane == 0) g0 = atomicAdd(&st->pair_ctr[2], (unsigned long long)turn);
+    const int64_t r0 = (int64_t)__shfl_sync(0xffffffffu, g0, 0);
+    if (r0 >= n) break;
+    const int records = (int)min((int64_t)turn, n - r0);
+    for (int w = 0; w < records;) {
+      int ncell = 0;
+      if (w + lane < records) {
+        const int64_t i = r0 + w + lane;
+        const int nr = (int)(rec[((i >> 5) * FxRecord::kWords + FxRecord::kInfo) * 32 + (i & 31)] & 0xff);
+        ncell = nr > 3 ? nr : (nr == 3 ? 1 : 0);
+      }
+      const CellSlot cs = assign_cells(ncell);
+      const int64_t i = r0 + w + cs.rec;
+      w += cs.taken;
+      bool ok = cs.cell >= 0;
+      int64_t u = 0;
+      FxScales sm;
+      int ke = 0;
+      long long weight = 0;
+      if (ok) {
+        const long long* o = rec + (i >> 5) * (32 * FxRecord::kWords) + (i & 31);
+        FxView f;
+        f.load<NSUB, NM>(o);
+        u = o[32 * FxRecord::kPair];
+        weight = f.weight(cs.cell);
+        sm = f.sm;
+        ke = f.ke;
+        ok = fx_back_project<NSUB, NM>(f, cs.cell, srec + (int64_t)SR_STRIDE * (4 * (int64_t)ps[u >> 2] + (u & 3)), xm,
+                                       conn_m, pm[u >> 2], pts, stride);
+      }
+      const unsigned bad = __ballot_sync(0xffffffffu, cs.cell >= 0 && !ok);
+      ok &= !(cs.cell >= 0 && (bad >> cs.first & ((1u << cs.cells) - 1u)) != 0);
+      double* out = U + 32 * u;
+      auto emit = [&](int a, int l, long long hh, long long cr) {
+        __stcs(out + 4 * a + l, fx_to_double(hh, cr, ke - sm.shape<NM>(l)));
+      };
+      long long* sums = pts + 28 * stride;
+      FxAcc g[4][4];
+      fx_cell_quadratic<NP, NM, 0>((int)(u & 3), sm, weight, pts, stride, g);
+      fx_sum_cells<NR, NM>(g, cs, ok, sums, stride, emit);
+      out += 4 * NR;
+      fx_cell_quadratic<NP, NM, 1>((int)(u & 3), sm, weight, pts, stride, g);
+      fx_sum_cells<NR, NM>(g, cs, ok, sums, stride, emit);
+      if (ok && (NP < 8 || NM < 4))   // the block is padded with zeros
+        for (int e = cs.cell; e < 32; e += cs.cells)
+          if ((e >> 2) >= NP || (e & 3) >= NM) __stcs(U + 32 * u + e, 0.0);
+      if (cs.cell == 0) {
+        if (ok) uflag[u] = 1;
+        else integrate_unit<NP, NM>(u, ps, pm, srec, xm, conn_m, U, uflag, slow);
+      }
+      __syncwarp();
+    }
+  }
+  // cells and points were counted by the clip kernel
+  block_count_add(&st->newton_fail, slow.newton_fail);
+}
+
+// Pair block = sum of its non-empty unit blocks in the order k = 0..3; flag = any.
 // Sixteen threads per pair, thread j summing the j-th 16-byte pair of entries
 // of the four blocks: every load and store of a half-warp is one contiguous
 // 256-byte segment.
@@ -233,16 +365,17 @@ __global__ void __launch_bounds__(256) k_quadratic_reduce(const double* __restri
   for (int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4; p < n;
        p += ((int64_t)gridDim.x * blockDim.x) >> 4) {
     const double2* u0 = reinterpret_cast<const double2*>(U + 128 * p) + j;
-    double2 acc = __ldcs(u0);
+    const uint32_t f = *reinterpret_cast<const uint32_t*>(uflag + 4 * p);
+    double2 acc = make_double2(0.0, 0.0);
 #pragma unroll
-    for (int k = 1; k < 4; ++k) {
+    for (int k = 0; k < 4; ++k) {
+      if ((f >> (8 * k) & 0xffu) == 0u) continue;   // an empty unit's block is not written
       const double2 t = __ldcs(u0 + 16 * k);
       acc.x += t.x;
       acc.y += t.y;
     }
     __stcs(reinterpret_cast<double2*>(Mblk + 32 * p) + j, acc);
     if (j == 0) {
-      const uint32_t f = *reinterpret_cast<const uint32_t*>(uflag + 4 * p);
       flag[p] = f != 0u ? 1 : 0;
       ne += f != 0u ? 1ull : 0ull;
     }
@@ -252,14 +385,26 @@ __global__ void __launch_bounds__(256) k_quadratic_reduce(const double* __restri
 
 template <int NP, int NM>
 void launch_q(mortar_ctx* c, const RunParams& rp) {
-  auto kern = k_integrate_quadratic<NP, NM>;
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kQThreads, 0);
-  if (per_sm < 1) per_sm = 1;
-  kern<<<(unsigned)(c->n_sm * per_sm), kQThreads, 0, c->stream>>>(
-      c->pairs_s.as<int32_t>(), c->pairs_m.as<int32_t>(), c->srec.as<double>(), c->xm.as<double>(),
-      c->conn_m.as<int32_t>(), rp, c->Qunit.as<double>(), c->Qflag.as<uint8_t>(), c->pair_cap,
-      c->dstat.as<DevStatus>());
+  constexpr int NSUB = NP == 8 ? 4 : 3;
+  IntegrateArgs a{c->pairs_s.as<int32_t>(), c->pairs_m.as<int32_t>(), c->srec.as<double>(), c->xm.as<double>(),
+                  c->conn_m.as<int32_t>(), nullptr, nullptr, nullptr, c->pair_cap, c->dstat.as<DevStatus>(), c->stream};
+  a.order = c->order.as<int32_t>();
+  auto clip = k_quadratic_clip<NP, NM>;
+  auto cells = k_quadratic_cells<NP, NM>;
+  const size_t shm = (size_t)kQThreads * kQPtsBytes;
+  cudaFuncSetAttribute(cells, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+  int clip_sm = 0, cell_sm = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&clip_sm, clip, kQThreads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cell_sm, cells, kQThreads, shm);
+  const unsigned gc = (unsigned)(c->n_sm * (clip_sm < 1 ? 1 : clip_sm)), gq = (unsigned)(c->n_sm * (cell_sm < 1 ? 1 : cell_sm));
+  for (int64_t first = 0; first < c->pair_cap; first += kPairChunk / 4) {
+    launch_pair_sort<NSUB, NM, 4>(a, rp, c->n_sm, kSortBatch, first);
+    clip<<<gc, kQThreads, 0, c->stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, c->Qunit.as<double>(),
+                                          c->Qflag.as<uint8_t>(), c->pair_cap, first, a.order, c->rec.as<long long>(),
+                                          a.st);
+    cells<<<gq, kQThreads, shm, c->stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, c->Qunit.as<double>(),
+                                             c->Qflag.as<uint8_t>(), c->pair_cap, first, c->rec.as<long long>(), a.st);
+  }
   k_quadratic_reduce<<<(unsigned)(c->n_sm * 8), 256, 0, c->stream>>>(c->Qunit.as<double>(), c->Qflag.as<uint8_t>(),
                                                                      c->pair_cap, c->Mblk.as<double>(),
                                                                      c->flag.as<uint8_t>(), c->dstat.as<DevStatus>());

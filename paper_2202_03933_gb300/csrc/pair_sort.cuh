@@ -37,7 +37,9 @@ __device__ __forceinline__ bool fetch_batch(unsigned long long* work_ctr, int64_
 // cell count + the edge intersections of an FP32 clip (0 = no pair); a cost
 // estimate only, the FP64 clip decides.  Counting sort over the key values
 // present, by ballots.  my: the warp's batch memory (batch_smem_bytes(B)).
-template <int NS, int NM>
+// SUB: units per pair (4 for quadratic slave elements: unit u is sub-element
+// u % 4 of pair u / 4, with a record of its own).
+template <int NS, int NM, int SUB>
 __device__ __forceinline__ int sort_batch(unsigned char* my, int B, int64_t base, int64_t lim, int rounds,
                                           const int32_t* __restrict__ ps, const int32_t* __restrict__ pm,
                                           const double* __restrict__ srec, const double* __restrict__ xm,
@@ -55,7 +57,9 @@ __device__ __forceinline__ int sort_batch(unsigned char* my, int B, int64_t base
     int key = 0;
     if (p < lim) {
       int n_int = 0;
-      const int nr = clip_count_f32<NS, NM>(srec + (int64_t)SR_STRIDE * ps[p], xm, conn_m, pm[p], n_int);
+      const int64_t pair = p / SUB;
+      const double* r = srec + (int64_t)SR_STRIDE * (SUB * (int64_t)ps[pair] + p % SUB);
+      const int nr = clip_count_f32<NS, NM>(r, xm, conn_m, pm[pair], n_int);
       key = 1 + 16 * (nr == 0 ? 0 : (nr == 3 ? 1 : min(nr, kPolyS))) + min(n_int, 15);
       atomicOr(&pres[key >> 5], 1u << (key & 31));
     }
@@ -93,7 +97,7 @@ __device__ __forceinline__ int sort_batch(unsigned char* my, int B, int64_t base
 // registers, many warps.
 constexpr int kSortThreads = 128;
 constexpr int kSortBatch = 1024;   // default pairs per warp batch, and the most
-template <int NS, int NM>
+template <int NS, int NM, int SUB>
 __global__ void __launch_bounds__(kSortThreads) k_pair_sort(
     const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
     const double* __restrict__ xm, const int32_t* __restrict__ conn_m, int64_t pair_cap, int64_t first, int B,
@@ -102,7 +106,7 @@ __global__ void __launch_bounds__(kSortThreads) k_pair_sort(
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* my = smem_raw + (size_t)(threadIdx.x >> 5) * batch_smem_bytes(B);
   const uint16_t* perm = reinterpret_cast<const uint16_t*>(my + 32);
-  const int64_t n = chunk_pairs(st, pair_cap, first, kPairChunk);
+  const int64_t n = SUB * chunk_pairs(st, pair_cap, first, kPairChunk / SUB);   // units
   ps += first;
   pm += first;
   const int64_t share = 2 * (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -113,16 +117,16 @@ __global__ void __launch_bounds__(kSortThreads) k_pair_sort(
     int fetch;
     if (!fetch_batch(&st->pair_ctr[0], n, share, B, base, fetch)) break;
     const int64_t lim = min(n, base + (int64_t)fetch);
-    const int live = sort_batch<NS, NM>(my, B, base, lim, (fetch + 31) >> 5, ps, pm, srec, xm, conn_m);
+    const int live = sort_batch<NS, NM, SUB>(my, B, base, lim, (fetch + 31) >> 5, ps, pm, srec, xm, conn_m);
     for (int i = threadIdx.x & 31; i < live; i += 32) order[base + i] = (int32_t)(base + perm[i]);
     __syncwarp();
   }
 }
 
-template <int NS, int NM>
+template <int NS, int NM, int SUB = 1>
 void launch_pair_sort(const IntegrateArgs& a, const RunParams& rp, int n_sm, int B, int64_t first) {
   cudaMemsetAsync(&a.st->pair_ctr, 0, sizeof(a.st->pair_ctr), a.stream);   // the chunk's kernels
-  auto kern = k_pair_sort<NS, NM>;
+  auto kern = k_pair_sort<NS, NM, SUB>;
   const size_t shm = (size_t)(kSortThreads / 32) * batch_smem_bytes(B);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSortThreads, shm);

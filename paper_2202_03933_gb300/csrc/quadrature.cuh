@@ -366,4 +366,34 @@ __device__ __forceinline__ CellSlot assign_cells(int ncell) {
   return s;
 }
 
+// Adds up the cells' sums g of every pair of the warp: the lanes of a pair take
+// its entries (a, l) in turn and pass each sum, hh + cr / 2^32, to emit.  buf:
+// this thread's slice of shared memory (24 words; entry i at buf[i * stride],
+// lane L's at buf - lane + L), free to use by the whole warp.
+template <int NR, int NC, class Emit>
+__device__ __forceinline__ void fx_sum_cells(const FxAcc g[4][4], const CellSlot& cs, bool ok,
+                                             long long* __restrict__ buf, int stride, Emit emit) {
+  __syncwarp();
+#pragma unroll
+  for (int a = 0; a < NR; ++a)
+#pragma unroll
+    for (int l = 0; l < NC; ++l) {
+      const int e = NC * a + l;
+      buf[e * stride] = g[a][l].hh + (g[a][l].cr >> 32);
+      reinterpret_cast<unsigned*>(buf + (16 + (e >> 1)) * stride)[e & 1] = (unsigned)g[a][l].cr;
+    }
+  __syncwarp();
+  const long long* pair = buf - (threadIdx.x & 31) + cs.first;
+  if (ok)
+#pragma unroll 1
+    for (int e = cs.cell; e < NR * NC; e += cs.cells) {
+      long long hh = 0, cr = 0;
+      for (int k = 0; k < cs.cells; ++k) {
+        hh += pair[e * stride + k];
+        cr += reinterpret_cast<const unsigned*>(pair + (16 + (e >> 1)) * stride + k)[e & 1];
+      }
+      emit(e / NC, e % NC, hh, cr);
+    }
+}
+
 }  // namespace mortar
