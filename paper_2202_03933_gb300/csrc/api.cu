@@ -502,8 +502,8 @@ void mortar_destroy(mortar_ctx* c) {
                     &c->srec, &c->De, &c->box_s, &c->box_m, &c->chunk_red, &c->grid, &c->mkey, &c->bin_cnt,
                     &c->bin_start, &c->bin_elems, &c->cand_cnt, &c->pair_off, &c->pairs_s, &c->pairs_m, &c->Mblk,
                     &c->Dblk, &c->flag, &c->row_cnt, &c->row_cnt2, &c->rowptr_D, &c->col_D, &c->val_D, &c->rowptr_M,
-                    &c->col_M, &c->val_M, &c->scan_tmp, &c->lambda, &c->gs_pair, &c->gm_pair, &c->abar_pair,
-                    &c->J_pair, &c->ge_elem, &c->mp_cnt, &c->mp_off, &c->mp_list, &c->grad_s, &c->grad_m,
+                    &c->col_M, &c->val_M, &c->scan_tmp, &c->lambda, &c->sl_pair, &c->gm_pair, &c->mult,
+                    &c->ge_elem, &c->mp_cnt, &c->mp_off, &c->mp_list, &c->grad_s, &c->grad_m,
                     &c->J_part, &c->dstat, &c->cta_t, &c->tan_ys, &c->tan_ym, &c->tan_Kp, &c->tan_Op,
                     &c->tan_Ke, &c->tan_rowptr, &c->tan_col, &c->tan_val, &c->rule_1d, &c->nrm_m,
                     &c->cn_normals, &c->cn_gap, &c->cn_lam, &c->cn_active, &c->cn_ncp, &c->Qunit, &c->Qflag, &c->rec, &c->order};

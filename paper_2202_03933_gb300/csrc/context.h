@@ -86,7 +86,8 @@ struct mortar_ctx {
 
   // ---- adjoint workspaces
   mortar::DevBuf lambda;                    // Ns x 3
-  mortar::DevBuf gs_pair, gm_pair, abar_pair, J_pair;   // per pair
+  mortar::DevBuf sl_pair, gm_pair;          // per pair: slave side (summed per element), master node gradients
+  mortar::DevBuf mult;                      // per slave element: multipliers, nodal and monomial (24)
   mortar::DevBuf ge_elem;                   // per slave element 4x3 + J
   mortar::DevBuf mp_cnt, mp_off, mp_list;   // master element -> pairs
   mortar::DevBuf grad_s, grad_m;            // Ns x 3, Nm x 3

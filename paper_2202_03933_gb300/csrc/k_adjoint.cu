@@ -68,19 +68,44 @@ struct FwdOut {
   uint8_t* flag;
 };
 
+// What a pair contributes to its slave element, summed per element by
+// k_adjoint_elems before the steps that depend on the element alone (dual
+// basis, J, auxiliary plane): Lb_c = dJ/dLambda_c (12), in-plane adjoints of the
+// slave nodes (4 + 4), adjoints of the plane from the master nodes (x0, t1, t2),
+// one word of padding, and (segment D) the direct slave node gradients (12).
+template <bool SEG>
+constexpr int kSlavePair = SEG ? 42 : 30;
+
+template <bool SEG>
+__device__ __forceinline__ void store_slave_pair(double* __restrict__ sl, int64_t p, const V3* Lb, const double* sbu,
+                                                 const double* sbv, const PlaneBar& pb, const double gX[4][3]) {
+  double2* o = reinterpret_cast<double2*>(sl + kSlavePair<SEG> * p);
+  auto put = [&](int k, double a, double b) { __stcs(o + k, make_double2(a, b)); };
+  for (int c = 0; c < 4; c += 2) {
+    put(3 * c / 2, Lb[c].x, Lb[c].y);
+    put(3 * c / 2 + 1, Lb[c].z, Lb[c + 1].x);
+    put(3 * c / 2 + 2, Lb[c + 1].y, Lb[c + 1].z);
+  }
+  put(6, sbu[0], sbu[1]); put(7, sbu[2], sbu[3]);
+  put(8, sbv[0], sbv[1]); put(9, sbv[2], sbv[3]);
+  put(10, pb.x0.x, pb.x0.y); put(11, pb.x0.z, pb.t1.x); put(12, pb.t1.y, pb.t1.z);
+  put(13, pb.t2.x, pb.t2.y); put(14, pb.t2.z, 0.0);
+  if (SEG)
+    for (int k = 0; k < 6; ++k) put(15 + k, gX[2 * k / 3][2 * k % 3], gX[(2 * k + 1) / 3][(2 * k + 1) % 3]);
+}
+
 template <int NS, int NM, bool SEG, bool DUAL>
 __device__ void adjoint_one(int64_t p, const int32_t* __restrict__ ps, const int32_t* __restrict__ pm,
                             const double* __restrict__ srec, const double* __restrict__ xs,
                             const double* __restrict__ xm, const int32_t* __restrict__ conn_s,
                             const int32_t* __restrict__ conn_m, const double* __restrict__ lambda,
-                            const RunParams& rp, double* __restrict__ gs_out, double* __restrict__ gm_out,
-                            double* __restrict__ ab_out, double* __restrict__ J_out, AdjCounters& ctr) {
+                            const RunParams& rp, double* __restrict__ sl_out, double* __restrict__ gm_out,
+                            AdjCounters& ctr) {
   const int32_t s = ps[p], m = pm[p];
   const double* r = srec + (int64_t)SR_STRIDE * s;
   double gX[4][3], gY[4][3], Lb[4][3];
   for (int a = 0; a < 4; ++a)
     for (int k = 0; k < 3; ++k) { gX[a][k] = 0.0; gY[a][k] = 0.0; Lb[a][k] = 0.0; }
-  double Jp = 0.0;
   const double eps_in = r[SR_EPSIN];
   bool nonempty = false;
   V3 X[4], Y[4], lam[4], Lam[4];
@@ -179,7 +204,6 @@ __device__ void adjoint_one(int64_t p, const int32_t* __restrict__ ps, const int
           for (int l = 0; l < NM; ++l) xmI = xmI + Nm[l] * Y[l];
           const V3 qv = xsI - xmI;
           const double f = dot(Lh, qv);
-          Jp += W * f;
           // ---- reverse of this quadrature point
           area_b += w * f;
           const V3 Lhb = W * qv, qb = W * Lh;
@@ -229,26 +253,16 @@ __device__ void adjoint_one(int64_t p, const int32_t* __restrict__ ps, const int
       cr.template reverse<NM>(r, Rbu, Rbv, srev, mrev, sbu, sbv, mbu, mbv);
       map_coeff_reverse<NS>(smb, sbu, sbv);
       map_coeff_reverse<NM>(mmb, mbu, mbv);
-      const V3 n0 = v3(r[SR_N0], r[SR_N0 + 1], r[SR_N0 + 2]);
-      plane_reverse<NS, NM>(X, Y, x0, t1, t2, n0, sbu, sbv, mbu, mbv, gX, gY);
+      PlaneBar pb{v3(0, 0, 0), v3(0, 0, 0), v3(0, 0, 0)};
+      project_reverse<NM>(Y, x0, t1, t2, mbu, mbv, gY, pb);
+      V3 L[4];
+      for (int c = 0; c < 4; ++c) L[c] = v3(Lb[c][0], Lb[c][1], Lb[c][2]);
+      store_slave_pair<SEG>(sl_out, p, L, sbu, sbv, pb, gX);
+      double* gmo = gm_out + 12 * p;
+      for (int a = 0; a < 4; ++a)
+        for (int k = 0; k < 3; ++k) gmo[3 * a + k] = gY[a][k];
     }
   }
-  double* go = gs_out + 12 * p;
-  double* gmo = gm_out + 12 * p;
-  for (int a = 0; a < 4; ++a)
-    for (int k = 0; k < 3; ++k) {
-      go[3 * a + k] = gX[a][k];
-      gmo[3 * a + k] = gY[a][k];
-    }
-  if (DUAL) {
-    double* ab = ab_out + 16 * p;
-    for (int a = 0; a < 4; ++a)
-      for (int c = 0; c < 4; ++c)
-        ab[4 * a + c] = (nonempty && a < NS && c < NS)
-                            ? lam[a].x * Lb[c][0] + lam[a].y * Lb[c][1] + lam[a].z * Lb[c][2]
-                            : 0.0;
-  }
-  J_out[p] = Jp;
 }
 
 template <int NS, int NM, bool SEG, bool DUAL>
@@ -256,8 +270,7 @@ __global__ void __launch_bounds__(kMaxPairBlock) k_adjoint_pairs(
     const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
     const double* __restrict__ xs, const double* __restrict__ xm, const int32_t* __restrict__ conn_s,
     const int32_t* __restrict__ conn_m, const double* __restrict__ lambda, RunParams rp, int64_t pair_cap,
-    int32_t chunk, double* __restrict__ gs_out, double* __restrict__ gm_out, double* __restrict__ ab_out,
-    double* __restrict__ J_out, DevStatus* st) {
+    int32_t chunk, double* __restrict__ sl_out, double* __restrict__ gm_out, DevStatus* st) {
   AdjCounters ctr;
   const int lane = threadIdx.x & 31;
   const bool ok = st->over_pairs == 0 && st->over_bins == 0;
@@ -271,8 +284,7 @@ __global__ void __launch_bounds__(kMaxPairBlock) k_adjoint_pairs(
     if (base >= n) break;
     const int64_t end = min(base + (int64_t)chunk, n);
     for (int64_t p = base + lane; p < end; p += 32)
-      adjoint_one<NS, NM, SEG, DUAL>(p, ps, pm, srec, xs, xm, conn_s, conn_m, lambda, rp, gs_out, gm_out, ab_out,
-                                     J_out, ctr);
+      adjoint_one<NS, NM, SEG, DUAL>(p, ps, pm, srec, xs, xm, conn_s, conn_m, lambda, rp, sl_out, gm_out, ctr);
   }
   block_count_add(&st->clip_overflow, ctr.clip_over);
   block_count_add(&st->newton_fail, ctr.newton_fail);
@@ -309,130 +321,133 @@ __device__ __forceinline__ void lm_weights(const double* __restrict__ r, const V
   }
 }
 
-// From a pair's sums (G, H, map-coefficient adjoints smb and mmb, adjoints Bu,
-// Bv of the polygon's vertices at their pool slots): the reverse of clip,
-// projection and plane, the direct terms and J; and the forward blocks if
-// `blocks`.  Outputs go out with streaming (evict-first) stores: each is
-// written once and read by a later kernel, and L2 keeps the threads' stack
-// lines instead.
-template <int NS, int NM, bool SEG, bool DUAL>
-__device__ __forceinline__ void adjoint_finish(int64_t p, int32_t s, int32_t m, const double* __restrict__ r,
-                                               const double* __restrict__ xs, const double* __restrict__ xm,
-                                               const int32_t* __restrict__ conn_s,
-                                               const int32_t* __restrict__ conn_m, const double* __restrict__ lambda,
-                                               const ClipPool<NS, NM>& cp, double* Bu, double* Bv, bool mrev,
-                                               const double* smb, const double* mmb, const double G[4][4],
-                                               const double H[4][4], bool blocks, double* __restrict__ gs_out,
-                                               double* __restrict__ gm_out, double* __restrict__ ab_out,
-                                               double* __restrict__ J_out, const FwdOut& fo) {
-  const int32_t* cs = conn_s + (int64_t)NS * s;
-  const int32_t* cm = conn_m + (int64_t)NM * m;
-  const V3 x0 = v3(r[SR_X0], r[SR_X0 + 1], r[SR_X0 + 2]);
-  const V3 t1 = v3(r[SR_T1], r[SR_T1 + 1], r[SR_T1 + 2]);
-  const V3 t2 = v3(r[SR_T2], r[SR_T2 + 1], r[SR_T2 + 2]);
-  const bool srev = r[SR_REV] != 0.0;
-  double Jp = 0.0;
-  V3 Lb[4];
-  if (blocks) {   // forward: M = A G, D = A H of this pair
-    double* mo = fo.Mblk + 16 * p;
-    for (int a = 0; a < 4; ++a)
-      for (int l = 0; l < 4; ++l) {
-        double v = 0.0;
-        if (a < NS && l < NM) {
-          if (DUAL)
-            for (int c = 0; c < NS; ++c) v += r[SR_A + 4 * a + c] * G[c][l];
-          else
-            v = G[a][l];
-        }
-        __stcs(mo + 4 * a + l, v);
-      }
-    if (SEG) {
-      double* dout = fo.Dblk + 16 * p;
-      for (int a = 0; a < 4; ++a)
-        for (int b = 0; b < 4; ++b) {
-          double v = 0.0;
-          if (a < NS && b < NS) {
-            if (DUAL)
-              for (int c = 0; c < NS; ++c) v += r[SR_A + 4 * a + c] * H[c][b];
-            else
-              v = H[a][b];
-          }
-          __stcs(dout + 4 * a + b, v);
-        }
-    }
-    __stcs(fo.flag + p, (uint8_t)1);
+// Lambda_c (12 words) and its monomial coefficients LM_i (12) of every slave
+// element: the pairs of an element share them.
+template <int NS, bool DUAL>
+__global__ void __launch_bounds__(kThreads) k_multipliers(const int32_t* __restrict__ conn_s,
+                                                          const double* __restrict__ lambda,
+                                                          const double* __restrict__ srec, int64_t Es,
+                                                          double* __restrict__ out) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= Es) return;
+  V3 lam[4], Lam[4], LM[4];
+  for (int a = 0; a < 4; ++a) Lam[a] = LM[a] = v3(0, 0, 0);
+  for (int a = 0; a < NS; ++a) {
+    const int64_t n = conn_s[(int64_t)NS * e + a];
+    lam[a] = v3(lambda[3 * n], lambda[3 * n + 1], lambda[3 * n + 2]);
   }
-  // ---- reverse merge and clipping (vertex pool) and the element maps
-  double sbu[4] = {0, 0, 0, 0}, sbv[4] = {0, 0, 0, 0}, mbu[4] = {0, 0, 0, 0}, mbv[4] = {0, 0, 0, 0};
-  cp.reverse(r, Bu, Bv, srev, mrev, sbu, sbv, mbu, mbv);
-  map_coeff_reverse<NS>(smb, sbu, sbv);
-  map_coeff_reverse<NM>(mmb, mbu, mbv);
-  // ---- direct terms and J from the forward accumulators, then the
-  //      reverse of the projection onto the auxiliary plane
-  V3 X[4], Y[4], lam[4], Lam[4];
-  load_pair_nodes<NS, NM>(cs, cm, xs, xm, lambda, X, Y, lam);
-  lm_weights<NS, DUAL>(r, lam, Lam);
-  double gX[4][3], gY[4][3];
-  for (int a = 0; a < 4; ++a)
-    for (int k = 0; k < 3; ++k) { gX[a][k] = 0.0; gY[a][k] = 0.0; }
-  for (int c = 0; c < NS; ++c) {
-    V3 acc = v3(0, 0, 0);
-    if (SEG)
-      for (int b = 0; b < NS; ++b) acc = acc + H[c][b] * X[b];
-    for (int l = 0; l < NM; ++l) acc = acc - G[c][l] * Y[l];
-    Lb[c] = acc;
-    Jp += dot(Lam[c], acc);
+  lm_weights<NS, DUAL>(srec + (int64_t)SR_STRIDE * e, lam, Lam);
+  nodal_to_mono<NS>(Lam, LM);
+  double* o = out + 24 * e;
+  for (int a = 0; a < 4; ++a) {
+    o[3 * a] = Lam[a].x; o[3 * a + 1] = Lam[a].y; o[3 * a + 2] = Lam[a].z;
+    o[12 + 3 * a] = LM[a].x; o[12 + 3 * a + 1] = LM[a].y; o[12 + 3 * a + 2] = LM[a].z;
   }
-  for (int l = 0; l < NM; ++l) {
-    V3 acc = v3(0, 0, 0);
-    for (int c = 0; c < NS; ++c) acc = acc + G[c][l] * Lam[c];
-    gY[l][0] -= acc.x; gY[l][1] -= acc.y; gY[l][2] -= acc.z;
-  }
-  if (SEG)
-    for (int b = 0; b < NS; ++b) {
-      V3 acc = v3(0, 0, 0);
-      for (int c = 0; c < NS; ++c) acc = acc + H[c][b] * Lam[c];
-      gX[b][0] += acc.x; gX[b][1] += acc.y; gX[b][2] += acc.z;
-    }
-  const V3 n0 = v3(r[SR_N0], r[SR_N0 + 1], r[SR_N0 + 2]);
-  plane_reverse<NS, NM>(X, Y, x0, t1, t2, n0, sbu, sbv, mbu, mbv, gX, gY);
-  double* go = gs_out + 12 * p;
-  double* gmo = gm_out + 12 * p;
-  for (int a = 0; a < 4; ++a)
-    for (int k = 0; k < 3; ++k) {
-      __stcs(go + 3 * a + k, gX[a][k]);
-      __stcs(gmo + 3 * a + k, gY[a][k]);
-    }
-  if (DUAL) {
-    double* ab = ab_out + 16 * p;
-    for (int a = 0; a < 4; ++a)
-      for (int c = 0; c < 4; ++c) __stcs(ab + 4 * a + c, (a < NS && c < NS) ? dot(lam[a], Lb[c]) : 0.0);
-  }
-  __stcs(J_out + p, Jp);
 }
 
-// Outputs of a pair without a polygon.
-template <bool SEG, bool DUAL>
-__device__ __forceinline__ void adjoint_empty(int64_t p, double* __restrict__ gs_out, double* __restrict__ gm_out,
-                                              double* __restrict__ ab_out, double* __restrict__ J_out,
-                                              const FwdOut& fo) {
-  double2* g1 = reinterpret_cast<double2*>(gs_out + 12 * p);
-  double2* g2 = reinterpret_cast<double2*>(gm_out + 12 * p);
-  for (int k = 0; k < 6; ++k) { __stcs(g1 + k, make_double2(0.0, 0.0)); __stcs(g2 + k, make_double2(0.0, 0.0)); }
-  if (DUAL) {
-    double2* a2 = reinterpret_cast<double2*>(ab_out + 16 * p);
-    for (int k = 0; k < 8; ++k) __stcs(a2 + k, make_double2(0.0, 0.0));
-  }
-  {
-    double2* mo = reinterpret_cast<double2*>(fo.Mblk + 16 * p);
-    for (int k = 0; k < 8; ++k) __stcs(mo + k, make_double2(0.0, 0.0));
-    if (SEG) {
-      double2* dd = reinterpret_cast<double2*>(fo.Dblk + 16 * p);
-      for (int k = 0; k < 8; ++k) __stcs(dd + k, make_double2(0.0, 0.0));
+template <int N>
+__device__ __forceinline__ void load_v3(const double* __restrict__ o, V3* v) {
+  for (int a = 0; a < N; ++a) v[a] = v3(o[3 * a], o[3 * a + 1], o[3 * a + 2]);
+}
+
+// M = A G and D = A H of a pair from FP64 sums.
+template <int NS, int NM, bool SEG, bool DUAL>
+__device__ __forceinline__ void adjoint_blocks(int64_t p, const double* __restrict__ r, const double G[4][4],
+                                               const double H[4][4], const FwdOut& fo) {
+  double* mo = fo.Mblk + 16 * p;
+  for (int a = 0; a < 4; ++a)
+    for (int l = 0; l < 4; ++l) {
+      double v = 0.0;
+      if (a < NS && l < NM) {
+        if (DUAL)
+          for (int c = 0; c < NS; ++c) v += r[SR_A + 4 * a + c] * G[c][l];
+        else
+          v = G[a][l];
+      }
+      __stcs(mo + 4 * a + l, v);
     }
-    __stcs(fo.flag + p, (uint8_t)0);
+  if (SEG) {
+    double* dout = fo.Dblk + 16 * p;
+    for (int a = 0; a < 4; ++a)
+      for (int b = 0; b < 4; ++b) {
+        double v = 0.0;
+        if (a < NS && b < NS) {
+          if (DUAL)
+            for (int c = 0; c < NS; ++c) v += r[SR_A + 4 * a + c] * H[c][b];
+          else
+            v = H[a][b];
+        }
+        __stcs(dout + 4 * a + b, v);
+      }
   }
-  __stcs(J_out + p, 0.0);
+  __stcs(fo.flag + p, (uint8_t)1);
+}
+
+// From a pair's sums (G, H, map-coefficient adjoints smb and mmb, adjoints Bu,
+// Bv of the polygon's vertices at their pool slots): the reverse of the clip,
+// the master's part of the projection, and the direct terms.  Outputs go out
+// with streaming (evict-first) stores: each is written once and read by a later
+// kernel, and L2 keeps the threads' stack lines instead.
+template <int NS, int NM, bool SEG>
+__device__ __forceinline__ void adjoint_finish(int64_t p, const int32_t* __restrict__ cs,
+                                               const int32_t* __restrict__ cm, const double* __restrict__ r,
+                                               const double* __restrict__ xs, const double* __restrict__ xm,
+                                               const V3* Lam, const ClipPool<NS, NM>& cp, double* Bu, double* Bv,
+                                               bool mrev, const double* smb, const double* mmb,
+                                               const double G[4][4], const double H[4][4],
+                                               double* __restrict__ sl_out, double* __restrict__ gm_out) {
+  double sbu[4] = {0, 0, 0, 0}, sbv[4] = {0, 0, 0, 0}, mbu[4] = {0, 0, 0, 0}, mbv[4] = {0, 0, 0, 0};
+  cp.reverse(r, Bu, Bv, r[SR_REV] != 0.0, mrev, sbu, sbv, mbu, mbv);
+  map_coeff_reverse<NS>(smb, sbu, sbv);
+  map_coeff_reverse<NM>(mmb, mbu, mbv);
+  V3 X[4], Y[4], Lb[4];
+  for (int l = 0; l < NM; ++l) {
+    const int64_t n = cm[l];
+    Y[l] = v3(xm[3 * n], xm[3 * n + 1], xm[3 * n + 2]);
+  }
+  if (SEG)
+    for (int a = 0; a < NS; ++a) {
+      const int64_t n = cs[a];
+      X[a] = v3(xs[3 * n], xs[3 * n + 1], xs[3 * n + 2]);
+    }
+  double gX[4][3], gY[4][3];
+  for (int c = 0; c < 4; ++c) {
+    V3 acc = v3(0, 0, 0);
+    if (c < NS) {
+      if (SEG)
+        for (int b = 0; b < NS; ++b) acc = acc + H[c][b] * X[b];
+      for (int l = 0; l < NM; ++l) acc = acc - G[c][l] * Y[l];
+    }
+    Lb[c] = acc;
+  }
+  for (int l = 0; l < 4; ++l) {
+    V3 acc = v3(0, 0, 0), acx = v3(0, 0, 0);
+    for (int c = 0; c < NS; ++c) {
+      if (l < NM) acc = acc - G[c][l] * Lam[c];
+      if (SEG && l < NS) acx = acx + H[c][l] * Lam[c];
+    }
+    gY[l][0] = acc.x; gY[l][1] = acc.y; gY[l][2] = acc.z;
+    if (SEG) { gX[l][0] = acx.x; gX[l][1] = acx.y; gX[l][2] = acx.z; }
+  }
+  PlaneBar pb{v3(0, 0, 0), v3(0, 0, 0), v3(0, 0, 0)};
+  project_reverse<NM>(Y, v3(r[SR_X0], r[SR_X0 + 1], r[SR_X0 + 2]), v3(r[SR_T1], r[SR_T1 + 1], r[SR_T1 + 2]),
+                      v3(r[SR_T2], r[SR_T2 + 1], r[SR_T2 + 2]), mbu, mbv, gY, pb);
+  store_slave_pair<SEG>(sl_out, p, Lb, sbu, sbv, pb, gX);
+  double2* gmo = reinterpret_cast<double2*>(gm_out + 12 * p);
+  for (int k = 0; k < 6; ++k)
+    __stcs(gmo + k, make_double2(gY[2 * k / 3][2 * k % 3], gY[(2 * k + 1) / 3][(2 * k + 1) % 3]));
+}
+
+// Forward outputs of a pair without a polygon.
+template <bool SEG>
+__device__ __forceinline__ void adjoint_empty(int64_t p, const FwdOut& fo) {
+  double2* mo = reinterpret_cast<double2*>(fo.Mblk + 16 * p);
+  for (int k = 0; k < 8; ++k) __stcs(mo + k, make_double2(0.0, 0.0));
+  if (SEG) {
+    double2* dd = reinterpret_cast<double2*>(fo.Dblk + 16 * p);
+    for (int k = 0; k < 8; ++k) __stcs(dd + k, make_double2(0.0, 0.0));
+  }
+  __stcs(fo.flag + p, (uint8_t)0);
 }
 
 // ---------------------------------------------------------------- variant 0
@@ -463,9 +478,8 @@ __device__ __noinline__ void adjoint_pair_fast(int64_t p, const int32_t* __restr
                                   const double* __restrict__ srec, const double* __restrict__ xs,
                                   const double* __restrict__ xm, const int32_t* __restrict__ conn_s,
                                   const int32_t* __restrict__ conn_m, const double* __restrict__ lambda,
-                                  double* __restrict__ gs_out, double* __restrict__ gm_out,
-                                  double* __restrict__ ab_out, double* __restrict__ J_out,
-                                  const FwdOut& fo, AdjCounters& ctr) {
+                                  double* __restrict__ sl_out, double* __restrict__ gm_out, const FwdOut& fo,
+                                  AdjCounters& ctr) {
   constexpr int KS = NS, KM = NM;   // monomials per side (quad4: 4, tri3: 3)
   double CYv[16], SXv[SEG ? 16 : 1];
   auto CYs = [&](int i, int j) -> double& { return CYv[4 * i + j]; };
@@ -700,11 +714,14 @@ ctr.cells++; ctr.gp += 7;
       const double inv = kInvCount[nr];
       for (int k = 0; k < nr; ++k) { const int sk = cp.id(k); Bu[sk] += cbu * inv; Bv[sk] += cbv * inv; }
     }
-    adjoint_finish<NS, NM, SEG, DUAL>(p, s, m, r, xs, xm, conn_s, conn_m, lambda, cp, Bu, Bv, mrev, smb, mmb, G, H, true,
-                                      gs_out, gm_out, ab_out, J_out, fo);
+    V3 X[4], Y[4], lam[4], Lam[4];
+    load_pair_nodes<NS, NM>(cs, cm, xs, xm, lambda, X, Y, lam);
+    lm_weights<NS, DUAL>(r, lam, Lam);
+    adjoint_blocks<NS, NM, SEG, DUAL>(p, r, G, H, fo);
+    adjoint_finish<NS, NM, SEG>(p, cs, cm, r, xs, xm, Lam, cp, Bu, Bv, mrev, smb, mmb, G, H, sl_out, gm_out);
     ctr.nonempty++;
   } else {
-    adjoint_empty<SEG, DUAL>(p, gs_out, gm_out, ab_out, J_out, fo);
+    adjoint_empty<SEG>(p, fo);
   }
 }
 
@@ -763,10 +780,9 @@ struct AdjArgs {
   int64_t first;   // first pair of the chunk
   const int32_t* order;
   long long* rec;
-  double* gs;
+  const double* mult;   // k_multipliers
+  double* sl;
   double* gm;
-  double* ab;
-  double* J;
   FwdOut fo;
   DevStatus* st;
   int32_t watchdog_us;
@@ -783,7 +799,7 @@ __device__ __forceinline__ bool next_group(unsigned long long* ctr, int64_t n, i
 // First kernel of the default adjoint (variant 0; the forward blocks come with
 // it): FP64 clip with its record, the pair's bilinear forms CY [and SX], and
 // the conversion to fixed point.  One record per pair, in sorted order.
-template <int NS, int NM, bool SEG, bool DUAL>
+template <int NS, int NM, bool SEG>
 __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, unsigned long long* cta_t) {
   cta_mark(cta_t, 0);
   constexpr int W = SEG ? AdjRecord::kWordsSeg : AdjRecord::kWords;
@@ -816,7 +832,7 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, un
       const bool mrev = ma2 < 0.0;
       ClipPool<NS, NM> cp;
       if (!cp.run(r, mu, mv, mrev, ctr.clip_over)) {
-        adjoint_empty<SEG, DUAL>(p, g.gs, g.gm, g.ab, g.J, g.fo);
+        adjoint_empty<SEG>(p, g.fo);
       } else {
         store_pool(o, cp, mrev);
         double pu[FxPolygon::kCap], pv[FxPolygon::kCap];
@@ -828,13 +844,12 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, un
         mark = kSlowPair;
         if (f.setup<NS, NM>(r, mmap, pu, pv, cp.nr)) {
           // bilinear forms of the pair, and their scales
-          V3 X[4], Y[4], lam[4], LM[4], YM[4];
-          load_pair_nodes<NS, NM>(g.conn_s + (int64_t)NS * s, cm, g.xs, g.xm, g.lambda, X, Y, lam);
-          {
-            V3 Lam[4];
-            lm_weights<NS, DUAL>(r, lam, Lam);
-            nodal_to_mono<NS>(Lam, LM);
+          V3 Y[4], LM[4], YM[4];
+          for (int l = 0; l < NM; ++l) {
+            const int64_t nd = cm[l];
+            Y[l] = v3(g.xm[3 * nd], g.xm[3 * nd + 1], g.xm[3 * nd + 2]);
           }
+          load_v3<NS>(g.mult + 24 * (int64_t)s + 12, LM);
           nodal_to_mono<NM>(Y, YM);
           double C[4][4], S[4][4];
 #pragma unroll
@@ -842,7 +857,11 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, un
 #pragma unroll
             for (int b = 0; b < NM; ++b) C[a][b] = dot(LM[a], YM[b]);
           if (SEG) {
-            V3 XM[4];
+            V3 X[4], XM[4];
+            for (int a = 0; a < NS; ++a) {
+              const int64_t nd = g.conn_s[(int64_t)NS * s + a];
+              X[a] = v3(g.xs[3 * nd], g.xs[3 * nd + 1], g.xs[3 * nd + 2]);
+            }
             nodal_to_mono<NS>(X, XM);
 #pragma unroll
             for (int a = 0; a < NS; ++a)
@@ -952,14 +971,14 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
     long long weight = 0, e1u = 0, e1v = 0, e2u = 0, e2v = 0;
     if (ok) {
       const int64_t p = o[32 * FxRecord::kPair];
+      const double* sr = ar.srec + (int64_t)SR_STRIDE * ar.ps[p];
       f.load<NS, NM>(o);
       sc.load(o[32 * AdjRecord::kScales], o[32 * AdjRecord::kScales2], f.ke, f.E);
       weight = f.weight(cs.cell);
       const int ib = f.ib(cs.cell), iw = f.iw(cs.cell);
       e1u = f.x(ib) - f.cu; e1v = f.y(ib) - f.cv;
       e2u = f.x(iw) - f.cu; e2v = f.y(iw) - f.cv;
-      ok = fx_back_project<NS, NM>(f, cs.cell, ar.srec + (int64_t)SR_STRIDE * ar.ps[p], ar.xm, ar.conn_m, ar.pm[p],
-                                   pts, stride);
+      ok = fx_back_project<NS, NM>(f, cs.cell, sr, ar.xm, ar.conn_m, ar.pm[p], pts, stride);
     }
     __syncthreads();
     long long area = 0;
@@ -1049,15 +1068,15 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
     __syncthreads();
     {
       FxAcc g[4][4];
-      FxAcc h[4][4];
-      if (SEG) fx_cell_products<NS, NS, true>(f.ss, f.ss, weight, pts, stride, h);
-      fx_cell_products<NS, NM, false>(f.ss, f.sm, weight, pts, stride, g);
-      if (SEG)
-        fx_sum_cells<NS, NS>(h, cs, ok, pts, stride, [&](int a, int b, long long hh, long long cr) {
+      if (SEG) {
+        fx_cell_products<NS, NS, true>(f.ss, f.ss, weight, pts, stride, g);
+        fx_sum_cells<NS, NS>(g, cs, ok, sums, stride, [&](int a, int b, long long hh, long long cr) {
           o[32 * (AdjRecord::kH + 4 * a + b)] =
               __double_as_longlong(fx_to_double(hh, cr, f.ke - f.ss.shape<NS>(a) - f.ss.shape<NS>(b)));
         });
-      fx_sum_cells<NS, NM>(g, cs, ok, pts, stride, [&](int a, int l, long long hh, long long cr) {
+      }
+      fx_cell_products<NS, NM, false>(f.ss, f.sm, weight, pts, stride, g);
+      fx_sum_cells<NS, NM>(g, cs, ok, sums, stride, [&](int a, int l, long long hh, long long cr) {
         o[32 * (AdjRecord::kG + 4 * a + l)] =
             __double_as_longlong(fx_to_double(hh, cr, f.ke - f.ss.shape<NS>(a) - f.sm.shape<NM>(l)));
       });
@@ -1066,8 +1085,8 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
   }
 }
 
-// Third kernel: per pair, the forward blocks, the reverse of clip, projection
-// and plane, the direct terms and J.
+// Third kernel: per pair, the forward blocks, the reverse of the clip and of
+// the master's projection, and the direct terms.
 template <int NS, int NM, bool SEG, bool DUAL>
 __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_finish(AdjArgs g) {
   constexpr int W = SEG ? AdjRecord::kWordsSeg : AdjRecord::kWords;
@@ -1081,7 +1100,7 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_finish(AdjArgs g) 
     const int nr = (int)(o[32 * FxRecord::kInfo] & 0xff);
     if (nr == kSlowPair) {
       adjoint_pair_fast<NS, NM, SEG, DUAL>(o[32 * FxRecord::kPair], g.ps, g.pm, g.srec, g.xs, g.xm, g.conn_s, g.conn_m,
-                                           g.lambda, g.gs, g.gm, g.ab, g.J, g.fo, ctr);
+                                           g.lambda, g.sl, g.gm, g.fo, ctr);
     } else if (nr != 0) {
       const int64_t p = o[32 * FxRecord::kPair];
       const int32_t s = g.ps[p], m = g.pm[p];
@@ -1109,8 +1128,12 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_finish(AdjArgs g) 
         Bu[id] += word(AdjRecord::kVertex + 2 * k);
         Bv[id] += word(AdjRecord::kVertex + 2 * k + 1);
       }
-      adjoint_finish<NS, NM, SEG, DUAL>(p, s, m, g.srec + (int64_t)SR_STRIDE * s, g.xs, g.xm, g.conn_s, g.conn_m,
-                                        g.lambda, cp, Bu, Bv, mrev, smb, mmb, G, H, true, g.gs, g.gm, g.ab, g.J, g.fo);
+      adjoint_blocks<NS, NM, SEG, DUAL>(p, g.srec + (int64_t)SR_STRIDE * s, G, H, g.fo);
+      V3 Lam[4];
+      load_v3<NS>(g.mult + 24 * (int64_t)s, Lam);
+      adjoint_finish<NS, NM, SEG>(p, g.conn_s + (int64_t)NS * s, g.conn_m + (int64_t)NM * m,
+                                  g.srec + (int64_t)SR_STRIDE * s, g.xs, g.xm, Lam, cp, Bu, Bv, mrev, smb, mmb, G, H,
+                                  g.sl, g.gm);
     }
     __syncwarp();
   }
@@ -1195,7 +1218,8 @@ template <int NS, bool DUAL, bool ELEMD>
 __global__ void __launch_bounds__(kThreads) k_adjoint_elems(
     const double* __restrict__ xs, const int32_t* __restrict__ conn_s, const double* __restrict__ lambda,
     const double* __restrict__ srec, const double* __restrict__ De, const int64_t* __restrict__ pair_off,
-    const double* __restrict__ ab_pair, int64_t Es, double* __restrict__ ge, const DevStatus* st) {
+    const uint8_t* __restrict__ flag, const double* __restrict__ sl, int64_t Es, double* __restrict__ ge,
+    const DevStatus* st) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= Es) return;
   double* out = ge + 16 * e;
@@ -1213,15 +1237,42 @@ __global__ void __launch_bounds__(kThreads) k_adjoint_elems(
     Dhb[a] = 0.0;
     for (int b = 0; b < 4; ++b) { A[a][b] = r[SR_A + 4 * a + b]; Ab[a][b] = 0.0; Meb[a][b] = 0.0; }
   }
-  if (DUAL) {
-    const int64_t p0 = pair_off[e], p1 = pair_off[e + 1];
-    for (int64_t p = p0; p < p1; ++p)
-      for (int a = 0; a < NS; ++a)
-        for (int b = 0; b < NS; ++b) Ab[a][b] += ab_pair[16 * p + 4 * a + b];
+  // what the element's pairs contribute (store_slave_pair)
+  constexpr int W = kSlavePair<!ELEMD>;
+  double sum[W];
+  for (int k = 0; k < W; ++k) sum[k] = 0.0;
+  for (int64_t p = pair_off[e]; p < pair_off[e + 1]; ++p) {
+    if (!flag[p]) continue;
+    const double2* o = reinterpret_cast<const double2*>(sl + W * p);
+#pragma unroll
+    for (int k = 0; k < W / 2; ++k) {
+      const double2 v = __ldcs(o + k);
+      sum[2 * k] += v.x;
+      sum[2 * k + 1] += v.y;
+    }
   }
   V3 Xb[4];
   for (int a = 0; a < 4; ++a) Xb[a] = v3(0, 0, 0);
   double Je = 0.0;
+  {   // pairs' part of J, dJ/dA (dual LMs), and the slave's side of projection and plane
+    V3 Lb[4], Lam[4];
+    load_v3<4>(sum, Lb);
+    lm_weights<NS, DUAL>(r, lam, Lam);
+    for (int c = 0; c < NS; ++c) {
+      Je += dot(Lam[c], Lb[c]);
+      if (DUAL)
+        for (int a = 0; a < NS; ++a) Ab[a][c] = dot(lam[a], Lb[c]);
+    }
+    double g[4][3];
+    for (int a = 0; a < 4; ++a)
+      for (int k = 0; k < 3; ++k) g[a][k] = ELEMD ? 0.0 : sum[(ELEMD ? 0 : 30) + 3 * a + k];
+    const V3 x0 = v3(r[SR_X0], r[SR_X0 + 1], r[SR_X0 + 2]), t1 = v3(r[SR_T1], r[SR_T1 + 1], r[SR_T1 + 2]),
+             t2 = v3(r[SR_T2], r[SR_T2 + 1], r[SR_T2 + 2]);
+    PlaneBar pb{v3(sum[20], sum[21], sum[22]), v3(sum[23], sum[24], sum[25]), v3(sum[26], sum[27], sum[28])};
+    project_reverse<NS>(X, x0, t1, t2, sum + 12, sum + 16, g, pb);
+    plane_basis_reverse<NS>(X, t1, t2, v3(r[SR_N0], r[SR_N0 + 1], r[SR_N0 + 2]), pb, g);
+    load_v3<NS>(&g[0][0], Xb);
+  }
   constexpr int nq = NS == 4 ? 9 : 7;
   // element integrals Me, Dh (recomputed).  A flat element (negligible
   // bilinear term: parallelograms, every tri3) has constant tangents g1, g2
@@ -1466,9 +1517,8 @@ __global__ void k_mp_sort(const int64_t* __restrict__ off, int64_t Em, int32_t* 
 }
 
 __global__ void k_grad_slave(const int64_t* __restrict__ n2e_ptr, const int64_t* __restrict__ n2e_ent,
-                             const int64_t* __restrict__ pair_off, const uint8_t* __restrict__ flag,
-                             const double* __restrict__ gs_pair, const double* __restrict__ ge, int64_t Ns,
-                             double* __restrict__ grad, const DevStatus* st) {
+                             const double* __restrict__ ge, int64_t Ns, double* __restrict__ grad,
+                             const DevStatus* st) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= Ns) return;
   double g0 = 0.0, g1 = 0.0, g2 = 0.0;
@@ -1477,10 +1527,6 @@ __global__ void k_grad_slave(const int64_t* __restrict__ n2e_ptr, const int64_t*
       const int64_t e = n2e_ent[q] >> 2;
       const int a = (int)(n2e_ent[q] & 3);
       g0 += ge[16 * e + 3 * a]; g1 += ge[16 * e + 3 * a + 1]; g2 += ge[16 * e + 3 * a + 2];
-      for (int64_t p = pair_off[e]; p < pair_off[e + 1]; ++p) {
-        if (!flag[p]) continue;
-        g0 += gs_pair[12 * p + 3 * a]; g1 += gs_pair[12 * p + 3 * a + 1]; g2 += gs_pair[12 * p + 3 * a + 2];
-      }
     }
   grad[3 * j] = g0;
   grad[3 * j + 1] = g1;
@@ -1510,16 +1556,12 @@ __global__ void k_grad_master(const int64_t* __restrict__ n2e_ptr, const int64_t
 
 constexpr int kJBlocks = 256;
 
-// Fixed-shape reduction of J over pairs and elements (deterministic).
-__global__ void __launch_bounds__(256) k_J_partial(const double* __restrict__ J_pair, int64_t pair_cap,
-                                                   const double* __restrict__ ge, int64_t Es,
-                                                   double* __restrict__ part, const DevStatus* st) {
-  const int64_t np = st->over_pairs ? 0 : (int64_t)min((unsigned long long)pair_cap, st->n_pairs);
-  const int64_t total = np + Es;
-  const int64_t per = (total + gridDim.x - 1) / gridDim.x;
-  const int64_t b0 = per * blockIdx.x, b1 = min(total, b0 + per);
+// Fixed-shape reduction of J over the elements (deterministic).
+__global__ void __launch_bounds__(256) k_J_partial(const double* __restrict__ ge, int64_t Es, double* __restrict__ part) {
+  const int64_t per = (Es + gridDim.x - 1) / gridDim.x;
+  const int64_t b0 = per * blockIdx.x, b1 = min(Es, b0 + per);
   double s = 0.0;
-  for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) s += i < np ? J_pair[i] : ge[16 * (i - np) + 12];
+  for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) s += ge[16 * i + 12];
   __shared__ double sh[256];
   sh[threadIdx.x] = s;
   __syncthreads();
@@ -1553,8 +1595,7 @@ void launch_pairs_t(mortar_ctx* c, const RunParams& rp, unsigned grid, unsigned 
   k_adjoint_pairs<NS, NM, SEG, DUAL><<<grid, block, 0, c->stream>>>(
       c->pairs_s.as<int32_t>(), c->pairs_m.as<int32_t>(), c->srec.as<double>(), c->xs.as<double>(),
       c->xm.as<double>(), c->conn_s.as<int32_t>(), c->conn_m.as<int32_t>(), c->lambda.as<double>(), rp, c->pair_cap,
-      chunk, c->gs_pair.as<double>(), c->gm_pair.as<double>(), c->abar_pair.as<double>(), c->J_pair.as<double>(),
-      c->dstat.as<DevStatus>());
+      chunk, c->sl_pair.as<double>(), c->gm_pair.as<double>(), c->dstat.as<DevStatus>());
 }
 
 // The default adjoint always produces the forward blocks as well (the run
@@ -1566,8 +1607,8 @@ void launch_fixed(mortar_ctx* c, const RunParams& rp, int block, int rounds) {
                    c->stream};
   ia.order = c->order.as<int32_t>();
   AdjArgs a{ia.ps, ia.pm, ia.srec, c->xs.as<double>(), ia.xm, c->conn_s.as<int32_t>(), ia.conn_m,
-            c->lambda.as<double>(), c->pair_cap, 0, ia.order, c->rec.as<long long>(), c->gs_pair.as<double>(),
-            c->gm_pair.as<double>(), c->abar_pair.as<double>(), c->J_pair.as<double>(),
+            c->lambda.as<double>(), c->pair_cap, 0, ia.order, c->rec.as<long long>(), c->mult.as<double>(),
+            c->sl_pair.as<double>(), c->gm_pair.as<double>(),
             FwdOut{c->Mblk.as<double>(), c->Dblk.as<double>(), c->flag.as<uint8_t>()}, ia.st, c->watchdog_us};
   auto grid = [&](auto kern, int threads, size_t shm) {
     int per_sm = 0;
@@ -1575,13 +1616,16 @@ void launch_fixed(mortar_ctx* c, const RunParams& rp, int block, int rounds) {
     return (unsigned)(c->n_sm * (per_sm < 1 ? 1 : per_sm));
   };
   unsigned long long* cta_t = (c->timing && c->cta_t.p) ? c->cta_t.as<unsigned long long>() : nullptr;
-  auto clip = k_adjoint_clip<NS, NM, SEG, DUAL>;
+  auto clip = k_adjoint_clip<NS, NM, SEG>;
   auto cells = k_adjoint_cells<NS, NM, SEG>;
   auto fin = k_adjoint_finish<NS, NM, SEG, DUAL>;
   const size_t shm = (size_t)kCellThreads * kAdjSlots * 8;
   cudaFuncSetAttribute(cells, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
   const unsigned gc = grid(clip, block, 0), gq = grid(cells, kCellThreads, shm), gf = grid(fin, block, 0);
   if (cta_t) c->pair_grid = (int)gc;
+  if (c->Es > 0)
+    k_multipliers<NS, DUAL><<<(unsigned)((c->Es + kThreads - 1) / kThreads), kThreads, 0, c->stream>>>(
+        a.conn_s, a.lambda, a.srec, c->Es, c->mult.as<double>());
   for (; a.first < c->pair_cap; a.first += kPairChunk) {
     launch_pair_sort<NS, NM>(ia, rp, c->n_sm, 32 * rounds, a.first);
     clip<<<gc, block, 0, c->stream>>>(a, cta_t);
@@ -1622,7 +1666,7 @@ void launch_elems_ns(mortar_ctx* c, const RunParams& rp) {
   auto args = [&](auto kern) {
     kern<<<g, kThreads, 0, c->stream>>>(c->xs.as<double>(), c->conn_s.as<int32_t>(), c->lambda.as<double>(),
                                         c->srec.as<double>(), c->De.as<double>(), c->pair_off.as<int64_t>(),
-                                        c->abar_pair.as<double>(), c->Es, c->ge_elem.as<double>(),
+                                        c->flag.as<uint8_t>(), c->sl_pair.as<double>(), c->Es, c->ge_elem.as<double>(),
                                         c->dstat.as<DevStatus>());
   };
   if (dual && elemd) args(k_adjoint_elems<NS, true, true>);
@@ -1645,13 +1689,13 @@ int prepare_adjoint_buffers(mortar_ctx* c) {
     }
     if ((r = buf_reserve(c->rec, need)) != MORTAR_OK) return r;
   }
-  if ((r = buf_reserve(c->gs_pair, P * 12 * 8)) != MORTAR_OK) return r;
+  const size_t sl = c->opt.d_domain == MORTAR_D_SEGMENT ? kSlavePair<true> : kSlavePair<false>;
+  if ((r = buf_reserve(c->sl_pair, P * sl * 8)) != MORTAR_OK) return r;
   if ((r = buf_reserve(c->gm_pair, P * 12 * 8)) != MORTAR_OK) return r;
-  if ((r = buf_reserve(c->J_pair, P * 8)) != MORTAR_OK) return r;
-  if (c->opt.lm == MORTAR_LM_DUAL && (r = buf_reserve(c->abar_pair, P * 16 * 8)) != MORTAR_OK) return r;
   if ((r = buf_reserve(c->mp_list, P * 4)) != MORTAR_OK) return r;
   const size_t Es = (size_t)std::max<int64_t>(c->Es, 1), Em = (size_t)std::max<int64_t>(c->Em, 1);
   if ((r = buf_reserve(c->ge_elem, Es * 16 * 8)) != MORTAR_OK) return r;
+  if ((r = buf_reserve(c->mult, Es * 24 * 8)) != MORTAR_OK) return r;
   if ((r = buf_reserve(c->mp_cnt, Em * 4)) != MORTAR_OK) return r;
   if ((r = buf_reserve(c->mp_off, (Em + 1) * 8)) != MORTAR_OK) return r;
   if ((r = buf_reserve(c->grad_s, (size_t)std::max<int64_t>(c->Ns, 1) * 24)) != MORTAR_OK) return r;
@@ -1690,14 +1734,13 @@ void launch_adjoint_rest(mortar_ctx* c, const RunParams& rp) {
         c->mp_off.as<int64_t>(), c->Em, c->mp_list.as<int32_t>());
   if (c->Ns > 0)
     k_grad_slave<<<(unsigned)((c->Ns + kThreads - 1) / kThreads), kThreads, 0, c->stream>>>(
-        c->n2e_s_ptr.as<int64_t>(), c->n2e_s_ent.as<int64_t>(), c->pair_off.as<int64_t>(), c->flag.as<uint8_t>(),
-        c->gs_pair.as<double>(), c->ge_elem.as<double>(), c->Ns, c->grad_s.as<double>(), st);
+        c->n2e_s_ptr.as<int64_t>(), c->n2e_s_ent.as<int64_t>(), c->ge_elem.as<double>(), c->Ns, c->grad_s.as<double>(),
+        st);
   if (c->Nm > 0)
     k_grad_master<<<(unsigned)((c->Nm + kThreads - 1) / kThreads), kThreads, 0, c->stream>>>(
         c->n2e_m_ptr.as<int64_t>(), c->n2e_m_ent.as<int64_t>(), c->mp_off.as<int64_t>(), c->mp_list.as<int32_t>(),
         c->gm_pair.as<double>(), c->Nm, c->grad_m.as<double>(), st);
-  k_J_partial<<<kJBlocks, 256, 0, c->stream>>>(c->J_pair.as<double>(), c->pair_cap, c->ge_elem.as<double>(), c->Es,
-                                               c->J_part.as<double>(), st);
+  k_J_partial<<<kJBlocks, 256, 0, c->stream>>>(c->ge_elem.as<double>(), c->Es, c->J_part.as<double>());
   k_J_final<<<1, 256, 0, c->stream>>>(c->J_part.as<double>(), st);
 }
 #endif  // MORTAR_PAIR_NS

@@ -429,43 +429,6 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_clip(
   cta_mark(cta_t, 1);
 }
 
-// Writes the 4x4 block M = A G (standard LMs: G) of every pair of the warp from
-// its cells' sums g (fx_sum_cells).
-template <int NS, int NC>
-__device__ __forceinline__ void write_block(const FxAcc g[4][4], const CellSlot& cs, bool ok, int ke,
-                                            const FxScales& ss, const FxScales& sc, bool dual,
-                                            const double* __restrict__ r, double* __restrict__ out,
-                                            long long* __restrict__ buf, int stride) {
-  double G[16];   // dual: this lane's entries, until every lane has read the sums
-  int n = 0;
-  fx_sum_cells<NS, NC>(g, cs, ok, buf, stride, [&](int a, int l, long long hh, long long cr) {
-    const double v = fx_to_double(hh, cr, ke - ss.shape<NS>(a) - sc.shape<NC>(l));
-    if (dual) G[n++] = v;
-    else __stcs(out + 4 * a + l, v);
-  });
-  if (ok && NS * NC < 16)   // the block is padded with zeros
-    for (int e = cs.cell; e < 16; e += cs.cells)
-      if ((e >> 2) >= NS || (e & 3) >= NC) __stcs(out + e, 0.0);
-  if (dual) {
-    __syncwarp();
-    double* Gs = reinterpret_cast<double*>(buf - (threadIdx.x & 31) + cs.first);
-    if (ok) {
-      n = 0;
-      for (int e = cs.cell; e < NS * NC; e += cs.cells) Gs[e * stride] = G[n++];
-    }
-    __syncwarp();
-    if (ok)
-#pragma unroll 1
-      for (int e = cs.cell; e < NS * NC; e += cs.cells) {
-        const int a = e / NC, l = e - NC * a;
-        double v = 0.0;
-#pragma unroll
-        for (int c = 0; c < NS; ++c) v = fma(r[SR_A + 4 * a + c], Gs[(NC * c + l) * stride], v);
-        __stcs(out + 4 * a + l, v);
-      }
-  }
-}
-
 // Quadrature of the clip kernel's records, one cell of a pair per lane (all
 // cells cost the same, so lanes idle only at the ends of warps): the cell's
 // back-projections, then its products, then the pair's sums through shared
@@ -527,10 +490,12 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_quadrature(
       FxAcc g[4][4];
       if (SEG) {   // the sums' memory is apart from the points', which M's products read again
         fx_cell_products<NS, NS, true>(ss, ss, weight, pts, stride, g);
-        write_block<NS, NS>(g, cs, ok, ke, ss, ss, rp.lm == 1, r, Dblk + 16 * p, pts + 28 * stride, stride);
+        write_block<NS, NS>(g, cs, ok, ke, ss, ss, rp.lm == 1, r, Dblk + 16 * p, pts + 28 * stride, stride,
+                            [](int, int, double) {});
       }
       fx_cell_products<NS, NM, false>(ss, sm, weight, pts, stride, g);
-      write_block<NS, NM>(g, cs, ok, ke, ss, sm, rp.lm == 1, r, Mblk + 16 * p, SEG ? pts + 28 * stride : pts, stride);
+      write_block<NS, NM>(g, cs, ok, ke, ss, sm, rp.lm == 1, r, Mblk + 16 * p, SEG ? pts + 28 * stride : pts, stride,
+                          [](int, int, double) {});
       if (cs.cell == 0) {
         if (ok) flag[p] = 1;
         else integrate_pair_fp64<NS, NM, SEG>(p, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, slow);

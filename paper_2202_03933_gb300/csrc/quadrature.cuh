@@ -396,4 +396,42 @@ __device__ __forceinline__ void fx_sum_cells(const FxAcc g[4][4], const CellSlot
     }
 }
 
+// Writes the 4x4 block M = A G (standard LMs: G) of every pair of the warp from
+// its cells' sums g (fx_sum_cells), and passes the entries (a, l) of G to keep.
+template <int NS, int NC, class Keep>
+__device__ __forceinline__ void write_block(const FxAcc g[4][4], const CellSlot& cs, bool ok, int ke,
+                                            const FxScales& ss, const FxScales& sc, bool dual,
+                                            const double* __restrict__ r, double* __restrict__ out,
+                                            long long* __restrict__ buf, int stride, Keep keep) {
+  double G[16];   // dual: this lane's entries, until every lane has read the sums
+  int n = 0;
+  fx_sum_cells<NS, NC>(g, cs, ok, buf, stride, [&](int a, int l, long long hh, long long cr) {
+    const double v = fx_to_double(hh, cr, ke - ss.shape<NS>(a) - sc.shape<NC>(l));
+    keep(a, l, v);
+    if (dual) G[n++] = v;
+    else __stcs(out + 4 * a + l, v);
+  });
+  if (ok && NS * NC < 16)   // the block is padded with zeros
+    for (int e = cs.cell; e < 16; e += cs.cells)
+      if ((e >> 2) >= NS || (e & 3) >= NC) __stcs(out + e, 0.0);
+  if (dual) {
+    __syncwarp();
+    double* Gs = reinterpret_cast<double*>(buf - (threadIdx.x & 31) + cs.first);
+    if (ok) {
+      n = 0;
+      for (int e = cs.cell; e < NS * NC; e += cs.cells) Gs[e * stride] = G[n++];
+    }
+    __syncwarp();
+    if (ok)
+#pragma unroll 1
+      for (int e = cs.cell; e < NS * NC; e += cs.cells) {
+        const int a = e / NC, l = e - NC * a;
+        double v = 0.0;
+#pragma unroll
+        for (int c = 0; c < NS; ++c) v = fma(r[SR_A + 4 * a + c], Gs[(NC * c + l) * stride], v);
+        __stcs(out + 4 * a + l, v);
+      }
+  }
+}
+
 }  // namespace mortar

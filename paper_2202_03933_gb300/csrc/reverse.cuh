@@ -61,10 +61,14 @@ __device__ __forceinline__ void elem_point_a(int k, double& xi, double& eta, dou
 template <int NEN>
 __device__ __forceinline__ void map_coeff_reverse(const double* cb, double* pbu, double* pbv) {
   if constexpr (NEN == 4) {
-    const double s1[4] = {-1.0, 1.0, 1.0, -1.0}, s2[4] = {-1.0, -1.0, 1.0, 1.0};
-    for (int a = 0; a < 4; ++a) {
-      pbu[a] += 0.25 * (cb[0] + s1[a] * cb[2] + s2[a] * cb[4] + s1[a] * s2[a] * cb[6]);
-      pbv[a] += 0.25 * (cb[1] + s1[a] * cb[3] + s2[a] * cb[5] + s1[a] * s2[a] * cb[7]);
+    for (int c = 0; c < 2; ++c) {   // corners (-1,-1), (1,-1), (1,1), (-1,1): sums and differences shared
+      double* pb = c == 0 ? pbu : pbv;
+      const double s0 = 0.25 * cb[c], s1 = 0.25 * cb[2 + c], s2 = 0.25 * cb[4 + c], s3 = 0.25 * cb[6 + c];
+      const double a = s0 - s2, b = s1 - s3, d = s0 + s2, e = s1 + s3;
+      pb[0] += a - b;
+      pb[1] += a + b;
+      pb[2] += d + e;
+      pb[3] += d - e;
     }
   } else {
     pbu[0] += cb[0] - cb[2] - cb[4];
@@ -414,32 +418,35 @@ struct ClipPool {
   }
 };
 
-// Reverse of the projection u = (P - x0).t1, v = (P - x0).t2 of every node of
-// the pair and of the auxiliary plane (x0 = element centre, n0 = unit normal
-// there, t1 = normalised projected first edge, t2 = n0 x t1) as functions of
-// the slave nodes X.  In-plane node adjoints (sbu, sbv, mbu, mbv) in; 3D
-// coordinate adjoints ADDED to gX (slave) and gY (master).
-template <int NS, int NM>
-__device__ __forceinline__ void plane_reverse(const V3* X, const V3* Y, V3 x0, V3 t1, V3 t2, V3 n0,
-                                              const double* sbu, const double* sbv, const double* mbu,
-                                              const double* mbv, double gX[4][3], double gY[4][3]) {
-  V3 x0b = v3(0, 0, 0), t1b = v3(0, 0, 0), t2b = v3(0, 0, 0);
-  for (int a = 0; a < NS; ++a) {
-    const V3 dd = X[a] - x0;
-    const V3 db = sbu[a] * t1 + sbv[a] * t2;
-    gX[a][0] += db.x; gX[a][1] += db.y; gX[a][2] += db.z;
-    x0b = x0b - db;
-    t1b = t1b + sbu[a] * dd;
-    t2b = t2b + sbv[a] * dd;
+// Adjoints of the auxiliary plane: point x0 and in-plane basis t1, t2.
+struct PlaneBar {
+  V3 x0, t1, t2;
+};
+
+// Reverse of the projection u = (P - x0).t1, v = (P - x0).t2 of N nodes P:
+// in-plane adjoints (bu, bv) in; 3D coordinate adjoints ADDED to g, the plane's
+// to pb.
+template <int N>
+__device__ __forceinline__ void project_reverse(const V3* P, V3 x0, V3 t1, V3 t2, const double* bu, const double* bv,
+                                                double g[4][3], PlaneBar& pb) {
+  for (int l = 0; l < N; ++l) {
+    const V3 dd = P[l] - x0;
+    const V3 db = bu[l] * t1 + bv[l] * t2;
+    g[l][0] += db.x; g[l][1] += db.y; g[l][2] += db.z;
+    pb.x0 = pb.x0 - db;
+    pb.t1 = pb.t1 + bu[l] * dd;
+    pb.t2 = pb.t2 + bv[l] * dd;
   }
-  for (int l = 0; l < NM; ++l) {
-    const V3 dd = Y[l] - x0;
-    const V3 db = mbu[l] * t1 + mbv[l] * t2;
-    gY[l][0] += db.x; gY[l][1] += db.y; gY[l][2] += db.z;
-    x0b = x0b - db;
-    t1b = t1b + mbu[l] * dd;
-    t2b = t2b + mbv[l] * dd;
-  }
+}
+
+// Reverse of the auxiliary plane (x0 = element centre, n0 = unit normal there,
+// t1 = normalised projected first edge, t2 = n0 x t1) as a function of the slave
+// nodes X; ADDED to gX.
+template <int NS>
+__device__ __forceinline__ void plane_basis_reverse(const V3* X, V3 t1, V3 t2, V3 n0, const PlaneBar& pb,
+                                                    double gX[4][3]) {
+  const V3 x0b = pb.x0, t2b = pb.t2;
+  V3 t1b = pb.t1;
   V3 g1, g2;
   if constexpr (NS == 4) {
     g1 = 0.25 * ((X[1] - X[0]) + (X[2] - X[3]));
@@ -483,6 +490,18 @@ __device__ __forceinline__ void plane_reverse(const V3* X, const V3* Y, V3 x0, V
   for (int a = 0; a < NS; ++a) {
     gX[a][0] += Xb[a].x; gX[a][1] += Xb[a].y; gX[a][2] += Xb[a].z;
   }
+}
+
+// Both: in-plane node adjoints (sbu, sbv, mbu, mbv) in; 3D coordinate adjoints
+// ADDED to gX (slave) and gY (master).
+template <int NS, int NM>
+__device__ __forceinline__ void plane_reverse(const V3* X, const V3* Y, V3 x0, V3 t1, V3 t2, V3 n0,
+                                              const double* sbu, const double* sbv, const double* mbu,
+                                              const double* mbv, double gX[4][3], double gY[4][3]) {
+  PlaneBar pb{v3(0, 0, 0), v3(0, 0, 0), v3(0, 0, 0)};
+  project_reverse<NS>(X, x0, t1, t2, sbu, sbv, gX, pb);
+  project_reverse<NM>(Y, x0, t1, t2, mbu, mbv, gY, pb);
+  plane_basis_reverse<NS>(X, t1, t2, n0, pb, gX);
 }
 
 // Monomial form of the element shape functions, N(xi) = T m(xi): quad4
