@@ -195,10 +195,10 @@ struct AdjSums {
 // into pts[(28 + 4 q + 0..3) * stride], and area = sum w f (Q61 at 2^s0).
 // o: the record (word w at o[32 w]); pts: back-projections.  False if an
 // inverse Jacobian leaves its range.
-template <int NS, int NM, bool SEG>
+template <int NS, int NM, bool SEG, int stride>
 __device__ __forceinline__ bool fx_cell_sweep(const FxMap& sm, const FxMap& mm, const AdjScale& sc,
                                               const long long* __restrict__ o, long long weight,
-                                              long long* __restrict__ pts, int stride, long long& area) {
+                                              long long* __restrict__ pts, long long& area) {
   constexpr int KS = NS, KM = NM;
   auto dg = [&](int w) { const long long v = o[32 * w]; return Dg{(int)(v >> 32), (int)v}; };
   auto val = [](Dg d) { return ((long long)d.h << 32) + d.l; };
@@ -304,8 +304,8 @@ __device__ __forceinline__ bool fx_cell_sweep(const FxMap& sm, const FxMap& mm, 
 
 // The cell's sums over the points' W y.  A loop of its own: the sweep holds the
 // element maps, this one the accumulators.
-template <int NS, int NM>
-__device__ __forceinline__ void fx_cell_moments(const long long* __restrict__ pts, int stride, AdjSums& r) {
+template <int NS, int NM, int stride>
+__device__ __forceinline__ void fx_cell_moments(const long long* __restrict__ pts, AdjSums& r) {
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     r.s1[k] = r.m1[k] = r.es1[k] = r.es2[k] = r.em1[k] = r.em2[k] = 0;

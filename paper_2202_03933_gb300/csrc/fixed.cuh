@@ -50,6 +50,7 @@ __device__ __forceinline__ long long mul_wide(int a, int b) {
   return d;
 }
 __device__ __forceinline__ int mul_hi(int a, int b) { return __mulhi(a, b); }
+__device__ __forceinline__ unsigned shift_in(unsigned lo, unsigned hi, int k) { return __funnelshift_l(lo, hi, k); }
 __device__ __forceinline__ float rcp_f32(float x) {   // about 1 ulp; seeds only
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -59,6 +60,9 @@ __device__ __forceinline__ float rcp_f32(float x) {   // about 1 ulp; seeds only
 inline long long mad_wide(int a, int b, long long c) { return (long long)a * b + c; }
 inline long long mul_wide(int a, int b) { return (long long)a * b; }
 inline int mul_hi(int a, int b) { return (int)(((long long)a * b) >> 32); }
+inline unsigned shift_in(unsigned lo, unsigned hi, int k) {
+  return (unsigned)((((unsigned long long)hi << 32 | lo) << k) >> 32);
+}
 inline float rcp_f32(float x) { return 1.0f / x; }
 #endif
 
@@ -74,14 +78,15 @@ struct FxAcc {
     hh = mad_wide(a.h, b.h, hh);
     cr = mad_wide(a.l, b.h, mad_wide(a.h, b.l, cr));
   }
-  // the sum times 2^K, 0 <= K < 32
-  template <int K>
-  __device__ __forceinline__ long long get() const {
-    return (long long)((unsigned long long)hh << K) + (cr >> (32 - K));
-  }
+  // the sum times 2^k, 0 <= k < 32: the cross sum's whole units are added by a
+  // multiply-add (one instruction), then both words shifted
   __device__ __forceinline__ long long get(int k) const {
-    return (long long)((unsigned long long)hh << k) + (cr >> (32 - k));
+    const long long t = mad_wide((int)(cr >> 32), 1, hh);
+    return (long long)((unsigned long long)shift_in((unsigned)t, (unsigned)((unsigned long long)t >> 32), k) << 32 |
+                       shift_in((unsigned)cr, (unsigned)t, k));
   }
+  template <int K>
+  __device__ __forceinline__ long long get() const { return get(K); }
   // the low digits' product of the last mul or mac, where 2^-2 unit matters
   __device__ __forceinline__ void low(Dg a, Dg b) { cr += mul_hi(a.l, b.l); }
   // moves the whole units of the cross sum into hh (keeps the fraction): bounds cr between runs of products

@@ -917,7 +917,7 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, un
   cta_mark(cta_t, 1);
 }
 
-constexpr int kAdjSlots = 58;      // shared 64-bit words per thread of the cell kernel: points, W y or sums
+constexpr int kAdjSlots = 56;      // shared 64-bit words per thread of the cell kernel: points, W y or sums
 constexpr int kCellThreads = 384;  // the registers of an SM at 168 a thread
 
 // Second kernel: one cell of a pair per lane, as k_pair_quadrature.  Leaves G
@@ -928,7 +928,7 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
   constexpr int W = SEG ? AdjRecord::kWordsSeg : AdjRecord::kWords;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   long long* pts = reinterpret_cast<long long*>(smem_raw) + threadIdx.x;
-  const int stride = (int)blockDim.x;
+  constexpr int stride = kCellThreads;
   long long* sums = pts + 28 * stride;
   const int lane = threadIdx.x & 31;
   DevStatus* st = ar.st;
@@ -966,23 +966,22 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
     w += cs.taken;
     long long* o = ar.rec + (i >> 5) * (32 * W) + (i & 31);
     bool ok = cs.cell >= 0;
+    // what later parts need they load again: registers are what bounds the warps
+    long long weight = 0, area = 0;
     FxView f;
-    AdjScale sc;
-    long long weight = 0, e1u = 0, e1v = 0, e2u = 0, e2v = 0;
     if (ok) {
       const int64_t p = o[32 * FxRecord::kPair];
       const double* sr = ar.srec + (int64_t)SR_STRIDE * ar.ps[p];
       f.load<NS, NM>(o);
-      sc.load(o[32 * AdjRecord::kScales], o[32 * AdjRecord::kScales2], f.ke, f.E);
       weight = f.weight(cs.cell);
-      const int ib = f.ib(cs.cell), iw = f.iw(cs.cell);
-      e1u = f.x(ib) - f.cu; e1v = f.y(ib) - f.cv;
-      e2u = f.x(iw) - f.cu; e2v = f.y(iw) - f.cv;
-      ok = fx_back_project<NS, NM>(f, cs.cell, sr, ar.xm, ar.conn_m, ar.pm[p], pts, stride);
+      ok = fx_back_project<NS, NM, stride>(f, cs.cell, sr, ar.xm, ar.conn_m, ar.pm[p], pts);
     }
     __syncthreads();
-    long long area = 0;
-    if (ok) ok = fx_cell_sweep<NS, NM, SEG>(f.s, f.m, sc, o, weight, pts, stride, area);
+    if (ok) {
+      AdjScale sc;
+      sc.load(o[32 * AdjRecord::kScales], o[32 * AdjRecord::kScales2], f.ke, f.E);
+      ok = fx_cell_sweep<NS, NM, SEG, stride>(f.s, f.m, sc, o, weight, pts, area);
+    }
     const unsigned bad = __ballot_sync(0xffffffffu, cs.cell >= 0 && !ok);
     const bool slow = cs.cell >= 0 && (bad >> cs.first & (cs.cells < 32 ? (1u << cs.cells) - 1u : ~0u)) != 0;
     ok &= !slow;
@@ -990,28 +989,32 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
     __syncthreads();
     {
       AdjSums r;
-      fx_cell_moments<NS, NM>(pts, stride, r);
+      fx_cell_moments<NS, NM, stride>(pts, r);
+      const long long info = o[32 * FxRecord::kInfo];
+      const int nr = (int)(info & 0xff);
+      AdjScale sc;
+      sc.load(o[32 * AdjRecord::kScales], o[32 * AdjRecord::kScales2], (int)(short)(info >> 32), (int)(short)(info >> 48));
       // map-coefficient adjoints: minus the sums of W y (x) (1, xi, eta, xi eta), units of 2^64 of Q61 x Q61
       __syncwarp();
       if (ok) {
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
+        for (int e = 0; e < 16; ++e) {   // the plain sums are whole; the others have a fraction, words 16..21
           const int c = e & 1, k = (e & 7) >> 1;
-          long long hh, cr;
           if (k == 0) {
-            const long long v = e < 8 ? r.s1[c] : r.m1[c];
-            hh = v >> 3;
-            cr = (v & 7) << 29;
+            sums[e * stride] = e < 8 ? r.s1[c] : r.m1[c];
           } else {
             const FxAcc& a = e < 8 ? r.sx[k - 1][c] : r.mx[k - 1][c];
-            hh = a.hh + (a.cr >> 32);
-            cr = (long long)(unsigned)a.cr;
+            const int i = e - (e < 8 ? 2 : 4);
+            sums[e * stride] = a.hh + (a.cr >> 32);
+            reinterpret_cast<unsigned*>(sums + (16 + (i >> 1)) * stride)[i & 1] = (unsigned)a.cr;
           }
-          sums[e * stride] = hh;
-          reinterpret_cast<unsigned*>(sums + (16 + (e >> 1)) * stride)[e & 1] = (unsigned)cr;
         }
         // vertex adjoints of the cell: moments of both sides and the area's part,
         // d area = +-(1/2)(e2v de1u - e2u de1v + e1u de2v - e1v de2u)
+        const int ib = nr > 3 ? cs.cell : 1, iw = nr > 3 ? (cs.cell + 1 == nr ? 0 : cs.cell + 1) : 2;
+        const long long cu = o[32 * 24], cv = o[32 * 25];
+        const long long e1u = o[64 * ib] - cu, e1v = o[64 * ib + 32] - cv;
+        const long long e2u = o[64 * iw] - cu, e2v = o[64 * iw + 32] - cv;
         FxAcc a;
         a.mul(fx_split(e1u), fx_split(e2v));
         FxAcc b;
@@ -1027,39 +1030,41 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
         const long long v1v = part(r.es1[1], r.em1[1], -e2u, sc.eu, sc.xau, sc.xvv);
         const long long v2u = part(r.es2[0], r.em2[0], -e1v, sc.ev, sc.xav, sc.xvu);
         const long long v2v = part(r.es2[1], r.em2[1], e1u, sc.eu, sc.xau, sc.xvv);
-        sums[24 * stride] = v1u; sums[25 * stride] = v1v;
-        sums[26 * stride] = v2u; sums[27 * stride] = v2v;
-        sums[28 * stride] = fx_down(r.s1[0], sc.xvu - sc.xs) + fx_down(r.m1[0], sc.xvu - sc.xm) - v1u - v2u;
-        sums[29 * stride] = fx_down(r.s1[1], sc.xvv - sc.xs) + fx_down(r.m1[1], sc.xvv - sc.xm) - v1v - v2v;
+        sums[22 * stride] = v1u; sums[23 * stride] = v1v;
+        sums[24 * stride] = v2u; sums[25 * stride] = v2v;
+        sums[26 * stride] = fx_down(r.s1[0], sc.xvu - sc.xs) + fx_down(r.m1[0], sc.xvu - sc.xm) - v1u - v2u;
+        sums[27 * stride] = fx_down(r.s1[1], sc.xvv - sc.xs) + fx_down(r.m1[1], sc.xvv - sc.xm) - v1v - v2v;
       }
       __syncwarp();
       if (ok) {
         const long long* pair = sums - lane + cs.first;
 #pragma unroll 1
         for (int e = cs.cell; e < 16; e += cs.cells) {
+          const bool plain = (e & 6) == 0;
+          const int i = e - (e < 8 ? 2 : 4);
           long long hh = 0, cr = 0;
           for (int k = 0; k < cs.cells; ++k) {
             hh += pair[e * stride + k];
-            cr += reinterpret_cast<const unsigned*>(pair + (16 + (e >> 1)) * stride + k)[e & 1];
+            if (!plain) cr += reinterpret_cast<const unsigned*>(pair + (16 + (i >> 1)) * stride + k)[i & 1];
           }
-          const double v = -fx_to_double(hh, cr, 3 + (e < 8 ? sc.xs : sc.xm));
+          const double v = -fx_to_double(hh, cr, (plain ? 0 : 3) + (e < 8 ? sc.xs : sc.xm));
           o[32 * (AdjRecord::kMapS + e)] = __double_as_longlong(v);
         }
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
           long long* ov = o + 32 * (AdjRecord::kVertex + c);
           const int xv = c == 0 ? sc.xvu : sc.xvv;
-          if (f.nr == 3) {   // one cell: its corner, then the two vertices
-            ov[0] = __double_as_longlong(fx_to_double(pair[(28 + c) * stride], 0, xv));
-            ov[64] = __double_as_longlong(fx_to_double(pair[(24 + c) * stride], 0, xv));
-            ov[128] = __double_as_longlong(fx_to_double(pair[(26 + c) * stride], 0, xv));
+          if (nr == 3) {   // one cell: its corner, then the two vertices
+            ov[0] = __double_as_longlong(fx_to_double(pair[(26 + c) * stride], 0, xv));
+            ov[64] = __double_as_longlong(fx_to_double(pair[(22 + c) * stride], 0, xv));
+            ov[128] = __double_as_longlong(fx_to_double(pair[(24 + c) * stride], 0, xv));
           } else {   // vertex k: cell k's first, cell k - 1's second, 1 / nr of the centre's
             long long centre = 0;
-            for (int k = 0; k < cs.cells; ++k) centre += pair[(28 + c) * stride + k];
+            for (int k = 0; k < cs.cells; ++k) centre += pair[(26 + c) * stride + k];
             FxAcc a;
-            a.mul(fx_split(centre), kInvCountFx.d[f.nr]);
+            a.mul(fx_split(centre), kInvCountFx.d[nr]);
             const int prev = cs.cell == 0 ? cs.cells - 1 : cs.cell - 1;
-            const long long v = a.get<2>() + pair[(24 + c) * stride + cs.cell] + pair[(26 + c) * stride + prev];
+            const long long v = a.get<2>() + pair[(22 + c) * stride + cs.cell] + pair[(24 + c) * stride + prev];
             ov[64 * cs.cell] = __double_as_longlong(fx_to_double(v, 0, xv));
           }
         }
@@ -1067,18 +1072,21 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
     }
     __syncthreads();
     {
+      FxScales ss, sm;
+      FxRecord::load_scales(o, ss, sm);
+      const int ke = (int)(short)(o[32 * FxRecord::kInfo] >> 32);
       FxAcc g[4][4];
       if (SEG) {
-        fx_cell_products<NS, NS, true>(f.ss, f.ss, weight, pts, stride, g);
-        fx_sum_cells<NS, NS>(g, cs, ok, sums, stride, [&](int a, int b, long long hh, long long cr) {
+        fx_cell_products<NS, NS, true, stride>(ss, ss, weight, pts, g);
+        fx_sum_cells<NS, NS, stride>(g, cs, ok, sums, [&](int a, int b, long long hh, long long cr) {
           o[32 * (AdjRecord::kH + 4 * a + b)] =
-              __double_as_longlong(fx_to_double(hh, cr, f.ke - f.ss.shape<NS>(a) - f.ss.shape<NS>(b)));
+              __double_as_longlong(fx_to_double(hh, cr, ke - ss.shape<NS>(a) - ss.shape<NS>(b)));
         });
       }
-      fx_cell_products<NS, NM, false>(f.ss, f.sm, weight, pts, stride, g);
-      fx_sum_cells<NS, NM>(g, cs, ok, sums, stride, [&](int a, int l, long long hh, long long cr) {
+      fx_cell_products<NS, NM, false, stride>(ss, sm, weight, pts, g);
+      fx_sum_cells<NS, NM, stride>(g, cs, ok, sums, [&](int a, int l, long long hh, long long cr) {
         o[32 * (AdjRecord::kG + 4 * a + l)] =
-            __double_as_longlong(fx_to_double(hh, cr, f.ke - f.ss.shape<NS>(a) - f.sm.shape<NM>(l)));
+            __double_as_longlong(fx_to_double(hh, cr, ke - ss.shape<NS>(a) - sm.shape<NM>(l)));
       });
     }
     if (slow && cs.cell == 0) o[32 * FxRecord::kInfo] = kSlowPair;

@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(kMaxPairBlock) k_integrate(const int32_t* __re
 }
 
 // ---------------------------------------------------------------- variant 0
+constexpr int kQuadThreads = 128;   // of the quadrature kernel's blocks
 // shared memory per thread: a cell's seven back-projections [and, SEG, its sums apart from them]
 template <bool SEG>
 constexpr int kPtsBytes = (SEG ? 52 : 28) * 8;
@@ -434,14 +435,13 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_clip(
 // back-projections, then its products, then the pair's sums through shared
 // memory.
 template <int NS, int NM, bool SEG>
-__global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_quadrature(
+__global__ void __launch_bounds__(kQuadThreads, 4) k_pair_quadrature(
     const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
     const double* __restrict__ xm, const int32_t* __restrict__ conn_m, RunParams rp, double* __restrict__ Mblk,
     double* __restrict__ Dblk, uint8_t* __restrict__ flag, int64_t pair_cap, int64_t first,
     const long long* __restrict__ rec, DevStatus* st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   long long* pts = reinterpret_cast<long long*>(smem_raw) + threadIdx.x;
-  const int stride = (int)blockDim.x;
   const int lane = threadIdx.x & 31;
   const int64_t n = chunk_pairs(st, pair_cap, first, kPairChunk);
   const int turn = cell_turn(n);
@@ -482,20 +482,19 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_quadrature(
         ss = f.ss;
         sm = f.sm;
         ke = f.ke;
-        ok = fx_back_project<NS, NM>(f, cs.cell, r, xm, conn_m, m, pts, stride);
+        ok = fx_back_project<NS, NM, kQuadThreads>(f, cs.cell, r, xm, conn_m, m, pts);
       }
       const unsigned bad = __ballot_sync(0xffffffffu, cs.cell >= 0 && !ok);
       const bool slow_pair = cs.cell >= 0 && (bad >> cs.first & ((1u << cs.cells) - 1u)) != 0;
       ok &= !slow_pair;
       FxAcc g[4][4];
       if (SEG) {   // the sums' memory is apart from the points', which M's products read again
-        fx_cell_products<NS, NS, true>(ss, ss, weight, pts, stride, g);
-        write_block<NS, NS>(g, cs, ok, ke, ss, ss, rp.lm == 1, r, Dblk + 16 * p, pts + 28 * stride, stride,
-                            [](int, int, double) {});
+        fx_cell_products<NS, NS, true, kQuadThreads>(ss, ss, weight, pts, g);
+        write_block<NS, NS, kQuadThreads>(g, cs, ok, ke, ss, ss, rp.lm == 1, r, Dblk + 16 * p, pts + 28 * kQuadThreads);
       }
-      fx_cell_products<NS, NM, false>(ss, sm, weight, pts, stride, g);
-      write_block<NS, NM>(g, cs, ok, ke, ss, sm, rp.lm == 1, r, Mblk + 16 * p, SEG ? pts + 28 * stride : pts, stride,
-                          [](int, int, double) {});
+      fx_cell_products<NS, NM, false, kQuadThreads>(ss, sm, weight, pts, g);
+      write_block<NS, NM, kQuadThreads>(g, cs, ok, ke, ss, sm, rp.lm == 1, r, Mblk + 16 * p,
+                                        SEG ? pts + 28 * kQuadThreads : pts);
       if (cs.cell == 0) {
         if (ok) flag[p] = 1;
         else integrate_pair_fp64<NS, NM, SEG>(p, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, slow);
@@ -513,18 +512,18 @@ template <int NS, int NM, bool SEG>
 void launch_split(const IntegrateArgs& a, const RunParams& rp, int n_sm, int rounds, int warps) {
   auto clip = k_pair_clip<NS, NM, SEG>;
   auto quad = k_pair_quadrature<NS, NM, SEG>;
-  const size_t shq = (size_t)warps * 32 * kPtsBytes<SEG>;
+  const size_t shq = (size_t)kQuadThreads * kPtsBytes<SEG>;
   cudaFuncSetAttribute(quad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shq);
   int clip_sm = 0, quad_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&clip_sm, clip, warps * 32, 0);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&quad_sm, quad, warps * 32, shq);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&quad_sm, quad, kQuadThreads, shq);
   const unsigned gc = (unsigned)(n_sm * (clip_sm < 1 ? 1 : clip_sm)), gq = (unsigned)(n_sm * (quad_sm < 1 ? 1 : quad_sm));
   if (a.grid_out) *a.grid_out = (int)gc;
   for (int64_t first = 0; first < a.pair_cap; first += kPairChunk) {
     launch_pair_sort<NS, NM>(a, rp, n_sm, 32 * rounds, first);
     clip<<<gc, warps * 32, 0, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag, a.pair_cap,
                                           first, a.order, a.rec, a.st, a.cta_t);
-    quad<<<gq, warps * 32, shq, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag,
+    quad<<<gq, kQuadThreads, shq, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag,
                                             a.pair_cap, first, a.rec, a.st);
   }
 }

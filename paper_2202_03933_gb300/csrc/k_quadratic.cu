@@ -194,9 +194,9 @@ __device__ __forceinline__ void fx_shape_quadratic(int k, long long xi, long lon
 
 // Sums over one cell's points of N_p (W N_m)^T for half of the parent's shape
 // functions (bounds as in fx_cell_products, with the roles exchanged).
-template <int NP, int NM, int HALF>
+template <int NP, int NM, int HALF, int stride>
 __device__ __forceinline__ void fx_cell_quadratic(int k, const FxScales& sm, long long weight,
-                                                  const long long* __restrict__ pts, int stride, FxAcc g[4][4]) {
+                                                  const long long* __restrict__ pts, FxAcc g[4][4]) {
   constexpr int NR = NP / 2;
 #pragma unroll
   for (int a = 0; a < NR; ++a)
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(kQThreads, 4) k_quadratic_cells(
   constexpr int NSUB = NP == 8 ? 4 : 3, NR = NP / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   long long* pts = reinterpret_cast<long long*>(smem_raw) + threadIdx.x;
-  const int stride = (int)blockDim.x;
+  constexpr int stride = kQThreads;
   const int lane = threadIdx.x & 31;
   const int64_t n = 4 * chunk_pairs(st, pair_cap, first, kPairChunk / 4);
   const int turn = cell_turn(n);
@@ -320,8 +320,8 @@ __global__ void __launch_bounds__(kQThreads, 4) k_quadratic_cells(
         weight = f.weight(cs.cell);
         sm = f.sm;
         ke = f.ke;
-        ok = fx_back_project<NSUB, NM>(f, cs.cell, srec + (int64_t)SR_STRIDE * (4 * (int64_t)ps[u >> 2] + (u & 3)), xm,
-                                       conn_m, pm[u >> 2], pts, stride);
+        ok = fx_back_project<NSUB, NM, stride>(f, cs.cell, srec + (int64_t)SR_STRIDE * (4 * (int64_t)ps[u >> 2] + (u & 3)), xm,
+                                       conn_m, pm[u >> 2], pts);
       }
       const unsigned bad = __ballot_sync(0xffffffffu, cs.cell >= 0 && !ok);
       ok &= !(cs.cell >= 0 && (bad >> cs.first & ((1u << cs.cells) - 1u)) != 0);
@@ -331,11 +331,11 @@ __global__ void __launch_bounds__(kQThreads, 4) k_quadratic_cells(
       };
       long long* sums = pts + 28 * stride;
       FxAcc g[4][4];
-      fx_cell_quadratic<NP, NM, 0>((int)(u & 3), sm, weight, pts, stride, g);
-      fx_sum_cells<NR, NM>(g, cs, ok, sums, stride, emit);
+      fx_cell_quadratic<NP, NM, 0, stride>((int)(u & 3), sm, weight, pts, g);
+      fx_sum_cells<NR, NM, stride>(g, cs, ok, sums, emit);
       out += 4 * NR;
-      fx_cell_quadratic<NP, NM, 1>((int)(u & 3), sm, weight, pts, stride, g);
-      fx_sum_cells<NR, NM>(g, cs, ok, sums, stride, emit);
+      fx_cell_quadratic<NP, NM, 1, stride>((int)(u & 3), sm, weight, pts, g);
+      fx_sum_cells<NR, NM, stride>(g, cs, ok, sums, emit);
       if (ok && (NP < 8 || NM < 4))   // the block is padded with zeros
         for (int e = cs.cell; e < 32; e += cs.cells)
           if ((e >> 2) >= NP || (e & 3) >= NM) __stcs(U + 32 * u + e, 0.0);

@@ -123,9 +123,9 @@ __device__ __forceinline__ void fx_shape(const FxScales& s, long long xi, long l
 // memory.  Records are stored in groups of 32, word w of lane i of group g at
 // rec[(g kWords + w) 32 + i]: a warp reads or writes 256 contiguous bytes.
 struct FxRecord {
-  static constexpr int kScale = 26, kMapS = 27, kMapM = 35, kPair = 43, kInfo = 44, kWords = 45;
+  static constexpr int kMapS = 26, kMapM = 34, kScale = 42, kPair = 43, kInfo = 44, kWords = 45;
   // words: 2k, 2k + 1: vertex k; 16 + c: weight of cell c; 24, 25: centre;
-  // 26: the eight factor scales; 27.., 35..: maps (c0, then the digits k1 k2 k3); 43: pair id;
+  // 26.., 34..: maps (c0, then the digits k1 k2 k3); 42: the eight factor scales; 43: pair id;
   // 44: nr | kb_s << 8 | kb_m << 16 | affine_s << 24 | affine_m << 25 | ke << 32 | E << 48
   static __device__ __forceinline__ void store_map(long long* o, const FxMap& m, bool bilinear_possible) {
     auto put = [&](int w, Dg d) { o[32 * w] = (long long)(((unsigned long long)(unsigned)d.h << 32) | (unsigned)d.l); };
@@ -142,6 +142,14 @@ struct FxRecord {
     if (bilinear_possible && !m.affine) {
       m.k3u = get(6); m.k3v = get(7);
       m.bilinear_floats();
+    }
+  }
+  static __device__ __forceinline__ void load_scales(const long long* o, FxScales& ss, FxScales& sm) {
+    const unsigned long long sc = (unsigned long long)o[32 * kScale];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      ss.k[k] = (int)(sc >> (8 * k)) & 0xff;
+      sm.k[k] = (int)(sc >> (32 + 8 * k)) & 0xff;
     }
   }
   template <int NS, int NM>
@@ -193,12 +201,7 @@ struct FxView {
     m.affine = (info >> 25) & 1;
     ke = (int)(short)(info >> 32);
     E = (int)(short)(info >> 48);
-    const unsigned long long sc = (unsigned long long)o[32 * FxRecord::kScale];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      ss.k[k] = (int)(sc >> (8 * k)) & 0xff;
-      sm.k[k] = (int)(sc >> (32 + 8 * k)) & 0xff;
-    }
+    FxRecord::load_scales(o, ss, sm);
     cu = o[32 * 24];
     cv = o[32 * 25];
     FxRecord::load_map(o + 32 * FxRecord::kMapS, s, NS == 4);
@@ -207,14 +210,15 @@ struct FxView {
 };
 
 // Back-projections of the seven points of cell c, in fixed point: xi, eta of the
-// slave and the master element into pts[(4 q + 0..3) * stride].  False if one
+// slave and the master element into pts[(4 q + 0..3) * stride] (pts: this
+// thread's slice of shared memory, stride: the block's threads).  False if one
 // fails.  The rule's points are c + (e1 + e2) / 3 and, per orbit (a, b),
 // c + a (e1 + e2) plus (b - a) e2, (b - a) e1 or nothing: three products a
 // coordinate for three points.
-template <int NS, int NM, class F>
+template <int NS, int NM, int stride, class F>
 __device__ __forceinline__ bool fx_back_project(F& f, int c, const double* __restrict__ r,
                                                 const double* __restrict__ xm, const int32_t* __restrict__ conn_m,
-                                                int32_t m, long long* __restrict__ pts, int stride) {
+                                                int32_t m, long long* __restrict__ pts) {
   const int ib = f.ib(c), iw = f.iw(c);
   const Dg e1u = fx_split(f.x(ib) - f.cu), e1v = fx_split(f.y(ib) - f.cv);
   const Dg e2u = fx_split(f.x(iw) - f.cu), e2v = fx_split(f.y(iw) - f.cv);
@@ -264,9 +268,9 @@ __device__ __forceinline__ bool fx_back_project(F& f, int c, const double* __res
 // keep their digits.  Bounds: a product's cross terms are l h of at most
 // 2^31 2^29, seven of them, and h l ones that sum to at most 2^29 2^31 (both
 // cannot be met at once: N = 1 at all seven points).
-template <int NS, int NC, bool SLAVE2>
+template <int NS, int NC, bool SLAVE2, int stride>
 __device__ __forceinline__ void fx_cell_products(const FxScales& ss, const FxScales& sc, long long weight,
-                                                 const long long* __restrict__ pts, int stride, FxAcc g[4][4]) {
+                                                 const long long* __restrict__ pts, FxAcc g[4][4]) {
 #pragma unroll
   for (int a = 0; a < NS; ++a)
 #pragma unroll
@@ -370,9 +374,9 @@ __device__ __forceinline__ CellSlot assign_cells(int ncell) {
 // its entries (a, l) in turn and pass each sum, hh + cr / 2^32, to emit.  buf:
 // this thread's slice of shared memory (24 words; entry i at buf[i * stride],
 // lane L's at buf - lane + L), free to use by the whole warp.
-template <int NR, int NC, class Emit>
+template <int NR, int NC, int stride, class Emit>
 __device__ __forceinline__ void fx_sum_cells(const FxAcc g[4][4], const CellSlot& cs, bool ok,
-                                             long long* __restrict__ buf, int stride, Emit emit) {
+                                             long long* __restrict__ buf, Emit emit) {
   __syncwarp();
 #pragma unroll
   for (int a = 0; a < NR; ++a)
@@ -397,17 +401,16 @@ __device__ __forceinline__ void fx_sum_cells(const FxAcc g[4][4], const CellSlot
 }
 
 // Writes the 4x4 block M = A G (standard LMs: G) of every pair of the warp from
-// its cells' sums g (fx_sum_cells), and passes the entries (a, l) of G to keep.
-template <int NS, int NC, class Keep>
+// its cells' sums g (fx_sum_cells).
+template <int NS, int NC, int stride>
 __device__ __forceinline__ void write_block(const FxAcc g[4][4], const CellSlot& cs, bool ok, int ke,
                                             const FxScales& ss, const FxScales& sc, bool dual,
                                             const double* __restrict__ r, double* __restrict__ out,
-                                            long long* __restrict__ buf, int stride, Keep keep) {
+                                            long long* __restrict__ buf) {
   double G[16];   // dual: this lane's entries, until every lane has read the sums
   int n = 0;
-  fx_sum_cells<NS, NC>(g, cs, ok, buf, stride, [&](int a, int l, long long hh, long long cr) {
+  fx_sum_cells<NS, NC, stride>(g, cs, ok, buf, [&](int a, int l, long long hh, long long cr) {
     const double v = fx_to_double(hh, cr, ke - ss.shape<NS>(a) - sc.shape<NC>(l));
-    keep(a, l, v);
     if (dual) G[n++] = v;
     else __stcs(out + 4 * a + l, v);
   });
