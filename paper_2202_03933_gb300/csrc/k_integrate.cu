@@ -27,11 +27,12 @@
 //    busy, 400 instructions a pair) and instruction fetch, the quadrature
 //    kernel by issue (0.52 per scheduler and clock) over the multiply-add and
 //    integer pipes.
-//  * one kernel with everything in FP64 (k_integrate_batched): for callers
-//    without workspace, and pairs that do not fit the fixed-point frame.  Each
-//    warp sorts a batch of up to 32 R pairs and runs rounds of 32; affine maps
-//    are inverted with one precomputed 2x2 inverse, bilinear ones by Newton in
-//    FP32, then one step with an FP64 residual (MapInverse in clip.cuh).
+//  * one kernel (k_integrate_fused): for callers without workspace.  Clip
+//    records in shared memory, then the same quadrature.
+//  * pairs that do not fit the fixed-point frame are integrated in FP64 in
+//    either form (integrate_pair_fp64): affine maps are inverted with one
+//    precomputed 2x2 inverse, bilinear ones by Newton in FP32, then one step
+//    with an FP64 residual (MapInverse in clip.cuh).
 //  * variant 1: one pair per thread, FP64 Newton from xi = 0 at every point
 //    (the oracle's iteration), kept as the reference schedule.
 //
@@ -227,8 +228,7 @@ constexpr int kQuadThreads = 128;   // of the quadrature kernel's blocks
 template <bool SEG>
 constexpr int kPtsBytes = (SEG ? 52 : 28) * 8;
 
-// One pair in FP64 (the one-kernel form, and pairs whose geometry does not fit
-// the fixed-point frame of the two-kernel form): FP64 clip, then the 7-point rule on the
+// One pair in FP64 (pairs whose geometry does not fit the fixed-point frame): FP64 clip, then the 7-point rule on the
 // centroid fan with the map inversions of MapInverse.
 template <int NS, int NM, bool SEG>
 __device__ __noinline__ void integrate_pair_fp64(int64_t p, const int32_t* __restrict__ ps,
@@ -334,45 +334,150 @@ __device__ __noinline__ void integrate_pair_fp64(int64_t p, const int32_t* __res
 }
 
 
+// FP64 clip of pair p, and its record at o (word w at o[32 w]).  Empty pairs
+// get zero blocks; pairs that do not fit the fixed-point frame are integrated
+// in FP64 here.  Either way the record says that no cells are left.
 template <int NS, int NM, bool SEG>
-__global__ void __launch_bounds__(kMaxPairBlock) k_integrate_batched(
+__device__ __forceinline__ void clip_record(bool has, int64_t p, const int32_t* __restrict__ ps,
+                                            const int32_t* __restrict__ pm, const double* __restrict__ srec,
+                                            const double* __restrict__ xm, const int32_t* __restrict__ conn_m,
+                                            const RunParams& rp, double* __restrict__ Mblk,
+                                            double* __restrict__ Dblk, uint8_t* __restrict__ flag,
+                                            long long* __restrict__ o, PairCounters& ctr) {
+  bool stored = false;
+  if (has) {
+    const double* r = srec + (int64_t)SR_STRIDE * ps[p];
+    PlaneMap mmap;
+    double pu[kPolyS], pv[kPolyS];
+    const int nr = clip_polygon<NS, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
+    if (nr == 0) {
+      write_zero_blocks(p, SEG, Mblk, Dblk);
+      flag[p] = 0;
+    } else {
+      FxPolygon f;
+      stored = f.setup<NS, NM>(r, mmap, pu, pv, nr);
+      if (stored) {
+        FxRecord::store<NS, NM>(o, f, p);
+        ctr.cells += f.ncell;
+        ctr.gp += 7 * f.ncell;
+        ctr.nonempty++;
+      } else {
+        integrate_pair_fp64<NS, NM, SEG>(p, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, ctr);
+      }
+    }
+  }
+  if (!stored) o[32 * FxRecord::kInfo] = 0;   // nr = 0
+}
+
+__device__ __forceinline__ int record_cells(long long info) {
+  const int nr = (int)(info & 0xff);
+  return nr > 3 ? nr : (nr == 3 ? 1 : 0);
+}
+
+// One cell of a record (at o, where this lane has one) per lane of the warp:
+// the cell's back-projections, then its products, then the pair's sums through
+// shared memory, and the pair's blocks.  STRIDE: the block's threads; pts:
+// this thread's slice of kPtsBytes.
+template <int NS, int NM, bool SEG, int STRIDE>
+__device__ __forceinline__ void integrate_cells(const CellSlot& cs, const long long* o,
+                                                const int32_t* __restrict__ ps, const int32_t* __restrict__ pm,
+                                                const double* __restrict__ srec, const double* __restrict__ xm,
+                                                const int32_t* __restrict__ conn_m, const RunParams& rp,
+                                                double* __restrict__ Mblk, double* __restrict__ Dblk,
+                                                uint8_t* __restrict__ flag, long long* __restrict__ pts,
+                                                PairCounters& slow) {
+  bool ok = cs.cell >= 0;
+  int64_t p = 0;
+  int32_t m = 0;
+  const double* r = srec;
+  FxScales ss, sm;
+  int ke = 0;
+  long long weight = 0;
+  if (ok) {
+    FxView f;
+    f.load<NS, NM>(o);
+    p = o[32 * FxRecord::kPair];
+    r = srec + (int64_t)SR_STRIDE * ps[p];
+    m = pm[p];
+    weight = f.weight(cs.cell);
+    ss = f.ss;
+    sm = f.sm;
+    ke = f.ke;
+    ok = fx_back_project<NS, NM, STRIDE>(f, cs.cell, r, xm, conn_m, m, pts);
+  }
+  const unsigned bad = __ballot_sync(0xffffffffu, cs.cell >= 0 && !ok);
+  const bool slow_pair = cs.cell >= 0 && (bad >> cs.first & ((1u << cs.cells) - 1u)) != 0;
+  ok &= !slow_pair;
+  FxAcc g[4][4];
+  if (SEG) {   // the sums' memory is apart from the points', which M's products read again
+    fx_cell_products<NS, NS, true, STRIDE>(ss, ss, weight, pts, g);
+    write_block<NS, NS, STRIDE>(g, cs, ok, ke, ss, ss, rp.lm == 1, r, Dblk + 16 * p, pts + 28 * STRIDE);
+  }
+  fx_cell_products<NS, NM, false, STRIDE>(ss, sm, weight, pts, g);
+  write_block<NS, NM, STRIDE>(g, cs, ok, ke, ss, sm, rp.lm == 1, r, Mblk + 16 * p, SEG ? pts + 28 * STRIDE : pts);
+  if (cs.cell == 0) {
+    if (ok) flag[p] = 1;
+    else integrate_pair_fp64<NS, NM, SEG>(p, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, slow);
+  }
+  __syncwarp();
+}
+
+// -------------------------------------------------------- one-kernel form
+// For callers without workspace: records live in shared memory, one group of
+// pairs per warp and turn.  Small pair lists are latency-bound (14,400 pairs
+// fill 3 of 16 warps of a scheduler at 8 pairs a warp), so a group is as small
+// as spreads the list over all warps, 8 pairs (about a warp full of cells) to 32.
+// 14,400 pairs of quad4 elements through the no-allocation entry point: 251 us a
+// call with the former FP64 kernel (one pair per lane, all of it in one round
+// of 450 warps), 170 us with this one.
+constexpr int kFusedThreads = 128;
+template <bool SEG>
+constexpr size_t kFusedSmem = (size_t)kFusedThreads * (kPtsBytes<SEG> + FxRecord::kWords * 8);
+template <int NS, int NM, bool SEG>
+__global__ void __launch_bounds__(kFusedThreads, 3) k_integrate_fused(
     const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
     const double* __restrict__ xm, const int32_t* __restrict__ conn_m, RunParams rp, double* __restrict__ Mblk,
-    double* __restrict__ Dblk, uint8_t* __restrict__ flag, int64_t pair_cap, int B, DevStatus* st,
+    double* __restrict__ Dblk, uint8_t* __restrict__ flag, int64_t pair_cap, DevStatus* st,
     unsigned long long* cta_t) {
   cta_mark(cta_t, 0);
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned char* my = smem_raw + (size_t)warp * batch_smem_bytes(B);
-  uint16_t* perm = reinterpret_cast<uint16_t*>(my + 32);
-
-  PairCounters ctr;
-  const bool ok = st->over_pairs == 0 && st->over_bins == 0;
-  const int64_t n = ok ? (int64_t)min((unsigned long long)pair_cap, st->n_pairs) : 0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  long long* pts = reinterpret_cast<long long*>(smem_raw) + threadIdx.x;
+  long long* rec = reinterpret_cast<long long*>(smem_raw) + kFusedThreads * (kPtsBytes<SEG> / 8) +
+                   warp * (32 * FxRecord::kWords);
+  PairCounters ctr, slow;
+  const int64_t n = chunk_pairs(st, pair_cap, 0, pair_cap);
+  const int64_t warps = (int64_t)gridDim.x * (kFusedThreads / 32);
+  const int turn = (int)max((int64_t)8, min((int64_t)32, (n + warps - 1) / warps));
   const Watchdog wd(rp.watchdog_us);
-  const int64_t share = 2 * (int64_t)gridDim.x * (blockDim.x >> 5);
   for (;;) {   // bounded: the shared counter only grows
     if (wd.expired(&st->timeout)) break;
-    int64_t base;
-    int fetch;
-    if (!fetch_batch(&st->work_ctr, n, share, B, base, fetch)) break;
-    const int n_live = sort_batch<NS, NM, 1>(my, B, base, min(n, base + (int64_t)fetch), (fetch + 31) >> 5, ps, pm, srec,
-                                          xm, conn_m);
-    // ---- phase B: one pair per lane, rounds of similar cost
-    for (int i0 = 0; i0 < n_live; i0 += 32) {
-      const int i = i0 + lane;
-      if (i < n_live)
-        integrate_pair_fp64<NS, NM, SEG>(base + perm[i], ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, ctr);
+    unsigned long long g0 = 0;
+    if (lane == 0) g0 = atomicAdd(&st->work_ctr, (unsigned long long)turn);
+    const int64_t p0 = (int64_t)__shfl_sync(0xffffffffu, g0, 0);
+    if (p0 >= n) break;
+    const int pairs = (int)min((int64_t)turn, n - p0);
+    clip_record<NS, NM, SEG>(lane < pairs, p0 + lane, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, rec + lane, ctr);
+    __syncwarp();
+    for (int w = 0; w < pairs;) {
+      int ncell = 0;
+      if (w + lane < pairs) ncell = record_cells(rec[32 * FxRecord::kInfo + w + lane]);
+      const CellSlot cs = assign_cells(ncell);
+      const long long* o = rec + w + cs.rec;
+      w += cs.taken;
+      integrate_cells<NS, NM, SEG, kFusedThreads>(cs, o, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, pts, slow);
     }
     __syncwarp();
   }
+  ctr.newton_fail += slow.newton_fail;   // slow pairs' cells and points were counted with their records
+  ctr.xi_oor += slow.xi_oor;
   ctr.add(st);
   __syncthreads();
   cta_mark(cta_t, 1);
 }
 
 // ------------------------------------------- three-kernel form (default)
-// The batched kernel's work, split where its character changes: a sort kernel
+// Split where the work's character changes: a sort kernel
 // (FP32 keys, k_pair_sort), a clip kernel (FP64 clip, and the polygon's
 // conversion to fixed point) that leaves one record per pair in sorted order,
 // and a quadrature kernel on the integer pipe.  One kernel with all of it does
@@ -398,31 +503,8 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_clip(
     g = __shfl_sync(0xffffffffu, g, 0);
     const int64_t i = 32 * (int64_t)g + lane;
     if (32 * (int64_t)g >= n) break;
-    long long* o = rec + (int64_t)g * (32 * FxRecord::kWords) + lane;
-    bool stored = false;
-    if (i < n) {
-      const int64_t p = first + order[i];
-      const double* r = srec + (int64_t)SR_STRIDE * ps[p];
-      PlaneMap mmap;
-      double pu[kPolyS], pv[kPolyS];
-      const int nr = clip_polygon<NS, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
-      if (nr == 0) {
-        write_zero_blocks(p, SEG, Mblk, Dblk);
-        flag[p] = 0;
-      } else {
-        FxPolygon f;
-        stored = f.setup<NS, NM>(r, mmap, pu, pv, nr);
-        if (stored) {
-          FxRecord::store<NS, NM>(o, f, p);
-          ctr.cells += f.ncell;
-          ctr.gp += 7 * f.ncell;
-          ctr.nonempty++;
-        } else {
-          integrate_pair_fp64<NS, NM, SEG>(p, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, ctr);
-        }
-      }
-    }
-    if (!stored) o[32 * FxRecord::kInfo] = 0;   // nr = 0: nothing left for the quadrature kernel
+    clip_record<NS, NM, SEG>(i < n, i < n ? first + order[i] : 0, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag,
+                             rec + (int64_t)g * (32 * FxRecord::kWords) + lane, ctr);
     __syncwarp();
   }
   ctr.add(st);
@@ -431,9 +513,7 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_clip(
 }
 
 // Quadrature of the clip kernel's records, one cell of a pair per lane (all
-// cells cost the same, so lanes idle only at the ends of warps): the cell's
-// back-projections, then its products, then the pair's sums through shared
-// memory.
+// cells cost the same, so lanes idle only at the ends of warps).
 template <int NS, int NM, bool SEG>
 __global__ void __launch_bounds__(kQuadThreads, 4) k_pair_quadrature(
     const int32_t* __restrict__ ps, const int32_t* __restrict__ pm, const double* __restrict__ srec,
@@ -458,48 +538,13 @@ __global__ void __launch_bounds__(kQuadThreads, 4) k_pair_quadrature(
       int ncell = 0;
       if (w + lane < records) {
         const int64_t i = r0 + w + lane;
-        const int nr = (int)(rec[((i >> 5) * FxRecord::kWords + FxRecord::kInfo) * 32 + (i & 31)] & 0xff);
-        ncell = nr > 3 ? nr : (nr == 3 ? 1 : 0);
+        ncell = record_cells(rec[((i >> 5) * FxRecord::kWords + FxRecord::kInfo) * 32 + (i & 31)]);
       }
       const CellSlot cs = assign_cells(ncell);
       const int64_t i = r0 + w + cs.rec;
       w += cs.taken;
-      bool ok = cs.cell >= 0;
-      int64_t p = 0;
-      int32_t m = 0;
-      const double* r = srec;
-      FxScales ss, sm;
-      int ke = 0;
-      long long weight = 0;
-      if (ok) {
-        const long long* o = rec + (i >> 5) * (32 * FxRecord::kWords) + (i & 31);
-        FxView f;
-        f.load<NS, NM>(o);
-        p = o[32 * FxRecord::kPair];
-        r = srec + (int64_t)SR_STRIDE * ps[p];
-        m = pm[p];
-        weight = f.weight(cs.cell);
-        ss = f.ss;
-        sm = f.sm;
-        ke = f.ke;
-        ok = fx_back_project<NS, NM, kQuadThreads>(f, cs.cell, r, xm, conn_m, m, pts);
-      }
-      const unsigned bad = __ballot_sync(0xffffffffu, cs.cell >= 0 && !ok);
-      const bool slow_pair = cs.cell >= 0 && (bad >> cs.first & ((1u << cs.cells) - 1u)) != 0;
-      ok &= !slow_pair;
-      FxAcc g[4][4];
-      if (SEG) {   // the sums' memory is apart from the points', which M's products read again
-        fx_cell_products<NS, NS, true, kQuadThreads>(ss, ss, weight, pts, g);
-        write_block<NS, NS, kQuadThreads>(g, cs, ok, ke, ss, ss, rp.lm == 1, r, Dblk + 16 * p, pts + 28 * kQuadThreads);
-      }
-      fx_cell_products<NS, NM, false, kQuadThreads>(ss, sm, weight, pts, g);
-      write_block<NS, NM, kQuadThreads>(g, cs, ok, ke, ss, sm, rp.lm == 1, r, Mblk + 16 * p,
-                                        SEG ? pts + 28 * kQuadThreads : pts);
-      if (cs.cell == 0) {
-        if (ok) flag[p] = 1;
-        else integrate_pair_fp64<NS, NM, SEG>(p, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, slow);
-      }
-      __syncwarp();
+      integrate_cells<NS, NM, SEG, kQuadThreads>(cs, rec + (i >> 5) * (32 * FxRecord::kWords) + (i & 31), ps, pm, srec,
+                                                 xm, conn_m, rp, Mblk, Dblk, flag, pts, slow);
     }
   }
   // pairs, cells and points were counted by the clip kernel
@@ -529,17 +574,15 @@ void launch_split(const IntegrateArgs& a, const RunParams& rp, int n_sm, int rou
 }
 
 template <int NS, int NM, bool SEG>
-void launch_batched(const IntegrateArgs& a, const RunParams& rp, int n_sm, int rounds, int warps) {
-  const size_t shm = (size_t)warps * batch_smem_bytes(32 * rounds);
-  auto kern = k_integrate_batched<NS, NM, SEG>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+void launch_fused(const IntegrateArgs& a, const RunParams& rp, int n_sm) {
+  auto kern = k_integrate_fused<NS, NM, SEG>;
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem<SEG>);
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, shm);
-  if (per_sm < 1) per_sm = 1;
-  const unsigned grid = (unsigned)(n_sm * per_sm);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFusedThreads, kFusedSmem<SEG>);
+  const unsigned grid = (unsigned)(n_sm * (per_sm < 1 ? 1 : per_sm));
   if (a.grid_out) *a.grid_out = (int)grid;
-  kern<<<grid, warps * 32, shm, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag,
-                                             a.pair_cap, 32 * rounds, a.st, a.cta_t);
+  kern<<<grid, kFusedThreads, kFusedSmem<SEG>, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk,
+                                                           a.flag, a.pair_cap, a.st, a.cta_t);
 }
 
 template <int NS, int NM, bool SEG>
@@ -568,8 +611,8 @@ void integrate_nsnm(const IntegrateArgs& a, const RunParams& rp, int n_sm, int v
     else launch_split<NS, NM, false>(a, rp, n_sm, rounds, block / 32);
     return;
   }
-  if (seg) launch_batched<NS, NM, true>(a, rp, n_sm, rounds, block / 32);
-  else launch_batched<NS, NM, false>(a, rp, n_sm, rounds, block / 32);
+  if (seg) launch_fused<NS, NM, true>(a, rp, n_sm);
+  else launch_fused<NS, NM, false>(a, rp, n_sm);
 }
 template void integrate_nsnm<MORTAR_PAIR_NS, MORTAR_PAIR_NM>(const IntegrateArgs&, const RunParams&, int, int, int,
                                                               int, int);
