@@ -107,6 +107,7 @@ struct mortar_ctx {
   mortar::DevBuf cn_normals, cn_gap, cn_lam, cn_active, cn_ncp;   // contact terms per slave node
   mortar::DevBuf rule_1d;                   // element-based rule: Gauss-Legendre points and weights
   int32_t rule_1d_n = 0;
+  int32_t rule_boost[2] = {-1, -1};         // of its fixed-point table, quad4 and tri3 slaves; -1: FP64
   mortar::DevBuf dstat;                     // mortar::DevStatus
   mortar::DevStatus* hstat = nullptr;       // pinned host copy
   bool search_valid = false;

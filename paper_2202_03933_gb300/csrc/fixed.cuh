@@ -252,7 +252,7 @@ struct FxMap {
     y -= d1;
     step = fabsf(d0) + fabsf(d1);
   }
-  __device__ __forceinline__ bool coarse(float tu, float tv, float& x, float& y) {
+  __device__ __forceinline__ bool settle(float tu, float tv, float& x, float& y) {
     float step;
     x = b00 * tu + b01 * tv;
     y = b10 * tu + b11 * tv;
@@ -262,7 +262,10 @@ struct FxMap {
 #pragma unroll 1
       for (int it = 0; it < 13 && !(step <= 1e-4f); ++it) newton_f32(tu, tv, x, y, step);
     }
-    return step <= 1e-4f && fabsf(x) < 1.01f && fabsf(y) < 1.01f;
+    return step <= 1e-4f;
+  }
+  __device__ __forceinline__ bool coarse(float tu, float tv, float& x, float& y) {
+    return settle(tu, tv, x, y) && fabsf(x) < 1.01f && fabsf(y) < 1.01f;
   }
 
   // FP32 xi of the point x (Q62), for bounds only; false if it did not settle
@@ -294,23 +297,20 @@ struct FxMap {
     rv = a.get<3>() - dv;
   }
 
-  // xi (Q61) of the point x (Q62); false if the FP32 or the fixed-point steps did not settle
-  template <int NEN>
-  __device__ __forceinline__ bool solve(long long xu, long long xv, long long& xi, long long& eta) {
-    const long long du = xu - c0u, dv = xv - c0v;
-    if (NEN == 3 || affine) {
-      const Dg a = fx_split(du), b = fx_split(dv);
-      FxAcc s;
-      s.mul(k1u, a);
-      s.mac(k1v, b);
-      xi = s.get(2 + kb);
-      s.mul(k2u, a);
-      s.mac(k2v, b);
-      eta = s.get(2 + kb);
-      return true;
-    }
-    float x, y;
-    if (!coarse(fx_f32(du), fx_f32(dv), x, y)) return false;
+  // affine: xi (Q61) at d = x - c0
+  __device__ __forceinline__ void solve_affine(long long du, long long dv, long long& xi, long long& eta) const {
+    const Dg a = fx_split(du), b = fx_split(dv);
+    FxAcc s;
+    s.mul(k1u, a);
+    s.mac(k1v, b);
+    xi = s.get(2 + kb);
+    s.mul(k2u, a);
+    s.mac(k2v, b);
+    eta = s.get(2 + kb);
+  }
+  // bilinear: the two fixed-point steps from the FP32 iterate (x, y)
+  __device__ __forceinline__ bool refine(long long du, long long dv, float x, float y, long long& xi,
+                                         long long& eta) const {
     xi = (long long)__float2int_rn(x * 0x1p30f) << 31;
     eta = (long long)__float2int_rn(y * 0x1p30f) << 31;
     long long ru, rv;
@@ -327,6 +327,17 @@ struct FxMap {
     xi -= (long long)__float2int_rn(d0);
     eta -= (long long)__float2int_rn(d1);
     return fmaxf(fabsf(d0), fabsf(d1)) < 0x1p25f;
+  }
+  // xi (Q61) of the point x (Q62); false if the FP32 or the fixed-point steps did not settle
+  template <int NEN>
+  __device__ __forceinline__ bool solve(long long xu, long long xv, long long& xi, long long& eta) {
+    const long long du = xu - c0u, dv = xv - c0v;
+    if (NEN == 3 || affine) {
+      solve_affine(du, dv, xi, eta);
+      return true;
+    }
+    float x, y;
+    return coarse(fx_f32(du), fx_f32(dv), x, y) && refine(du, dv, x, y, xi, eta);
   }
 };
 
