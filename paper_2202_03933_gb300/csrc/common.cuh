@@ -149,6 +149,36 @@ __device__ __forceinline__ double f64_of_f32(float f) {
   return __longlong_as_double((long long)(sign | (e64 << 52) | ((unsigned long long)(u & 0x7fffffu) << 29)));
 }
 
+// FP32 seed of 1 / x (relative error about 2^-22) as a double, by integer
+// operations and one FP32 reciprocal; false for zero, subnormal, very large or
+// very small x, infinities and NaN.
+__device__ __forceinline__ bool rcp_seed(double x, double& y) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ffu);
+  const float m = __uint_as_float(0x3f800000u | (unsigned)((b >> 29) & 0x7fffffull));   // [1, 2)
+  const unsigned f = __float_as_uint(__fdividef(1.0f, m));                              // (1/2, 1]
+  const unsigned long long ye = (unsigned long long)((int)(f >> 23) - 127 + 2046 - e);
+  y = __longlong_as_double((long long)((b & 0x8000000000000000ull) | ye << 52 | (unsigned long long)(f & 0x7fffffu) << 29));
+  return e > 64 && e < 1980;
+}
+// 1 / x: the seed and two Newton steps y + y (1 - x y), each squaring the
+// error; 4 FP64 operations, where an IEEE division costs about 10.
+__device__ __forceinline__ double rcp_newton(double x) {
+  double y;
+  if (!rcp_seed(x, y)) return 1.0 / x;
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+// a / x to about an ulp: one Newton step (error 2^-44), the quotient, and its
+// remainder's correction; 5 FP64 operations.
+__device__ __forceinline__ double quotient(double a, double x) {
+  double y;
+  if (!rcp_seed(x, y)) return a / x;
+  y = fma(y, fma(-x, y, 1.0), y);
+  const double q = a * y;
+  return fma(fma(-x, q, a), y, q);
+}
+
 template <int NEN>
 __device__ __forceinline__ void shape_fn(double xi, double eta, double N[4]) {
   if constexpr (NEN == 4) {

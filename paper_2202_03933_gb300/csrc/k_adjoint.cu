@@ -133,9 +133,7 @@ __device__ void adjoint_one(int64_t p, const int32_t* __restrict__ ps, const int
     PlaneMap smap;
     smap.c0u = r[SR_C + 0]; smap.c0v = r[SR_C + 1]; smap.c1u = r[SR_C + 2]; smap.c1v = r[SR_C + 3];
     smap.c2u = r[SR_C + 4]; smap.c2v = r[SR_C + 5]; smap.c3u = r[SR_C + 6]; smap.c3v = r[SR_C + 7];
-    double ma2 = 0.0;
-    for (int l = 0; l < NM; ++l) ma2 += cross2(mu[l], mv[l], mu[(l + 1) % NM], mv[(l + 1) % NM]);
-    const bool mrev = ma2 < 0.0;
+    const bool mrev = polygon_reversed<NM>(mu, mv);
     const bool srev = r[SR_REV] != 0.0;
     // ---- forward clip with recorded stages and merge
     ClipRec<NS> cr;
@@ -502,9 +500,7 @@ __device__ __noinline__ void adjoint_pair_fast(int64_t p, const int32_t* __restr
   PlaneMap smap;
   smap.c0u = r[SR_C + 0]; smap.c0v = r[SR_C + 1]; smap.c1u = r[SR_C + 2]; smap.c1v = r[SR_C + 3];
   smap.c2u = r[SR_C + 4]; smap.c2v = r[SR_C + 5]; smap.c3u = r[SR_C + 6]; smap.c3v = r[SR_C + 7];
-  double ma2 = 0.0;
-  for (int l = 0; l < NM; ++l) ma2 += cross2(mu[l], mv[l], mu[(l + 1) % NM], mv[(l + 1) % NM]);
-  const bool mrev = ma2 < 0.0;
+  const bool mrev = polygon_reversed<NM>(mu, mv);
   // ---- forward clip recorded as a vertex pool, and merge (same decisions as clip_polygon)
   ClipPool<NS, NM> cp;
   const bool nonempty = cp.run(r, mu, mv, mrev, ctr.clip_over);
@@ -827,9 +823,7 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, un
         mv[l] = dx * r[SR_T2] + dy * r[SR_T2 + 1] + dz * r[SR_T2 + 2];
       }
       const PlaneMap mmap = plane_map<NM>(mu, mv);
-      double ma2 = 0.0;
-      for (int l = 0; l < NM; ++l) ma2 += cross2(mu[l], mv[l], mu[(l + 1) % NM], mv[(l + 1) % NM]);
-      const bool mrev = ma2 < 0.0;
+      const bool mrev = polygon_reversed<NM>(mu, mv);
       ClipPool<NS, NM> cp;
       if (!cp.run(r, mu, mv, mrev, ctr.clip_over)) {
         adjoint_empty<SEG>(p, g.fo);

@@ -42,6 +42,7 @@
 #include "context.h"
 #include "pair_sort.cuh"
 #include "quadrature.cuh"
+#include "reverse.cuh"
 
 namespace mortar {
 
@@ -240,7 +241,7 @@ __device__ __noinline__ void integrate_pair_fp64(int64_t p, const int32_t* __res
   const double* r = srec + (int64_t)SR_STRIDE * ps[p];
   PlaneMap mmap;
   double pu[kPolyS], pv[kPolyS];
-  const int nr = clip_polygon<NS, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
+  const int nr = clip_polygon_pool<NS, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
   if (nr == 0) {
     write_zero_blocks(p, SEG, Mblk, Dblk);
     flag[p] = 0;
@@ -349,7 +350,7 @@ __device__ __forceinline__ void clip_record(bool has, int64_t p, const int32_t* 
     const double* r = srec + (int64_t)SR_STRIDE * ps[p];
     PlaneMap mmap;
     double pu[kPolyS], pv[kPolyS];
-    const int nr = clip_polygon<NS, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
+    const int nr = clip_polygon_pool<NS, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
     if (nr == 0) {
       write_zero_blocks(p, SEG, Mblk, Dblk);
       flag[p] = 0;

@@ -25,6 +25,7 @@
 #include "context.h"
 #include "pair_sort.cuh"
 #include "quadrature.cuh"
+#include "reverse.cuh"
 #include "quadratic.cuh"
 
 namespace mortar {
@@ -53,7 +54,7 @@ __device__ __noinline__ void integrate_unit(int64_t u, const int32_t* __restrict
   double2* out = reinterpret_cast<double2*>(U + 32 * u);
   PlaneMap mmap;
   double Pu[kPolyS], Pv[kPolyS];
-  const int nr = clip_polygon<NSUB, NM, kPolyS>(r, xm, conn_m, m, mmap, Pu, Pv, ctr.clip_over);
+  const int nr = clip_polygon_pool<NSUB, NM, kPolyS>(r, xm, conn_m, m, mmap, Pu, Pv, ctr.clip_over);
   if (nr == 0) {
 #pragma unroll
     for (int i = 0; i < 16; ++i) __stcs(out + i, make_double2(0.0, 0.0));
@@ -249,7 +250,7 @@ __global__ void __launch_bounds__(kQThreads, 4) k_quadratic_clip(
       const double* r = srec + (int64_t)SR_STRIDE * (4 * (int64_t)ps[p] + (u & 3));
       PlaneMap mmap;
       double pu[kPolyS], pv[kPolyS];
-      const int nr = clip_polygon<NSUB, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
+      const int nr = clip_polygon_pool<NSUB, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
       if (nr == 0) {
         uflag[u] = 0;
       } else {

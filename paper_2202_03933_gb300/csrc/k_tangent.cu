@@ -94,9 +94,7 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
   PlaneMap smap;
   smap.c0u = r[SR_C + 0]; smap.c0v = r[SR_C + 1]; smap.c1u = r[SR_C + 2]; smap.c1v = r[SR_C + 3];
   smap.c2u = r[SR_C + 4]; smap.c2v = r[SR_C + 5]; smap.c3u = r[SR_C + 6]; smap.c3v = r[SR_C + 7];
-  double ma2 = 0.0;
-  for (int l = 0; l < NM; ++l) ma2 += cross2(mu[l], mv[l], mu[(l + 1) % NM], mv[(l + 1) % NM]);
-  const bool mrev = ma2 < 0.0;
+  const bool mrev = polygon_reversed<NM>(mu, mv);
   const bool srev = r[SR_REV] != 0.0;
   ClipPool<NS, NM> clip;   // compact record: master corners + intersections
   unsigned long long clip_dummy = 0;
