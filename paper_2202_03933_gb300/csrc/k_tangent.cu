@@ -9,12 +9,16 @@
 //     Z_c   = [segment D] sum_b N_b(xi_s) ys_b,c - sum_l N_l(xi_m) ym_l,c,
 // and the pair's rows are sum_e A[a][e] O_e,c (A = I for standard LMs).
 // Three lanes own one pair, one component c each, and run the reverse sweep
-// of the four outputs O_0..3,c together: each lane computes every third
-// quadrature point's back-projections and shape functions and shares them
-// with the other two through shared memory, the per-point adjoints of the
-// four seeds are accumulated side by side (their map-coefficient adjoints in
-// shared memory), and only the reverse of the clip and of the projection runs
-// once per seed.  The derivatives through A (dual LMs) and of
+// of the four outputs together: each lane computes every third quadrature
+// point's back-projections and shares them with the other two through shared
+// memory, the per-point adjoints of the four seeds are accumulated side by
+// side (their map-coefficient adjoints in shared memory), and only the reverse
+// of the clip and of the projection runs once per seed.  The seeds are the
+// monomials 1, xi, eta, xi eta, of which the N_e are combinations: a seed's
+// point adjoint is then a product or two, and the slave map's adjoints of all
+// four follow from 12 moments.  Bound by the FP64 pipe (about 75 % busy);
+// 300x260 quads, dual (0.31 M pairs): 21.7 ms with the N_e as seeds, 18.7 ms
+// this way, square roots and divisions of the plane once per pair.  The derivatives through A (dual LMs) and of
 // the element-domain D depend on the slave element alone: a per-element
 // kernel pushes the pair sums of O and the D term through A = Dh Me^-1 and
 // the element integrals in forward mode over the 12 slave coordinates.  Rows
@@ -33,8 +37,6 @@ namespace {
 constexpr int kTanWarps = 4;
 constexpr int kTanThreads = 32 * kTanWarps;
 constexpr int kThreads = 128;
-// map-coefficient adjoints of 4 seeds per thread, then 32 exchange slots per warp
-constexpr size_t kTanSmem = sizeof(double) * 16 * 4 * kTanThreads + 32 * kTanWarps * 28 * sizeof(double);
 
 struct TanArgs {
   const int32_t* ps;
@@ -55,13 +57,39 @@ struct TanArgs {
 };
 
 // Quadrature-point data one lane computes and the other two lanes of its
-// pair group read (shared memory): back-projections, shape-function state of
-// both sides and both inverse Jacobians.
+// pair group read (shared memory), what does not depend on the component:
+// back-projections and their products, and W J_s^-1, -W J_m^-1 with the
+// seeds' scale (a quarter on quad4 slaves).
 struct GPX {
-  double xs1, xs2, xm1, xm2;
-  double sN[4], sq[4], mN[4], mq[4];
+  double s1, s2, s12, m1, m2, m12;
   double a[4], b[4];
+  double s11, s22, s122, s112;
 };
+
+// One value in the basis (1, xi, eta, xi eta) of an element
+template <int NEN>
+__device__ __forceinline__ double mono_value(const double* y, double x1, double x2, double x12) {
+  const double v = fma(y[2], x2, fma(y[1], x1, y[0]));
+  return NEN == 4 ? fma(y[3], x12, v) : v;
+}
+template <int NEN>
+__device__ __forceinline__ void mono_grad(const double* y, double x1, double x2, double& g0, double& g1) {
+  g0 = NEN == 4 ? fma(y[3], x2, y[1]) : y[1];
+  g1 = NEN == 4 ? fma(y[3], x1, y[2]) : y[2];
+}
+
+// Accumulators of a thread (shared memory).  Slave side, element D: moments of
+// su_1, su_2 = W J_s^-T e_1, e_2 times Z, with (1, xi, eta, xi eta) and, on
+// quad4, (eta^2, xi eta^2) for su_1, (xi^2, xi^2 eta) for su_2, from which the
+// map adjoints of all seeds follow (grad xi eta = eta e_1 + xi e_2); segment D:
+// the map adjoints themselves.  Then the master map adjoints.
+template <int NS, bool SEG>
+constexpr int kSlaveSums = SEG ? 8 * NS : (NS == 4 ? 24 : 12);
+template <int NS, int NM, bool SEG>
+constexpr int kTanSums = kSlaveSums<NS, SEG> + (NM == 4 ? 8 : 6) * NS;
+// the sums of every thread, then 32 exchange slots per warp
+template <int NS, int NM, bool SEG>
+constexpr size_t kTanSmem = sizeof(double) * kTanSums<NS, NM, SEG> * kTanThreads + sizeof(GPX) * kTanThreads;
 
 // Pair p, component cp, for the lanes of one pair group (lanes 3g, 3g + 1,
 // 3g + 2 hold components 0, 1, 2 of the same pair).  Every lane of the warp
@@ -78,8 +106,13 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
   const int32_t* cs = g.conn_s + (int64_t)NS * s;
   const int32_t* cm = g.conn_m + (int64_t)NM * m;
   double yS[4] = {0, 0, 0, 0}, yM[4] = {0, 0, 0, 0};
-  for (int a = 0; a < NS; ++a) yS[a] = g.ys[3 * (int64_t)cs[a] + cp];
-  for (int l = 0; l < NM; ++l) yM[l] = g.ym[3 * (int64_t)cm[l] + cp];
+  {   // monomial coefficients of the held fields
+    double y[4] = {0, 0, 0, 0};
+    for (int a = 0; a < NS; ++a) y[a] = g.ys[3 * (int64_t)cs[a] + cp];
+    if (SEG) nodal_to_mono<NS>(y, yS);
+    for (int l = 0; l < NM; ++l) y[l] = g.ym[3 * (int64_t)cm[l] + cp];
+    nodal_to_mono<NM>(y, yM);
+  }
   const V3 x0 = v3(r[SR_X0], r[SR_X0 + 1], r[SR_X0 + 2]);
   const V3 t1 = v3(r[SR_T1], r[SR_T1 + 1], r[SR_T1 + 2]);
   const V3 t2 = v3(r[SR_T2], r[SR_T2 + 1], r[SR_T2 + 2]);
@@ -128,7 +161,8 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
     ncell = nr;
   }
   if (!live) ncell = 0;
-  for (int i = 0; i < 16 * NS; ++i) acc[i * kTanThreads] = 0.0;
+  constexpr int KS = kSlaveSums<NS, SEG>, KM = NM == 4 ? 8 : 6;   // master sums per seed
+  for (int i = 0; i < KS + KM * NS; ++i) acc[i * kTanThreads] = 0.0;
   double O[4] = {0, 0, 0, 0}, cbu[4] = {0, 0, 0, 0}, cbv[4] = {0, 0, 0, 0};
   const int ncell_w = __reduce_max_sync(0xffffffffu, ncell);
   const int gbase = 3 * (lane / 3);
@@ -159,23 +193,24 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
       if (cell_ok && qo < 7) {
         double l1, l2, w;
         tri7_point(qo, l1, l2, w);
+        if (NS == 4) w *= 0.25;
+        const double W = w * area;
         const double xu = au + l1 * e1u + l2 * e2u;
         const double xv = av + l1 * e1v + l2 * e2v;
         GPX& o = gx[lane];
-        double xs1, xs2, xm1, xm2;
+        double xs1, xs2, xm1, xm2, a00, a01, a10, a11;
         if (!si.solve(xu, xv, xs1, xs2)) newton_fail++;
         if (!mi.solve(xu, xv, xm1, xm2)) newton_fail++;
-        ShapeAD<NS> SA;
-        ShapeAD<NM> MA;
-        SA.eval(xs1, xs2);
-        MA.eval(xm1, xm2);
-        o.xs1 = xs1; o.xs2 = xs2; o.xm1 = xm1; o.xm2 = xm2;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) { o.sN[k] = SA.N[k]; o.mN[k] = MA.N[k]; }
-        o.sq[0] = SA.qa; o.sq[1] = SA.qb; o.sq[2] = SA.qc; o.sq[3] = SA.qd;
-        o.mq[0] = MA.qa; o.mq[1] = MA.qb; o.mq[2] = MA.qc; o.mq[3] = MA.qd;
-        si.jinv(xs1, xs2, o.a[0], o.a[1], o.a[2], o.a[3]);
-        mi.jinv(xm1, xm2, o.b[0], o.b[1], o.b[2], o.b[3]);
+        o.s1 = xs1; o.s2 = xs2; o.s12 = xs1 * xs2;
+        o.m1 = xm1; o.m2 = xm2; o.m12 = xm1 * xm2;
+        si.jinv(xs1, xs2, a00, a01, a10, a11);
+        o.a[0] = W * a00; o.a[1] = W * a01; o.a[2] = W * a10; o.a[3] = W * a11;
+        mi.jinv(xm1, xm2, a00, a01, a10, a11);
+        o.b[0] = -W * a00; o.b[1] = -W * a01; o.b[2] = -W * a10; o.b[3] = -W * a11;
+        if (NS == 4 && !SEG) {
+          o.s11 = xs1 * xs1; o.s22 = xs2 * xs2;
+          o.s122 = o.s12 * xs2; o.s112 = o.s12 * xs1;
+        }
       }
       __syncwarp();
 #pragma unroll 1
@@ -185,74 +220,68 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
         const GPX& x = gx[gbase + jj];
         double l1, l2, w;
         tri7_point(q, l1, l2, w);
-        const double W = w * area;
-        const double xs1 = x.xs1, xs2 = x.xs2, xm1 = x.xm1, xm2 = x.xm2;
-        ShapeAD<NS> SA;
-        ShapeAD<NM> MA;
+        const double s1 = x.s1, s2 = x.s2, s12 = x.s12, m1 = x.m1, m2 = x.m2, m12 = x.m12;
+        double Z = -mono_value<NM>(yM, m1, m2, m12);
+        if (SEG) Z += mono_value<NS>(yS, s1, s2, s12);
+        const double wZ = (NS == 4 ? 0.25 * w : w) * Z;
+        arb[0] += wZ;
+        arb[1] = fma(wZ, s1, arb[1]);
+        arb[2] = fma(wZ, s2, arb[2]);
+        if (NS == 4) arb[3] = fma(wZ, s12, arb[3]);
+        // J_m^-T (adjoint of xi_m) of the seed 1
+        double g0, g1;
+        mono_grad<NM>(yM, m1, m2, g0, g1);
+        double tu[4], tv[4], su[4], sv[4];   // master and slave point adjoints of the seeds 1, xi, eta, xi eta
+        tu[0] = fma(x.b[0], g0, x.b[2] * g1);
+        tv[0] = fma(x.b[1], g0, x.b[3] * g1);
+        tu[1] = s1 * tu[0]; tv[1] = s1 * tv[0];
+        tu[2] = s2 * tu[0]; tv[2] = s2 * tv[0];
+        if (NS == 4) { tu[3] = s12 * tu[0]; tv[3] = s12 * tv[0]; }
+        su[0] = 0.0; sv[0] = 0.0;
+        su[1] = x.a[0] * Z; sv[1] = x.a[1] * Z;
+        su[2] = x.a[2] * Z; sv[2] = x.a[3] * Z;
+        if (NS == 4) {
+          su[3] = fma(s2, su[1], s1 * su[2]);
+          sv[3] = fma(s2, sv[1], s1 * sv[2]);
+        }
+        auto add = [&](int i, double f, double v) { acc[i * kTanThreads] = fma(f, v, acc[i * kTanThreads]); };
+        if constexpr (SEG) {
+          mono_grad<NS>(yS, s1, s2, g0, g1);
+          const double gu = fma(x.a[0], g0, x.a[2] * g1), gv = fma(x.a[1], g0, x.a[3] * g1);
+          su[0] = gu; sv[0] = gv;
+          su[1] = fma(s1, gu, su[1]); sv[1] = fma(s1, gv, sv[1]);
+          su[2] = fma(s2, gu, su[2]); sv[2] = fma(s2, gv, sv[2]);
+          if (NS == 4) { su[3] = fma(s12, gu, su[3]); sv[3] = fma(s12, gv, sv[3]); }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) { SA.N[k] = x.sN[k]; MA.N[k] = x.mN[k]; }
-        SA.qa = x.sq[0]; SA.qb = x.sq[1]; SA.qc = x.sq[2]; SA.qd = x.sq[3];
-        MA.qa = x.mq[0]; MA.qb = x.mq[1]; MA.qc = x.mq[2]; MA.qd = x.mq[3];
-        double Z = 0.0;
-        if (SEG)
-#pragma unroll
-          for (int b = 0; b < NS; ++b) Z = fma(SA.N[b], yS[b], Z);
-#pragma unroll
-        for (int l = 0; l < NM; ++l) Z = fma(-MA.N[l], yM[l], Z);
-        // gradients in the plane: J_s^-T grad_xi N_e, J^-T grad_xi of the interpolated y
-        const double a00 = x.a[0], a01 = x.a[1], a10 = x.a[2], a11 = x.a[3];
-        double dx[4], de[4];
-        if constexpr (NS == 4) {
-          dx[0] = -SA.qc; dx[1] = SA.qc; dx[2] = SA.qd; dx[3] = -SA.qd;
-          de[0] = -SA.qa; de[1] = -SA.qb; de[2] = SA.qb; de[3] = SA.qa;
+          for (int e = 0; e < NS; ++e) {
+            add(8 * e + 0, 1.0, su[e]); add(8 * e + 1, 1.0, sv[e]);
+            add(8 * e + 2, s1, su[e]); add(8 * e + 3, s1, sv[e]);
+            add(8 * e + 4, s2, su[e]); add(8 * e + 5, s2, sv[e]);
+            if (NS == 4) { add(8 * e + 6, s12, su[e]); add(8 * e + 7, s12, sv[e]); }
+          }
         } else {
-          dx[0] = -1.0; dx[1] = 1.0; dx[2] = 0.0; dx[3] = 0.0;
-          de[0] = -1.0; de[1] = 0.0; de[2] = 1.0; de[3] = 0.0;
-        }
-        // gu_e = J_s^-T grad N_e = (a00 dx_e + a10 de_e, a01 dx_e + a11 de_e) enters
-        // only scaled by W Z (and, segment mode, through sum_e yS_e gu_e): the
-        // scale is folded into the coefficients once per point
-        const double WZ = W * Z, wZ = w * Z;
-        const double p00 = WZ * a00, p10 = WZ * a10, p01 = WZ * a01, p11 = WZ * a11;
-        double WgYsu = 0.0, WgYsv = 0.0;
-        if (SEG) {
-          double sdx = 0.0, sde = 0.0;
 #pragma unroll
-          for (int e = 0; e < NS; ++e) { sdx = fma(yS[e], dx[e], sdx); sde = fma(yS[e], de[e], sde); }
-          WgYsu = W * fma(a00, sdx, a10 * sde);
-          WgYsv = W * fma(a01, sdx, a11 * sde);
+          for (int e = 1; e < 3; ++e) {
+            constexpr int N = NS == 4 ? 12 : 6;
+            const int o = N * (e - 1);
+            add(o + 0, 1.0, su[e]); add(o + 1, 1.0, sv[e]);
+            add(o + 2, s1, su[e]); add(o + 3, s1, sv[e]);
+            add(o + 4, s2, su[e]); add(o + 5, s2, sv[e]);
+            if (NS == 4) {
+              add(o + 6, s12, su[e]); add(o + 7, s12, sv[e]);
+              add(o + 8, e == 1 ? x.s22 : x.s11, su[e]); add(o + 9, e == 1 ? x.s22 : x.s11, sv[e]);
+              add(o + 10, e == 1 ? x.s122 : x.s112, su[e]); add(o + 11, e == 1 ? x.s122 : x.s112, sv[e]);
+            }
+          }
         }
-        double ym0, ym1;
-        MA.pull(yM, ym0, ym1);
-        const double b00 = x.b[0], b01 = x.b[1], b10 = x.b[2], b11 = x.b[3];
-        const double mWu = -W * fma(b00, ym0, b10 * ym1), mWv = -W * fma(b01, ym0, b11 * ym1);
-        const double s12 = xs1 * xs2, m12 = xm1 * xm2;
 #pragma unroll
         for (int e = 0; e < NS; ++e) {
-          const double ne = SA.N[e];
-          O[e] = fma(ne, WZ, O[e]);
-          arb[e] = fma(wZ, ne, arb[e]);
-          double su = fma(p00, dx[e], p10 * de[e]), sv = fma(p01, dx[e], p11 * de[e]);   // J_s^-T (adjoint of xi_s)
-          if (SEG) { su = fma(ne, WgYsu, su); sv = fma(ne, WgYsv, sv); }
-          const double tu = ne * mWu, tv = ne * mWv;   // J_m^-T (adjoint of xi_m)
-          double* A = acc + (16 * e) * kTanThreads;
-          A[0 * kTanThreads] -= su;
-          A[1 * kTanThreads] -= sv;
-          A[2 * kTanThreads] = fma(-xs1, su, A[2 * kTanThreads]);
-          A[3 * kTanThreads] = fma(-xs1, sv, A[3 * kTanThreads]);
-          A[4 * kTanThreads] = fma(-xs2, su, A[4 * kTanThreads]);
-          A[5 * kTanThreads] = fma(-xs2, sv, A[5 * kTanThreads]);
-          A[6 * kTanThreads] = fma(-s12, su, A[6 * kTanThreads]);
-          A[7 * kTanThreads] = fma(-s12, sv, A[7 * kTanThreads]);
-          A[8 * kTanThreads] -= tu;
-          A[9 * kTanThreads] -= tv;
-          A[10 * kTanThreads] = fma(-xm1, tu, A[10 * kTanThreads]);
-          A[11 * kTanThreads] = fma(-xm1, tv, A[11 * kTanThreads]);
-          A[12 * kTanThreads] = fma(-xm2, tu, A[12 * kTanThreads]);
-          A[13 * kTanThreads] = fma(-xm2, tv, A[13 * kTanThreads]);
-          A[14 * kTanThreads] = fma(-m12, tu, A[14 * kTanThreads]);
-          A[15 * kTanThreads] = fma(-m12, tv, A[15 * kTanThreads]);
-          const double xbu = su + tu, xbv = sv + tv;
+          const int o = KS + KM * e;
+          add(o + 0, 1.0, tu[e]); add(o + 1, 1.0, tv[e]);
+          add(o + 2, m1, tu[e]); add(o + 3, m1, tv[e]);
+          add(o + 4, m2, tu[e]); add(o + 5, m2, tv[e]);
+          if (NM == 4) { add(o + 6, m12, tu[e]); add(o + 7, m12, tv[e]); }
+          const double xbu = e == 0 && !SEG ? tu[e] : su[e] + tu[e], xbv = e == 0 && !SEG ? tv[e] : sv[e] + tv[e];
           xbu_c[e] += xbu; xbv_c[e] += xbv;
           e1bu[e] = fma(l1, xbu, e1bu[e]); e1bv[e] = fma(l1, xbv, e1bv[e]);
           e2bu[e] = fma(l2, xbu, e2bu[e]); e2bv[e] = fma(l2, xbv, e2bv[e]);
@@ -263,6 +292,7 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
     if (cell_ok) {
 #pragma unroll
       for (int e = 0; e < NS; ++e) {   // area = |cross| / 2, cell vertices, centroid
+        O[e] = fma(area, arb[e], O[e]);
         const double crb = 0.5 * (crs < 0.0 ? -arb[e] : arb[e]);
         e1bu[e] += crb * e2v; e1bv[e] -= crb * e2u;
         e2bu[e] -= crb * e1v; e2bv[e] += crb * e1u;
@@ -307,49 +337,79 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
     const int64_t n = cm[l];
     Y[l] = v3(g.xm[3 * n], g.xm[3 * n + 1], g.xm[3 * n + 2]);
   }
-  double Ks[DUAL ? 4 : 1][24];   // seed rows, combined through A at the end (dual LMs)
+  const PlaneBasis<NS> basis(X, t1, t2, n0);
+  double Ks[NS][24];   // rows of the seeds 1, xi, eta, xi eta (a quarter of them on quad4)
+#pragma unroll 1
   for (int e = 0; e < NS; ++e) {
     double sbu[4] = {0, 0, 0, 0}, sbv[4] = {0, 0, 0, 0}, mbu[4] = {0, 0, 0, 0}, mbv[4] = {0, 0, 0, 0};
     clip.reverse(r, Rbu[e], Rbv[e], srev, mrev, sbu, sbv, mbu, mbv);
-    double smb[8], mmb[8];
+    double smb[8], mmb[8];   // map adjoints: minus the sums
+    auto sum = [&](int i) { return acc[i * kTanThreads]; };
     for (int k = 0; k < 8; ++k) {
-      smb[k] = acc[(16 * e + k) * kTanThreads];
-      mmb[k] = acc[(16 * e + 8 + k) * kTanThreads];
+      const int c = k & 1;
+      if constexpr (SEG) {
+        smb[k] = NS == 4 || k < 6 ? -sum(8 * e + k) : 0.0;
+      } else if constexpr (NS == 3) {
+        smb[k] = e > 0 && k < 6 ? -sum(6 * (e - 1) + k) : 0.0;
+      } else {
+        if (e == 0) smb[k] = 0.0;
+        else if (e < 3) smb[k] = -sum(12 * (e - 1) + k);
+        else   // eta su_1 + xi su_2 with 1, xi, eta, xi eta
+          smb[k] = -(sum((k < 2 ? 4 : (k < 4 ? 6 : (k < 6 ? 8 : 10))) + c) +
+                     sum(12 + (k < 2 ? 2 : (k < 4 ? 8 : (k < 6 ? 6 : 10))) + c));
+      }
+      mmb[k] = k < KM ? -sum(KS + KM * e + k) : 0.0;
     }
     map_coeff_reverse<NS>(smb, sbu, sbv);
     map_coeff_reverse<NM>(mmb, mbu, mbv);
     double gX[4][3], gY[4][3];
     for (int a = 0; a < 4; ++a)
       for (int d = 0; d < 3; ++d) { gX[a][d] = 0.0; gY[a][d] = 0.0; }
-    plane_reverse<NS, NM>(X, Y, x0, t1, t2, n0, sbu, sbv, mbu, mbv, gX, gY);
-    if (DUAL) {
-      for (int a = 0; a < 4; ++a)
-        for (int d = 0; d < 3; ++d) {
-          Ks[DUAL ? e : 0][3 * a + d] = gX[a][d];
-          Ks[DUAL ? e : 0][12 + 3 * a + d] = gY[a][d];
-        }
-    } else {   // standard LMs: seed e is row e
-      for (int a = 0; a < 4; ++a)
-        for (int d = 0; d < 3; ++d) {
-          __stcs(kout + 72 * e + 3 * a + d, gX[a][d]);
-          __stcs(kout + 72 * e + 12 + 3 * a + d, gY[a][d]);
-        }
+    PlaneBar pb{v3(0, 0, 0), v3(0, 0, 0), v3(0, 0, 0)};
+    project_reverse<NS>(X, x0, t1, t2, sbu, sbv, gX, pb);
+    project_reverse<NM>(Y, x0, t1, t2, mbu, mbv, gY, pb);
+    basis.reverse(pb, gX);
+    for (int a = 0; a < 4; ++a)
+      for (int d = 0; d < 3; ++d) {
+        Ks[e][3 * a + d] = gX[a][d];
+        Ks[e][12 + 3 * a + d] = gY[a][d];
+      }
+  }
+  // N_e from the seeds: corners (-1,-1), (1,-1), (1,1), (-1,1) of quad4; (1 - xi - eta, xi, eta) of tri3
+  auto nodal = [&](const double* f, double* out) {
+    if constexpr (NS == 4) {
+      const double a = f[0] - f[2], b = f[1] - f[3], d = f[0] + f[2], e = f[1] + f[3];
+      out[0] = a - b; out[1] = a + b; out[2] = d + e; out[3] = d - e;
+    } else {
+      out[0] = f[0] - f[1] - f[2]; out[1] = f[1]; out[2] = f[2]; out[3] = 0.0;
     }
+  };
+  double AT[4][4];   // dual: rows of A in the seeds
+  if (DUAL)
+    for (int a = 0; a < NS; ++a) {
+      double v[4];
+      for (int e = 0; e < NS; ++e) v[e] = (NS == 4 ? 4.0 : 1.0) * r[SR_A + 4 * a + e];
+      nodal_to_mono<NS>(v, AT[a]);
+    }
+  for (int k = 0; k < 24; ++k) {
+    double f[4], row[4];
+    for (int e = 0; e < NS; ++e) f[e] = Ks[e][k];
+    if (DUAL) {
+      for (int a = 0; a < NS; ++a) {
+        double v = 0.0;
+        for (int e = 0; e < NS; ++e) v = fma(AT[a][e], f[e], v);
+        row[a] = v;
+      }
+    } else {
+      nodal(f, row);
+    }
+    for (int a = 0; a < 4; ++a) __stcs(kout + 72 * a + k, a < NS ? row[a] : 0.0);
   }
   if (DUAL) {
-    for (int a = 0; a < 4; ++a)
-      for (int k = 0; k < 24; ++k) {
-        double v = 0.0;
-        if (a < NS)
-          for (int e = 0; e < NS; ++e) v = fma(r[SR_A + 4 * a + e], Ks[e][k], v);
-        __stcs(kout + 72 * a + k, v);
-      }
-  } else {
-    for (int a = NS; a < 4; ++a)
-      for (int k = 0; k < 24; ++k) __stcs(kout + 72 * a + k, 0.0);
+    double On[4];
+    nodal(O, On);
+    for (int e = 0; e < 4; ++e) __stcs(g.Op + 12 * p + 3 * e + cp, e < NS ? On[e] : 0.0);
   }
-  if (DUAL)
-    for (int e = 0; e < 4; ++e) __stcs(g.Op + 12 * p + 3 * e + cp, e < NS ? O[e] : 0.0);
 }
 
 // Persistent kernel over warp batches of 32 R pairs, each sorted by the cell
@@ -371,7 +431,7 @@ __global__ void __launch_bounds__(kTanThreads) k_tangent_pairs(TanArgs g) {
   const bool ok = st->over_pairs == 0 && st->over_bins == 0;
   const int64_t n = ok ? (int64_t)min((unsigned long long)g.pair_cap, st->n_pairs) : 0;
   const int64_t items = (n + B - 1) / B;
-  GPX* gx = reinterpret_cast<GPX*>(tan_acc + 16 * 4 * kTanThreads) + 32 * (threadIdx.x >> 5);
+  GPX* gx = reinterpret_cast<GPX*>(tan_acc + kTanSums<NS, NM, SEG> * kTanThreads) + 32 * (threadIdx.x >> 5);
   const Watchdog wd(g.watchdog_us);
   for (;;) {   // bounded: the shared counter only grows
     if (wd.expired(&st->timeout)) break;
@@ -833,11 +893,11 @@ void launch_pairs_t(mortar_ctx* c) {
             c->tan_pair_cap, c->dstat.as<DevStatus>(), c->watchdog_us};
   // batches of 160 pairs: 16 full rounds of 10 pair groups (lanes 30, 31 idle)
   auto kern = k_tangent_pairs<NS, NM, SEG, DUAL, 5>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTanSmem);
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTanSmem<NS, NM, SEG>);
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTanThreads, kTanSmem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTanThreads, kTanSmem<NS, NM, SEG>);
   if (per_sm < 1) per_sm = 1;
-  kern<<<(unsigned)(c->n_sm * per_sm), kTanThreads, kTanSmem, c->stream>>>(g);
+  kern<<<(unsigned)(c->n_sm * per_sm), kTanThreads, kTanSmem<NS, NM, SEG>, c->stream>>>(g);
 }
 
 template <int NS, int NM, bool SEG, bool DUAL, bool ELEMD>

@@ -516,67 +516,66 @@ __device__ __forceinline__ void project_reverse(const V3* P, V3 x0, V3 t1, V3 t2
 
 // Reverse of the auxiliary plane (x0 = element centre, n0 = unit normal there,
 // t1 = normalised projected first edge, t2 = n0 x t1) as a function of the slave
-// nodes X; ADDED to gX.
+// nodes X: what several reverse sweeps of one element share (the square roots
+// and divisions), and one sweep, ADDED to gX.
+template <int NS>
+struct PlaneBasis {
+  V3 t1, t2, n0, g1, g2, ed;
+  double iln, ile, en;
+  __device__ __forceinline__ PlaneBasis(const V3* X, V3 t1_, V3 t2_, V3 n0_) : t1(t1_), t2(t2_), n0(n0_) {
+    if constexpr (NS == 4) {
+      g1 = 0.25 * ((X[1] - X[0]) + (X[2] - X[3]));
+      g2 = 0.25 * ((X[2] - X[1]) + (X[3] - X[0]));
+    } else {
+      g1 = X[1] - X[0];
+      g2 = X[2] - X[0];
+    }
+    const V3 nn = cross(g1, g2);
+    iln = 1.0 / sqrt(dot(nn, nn));
+    ed = X[1] - X[0];
+    en = dot(ed, n0);
+    const V3 ep = ed - en * n0;
+    ile = 1.0 / sqrt(dot(ep, ep));
+  }
+  __device__ __forceinline__ void reverse(const PlaneBar& pb, double gX[4][3]) const {
+    const V3 x0b = pb.x0, t2b = pb.t2;
+    V3 t1b = pb.t1;
+    V3 n0b = cross(t1, t2b);   // t2 = n0 x t1
+    t1b = t1b + cross(t2b, n0);
+    const V3 epb = ile * (t1b - dot(t1, t1b) * t1);
+    V3 edb = epb;
+    const double enb = -dot(epb, n0);
+    n0b = n0b - en * epb;
+    edb = edb + enb * n0;
+    n0b = n0b + enb * ed;
+    const V3 nb = iln * (n0b - dot(n0, n0b) * n0);
+    const V3 g1b = cross(g2, nb), g2b = cross(nb, g1);
+    V3 Xb[4];
+    for (int a = 0; a < 4; ++a) Xb[a] = v3(0, 0, 0);
+    Xb[1] = Xb[1] + edb;
+    Xb[0] = Xb[0] - edb;
+    if constexpr (NS == 4) {
+      const V3 a1 = 0.25 * g1b, a2 = 0.25 * g2b, ax = 0.25 * x0b;
+      Xb[0] = Xb[0] - a1 - a2 + ax;
+      Xb[1] = Xb[1] + a1 - a2 + ax;
+      Xb[2] = Xb[2] + a1 + a2 + ax;
+      Xb[3] = Xb[3] - a1 + a2 + ax;
+    } else {
+      const V3 ax = (1.0 / 3.0) * x0b;
+      Xb[0] = Xb[0] - g1b - g2b + ax;
+      Xb[1] = Xb[1] + g1b + ax;
+      Xb[2] = Xb[2] + g2b + ax;
+    }
+    for (int a = 0; a < NS; ++a) {
+      gX[a][0] += Xb[a].x; gX[a][1] += Xb[a].y; gX[a][2] += Xb[a].z;
+    }
+  }
+};
+
 template <int NS>
 __device__ __forceinline__ void plane_basis_reverse(const V3* X, V3 t1, V3 t2, V3 n0, const PlaneBar& pb,
                                                     double gX[4][3]) {
-  const V3 x0b = pb.x0, t2b = pb.t2;
-  V3 t1b = pb.t1;
-  V3 g1, g2;
-  if constexpr (NS == 4) {
-    g1 = 0.25 * ((X[1] - X[0]) + (X[2] - X[3]));
-    g2 = 0.25 * ((X[2] - X[1]) + (X[3] - X[0]));
-  } else {
-    g1 = X[1] - X[0];
-    g2 = X[2] - X[0];
-  }
-  const V3 nn = cross(g1, g2);
-  const double ln = sqrt(dot(nn, nn));
-  const V3 ed = X[1] - X[0];
-  const double en = dot(ed, n0);
-  const V3 ep = ed - en * n0;
-  const double le = sqrt(dot(ep, ep));
-  V3 n0b = cross(t1, t2b);   // t2 = n0 x t1
-  t1b = t1b + cross(t2b, n0);
-  const V3 epb = (1.0 / le) * (t1b - dot(t1, t1b) * t1);
-  V3 edb = epb;
-  const double enb = -dot(epb, n0);
-  n0b = n0b - en * epb;
-  edb = edb + enb * n0;
-  n0b = n0b + enb * ed;
-  const V3 nb = (1.0 / ln) * (n0b - dot(n0, n0b) * n0);
-  const V3 g1b = cross(g2, nb), g2b = cross(nb, g1);
-  V3 Xb[4];
-  for (int a = 0; a < 4; ++a) Xb[a] = v3(0, 0, 0);
-  Xb[1] = Xb[1] + edb;
-  Xb[0] = Xb[0] - edb;
-  if constexpr (NS == 4) {
-    const V3 a1 = 0.25 * g1b, a2 = 0.25 * g2b, ax = 0.25 * x0b;
-    Xb[0] = Xb[0] - a1 - a2 + ax;
-    Xb[1] = Xb[1] + a1 - a2 + ax;
-    Xb[2] = Xb[2] + a1 + a2 + ax;
-    Xb[3] = Xb[3] - a1 + a2 + ax;
-  } else {
-    const V3 ax = (1.0 / 3.0) * x0b;
-    Xb[0] = Xb[0] - g1b - g2b + ax;
-    Xb[1] = Xb[1] + g1b + ax;
-    Xb[2] = Xb[2] + g2b + ax;
-  }
-  for (int a = 0; a < NS; ++a) {
-    gX[a][0] += Xb[a].x; gX[a][1] += Xb[a].y; gX[a][2] += Xb[a].z;
-  }
-}
-
-// Both: in-plane node adjoints (sbu, sbv, mbu, mbv) in; 3D coordinate adjoints
-// ADDED to gX (slave) and gY (master).
-template <int NS, int NM>
-__device__ __forceinline__ void plane_reverse(const V3* X, const V3* Y, V3 x0, V3 t1, V3 t2, V3 n0,
-                                              const double* sbu, const double* sbv, const double* mbu,
-                                              const double* mbv, double gX[4][3], double gY[4][3]) {
-  PlaneBar pb{v3(0, 0, 0), v3(0, 0, 0), v3(0, 0, 0)};
-  project_reverse<NS>(X, x0, t1, t2, sbu, sbv, gX, pb);
-  project_reverse<NM>(Y, x0, t1, t2, mbu, mbv, gY, pb);
-  plane_basis_reverse<NS>(X, t1, t2, n0, pb, gX);
+  PlaneBasis<NS>(X, t1, t2, n0).reverse(pb, gX);
 }
 
 // Monomial form of the element shape functions, N(xi) = T m(xi): quad4
@@ -587,10 +586,10 @@ __device__ __forceinline__ void plane_reverse(const V3* X, const V3* Y, V3 x0, V
 // quadrature point evaluates without forming N.
 
 // out_i = sum_a T[a][i] in_a: monomial coefficients of the nodal field `in`.
-template <int NEN>
-__device__ __forceinline__ void nodal_to_mono(const V3* in, V3* out) {
+template <int NEN, class T>
+__device__ __forceinline__ void nodal_to_mono(const T* in, T* out) {
   if constexpr (NEN == 4) {
-    const V3 s02 = in[0] + in[2], s13 = in[1] + in[3], d20 = in[2] - in[0], d13 = in[1] - in[3];
+    const T s02 = in[0] + in[2], s13 = in[1] + in[3], d20 = in[2] - in[0], d13 = in[1] - in[3];
     out[0] = 0.25 * (s02 + s13);
     out[1] = 0.25 * (d20 + d13);
     out[2] = 0.25 * (d20 - d13);
