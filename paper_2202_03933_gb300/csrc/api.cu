@@ -118,6 +118,8 @@ int alloc_pair_buffers(mortar_ctx* c, int64_t cap) {
     const size_t chunk = std::min<size_t>(quadratic_slave(c) ? 4 * n : n, kPairChunk);
     MORTAR_TRY(buf_reserve(c->rec, (chunk + 31) / 32 * kRecordGroupBytes));
     MORTAR_TRY(buf_reserve(c->order, chunk * 4));
+  } else {   // element-based: no records, only the staged candidates and rows
+    MORTAR_TRY(buf_reserve(c->rec, n * 48));
   }
   c->pair_cap = cap;
   return MORTAR_OK;

@@ -83,6 +83,7 @@ struct DevStatus {
   unsigned long long nnzb_K;       // 3x3 blocks of the linearisation
   unsigned long long over_K;       // linearisation block buffer too small
   unsigned long long nonfinite;    // elements with a non-finite node coordinate
+  unsigned long long stage_ctr[2]; // entries staged by the candidate and the row kernel
   unsigned long long pair_ctr[4];  // work counters of a chunk's sort, clip, quadrature and finish kernels
   double J;
 };

@@ -12,6 +12,7 @@
 // Topology (node -> element adjacency of each side) is built once per
 // interface with a counting sort plus a per-node sort of the short lists.
 #include "context.h"
+#include "staging.cuh"
 
 namespace mortar {
 
@@ -155,52 +156,74 @@ __device__ int row_slow(const Src& src, int64_t j, int64_t out, int32_t* __restr
 }
 
 // One thread per slave node (row): both D and M.  MODE 0 counts the unique
-// columns of each row, MODE 1 writes the rows.
+// columns of each row and stages the rows; MODE 1 writes them, by a contiguous
+// copy of the block's staged rows where it has them.
+// Visiting a row (gathering 50 to 100 entries into a sorted list in
+// thread-local memory) is what both passes used to cost: 1000x866 quads 0.73 +
+// 0.82 ms without staging, 0.87 + 0.10 ms with it.
 template <int MODE, class SrcD, class SrcM>
 __global__ void __launch_bounds__(kThreads) k_rows(SrcD srcD, SrcM srcM, int64_t N, int32_t* __restrict__ cntD,
                                                    int32_t* __restrict__ cntM, const int64_t* __restrict__ rpD,
                                                    const int64_t* __restrict__ rpM, int64_t capD, int64_t capM,
                                                    int32_t* __restrict__ colD, double* __restrict__ valD,
                                                    int32_t* __restrict__ colM, double* __restrict__ valM,
-                                                   DevStatus* st) {
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= N) return;
+                                                   Staging stage, DevStatus* st) {
+  const int64_t j0 = (int64_t)blockIdx.x * blockDim.x, j = j0 + threadIdx.x;
+  const bool has = j < N;
   if (st->over_pairs) {   // pair buffers incomplete: the run is repeated with larger ones
-    if (MODE == 0) { cntD[j] = 0; cntM[j] = 0; }
+    if (MODE == 0 && has) { cntD[j] = 0; cntM[j] = 0; }
     return;
   }
   if (MODE == 1 && (rpD[N] > capD || rpM[N] > capM)) {
     if (j == 0) atomicMax(&st->over_nnz, 1ull);
     return;
   }
-  {
-    RowAcc<32> acc;
-    srcD.visit(j, [&](int32_t c, double v) { acc.add(c, v); });
+  constexpr int64_t kEntry = sizeof(double) + sizeof(int32_t);
+  double* sval = reinterpret_cast<double*>(stage.data);
+  int32_t* scol = reinterpret_cast<int32_t*>(sval + stage.bytes / kEntry);
+  if (MODE == 1 && stage.base && stage.base[blockIdx.x] != kNotStaged) {
+    const int64_t j1 = min(j0 + (int64_t)blockDim.x, N), at = stage.base[blockIdx.x];
+    const int64_t outD = rpD[j0], nD = rpD[j1] - outD, outM = rpM[j0], nM = rpM[j1] - outM;
+    for (int64_t k = threadIdx.x; k < nD; k += blockDim.x) { colD[outD + k] = scol[at + k]; valD[outD + k] = sval[at + k]; }
+    for (int64_t k = threadIdx.x; k < nM; k += blockDim.x) {
+      colM[outM + k] = scol[at + nD + k];
+      valM[outM + k] = sval[at + nD + k];
+    }
+    return;
+  }
+  RowAcc<32> aD;
+  RowAcc<64> aM;
+  if (has) {
+    srcD.visit(j, [&](int32_t c, double v) { aD.add(c, v); });
+    srcM.visit(j, [&](int32_t c, double v) { aM.add(c, v); });
+  }
+  if (MODE == 0) {
+    const bool fits = !__syncthreads_or(aD.over || aM.over);
+    unsigned total;
+    const unsigned before = block_exclusive((unsigned)aD.u | (unsigned)aM.u << 16, total);   // sums below 2^13, 2^14
+    const int64_t nD = total & 0xffffu;
+    const long long at = stage_block(stage, fits, nD + (total >> 16), kEntry);
+    if (at != kNotStaged) {
+      const int64_t oD = at + (before & 0xffffu), oM = at + nD + (before >> 16);
+      for (int k = 0; k < aD.u; ++k) { scol[oD + k] = aD.col[k]; sval[oD + k] = aD.val[k]; }
+      for (int k = 0; k < aM.u; ++k) { scol[oM + k] = aM.col[k]; sval[oM + k] = aM.val[k]; }
+    }
+  }
+  if (!has) return;
+  auto finish = [&](auto& acc, auto& src, int32_t* cnt, const int64_t* rp, int32_t* col, double* val) {
     int u = acc.u;
-    const int64_t out = MODE == 1 ? rpD[j] : 0;
+    const int64_t out = MODE == 1 ? rp[j] : 0;
     if (!acc.over) {
       if (MODE == 1)
-        for (int k = 0; k < u; ++k) { colD[out + k] = acc.col[k]; valD[out + k] = acc.val[k]; }
+        for (int k = 0; k < u; ++k) { col[out + k] = acc.col[k]; val[out + k] = acc.val[k]; }
     } else {
       if (MODE == 0) atomicAdd(&st->row_slow, 1ull);
-      u = row_slow<MODE>(srcD, j, out, colD, valD);
+      u = row_slow<MODE>(src, j, out, col, val);
     }
-    if (MODE == 0) cntD[j] = u;
-  }
-  {
-    RowAcc<64> acc;
-    srcM.visit(j, [&](int32_t c, double v) { acc.add(c, v); });
-    int u = acc.u;
-    const int64_t out = MODE == 1 ? rpM[j] : 0;
-    if (!acc.over) {
-      if (MODE == 1)
-        for (int k = 0; k < u; ++k) { colM[out + k] = acc.col[k]; valM[out + k] = acc.val[k]; }
-    } else {
-      if (MODE == 0) atomicAdd(&st->row_slow, 1ull);
-      u = row_slow<MODE>(srcM, j, out, colM, valM);
-    }
-    if (MODE == 0) cntM[j] = u;
-  }
+    if (MODE == 0) cnt[j] = u;
+  };
+  finish(aD, srcD, cntD, rpD, colD, valD);
+  finish(aM, srcM, cntM, rpM, colM, valM);
 }
 
 __global__ void k_finalize(const int64_t* __restrict__ rpD, const int64_t* __restrict__ rpM, int64_t N,
@@ -224,16 +247,17 @@ void assemble_t(mortar_ctx* c, const double* blkD) {
   const unsigned g = (unsigned)((N + kThreads - 1) / kThreads);
   int32_t* cntD = c->row_cnt.as<int32_t>();
   int32_t* cntM = c->row_cnt2.as<int32_t>();
+  const Staging stage = staging_area(c->rec, g, &st->stage_ctr[1]);
   if (N > 0)
     k_rows<0><<<g, kThreads, 0, c->stream>>>(srcD, srcM, N, cntD, cntM, nullptr, nullptr, 0, 0, nullptr, nullptr,
-                                              nullptr, nullptr, st);
+                                              nullptr, nullptr, stage, st);
   launch_exclusive_scan_i32(cntD, c->rowptr_D.as<int64_t>(), nullptr, N, c->scan_tmp.as<int64_t>(), c->stream);
   launch_exclusive_scan_i32(cntM, c->rowptr_M.as<int64_t>(), nullptr, N, c->scan_tmp.as<int64_t>(), c->stream);
   if (N > 0)
     k_rows<1><<<g, kThreads, 0, c->stream>>>(srcD, srcM, N, nullptr, nullptr, c->rowptr_D.as<int64_t>(),
                                               c->rowptr_M.as<int64_t>(), c->nnz_cap_D, c->nnz_cap_M,
                                               c->col_D.as<int32_t>(), c->val_D.as<double>(), c->col_M.as<int32_t>(),
-                                              c->val_M.as<double>(), st);
+                                              c->val_M.as<double>(), stage, st);
 }
 
 template <int NS, int NM>
