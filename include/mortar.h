@@ -135,7 +135,7 @@ typedef struct mortar_stats {
    * adjoint = the remaining adjoint kernels, of which adjoint_pairs is the
    * separate per-pair reverse sweep (0 when fused). */
   float ms_search, ms_integrate, ms_assemble, ms_adjoint, ms_adjoint_pairs, ms_total;
-  /* CTA busy-time imbalance max/min of the batched pair kernel in the last run
+  /* CTA busy-time imbalance max/min of the clip kernel (first chunk of pairs) in the last run
    * (timing on; the measure eta_t of the paper's load-balancing trigger,
    * Sec. 4.4, taken over CTAs instead of processes); 0 if not measured */
   float eta_t;
@@ -302,10 +302,11 @@ int mortar_set_timing(mortar_ctx* ctx, int32_t enabled);
 int mortar_set_watchdog(mortar_ctx* ctx, int32_t watchdog_us);
 
 /* Launch shape of the pair kernels (used by the autotuner; 0 = default):
- * variant 0 = integration and adjoint in warp batches of up to 32 * rounds
- * pairs sorted by their clip's cell count and edge intersections (rounds 1,
- * 2, 4, 8, 16 or 32), variant 1 = one pair per thread; block_size = threads per block of either variant (a
- * multiple of 32 up to 256; default 128); chunk_pairs = pairs per
+ * variant 0 = integration and adjoint over pairs sorted by their clip's cell
+ * count and edge intersections in warp batches of up to 32 * rounds pairs (rounds 1,
+ * 2, 4, 8, 16 or 32), variant 1 = one pair per thread; block_size = threads per
+ * block (a multiple of 32 up to 256; default 128; of variant 0's clip and
+ * finish kernels, its other kernels have one shape); chunk_pairs = pairs per
  * work-counter fetch of variant 1 (default 32).  MORTAR_ERR_INVALID_ARG for
  * other values. */
 int mortar_set_launch(mortar_ctx* ctx, int32_t variant, int32_t block_size, int32_t chunk_pairs, int32_t rounds);

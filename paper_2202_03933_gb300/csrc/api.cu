@@ -177,7 +177,7 @@ void enqueue_run(mortar_ctx* c, const Phases& ph) {
     launch_candidates(c);
   }
   if (c->timing) record_event(c->ev[1], st);
-  // with the adjoint, the batched adjoint pair kernel also produces the
+  // with the adjoint, the default adjoint pair kernels also produce the
   // forward blocks (one pass over the pairs instead of two)
   const bool fused = ph.adjoint && ph.integrate && adjoint_fuses_forward(c);
   {
@@ -845,8 +845,8 @@ int mortar_autotune(mortar_ctx* c, const double* lambda, int32_t on_device, int3
     MORTAR_TRY(buf_reserve(c->lambda, (size_t)std::max<int64_t>(c->Ns, 1) * 24));
     MORTAR_TRY(copy_in(c->lambda.p, lambda, (size_t)c->Ns * 24, on_device, c->stream));
   }
-  // candidate launch shapes: the warp-batched kernels with 32 R pairs per
-  // warp batch (R = rounds 1, 2, 4, 8, 16, 32) and 2, 4 or 8 warps per block, and
+  // candidate launch shapes: the default kernels with 32 R pairs per sorted
+  // batch (R = rounds 1, 2, 4, 8, 16, 32) and 2, 4 or 8 warps per block, and
   // the one-pair-per-thread kernels with 64, 128 or 256 threads per block and
   // 32 or 128 pairs per work-counter fetch
   struct Cand { int32_t variant, rounds, block, chunk; };

@@ -38,10 +38,10 @@ struct mortar_ctx {
   int device = 0;
   int n_sm = 0;
   bool timing = false;
-  int32_t variant = 0;        // integration kernel: 0 batched + sorted (default), 1 one pair per thread
+  int32_t variant = 0;        // pair kernels: 0 sorted, fixed point (default), 1 one pair per thread, FP64
   int32_t block_size = 0;     // pair kernels (0 = default)
   int32_t chunk_pairs = 0;    // pairs per work item of the one-pair-per-thread kernels (0 = default)
-  int32_t rounds = 0;         // batched kernel: 32 * rounds pairs per warp batch (0 = default)
+  int32_t rounds = 0;         // sort kernel: 32 * rounds pairs per warp batch (0 = default)
   int32_t watchdog_us = 0;    // per-CTA time budget of the persistent pair kernels (0 = none)
 
   // ---- interface definition
@@ -81,7 +81,7 @@ struct mortar_ctx {
   int64_t nnz_cap_D = 0, nnz_cap_M = 0;
   mortar::DevBuf scan_tmp;                  // block partials of the scans
   mortar::DevBuf cta_t;                     // per-CTA busy intervals of the pair kernel (timing)
-  int pair_grid = 0;                        // CTAs of the last batched pair kernel (timing)
+  int pair_grid = 0;                        // CTAs of the clip kernel (timing)
   std::vector<unsigned long long> h_cta_t;
 
   // ---- adjoint workspaces
@@ -142,7 +142,7 @@ void launch_candidates(mortar_ctx* c);
 
 // k_integrate.cu
 void launch_integrate(mortar_ctx* c, const RunParams& rp);
-bool integrate_batched_fits(int rounds, int block);   // shared memory of the batched kernel fits
+bool integrate_batched_fits(int rounds, int block);   // shared memory of the sort kernel's batches fits
 int integrate_rounds(int rounds, int block);          // rounds the integration kernel uses for a setting
 
 // k_contact.cu

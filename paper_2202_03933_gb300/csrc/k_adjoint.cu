@@ -448,8 +448,9 @@ __device__ __forceinline__ void adjoint_empty(int64_t p, const FwdOut& fo) {
   __stcs(fo.flag + p, (uint8_t)0);
 }
 
-// ---------------------------------------------------------------- variant 0
-// Same functional, reorganised for the FP64 pipe:
+// ------------------------------------------------- variant 0, FP64 fallback
+// Pairs that do not fit the fixed-point frame.  Same functional, reorganised
+// for the FP64 pipe:
 //  * the per-point work is written in the monomial basis of the shape
 //    functions, N = T m with m = (1, xi, eta, xi eta) (quad4) or (1, xi, eta)
 //    (tri3).  With the monomial coefficients LM_i = sum_c T_s[c][i] Lambda_c,
@@ -464,13 +465,11 @@ __device__ __forceinline__ void adjoint_empty(int64_t p, const FwdOut& fo) {
 //    basis: non-negative terms keep small entries accurate) at the end:
 //      dJ/dY_l |direct = -sum_c G[c][l] Lambda_c,  dJ/dX_b |direct = sum_c H[c][b] Lambda_c,
 //      dJ/dLambda_c = sum_b H[c][b] X_b - sum_l G[c][l] Y_l,  J = sum_c Lambda_c . dJ/dLambda_c;
-//  * element maps are inverted as in the batched integration kernel (affine
-//    2x2 inverse, or FP32 Newton + one Newton step on the FP64 residual), and the
+//  * element maps are inverted with MapInverse (affine 2x2 inverse, or FP32
+//    Newton + one Newton step on the FP64 residual), and the
 //    implicit-function step applies the FP64 inverse Jacobian at the
 //    converged xi (MapInverse::jinvT);
-//  * the clip is recorded as a compact vertex pool (ClipPool);
-//  * a warp sorts its batch of pairs by the cell count and edge
-//    intersections of an FP32 clip before the sweep.
+//  * the clip is recorded as a compact vertex pool (ClipPool).
 template <int NS, int NM, bool SEG, bool DUAL>
 __device__ __noinline__ void adjoint_pair_fast(int64_t p, const int32_t* __restrict__ ps, const int32_t* __restrict__ pm,
                                   const double* __restrict__ srec, const double* __restrict__ xs,
@@ -792,9 +791,16 @@ __device__ __forceinline__ bool next_group(unsigned long long* ctr, int64_t n, i
   return 32 * g < n;
 }
 
-// First kernel of the default adjoint (variant 0; the forward blocks come with
-// it): FP64 clip with its record, the pair's bilinear forms CY [and SX], and
-// the conversion to fixed point.  One record per pair, in sorted order.
+// Variant 0 (default; the forward blocks come with it) is split like the
+// forward integration, where the work's character changes: k_pair_sort,
+// k_adjoint_clip, k_adjoint_cells, k_adjoint_finish, with a record per pair in
+// between (832 B, 960 B with segment D).  planar 600x520, dual (1.35 M pairs):
+// 0.25 + 1.1 + 4.3 + 1.2 ms against 14.5 to 16.8 ms (by batch size) of one FP64
+// kernel with the same sweep.
+//
+// First kernel: FP64 clip with its record, the pair's bilinear forms CY [and
+// SX], and the conversion to fixed point.  Bound by the FP64 pipe and the
+// latency of its chains.  One record per pair, in sorted order.
 template <int NS, int NM, bool SEG>
 __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, unsigned long long* cta_t) {
   cta_mark(cta_t, 0);
@@ -916,7 +922,14 @@ constexpr int kCellThreads = 384;  // the registers of an SM at 168 a thread
 
 // Second kernel: one cell of a pair per lane, as k_pair_quadrature.  Leaves G
 // [and H], the map-coefficient adjoints and the polygon vertices' adjoints in
-// the record.
+// the record.  Bound by issue (0.4 per scheduler and clock) over the
+// multiply-add pipe (43 %) and the integer pipe (38 %), with 3 warps per
+// scheduler.  Its loop is beyond the instruction cache's full-rate size (about
+// 2,300 instructions), so the warps of a block stay in the same part
+// (__syncthreads): 5.2 ms at 600x520, 5.8 ms with every warp on its own.  4.3 ms
+// with what later parts need read again from the record instead of held.
+// Other shapes (all adjoint kernels together 7.9 ms): 512 threads of 128
+// registers 8.6, two blocks of 256 threads of 128 registers 8.3.
 template <int NS, int NM, bool SEG>
 __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
   constexpr int W = SEG ? AdjRecord::kWordsSeg : AdjRecord::kWords;
@@ -1088,7 +1101,11 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
 }
 
 // Third kernel: per pair, the forward blocks, the reverse of the clip and of
-// the master's projection, and the direct terms.
+// the master's projection, and the direct terms; bound by the FP64 pipe.  The
+// blocks M = A G belong here: inside the cell kernel they cost 0.8 ms more at
+// 600x520 (4.5 -> 5.3) than they save.  What depends on the slave element alone
+// (the plane's reverse) is done once per element (k_adjoint_elems): pairs
+// leave 30 words, 42 with dual LMs.
 template <int NS, int NM, bool SEG, bool DUAL>
 __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_finish(AdjArgs g) {
   constexpr int W = SEG ? AdjRecord::kWordsSeg : AdjRecord::kWords;
@@ -1630,7 +1647,7 @@ void launch_fixed(mortar_ctx* c, const RunParams& rp, int block, int rounds) {
         a.conn_s, a.lambda, a.srec, c->Es, c->mult.as<double>());
   for (; a.first < c->pair_cap; a.first += kPairChunk) {
     launch_pair_sort<NS, NM>(ia, rp, c->n_sm, 32 * rounds, a.first);
-    clip<<<gc, block, 0, c->stream>>>(a, cta_t);
+    clip<<<gc, block, 0, c->stream>>>(a, a.first == 0 ? cta_t : nullptr);   // a full chunk's balance
     cells<<<gq, kCellThreads, shm, c->stream>>>(a);
     fin<<<gf, block, 0, c->stream>>>(a);
   }

@@ -21,7 +21,7 @@
 //    element maps and the cell weights into a fixed-point record;
 //    k_pair_quadrature integrates the records on the integer pipe, one cell of
 //    a pair per lane (fixed.cuh, quadrature.cuh).
-//    planar_600x520 (1.35 M pairs, dual LMs): 0.20 + 1.16 + 1.65 ms, against
+//    planar_600x520 (1.35 M pairs, dual LMs): 0.24 + 1.0 + 1.65 ms, against
 //    6.2 ms (batches of 64 pairs, the former default) and 5.6 ms (1024) of the
 //    one-kernel FP64 form.  The clip kernel is bound by the FP64 pipe (50 %
 //    busy, 400 instructions a pair) and instruction fetch, the quadrature
@@ -568,7 +568,7 @@ void launch_split(const IntegrateArgs& a, const RunParams& rp, int n_sm, int rou
   for (int64_t first = 0; first < a.pair_cap; first += kPairChunk) {
     launch_pair_sort<NS, NM>(a, rp, n_sm, 32 * rounds, first);
     clip<<<gc, warps * 32, 0, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag, a.pair_cap,
-                                          first, a.order, a.rec, a.st, a.cta_t);
+                                          first, a.order, a.rec, a.st, first == 0 ? a.cta_t : nullptr);   // a full chunk's balance
     quad<<<gq, kQuadThreads, shq, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag,
                                             a.pair_cap, first, a.rec, a.st);
   }
