@@ -29,6 +29,8 @@ constexpr int kMaxRule = 16;
 constexpr double kInsideTol = 1e-10;
 
 constexpr int kChunk = 8;   // candidate pairs held per pass over the points
+constexpr int kFixedPairs = 12;   // ... in the fixed-point form
+constexpr int kMaxFixedRule = 12;   // n of the largest fixed-point rule (rule_boost)
 
 // One element in FP64, points outermost: for each rule point the
 // element's candidate pairs (a chunk of up to kChunk, with their projected
@@ -256,14 +258,16 @@ __global__ void __launch_bounds__(kThreads) k_integrate_elembased(
 // element's edge, the fixed-point back-projection (2^-57 in xi) for the others
 // with the same 1e-10 tolerance.  The owner's sums stay in registers while
 // consecutive points have the same owner, and are exchanged with thread-local
-// memory when it changes.  Digits: the products'
-// low x low terms are kept and a sum holds 96 bits, so an entry's error is the
-// table's rounding, 2^-62-boost of the element's weight a product.
-// 600x520 quad4, n = 8, dual: 5.95 ms in FP64 (FP64 pipe), 3.25 ms here, of which
+// memory when it changes.  Digits: the products' low x low terms are kept and a
+// sum holds 96 bits, so an entry's error is the table's rounding, 2^-62-boost
+// of the element's weight a product.
+// 600x520 quad4, n = 8, dual: 5.95 ms in FP64 (FP64 pipe), 3.14 ms here, of which
 // the instructions would take half: the candidates' maps and the exchanged sums
 // (about 2 KB a thread) miss L1 in 58 % of their sectors.  Sums added in memory
 // point by point: 4.07 ms; without the warp in step: 9.0 ms; 2 or 4 blocks per SM
-// instead of 3: 3.6, 3.8 ms.
+// instead of 3: 3.6, 3.8 ms.  An element that falls back to FP64 holds up its
+// warp: with 8 pairs the most, 275x332 quads (nine pairs here and there) took
+// 1.2 times the FP64 form's call, with chunks of 12 0.84 times.
 struct ElemCandidate {
   FxMap map;
   int lo_u, hi_u, lo_v, hi_v;   // box in 2^-29 of the frame, widened by 2^-13 of its size
@@ -356,8 +360,10 @@ __device__ __forceinline__ void put_block(const FxAcc* __restrict__ acc, int ke,
 
 // One element per lane, the warp in step (__syncwarp between the parts, which
 // lanes with another owner or candidate would otherwise run one by one).
-// False (nothing written) for a lane whose element does not fit: more than
-// kChunk pairs, a degenerate element, or sizes more than 2^6 apart (fx_frame).
+// Candidate pairs in chunks of kFixedPairs: 12 holds what meshes of about the
+// same size have (three by three, four by three), further chunks take the
+// points without an owner yet.  False (blocks not final) for a lane whose
+// element does not fit: degenerate, or sizes more than 2^6 apart (fx_frame).
 // tab: per point xi, eta, then NS products.
 template <int NS, int NM, bool SEG, bool DUAL>
 __device__ __forceinline__ bool element_fixed(bool valid, int64_t e, const int64_t* __restrict__ pair_off,
@@ -367,172 +373,185 @@ __device__ __forceinline__ bool element_fixed(bool valid, int64_t e, const int64
                                               double* __restrict__ Mblk, double* __restrict__ Dblk,
                                               uint8_t* __restrict__ flag, unsigned long long& n_live,
                                               unsigned long long& n_gp) {
-  int64_t p0 = 0;
-  int kc = 0;
+  int64_t p0 = 0, p1 = 0;
   const double* r = srec;
   if (valid) {
     p0 = pair_off[e];
-    kc = (int)min(pair_off[e + 1] - p0, (int64_t)(kChunk + 1));
+    p1 = pair_off[e + 1];
     r = srec + (int64_t)SR_STRIDE * e;
   }
-  bool ok = kc <= kChunk && (kc == 0 || r[SR_EPSIN] >= 0.0);
-  if (!ok) kc = 0;
-  __syncwarp();
-  const PlaneMap smap = kc > 0 ? slave_plane_map(r) : PlaneMap{0.0, 0.0, 1.0, 0.0, 0.0, 1.0, 0.0, 0.0};
-  PlaneMap maps[kChunk];
-  int E = -1000, small = 1000;
-  for (int k = 0; k < kc; ++k) {
-    maps[k] = master_plane_map<NM>(r, xm, conn_m, pm[p0 + k]);
-    const FxFrame f = fx_frame<NS, NM>(r, smap, maps[k]);
-    E = max(E, f.E);
-    small = min(small, fx_exponent(max(max(fx_hi_abs(maps[k].c1u), fx_hi_abs(maps[k].c1v)),
-                                       max(fx_hi_abs(maps[k].c2u), fx_hi_abs(maps[k].c2v)))));
-  }
-  __syncwarp();
-  small = min(small, fx_exponent(max(max(fx_hi_abs(smap.c1u), fx_hi_abs(smap.c1v)),
-                                     max(fx_hi_abs(smap.c2u), fx_hi_abs(smap.c2v)))));
-  // det J_s = d0 + d1 xi + d2 eta, in units of 2^ED (Q61)
-  const double f0 = cross2(smap.c1u, smap.c1v, smap.c2u, smap.c2v), f1 = cross2(smap.c1u, smap.c1v, smap.c3u, smap.c3v);
-  const double f2 = cross2(smap.c3u, smap.c3v, smap.c2u, smap.c2v);
-  const int ED = fx_exponent(fx_hi_abs(fabs(f0) + fabs(f1) + fabs(f2)));
-  if (kc > 0 && !(E > -200 && E < 200 && small > E - 7 && ED > -500 && ED < 500)) {
-    ok = false;
-    kc = 0;
-  }
-  if (kc == 0) E = 4;   // lanes without work run along on the unit map
-  const long long d0 = fx_of_double(f0, 61 - ED);
-  const Dg d1 = fx_split(fx_of_double(f1, 61 - ED)), d2 = fx_split(fx_of_double(f2, 61 - ED));
-  const bool varies = NS == 4 && !(f1 == 0.0 && f2 == 0.0);
-  FxMap sm;
-  sm.setup_bilinear(smap, E);
-  ElemCandidate cand[kChunk];
-  FxAcc acc[kChunk][NS * NM], accD[SEG ? kChunk : 1][SEG ? NS * NS : 1];
-  for (int k = 0; k < kc; ++k) {
-    FxMap& m = cand[k].map;
-    m.setup_bilinear(maps[k], E);   // for the box
-    corner_range<NM>(m.c0u, m.k1u, m.k2u, m.k3u, cand[k].lo_u, cand[k].hi_u);
-    corner_range<NM>(m.c0v, m.k1v, m.k2v, m.k3v, cand[k].lo_v, cand[k].hi_v);
-    if (NM == 3 || map_is_affine(maps[k])) {
-      const double id = 1.0 / (maps[k].c1u * maps[k].c2v - maps[k].c2u * maps[k].c1v);
-      ok &= m.setup_affine(maps[k], maps[k].c2v * id, -maps[k].c2u * id, -maps[k].c1v * id, maps[k].c1u * id, E);
-    }
-    for (int t = 0; t < NS * NM; ++t) acc[k][t].zero();
-    if (SEG)
-      for (int t = 0; t < NS * NS; ++t) accD[SEG ? k : 0][SEG ? t : 0].zero();
-  }
-  if (!ok) kc = 0;
-  __syncwarp();
-  const FxScales none = {{0, 0, 0, 0}};
-  FxAcc g[4][4], h[4][4];   // sums of pair cur
+  bool ok = p0 == p1 || r[SR_EPSIN] >= 0.0;
+  unsigned taken[(kMaxFixedRule * kMaxFixedRule + 31) / 32];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int l = 0; l < 4; ++l) { g[i][l].zero(); h[i][l].zero(); }
-  int cur = -1;
-  unsigned long long got = 0;   // points of pair k in byte k (at most 144)
-#pragma unroll 1
-  for (int q = 0; q < nq; ++q) {
-    const long long* t = tab + (2 + NS) * q;
-    const long long xs = t[0], es = t[1];
-    long long xu, xv;
-    sm.residual(-sm.c0u, -sm.c0v, xs, es, xu, xv);
-    const int iu = (int)(xu >> 33), iv = (int)(xv >> 33);
-    unsigned near_box = 0;   // candidates left to try, in pair order
-    for (int k = 0; k < kc; ++k)
-      near_box |= (iu >= cand[k].lo_u && iu <= cand[k].hi_u && iv >= cand[k].lo_v && iv <= cand[k].hi_v ? 1u : 0u) << k;
-    int owner = -1;
-    long long x1 = 0, x2 = 0;
-    while (__any_sync(0xffffffffu, near_box != 0u)) {   // at most kChunk rounds: each takes a bit of every lane
-      bool near = false, settled = true;
-      float x = 0.0f, y = 0.0f;
-      const int k = near_box != 0u ? __ffs(near_box) - 1 : 0;
-      FxMap m;
-      if (near_box != 0u) {
-        m = cand[k].map;
-        near_box &= near_box - 1u;
-        const float tu = fx_f32(xu - m.c0u), tv = fx_f32(xv - m.c0v);
-        float band = 1e-5f;
-        if (NM == 3 || m.affine) {
-          const float xa = m.b00 * tu, xb = m.b01 * tv, ya = m.b10 * tu, yb = m.b11 * tv;
-          x = xa + xb;
-          y = ya + yb;
-          band = fmaf(1e-6f, fabsf(xa) + fabsf(xb) + fabsf(ya) + fabsf(yb), band);   // FP32 rounding of a needle's sums
-          if (!(band < 0.25f)) ok = false;   // nothing is written before the end
-        } else {
-          settled = m.settle(tu, tv, x, y);
-        }
-        // points clearly outside skip the fixed-point step
-        near = !settled || (NM == 4 ? (fabsf(x) <= 1.0f + band && fabsf(y) <= 1.0f + band)
-                                    : (x >= -band && y >= -band && x + y <= 1.0f + band));
-      }
-      __syncwarp();
-      if (near) {
-        bool solved = settled;
-        if (NM == 3 || m.affine) m.solve_affine(xu - m.c0u, xv - m.c0v, x1, x2);
-        else if (settled) solved = m.refine(xu - m.c0u, xv - m.c0v, x, y, x1, x2);
-        if (!solved) solved = fx_slow_solve(maps[k], E, xu, xv, x1, x2);
-        constexpr long long one = 1ll << 61, tol = (long long)(kInsideTol * (double)(1ll << 61));
-        const bool inside = NM == 4
-            ? (x1 <= one + tol && x1 >= -(one + tol) && x2 <= one + tol && x2 >= -(one + tol))
-            : (x1 >= -tol && x2 >= -tol && x1 + x2 <= one + tol);
-        if (solved && inside) {
-          owner = k;
-          near_box = 0u;
-        }
-      }
-      __syncwarp();
-    }
-    if (owner >= 0 && owner != cur) {
-      exchange<NS, NM>(g, cur >= 0 ? acc[cur] : nullptr, acc[owner]);
-      if (SEG) exchange<NS, NS>(h, cur >= 0 ? accD[SEG ? cur : 0] : nullptr, accD[SEG ? owner : 0]);
-      cur = owner;
+  for (int k = 0; k < (int)(sizeof(taken) / sizeof(taken[0])); ++k) taken[k] = 0u;
+  unsigned live = 0, owned = 0;
+  const bool more = __any_sync(0xffffffffu, p1 - p0 > kFixedPairs);
+  for (; __any_sync(0xffffffffu, ok && p0 < p1); p0 += kFixedPairs) {   // p0 of a finished lane moves on, unused
+    int kc = ok ? (int)max((int64_t)0, min(p1 - p0, (int64_t)kFixedPairs)) : 0;
+    const PlaneMap smap = kc > 0 ? slave_plane_map(r) : PlaneMap{0.0, 0.0, 1.0, 0.0, 0.0, 1.0, 0.0, 0.0};
+    PlaneMap maps[kFixedPairs];
+    int E = -1000, small = 1000;
+    for (int k = 0; k < kc; ++k) {
+      maps[k] = master_plane_map<NM>(r, xm, conn_m, pm[p0 + k]);
+      const FxFrame f = fx_frame<NS, NM>(r, smap, maps[k]);
+      E = max(E, f.E);
+      small = min(small, fx_exponent(max(max(fx_hi_abs(maps[k].c1u), fx_hi_abs(maps[k].c1v)),
+                                         max(fx_hi_abs(maps[k].c2u), fx_hi_abs(maps[k].c2v)))));
     }
     __syncwarp();
-    long long det = d0;
-    FxAcc a;
-    if (varies) {
-      a.mul(d1, fx_split(xs));
-      a.mac(d2, fx_split(es));
-      det += a.get<3>();
+    small = min(small, fx_exponent(max(max(fx_hi_abs(smap.c1u), fx_hi_abs(smap.c1v)),
+                                       max(fx_hi_abs(smap.c2u), fx_hi_abs(smap.c2v)))));
+    // det J_s = d0 + d1 xi + d2 eta, in units of 2^ED (Q61)
+    const double f0 = cross2(smap.c1u, smap.c1v, smap.c2u, smap.c2v), f1 = cross2(smap.c1u, smap.c1v, smap.c3u, smap.c3v);
+    const double f2 = cross2(smap.c3u, smap.c3v, smap.c2u, smap.c2v);
+    const int ED = fx_exponent(fx_hi_abs(fabs(f0) + fabs(f1) + fabs(f2)));
+    if (kc > 0 && !(E > -200 && E < 200 && small > E - 7 && ED > -500 && ED < 500)) {
+      ok = false;
+      kc = 0;
     }
-    const Dg W = fx_split(det < 0 ? -det : det);
-    if (owner >= 0) {
-      got += 1ull << (8 * owner);
-      Dg Ns[4], Nc[4];
+    if (kc == 0) E = 4;   // lanes without work run along on the unit map
+    const long long d0 = fx_of_double(f0, 61 - ED);
+    const Dg d1 = fx_split(fx_of_double(f1, 61 - ED)), d2 = fx_split(fx_of_double(f2, 61 - ED));
+    const bool varies = NS == 4 && !(f1 == 0.0 && f2 == 0.0);
+    FxMap sm;
+    sm.setup_bilinear(smap, E);
+    ElemCandidate cand[kFixedPairs];
+    FxAcc acc[kFixedPairs][NS * NM], accD[SEG ? kFixedPairs : 1][SEG ? NS * NS : 1];
+    for (int k = 0; k < kc; ++k) {
+      FxMap& m = cand[k].map;
+      m.setup_bilinear(maps[k], E);   // for the box
+      corner_range<NM>(m.c0u, m.k1u, m.k2u, m.k3u, cand[k].lo_u, cand[k].hi_u);
+      corner_range<NM>(m.c0v, m.k1v, m.k2v, m.k3v, cand[k].lo_v, cand[k].hi_v);
+      if (NM == 3 || map_is_affine(maps[k])) {
+        const double id = 1.0 / (maps[k].c1u * maps[k].c2v - maps[k].c2u * maps[k].c1v);
+        ok &= m.setup_affine(maps[k], maps[k].c2v * id, -maps[k].c2u * id, -maps[k].c1v * id, maps[k].c1u * id, E);
+      }
+      for (int t = 0; t < NS * NM; ++t) acc[k][t].zero();
+      if (SEG)
+        for (int t = 0; t < NS * NS; ++t) accD[SEG ? k : 0][SEG ? t : 0].zero();
+    }
+    if (!ok) kc = 0;
+    __syncwarp();
+    const FxScales none = {{0, 0, 0, 0}};
+    FxAcc g[4][4], h[4][4];   // sums of pair cur
 #pragma unroll
-      for (int i = 0; i < NS; ++i) {
-        const Dg T = fx_split(t[2 + i]);
-        a.mul(T, W);
-        a.low(T, W);
-        Ns[i] = fx_split(a.get<3>());
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int l = 0; l < 4; ++l) { g[i][l].zero(); h[i][l].zero(); }
+    int cur = -1;
+    unsigned got[3] = {0u, 0u, 0u};   // points of pair k in byte k (at most 144)
+#pragma unroll 1
+    for (int q = 0; q < nq; ++q) {
+      const long long* t = tab + (2 + NS) * q;
+      const long long xs = t[0], es = t[1];
+      long long xu, xv;
+      sm.residual(-sm.c0u, -sm.c0v, xs, es, xu, xv);
+      const int iu = (int)(xu >> 33), iv = (int)(xv >> 33);
+      unsigned near_box = 0;   // candidates left to try, in pair order
+      const bool open = !more || !(taken[q >> 5] >> (q & 31) & 1u);
+      for (int k = 0; k < (open ? kc : 0); ++k)
+        near_box |= (iu >= cand[k].lo_u && iu <= cand[k].hi_u && iv >= cand[k].lo_v && iv <= cand[k].hi_v ? 1u : 0u) << k;
+      int owner = -1;
+      long long x1 = 0, x2 = 0;
+      while (__any_sync(0xffffffffu, near_box != 0u)) {   // at most kFixedPairs rounds: each takes a bit of every lane
+        bool near = false, settled = true;
+        float x = 0.0f, y = 0.0f;
+        const int k = near_box != 0u ? __ffs(near_box) - 1 : 0;
+        FxMap m;
+        if (near_box != 0u) {
+          m = cand[k].map;
+          near_box &= near_box - 1u;
+          const float tu = fx_f32(xu - m.c0u), tv = fx_f32(xv - m.c0v);
+          float band = 1e-5f;
+          if (NM == 3 || m.affine) {
+            const float xa = m.b00 * tu, xb = m.b01 * tv, ya = m.b10 * tu, yb = m.b11 * tv;
+            x = xa + xb;
+            y = ya + yb;
+            band = fmaf(1e-6f, fabsf(xa) + fabsf(xb) + fabsf(ya) + fabsf(yb), band);   // FP32 rounding of a needle's sums
+            if (!(band < 0.25f)) ok = false;   // nothing is written before the end
+          } else {
+            settled = m.settle(tu, tv, x, y);
+          }
+          // points clearly outside skip the fixed-point step
+          near = !settled || (NM == 4 ? (fabsf(x) <= 1.0f + band && fabsf(y) <= 1.0f + band)
+                                      : (x >= -band && y >= -band && x + y <= 1.0f + band));
+        }
+        __syncwarp();
+        if (near) {
+          bool solved = settled;
+          if (NM == 3 || m.affine) m.solve_affine(xu - m.c0u, xv - m.c0v, x1, x2);
+          else if (settled) solved = m.refine(xu - m.c0u, xv - m.c0v, x, y, x1, x2);
+          if (!solved) solved = fx_slow_solve(maps[k], E, xu, xv, x1, x2);
+          constexpr long long one = 1ll << 61, tol = (long long)(kInsideTol * (double)(1ll << 61));
+          const bool inside = NM == 4
+              ? (x1 <= one + tol && x1 >= -(one + tol) && x2 <= one + tol && x2 >= -(one + tol))
+              : (x1 >= -tol && x2 >= -tol && x1 + x2 <= one + tol);
+          if (solved && inside) {
+            owner = k;
+            near_box = 0u;
+          }
+        }
+        __syncwarp();
       }
-      fx_shape<NM>(none, x1, x2, Nc);
-      add_products<NS, NM>(g, Ns, Nc);
-      if (SEG) {
-        fx_shape<NS>(none, xs, es, Nc);
-        add_products<NS, NS>(h, Ns, Nc);
+      if (owner >= 0 && owner != cur) {
+        exchange<NS, NM>(g, cur >= 0 ? acc[cur] : nullptr, acc[owner]);
+        if (SEG) exchange<NS, NS>(h, cur >= 0 ? accD[SEG ? cur : 0] : nullptr, accD[SEG ? owner : 0]);
+        cur = owner;
       }
+      __syncwarp();
+      long long det = d0;
+      FxAcc a;
+      if (varies) {
+        a.mul(d1, fx_split(xs));
+        a.mac(d2, fx_split(es));
+        det += a.get<3>();
+      }
+      const Dg W = fx_split(det < 0 ? -det : det);
+      if (owner >= 0) {
+        const unsigned one = 1u << (8 * (owner & 3));
+        got[0] += owner < 4 ? one : 0u;
+        got[1] += owner >= 4 && owner < 8 ? one : 0u;
+        got[2] += owner >= 8 ? one : 0u;
+        if (more) taken[q >> 5] |= 1u << (q & 31);
+        Dg Ns[4], Nc[4];
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+          const Dg T = fx_split(t[2 + i]);
+          a.mul(T, W);
+          a.low(T, W);
+          Ns[i] = fx_split(a.get<3>());
+        }
+        fx_shape<NM>(none, x1, x2, Nc);
+        add_products<NS, NM>(g, Ns, Nc);
+        if (SEG) {
+          fx_shape<NS>(none, xs, es, Nc);
+          add_products<NS, NS>(h, Ns, Nc);
+        }
+      }
+      if ((q & 3) == 3) {   // four products: cross sums below 2^63
+        carry_all<NS, NM>(g);
+        if (SEG) carry_all<NS, NS>(h);
+      }
+      __syncwarp();
     }
-    if ((q & 3) == 3) {   // four products: cross sums below 2^63
-      carry_all<NS, NM>(g);
-      if (SEG) carry_all<NS, NS>(h);
+    if (ok && cur >= 0) {
+      exchange<NS, NM>(g, acc[cur], acc[cur]);
+      if (SEG) exchange<NS, NS>(h, accD[SEG ? cur : 0], accD[SEG ? cur : 0]);
+    }
+    const int ke = ED - 59 - boost + (NS == 4 ? 2 : -1);   // sum w = 4 or 1/2
+    for (int k = 0; k < (ok ? kc : 0); ++k) {
+      const unsigned points = (k < 4 ? got[0] : (k < 8 ? got[1] : got[2])) >> (8 * (k & 3)) & 0xffu;
+      put_block<NS, NM, DUAL>(acc[k], ke, r + SR_A, Mblk + 16 * (p0 + k));
+      if (SEG) put_block<NS, NS, DUAL>(accD[SEG ? k : 0], ke, r + SR_A, Dblk + 16 * (p0 + k));
+      flag[p0 + k] = points > 0 ? 1 : 0;
+      live += points > 0 ? 1u : 0u;
+      owned += points;
     }
     __syncwarp();
   }
   if (!ok) return false;
-  if (cur >= 0) {
-    exchange<NS, NM>(g, acc[cur], acc[cur]);
-    if (SEG) exchange<NS, NS>(h, accD[SEG ? cur : 0], accD[SEG ? cur : 0]);
-  }
-  const int ke = ED - 59 - boost + (NS == 4 ? 2 : -1);   // sum w = 4 or 1/2
-  for (int k = 0; k < kc; ++k) {
-    const int points = (int)(got >> (8 * k)) & 0xff;
-    put_block<NS, NM, DUAL>(acc[k], ke, r + SR_A, Mblk + 16 * (p0 + k));
-    if (SEG) put_block<NS, NS, DUAL>(accD[SEG ? k : 0], ke, r + SR_A, Dblk + 16 * (p0 + k));
-    flag[p0 + k] = points > 0 ? 1 : 0;
-    n_live += points > 0 ? 1 : 0;
-    n_gp += (unsigned long long)points;
-  }
+  n_live += live;
+  n_gp += owned;
   return true;
 }
 
@@ -616,7 +635,7 @@ int rule_boost(int nen, const double* rule, int n) {
   }
   int b = 0;
   while (b < 3 && std::ldexp(hi, b + 1) < 0.25) ++b;
-  return n <= 12 && std::ldexp(lo, b) >= std::ldexp(1.0, -22) ? b : -1;
+  return n <= kMaxFixedRule && std::ldexp(lo, b) >= std::ldexp(1.0, -22) ? b : -1;
 }
 
 }  // namespace

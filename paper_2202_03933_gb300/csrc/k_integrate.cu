@@ -568,7 +568,8 @@ void launch_split(const IntegrateArgs& a, const RunParams& rp, int n_sm, int rou
   for (int64_t first = 0; first < a.pair_cap; first += kPairChunk) {
     launch_pair_sort<NS, NM>(a, rp, n_sm, 32 * rounds, first);
     clip<<<gc, warps * 32, 0, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag, a.pair_cap,
-                                          first, a.order, a.rec, a.st, first == 0 ? a.cta_t : nullptr);   // a full chunk's balance
+                                          first, a.order, a.rec, a.st,
+                                          first == 0 ? a.cta_t : nullptr);   // a full chunk's balance
     quad<<<gq, kQuadThreads, shq, a.stream>>>(a.ps, a.pm, a.srec, a.xm, a.conn_m, rp, a.Mblk, a.Dblk, a.flag,
                                             a.pair_cap, first, a.rec, a.st);
   }

@@ -18,12 +18,13 @@
 // point adjoint is then a product or two, and the slave map's adjoints of all
 // four follow from 12 moments.  Bound by the FP64 pipe (about 75 % busy);
 // 300x260 quads, dual (0.31 M pairs): 21.7 ms with the N_e as seeds, 18.7 ms
-// this way, square roots and divisions of the plane once per pair.  The derivatives through A (dual LMs) and of
-// the element-domain D depend on the slave element alone: a per-element
-// kernel pushes the pair sums of O and the D term through A = Dh Me^-1 and
-// the element integrals in forward mode over the 12 slave coordinates.  Rows
-// are gathered per slave node in a fixed order into BSR with no
-// floating-point atomics: bitwise reproducible.
+// this way, square roots and divisions of the plane once per pair.
+//
+// The derivatives through A (dual LMs) and of the element-domain D depend on
+// the slave element alone: a per-element kernel pushes the pair sums of O and
+// the D term through A = Dh Me^-1 and the element integrals in forward mode
+// over the 12 slave coordinates.  Rows are gathered per slave node in a fixed
+// order into BSR with no floating-point atomics: bitwise reproducible.
 #include <algorithm>
 
 #include "clip.cuh"

@@ -134,7 +134,7 @@ def _tri_slave(seed):
 
 
 # element-based: rules on both sides of the FP64 lines (12 on quad4, 8 on tri3),
-# elements with more than eight pairs, sizes beyond 2^6, units
+# elements with more pairs than a chunk (12), sizes beyond 2^6, units
 ELEMENT = {
     "n1": (lambda: inputs.planar_noisy(6, 5, 0, 90, "e1"), 1),
     "n12": (lambda: _both_noisy(5, 6, 1, 91), 12),
