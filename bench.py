@@ -1,5 +1,5 @@
 """Benchmark: mortar pairs integrated per second (D + M, FP64) with the adjoint,
-on one GB300, against the FP64 roofline.
+on one GB300, against its issue and FP64 rooflines.
 
 One step = the whole hot path on one synthetic interface, replayed as one
 CUDA graph: element precompute, binned search, per-pair segment integration,
@@ -48,14 +48,18 @@ sys.path.insert(0, ROOT)
 METRIC = "mortar pairs integrated/sec (D+M, FP64) and fwd+adjoint time on 1 GB300 vs FP64 roofline"
 UNIT = "pairs/s"
 
-# Executed FP64 flops (2 x DFMA + DADD + DMUL thread instructions, predicated
-# on) and DRAM bytes per pair of the per-pair kernels, from ncu counters of
-# this build on planar_600x520 (same element types and density as the full
-# workload, so per-pair figures carry over); see profiles/.
+# Executed warp instructions, FP64 flops (2 x DFMA + DADD + DMUL thread
+# instructions, predicated on) and DRAM bytes per pair of the per-pair kernels
+# together, from ncu counters of this build on planar_600x520 (same element
+# types and density as the full workload, so per-pair figures carry over); see
+# profiles/.  The quadrature is 64-bit fixed point on the integer pipes, so the
+# kernels' common roofline is the issue rate.
 EXEC_PER_PAIR = {
-    "fused": {"flops": 8492.3, "dram_bytes": 880.0},
-    "integrate": {"flops": 2994.6, "dram_bytes": 283.0},
+    "fused": {"warp_inst": 2056.0, "flops": 1084.4, "dram_bytes": 4109.0, "fp64_form": 8492.3},
+    "integrate": {"warp_inst": 1061.2, "flops": 381.4, "dram_bytes": 1584.0, "fp64_form": 2994.6},
 }
+# fp64_form: executed FP64 flops per pair of the same integration with the
+# quadrature on the FP64 pipe (this library's former kernels).
 
 # FP64 peak derived from unit counts and clocks: 152 SMs x 2 FP64 FMA lanes
 # per SM per clock (4 flop/clk/SM) x 2070 MHz maximum SM clock = 1.259 TFLOP/s,
@@ -64,6 +68,36 @@ SM_COUNT = 152
 FP64_FLOP_PER_CLK_PER_SM = 4
 SM_MAX_MHZ = 2070.0
 FP64_PEAK_TFLOPS = SM_COUNT * FP64_FLOP_PER_CLK_PER_SM * SM_MAX_MHZ * 1e6 / 1e12
+# issue peak: 4 schedulers per SM, one warp instruction per clock each
+ISSUE_PEAK_GINST = SM_COUNT * 4 * SM_MAX_MHZ * 1e6 / 1e9
+
+
+def pair_roofline(kernel: str, ex: dict, n_pairs: int, ms: float, same_family: bool) -> dict:
+    """Executed warp instructions over the pair kernels' CUDA-event time against
+    the issue peak, and their FP64 flops against the FP64 peak."""
+    roof = {"bound": "issue", "kernel": kernel, "ms_per_launch": round(ms, 4),
+            "peak": round(ISSUE_PEAK_GINST, 1), "unit": "Ginst/s",
+            "peak_kind": "derived issue rate: 152 SM x 4 schedulers x 2070 MHz",
+            "counted": "executed warp instructions (ncu, per pair on planar_600x520) x pairs",
+            "achieved": None, "frac": None, "traffic": None}
+    # the per-pair counters were taken on the planar quad4/quad4 dual family;
+    # other element types execute other per-pair work, so they get no fraction
+    if not same_family:
+        roof["note"] = "executed work per pair measured on the planar quad4/quad4 dual family only"
+        return roof
+    s = ms / 1e3
+    inst = ex["warp_inst"] * n_pairs / s / 1e9
+    fp64 = ex["flops"] * n_pairs / s / 1e12
+    roof.update(achieved=round(inst, 1), frac=round(inst / ISSUE_PEAK_GINST, 4),
+                warp_inst_per_pair=ex["warp_inst"], traffic=int(ex["dram_bytes"] * n_pairs),
+                fp64={"achieved": round(fp64, 4), "peak": round(FP64_PEAK_TFLOPS, 4), "unit": "TFLOP/s",
+                      "frac": round(fp64 / FP64_PEAK_TFLOPS, 4), "flops_per_pair": ex["flops"],
+                      "peak_kind": "derived FP64: 152 SM x 4 flop/clk x 2070 MHz (measured probe below)"})
+    eq = ex["fp64_form"] * n_pairs / s / 1e12
+    roof["fp64_form"] = {"rate": round(eq, 4), "unit": "TFLOP/s", "of_fp64_peak": round(eq / FP64_PEAK_TFLOPS, 4),
+                         "flops_per_pair": ex["fp64_form"],
+                         "note": "flops of the all-FP64 form of the same integration over this time; not executed FP64"}
+    return roof
 
 
 def measured_peaks() -> dict:
@@ -435,25 +469,11 @@ def run_ours(args, world, rank, local):
     med = statistics.median
     ms_pair = med(t_int)   # the pair kernel that produced the forward blocks (fused with the adjoint)
     fused = bool(st.get("fused", 0))
-    # ---- roofline of the dominant kernel: executed FP64 flops / its CUDA-event time
-    ex = EXEC_PER_PAIR["fused" if fused else "integrate"]
-    roof = {"bound": "alu", "kernel": ("k_adjoint_batched: fused forward blocks + adjoint per pair" if fused
-                                       else "k_integrate_batched"),
-            "ms_per_launch": round(ms_pair, 4), "peak": round(FP64_PEAK_TFLOPS, 4), "unit": "TFLOP/s",
-            "peak_kind": "derived FP64: 152 SM x 4 flop/clk x 2070 MHz (of derived; measured probe below)",
-            "flops": "executed FP64 (ncu 2 DFMA + DADD + DMUL per pair, planar_600x520) x pairs",
-            "achieved": None, "frac": None, "traffic": None}
-    # the per-pair counters were taken on the planar quad4/quad4 dual family;
-    # other element types execute other per-pair work, so they get no fraction
+    # ---- roofline of the pair kernels
     same_family = args.workload.startswith("planar_") and itf.lm == 1
-    if ex["flops"] and same_family:
-        achieved = ex["flops"] * n_pairs / (ms_pair / 1e3) / 1e12
-        roof.update(achieved=round(achieved, 4), frac=round(achieved / FP64_PEAK_TFLOPS, 4),
-                    flops_per_pair=ex["flops"])
-    elif ex["flops"]:
-        roof["note"] = "executed FP64 per pair measured on the planar quad4/quad4 dual family only"
-    if ex["dram_bytes"] and same_family:
-        roof["traffic"] = int(ex["dram_bytes"] * n_pairs)
+    roof = pair_roofline("k_pair_sort, k_adjoint_clip, _cells, _finish: forward blocks + adjoint per pair" if fused
+                         else "k_pair_sort, k_pair_clip, k_pair_quadrature",
+                         EXEC_PER_PAIR["fused" if fused else "integrate"], n_pairs, ms_pair, same_family)
 
     # ---- HBM rates of the two memory-bound phases (algorithmic bytes / phase
     #      time): search = element boxes read (64 B per element, both sides) +
@@ -475,7 +495,7 @@ def run_ours(args, world, rank, local):
         phase_bw = {"error": str(ex_)}
 
     # ---- forward only (search + integration + assembly graph): forward pairs/s
-    #      and the integration kernel's executed-FP64 roofline fraction
+    #      and the integration kernels' roofline fractions
     fwd = None
     try:
         if "forward" not in sections:
@@ -501,15 +521,9 @@ def run_ours(args, world, rank, local):
         mf.close()
         fwd = {"ms_per_step": round(ms_f, 4), "pairs_per_s": world * n_pairs / (ms_f / 1e3),
                "ms_integrate": round(med(t_fi), 4), "autotune": pick_f}
-        exf = EXEC_PER_PAIR["integrate"]
-        if exf["flops"] and args.workload.startswith("planar_") and itf.lm == 1:
-            a = exf["flops"] * n_pairs / (med(t_fi) / 1e3) / 1e12
-            fwd["roofline"] = {
-                "bound": "alu", "kernel": "k_integrate_batched", "ms_per_launch": round(med(t_fi), 4),
-                "achieved": round(a, 4), "peak": round(FP64_PEAK_TFLOPS, 4), "unit": "TFLOP/s",
-                "frac": round(a / FP64_PEAK_TFLOPS, 4), "flops_per_pair": exf["flops"],
-                "flops": "executed FP64 (ncu 2 DFMA + DADD + DMUL per pair, planar_600x520) x pairs",
-                "traffic": int(exf["dram_bytes"] * n_pairs) if exf["dram_bytes"] else None}
+        if same_family:
+            fwd["roofline"] = pair_roofline("k_pair_sort, k_pair_clip, k_pair_quadrature", EXEC_PER_PAIR["integrate"],
+                                            n_pairs, med(t_fi), True)
     except _Skip:
         pass
     except Exception as ex_:   # reported, not fatal
