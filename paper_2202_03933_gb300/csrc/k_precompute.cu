@@ -32,6 +32,27 @@ __device__ __forceinline__ V3 cross(V3 a, V3 b) {
   return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
 }
 
+// Surface Jacobian |x,xi x x,eta| of an element at (xi, eta).
+template <int NEN>
+__device__ double surface_jac(const V3* X, double xi, double eta) {
+  V3 g1, g2;
+  if constexpr (NEN == 4) {
+    const double em = 0.25 * (1.0 - eta), ep = 0.25 * (1.0 + eta);
+    const double xm = 0.25 * (1.0 - xi), xp = 0.25 * (1.0 + xi);
+    g1 = {-em * X[0].x + em * X[1].x + ep * X[2].x - ep * X[3].x,
+          -em * X[0].y + em * X[1].y + ep * X[2].y - ep * X[3].y,
+          -em * X[0].z + em * X[1].z + ep * X[2].z - ep * X[3].z};
+    g2 = {-xm * X[0].x - xp * X[1].x + xp * X[2].x + xm * X[3].x,
+          -xm * X[0].y - xp * X[1].y + xp * X[2].y + xm * X[3].y,
+          -xm * X[0].z - xp * X[1].z + xp * X[2].z + xm * X[3].z};
+  } else {
+    g1 = sub(X[1], X[0]);
+    g2 = sub(X[2], X[0]);
+  }
+  V3 n = cross(g1, g2);
+  return sqrt(dot(n, n));
+}
+
 // Element rule point k: 3x3 Gauss-Legendre (quad4, weights sum 4) or the
 // 7-point triangle rule (tri3, weights sum 1/2).
 template <int NEN>
@@ -149,9 +170,6 @@ __device__ __forceinline__ void set_nan_box(double* b) {
   for (int k = 0; k < 7; ++k) b[k] = q;
 }
 
-// Bound by the FP64 pipe.  600x520, distorted slave quads (0.36 M): 0.60 ms with
-// the tangents, normal and 16 products formed at each of the 9 points, 0.42 ms
-// with the linear normal and the products summed one direction at a time.
 template <int NS>
 __global__ void __launch_bounds__(kThreads) k_slave_precompute(
     const double* __restrict__ xs, const int32_t* __restrict__ conn, int64_t Es, RunParams rp,
@@ -178,10 +196,9 @@ __global__ void __launch_bounds__(kThreads) k_slave_precompute(
       for (int b = 0; b < 4; ++b) Me[a][b] = 0.0;
     }
     bool flat_jac = NS == 3;
-    V3 d3 = {0.0, 0.0, 0.0};
     if constexpr (NS == 4) {
-      d3 = {0.25 * ((X[0].x - X[1].x) + (X[2].x - X[3].x)), 0.25 * ((X[0].y - X[1].y) + (X[2].y - X[3].y)),
-            0.25 * ((X[0].z - X[1].z) + (X[2].z - X[3].z))};
+      const V3 d3 = {0.25 * ((X[0].x - X[1].x) + (X[2].x - X[3].x)), 0.25 * ((X[0].y - X[1].y) + (X[2].y - X[3].y)),
+                     0.25 * ((X[0].z - X[1].z) + (X[2].z - X[3].z))};
       const double s3 = fabs(d3.x) + fabs(d3.y) + fabs(d3.z);
       const double s12 = fabs(g1.x) + fabs(g1.y) + fabs(g1.z) + fabs(g2.x) + fabs(g2.y) + fabs(g2.z);
       flat_jac = s3 <= 1e-15 * s12;
@@ -205,40 +222,18 @@ __global__ void __launch_bounds__(kThreads) k_slave_precompute(
         }
       }
     } else {
-      // distorted quad4, 3x3 Gauss-Legendre: the normal is linear in xi and eta
-      // (g1 = g1_0 + eta d3, g2 = g2_0 + xi d3, d3 x d3 = 0), and the products of
-      // 1D shape functions p0 p0, p0 p1, p1 p1 are summed one direction at a time
-      const V3 n0 = cross(g1, g2), nx = cross(g1, d3), ne = cross(d3, g2);
-      const double g = 0.7745966692414834;
-      const double pt[3] = {-g, 0.0, g}, pw[3] = {5.0 / 9.0, 8.0 / 9.0, 5.0 / 9.0};
-      double S[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};   // [xi products][eta products]
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const V3 nj = {n0.x + pt[j] * ne.x, n0.y + pt[j] * ne.y, n0.z + pt[j] * ne.z};
-        double R[3] = {0, 0, 0};
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          const V3 n = {nj.x + pt[i] * nx.x, nj.y + pt[i] * nx.y, nj.z + pt[i] * nx.z};
-          const double J = sqrt(dot(n, n));
-          const double p0 = 0.5 - 0.5 * pt[i], p1 = 0.5 + 0.5 * pt[i];
-          R[0] = fma(pw[i] * p0 * p0, J, R[0]);
-          R[1] = fma(pw[i] * p0 * p1, J, R[1]);
-          R[2] = fma(pw[i] * p1 * p1, J, R[2]);
+      constexpr int nq = NS == 4 ? 9 : 7;
+      for (int q = 0; q < nq; ++q) {
+        double xi, eta, w;
+        elem_point<NS>(q, xi, eta, w);
+        double N[4];
+        shape_fn<NS>(xi, eta, N);
+        const double wj = w * surface_jac<NS>(X, xi, eta);
+        for (int a = 0; a < NS; ++a) {
+          const double wn = wj * N[a];
+          Dh[a] += wn;
+          for (int b = 0; b < NS; ++b) Me[a][b] += wn * N[b];
         }
-        const double p0 = 0.5 - 0.5 * pt[j], p1 = 0.5 + 0.5 * pt[j];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          S[k][0] = fma(pw[j] * p0 * p0, R[k], S[k][0]);
-          S[k][1] = fma(pw[j] * p0 * p1, R[k], S[k][1]);
-          S[k][2] = fma(pw[j] * p1 * p1, R[k], S[k][2]);
-        }
-      }
-      constexpr int px[4] = {0, 1, 1, 0}, pe[4] = {0, 0, 1, 1};   // corners (-1,-1), (1,-1), (1,1), (-1,1)
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-#pragma unroll
-        for (int b = 0; b < 4; ++b) Me[a][b] = S[px[a] + px[b]][pe[a] + pe[b]];
-        Dh[a] = (Me[a][0] + Me[a][1]) + (Me[a][2] + Me[a][3]);   // sum_b N_b = 1
       }
     }
     // ---- LM coefficients: standard A = I; dual A = Dh Me^-1 (Me A^T = diag(Dh))
@@ -296,7 +291,7 @@ __global__ void __launch_bounds__(kThreads) k_slave_precompute(
         if (rp.lm == 1) {
           v = a == b ? Dh[a] : 0.0;
         } else {
-          v = Me[a][b];
+          for (int c = 0; c < NS; ++c) v += A[a][c] * Me[c][b];
         }
         d[4 * a + b] = (a < NS && b < NS) ? v : 0.0;
       }
