@@ -844,10 +844,14 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, un
         mark = kSlowPair;
         if (f.setup<NS, NM>(r, mmap, pu, pv, cp.nr)) {
           // bilinear forms of the pair, and their scales
+          // (segment D: x_s - x_m does not change with the origin, and about the
+          // element's centre the forms are as large as the element, not as the
+          // coordinates: what cancels in fixed point is small)
+          const V3 org = SEG ? v3(r[SR_X0], r[SR_X0 + 1], r[SR_X0 + 2]) : v3(0.0, 0.0, 0.0);
           V3 Y[4], LM[4], YM[4];
           for (int l = 0; l < NM; ++l) {
             const int64_t nd = cm[l];
-            Y[l] = v3(g.xm[3 * nd], g.xm[3 * nd + 1], g.xm[3 * nd + 2]);
+            Y[l] = v3(g.xm[3 * nd], g.xm[3 * nd + 1], g.xm[3 * nd + 2]) - org;
           }
           load_v3<NS>(g.mult + 24 * (int64_t)s + 12, LM);
           nodal_to_mono<NM>(Y, YM);
@@ -860,7 +864,7 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, un
             V3 X[4], XM[4];
             for (int a = 0; a < NS; ++a) {
               const int64_t nd = g.conn_s[(int64_t)NS * s + a];
-              X[a] = v3(g.xs[3 * nd], g.xs[3 * nd + 1], g.xs[3 * nd + 2]);
+              X[a] = v3(g.xs[3 * nd], g.xs[3 * nd + 1], g.xs[3 * nd + 2]) - org;
             }
             nodal_to_mono<NS>(X, XM);
 #pragma unroll
