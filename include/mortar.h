@@ -108,9 +108,11 @@ typedef struct mortar_options {
   int32_t element_rule_n;   /* points per direction of the element-based rule, 1..16 (8) */
   int32_t facing_test;      /* 1: keep only candidate pairs whose slave and master element normals (at
                                the element centres) point against each other, n_s . n_m < 0 (0) */
-  int32_t watchdog_us;      /* time budget of the persistent pair kernels in microseconds, 0 = none (0):
-                               a kernel whose thread blocks run longer stops taking work and the call
-                               returns MORTAR_ERR_TIMEOUT (results not valid; the context stays usable) */
+  int32_t watchdog_us;      /* time budget of a persistent pair kernel in microseconds, 0 = none (0): a
+                               kernel whose thread blocks run longer stops taking work, the pair kernels
+                               after it take none, and the call returns MORTAR_ERR_TIMEOUT (results not
+                               valid; the context stays usable).  The budget is of each kernel: a run
+                               has up to four for every 4 M pairs */
 } mortar_options;
 
 typedef struct mortar_stats {

@@ -210,6 +210,12 @@ int finish_run(mortar_ctx* c, const Phases& ph) {
   MORTAR_TRY(check_cuda());
   const DevStatus& h = *c->hstat;
   bool again = false;
+  // a captured run holds the addresses of what is about to grow, whatever this
+  // run then returns
+  if ((h.over_pairs || (ph.assemble && h.over_nnz)) && c->graph_exec) {
+    cudaGraphExecDestroy(c->graph_exec);
+    c->graph_exec = nullptr;
+  }
   if (h.over_pairs) {
     MORTAR_TRY(alloc_pair_buffers(c, (int64_t)(h.over_pairs + h.over_pairs / 8 + 1024)));
     again = true;
@@ -223,13 +229,7 @@ int finish_run(mortar_ctx* c, const Phases& ph) {
   if (ph.adjoint && h.over_mlist) again = true;   // list buffers are sized from n_pairs below
   if (h.over_bins) return MORTAR_ERR_CAPACITY;
   if (h.timeout) return MORTAR_ERR_TIMEOUT;
-  if (again) {
-    if (c->graph_exec) {
-      cudaGraphExecDestroy(c->graph_exec);
-      c->graph_exec = nullptr;
-    }
-    return 1;
-  }
+  if (again) return 1;
   c->n_pairs = (int64_t)h.n_pairs;
   c->nnz_D = (int64_t)h.nnz_D;
   c->nnz_M = (int64_t)h.nnz_M;

@@ -315,7 +315,8 @@ __device__ __forceinline__ unsigned long long global_ns() {
 
 // Watchdog of the persistent pair kernels: a warp stops fetching work once
 // its CTA has run longer than the budget (watchdog_us > 0) and flags
-// st->timeout; the host then reports MORTAR_ERR_TIMEOUT and the context stays
+// st->timeout; later kernels of the run that read what it leaves take no work
+// (chunk_pairs), the host reports MORTAR_ERR_TIMEOUT and the context stays
 // usable (every run starts from cleared counters).
 struct Watchdog {
   unsigned long long t0, budget_ns;

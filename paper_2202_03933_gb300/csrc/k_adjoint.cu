@@ -969,8 +969,7 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
     int ncell = 0;
     if (w + lane < records) {
       const int64_t i = r0 + w + lane;
-      const int nr = (int)(ar.rec[((i >> 5) * W + FxRecord::kInfo) * 32 + (i & 31)] & 0xff);
-      ncell = nr == kSlowPair ? 0 : (nr > 3 ? nr : (nr == 3 ? 1 : 0));
+      ncell = record_cells(ar.rec[((i >> 5) * W + FxRecord::kInfo) * 32 + (i & 31)]);
     }
     const CellSlot cs = assign_cells(ncell);
     const int64_t i = w < records ? r0 + w + cs.rec : 0;

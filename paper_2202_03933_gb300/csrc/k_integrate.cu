@@ -370,11 +370,6 @@ __device__ __forceinline__ void clip_record(bool has, int64_t p, const int32_t* 
   if (!stored) o[32 * FxRecord::kInfo] = 0;   // nr = 0
 }
 
-__device__ __forceinline__ int record_cells(long long info) {
-  const int nr = (int)(info & 0xff);
-  return nr > 3 ? nr : (nr == 3 ? 1 : 0);
-}
-
 // One cell of a record (at o, where this lane has one) per lane of the warp:
 // the cell's back-projections, then its products, then the pair's sums through
 // shared memory, and the pair's blocks.  STRIDE: the block's threads; pts:

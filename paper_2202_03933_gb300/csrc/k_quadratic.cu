@@ -304,8 +304,7 @@ __global__ void __launch_bounds__(kQThreads, 4) k_quadratic_cells(
       int ncell = 0;
       if (w + lane < records) {
         const int64_t i = r0 + w + lane;
-        const int nr = (int)(rec[((i >> 5) * FxRecord::kWords + FxRecord::kInfo) * 32 + (i & 31)] & 0xff);
-        ncell = nr > 3 ? nr : (nr == 3 ? 1 : 0);
+        ncell = record_cells(rec[((i >> 5) * FxRecord::kWords + FxRecord::kInfo) * 32 + (i & 31)]);
       }
       const CellSlot cs = assign_cells(ncell);
       const int64_t i = r0 + w + cs.rec;

@@ -315,11 +315,24 @@ __device__ __forceinline__ void fx_cell_products(const FxScales& ss, const FxSca
   }
 }
 
-// Pairs [first, first + count) that the run has; 0 after an overflow.
+// Pairs [first, first + count) that the run has; 0 after an overflow, and when
+// an earlier kernel of the run stopped early (Watchdog): the kernels of a chunk
+// hand each other an order and records, of which such a kernel has left a part
+// unwritten.  Lane 0 decides for its warp, since a block of the same kernel may
+// set the flag meanwhile.  Every lane of the warp calls it.
 __device__ __forceinline__ int64_t chunk_pairs(const DevStatus* st, int64_t pair_cap, int64_t first, int64_t count) {
-  if (st->over_pairs != 0 || st->over_bins != 0) return 0;
-  const int64_t n = (int64_t)min((unsigned long long)pair_cap, st->n_pairs) - first;
-  return max((int64_t)0, min(n, count));
+  int64_t n = 0;
+  if ((threadIdx.x & 31) == 0 && st->over_pairs == 0 && st->over_bins == 0 &&
+      *reinterpret_cast<const volatile unsigned long long*>(&st->timeout) == 0)
+    n = max((int64_t)0, min((int64_t)min((unsigned long long)pair_cap, st->n_pairs) - first, count));
+  return __shfl_sync(0xffffffffu, n, 0);
+}
+
+// Cells of a record with nr vertices: none for an empty pair's, or one that is
+// not the cell kernels' to run (nr beyond the polygon's capacity).
+__device__ __forceinline__ int record_cells(long long info) {
+  const int nr = (int)(info & 0xff);
+  return nr < 3 || nr > FxPolygon::kCap ? 0 : (nr > 3 ? nr : 1);
 }
 
 // Records per turn of a cell kernel's warp: about 16 turns a warp, 8 (a warp's
@@ -336,7 +349,7 @@ struct CellSlot {
   int cell;     // cell of this lane within its pair, -1: none
   int first;    // lane of the pair's cell 0
   int cells;    // cells of the pair
-  int taken;    // records used up by this round
+  int taken;    // records used up by this round, at least 1
 };
 // ncell: this lane's record's cells (lane i: record i of the window; at most 8)
 __device__ __forceinline__ CellSlot assign_cells(int ncell) {
@@ -350,7 +363,7 @@ __device__ __forceinline__ CellSlot assign_cells(int ncell) {
   }
   const unsigned fit = __ballot_sync(kAll, cum <= 32);   // a prefix of the lanes
   CellSlot s;
-  s.taken = __popc(fit);
+  s.taken = max(__popc(fit), 1);   // a lane's cells fit a warp (record_cells), so that 0 does not happen
   const bool has = cum <= 32 && ncell > 0;
   const int start = cum - ncell;
   const unsigned starts = __reduce_or_sync(kAll, has ? 1u << start : 0u);
