@@ -760,7 +760,9 @@ __device__ __forceinline__ bool load_pool(const long long* o, ClipPool<NS, NM>& 
   return (n >> 16 & 1) != 0;
 }
 
-constexpr int kSlowPair = 0xff;   // nr of a record whose pair the finish kernel runs in FP64
+// nr of a record whose pair the finish kernel runs in FP64: set by the clip
+// kernel, or by the cell kernel (the clip kernel has counted the pair then)
+constexpr int kSlowPair = 0xff, kSlowCounted = 0xfe;
 
 struct AdjArgs {
   const int32_t* ps;
@@ -1099,7 +1101,7 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
             __double_as_longlong(fx_to_double(hh, cr, ke - ss.shape<NS>(a) - sm.shape<NM>(l)));
       });
     }
-    if (slow && cs.cell == 0) o[32 * FxRecord::kInfo] = kSlowPair;
+    if (slow && cs.cell == 0) o[32 * FxRecord::kInfo] = kSlowCounted;
   }
 }
 
@@ -1112,7 +1114,7 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
 template <int NS, int NM, bool SEG, bool DUAL>
 __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_finish(AdjArgs g) {
   constexpr int W = SEG ? AdjRecord::kWordsSeg : AdjRecord::kWords;
-  AdjCounters ctr;
+  AdjCounters ctr, counted;
   DevStatus* st = g.st;
   const int64_t n = chunk_pairs(st, g.pair_cap, g.first, kPairChunk);
   const Watchdog wd(g.watchdog_us);
@@ -1120,9 +1122,9 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_finish(AdjArgs g) 
   while (!wd.expired(&st->timeout) && next_group(&st->pair_ctr[3], n, grp)) {   // bounded: the counter only grows
     const long long* o = g.rec + grp * (32 * W) + (threadIdx.x & 31);
     const int nr = (int)(o[32 * FxRecord::kInfo] & 0xff);
-    if (nr == kSlowPair) {
+    if (nr == kSlowPair || nr == kSlowCounted) {
       adjoint_pair_fast<NS, NM, SEG, DUAL>(o[32 * FxRecord::kPair], g.ps, g.pm, g.srec, g.xs, g.xm, g.conn_s, g.conn_m,
-                                           g.lambda, g.sl, g.gm, g.fo, ctr);
+                                           g.lambda, g.sl, g.gm, g.fo, nr == kSlowPair ? ctr : counted);
     } else if (nr != 0) {
       const int64_t p = o[32 * FxRecord::kPair];
       const int32_t s = g.ps[p], m = g.pm[p];
@@ -1159,9 +1161,9 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_finish(AdjArgs g) 
     }
     __syncwarp();
   }
-  // pairs run here in FP64; the others were counted by the clip kernel
+  // pairs that the clip kernel did not count
   block_count_add(&st->clip_overflow, ctr.clip_over);
-  block_count_add(&st->newton_fail, ctr.newton_fail);
+  block_count_add(&st->newton_fail, ctr.newton_fail + counted.newton_fail);
   block_count_add(&st->nonempty, ctr.nonempty);
   block_count_add(&st->cells, ctr.cells);
   block_count_add(&st->gauss_points, ctr.gp);
