@@ -15,7 +15,10 @@
 //   s11: CY[i][j], i, j >= 1;  sv: CY[i][0], i >= 1, v and b_s;
 //   s1: CY[0][j], u and b_m;   s0: CY[0][0] and f.
 // y is held as y 2^-ky in the pair's frame, with 2^ky a bound of the inverse
-// Jacobian over the element.
+// Jacobian over the element; on stretched elements, where one component is
+// smaller than the other by the aspect and W y (the fewest bits of the sweep) would
+// lose as many of it, times 2^l with a shift of its own for each component, from a
+// bound of that component over the pair (bound_y).
 #pragma once
 
 #include "quadrature.cuh"
@@ -34,20 +37,55 @@ struct AdjRecord {
   static constexpr int kG = 0, kMapS = 16, kMapM = 24, kVertex = 45, kH = 104;
 };
 
+// Lower bound of a bilinear map's |determinant| over the element (xi to 1.01),
+// in units of 2^-60 of the frame: it is linear in xi and eta.
+__device__ __forceinline__ float fx_smallest_det(const FxMap& m) {
+  const float d = fabsf(m.f1u * m.f2v - m.f2u * m.f1v), d1 = fabsf(m.f1u * m.f3v - m.f3u * m.f1v),
+              d2 = fabsf(m.f3u * m.f2v - m.f2u * m.f3v);
+  const float dmin = d - 1.01f * (d1 + d2);
+  return dmin > 1e-3f * d ? dmin : 0.0f;   // 0: nearly singular somewhere
+}
+
+// 2^ky above |J^-T b| for |b| <= 1/2, in the frame (99: nearly singular somewhere in the element).
+__device__ __forceinline__ int fx_inverse_exponent(const FxMap& m) {
+  if (m.affine) return m.kb;
+  const float a = fmaxf(fmaxf(fabsf(m.f1u), fabsf(m.f1v)), fmaxf(fabsf(m.f2u), fabsf(m.f2v))) +
+                  fmaxf(fabsf(m.f3u), fabsf(m.f3v));
+  const float dmin = fx_smallest_det(m);
+  if (!(dmin > 0.0f)) return 99;
+  return max(0, (int)(__float_as_uint(a / dmin) >> 23) - 126 + 30);   // f in units of 2^-30
+}
+
+// Pairs whose frame is stretched by more than 2^kMaxStretch = 2^|Eu - Ev| take
+// the FP64 path: the smaller component of the master's y is smaller by about as
+// much, either because its b is (the forms' resolution is 2^-62 of their scale)
+// or, on sheared elements, by cancellation.  From a stretch of 2^2 on, its bound
+// is used to hold it at full width.  Errors of the master's map adjoints relative
+// to their largest (400 random pairs, geometric mean; here, FP64), aspects 1, 16,
+// 100: parallelograms along the axes 1.8e-16, 1.4e-16, 2.3e-16 (2.5e-16, 2.3e-16,
+// 2.1e-16), sheared ones 2.3e-16, 5.7e-16, 2.5e-15 (3.1e-16, 6.3e-16, 2.1e-15),
+// distorted quads 6e-17, 1.3e-16, 7e-16 (1.4e-14).
+constexpr int kMaxStretch = 7;
+
 // Exponents: of the pair's forms (a Q62 value c stands for c 2^s), of y, and
 // the shifts su, sv that bring the fan's edges to full width; and of a cell's
 // sums (an integer stands for integer 2^x).
 struct AdjScale {
   int s0, sv, s1, s11, kys, kym, eu, ev;
-  int xs, xm;     // W y of slave, master
+  unsigned l;                   // shifts of y of slave u, v, master u, v, in 8 bits each
+  int xsu, xsv, xmu, xmv;       // W y of slave, master
   int xau, xav;   // half the area adjoint times an edge's u (v) component: (Q61 x Q62) / 2^64
   int xvu, xvv;   // common scale of the vertex adjoints' u and v components
   __device__ __forceinline__ long long word1() const {
     return (long long)((unsigned long long)(unsigned short)s0 | (unsigned long long)(unsigned short)sv << 16 |
                        (unsigned long long)(unsigned short)s1 << 32 | (unsigned long long)(unsigned short)s11 << 48);
   }
-  __device__ __forceinline__ long long word2() const { return kys | kym << 8 | eu << 16 | ev << 24; }
-  __device__ __forceinline__ void load(long long w1, long long w2, int ke, int E) {
+  __device__ __forceinline__ long long word2() const {
+    return (long long)((unsigned long long)(unsigned)(kys | kym << 8 | eu << 16 | ev << 24) |
+                       (unsigned long long)l << 32);
+  }
+  __device__ __forceinline__ int shift(int k) const { return (int)(l >> (8 * k) & 0xffu); }
+  __device__ __forceinline__ void load(long long w1, long long w2, int ke, int Eu, int Ev) {
     s0 = (int)(short)w1;
     sv = (int)(short)(w1 >> 16);
     s1 = (int)(short)(w1 >> 32);
@@ -56,18 +94,27 @@ struct AdjScale {
     kym = (int)(w2 >> 8) & 0xff;
     eu = (int)(w2 >> 16) & 0xff;
     ev = (int)(w2 >> 24) & 0xff;
-    const int kw = ke - 5 - E;   // weights are 4 omega w
-    xs = kw + kys + sv;
-    xm = kw + kym + s1;
-    xau = s0 + E - 60 - eu;
-    xav = s0 + E - 60 - ev;
-    xvu = max(xs, max(xm, xav)) + 2;   // the u adjoint takes the area times v components
-    xvv = max(xs, max(xm, xau)) + 2;
+    l = (unsigned)((unsigned long long)w2 >> 32);
+    const int ku = ke - 5 - Eu, kv = ke - 5 - Ev;   // weights are 4 omega w
+    xsu = ku + kys + sv - shift(0);
+    xsv = kv + kys + sv - shift(1);
+    xmu = ku + kym + s1 - shift(2);
+    xmv = kv + kym + s1 - shift(3);
+    xau = s0 + Eu - 60 - eu;
+    xav = s0 + Ev - 60 - ev;
+    xvu = max(xsu, max(xmu, xav)) + 2;   // the u adjoint takes the area times v components
+    xvv = max(xsv, max(xmv, xau)) + 2;
   }
-  // From the forms C (and, SEG, S).  False if they leave the FP32 range that the bounds are formed in.
+  __device__ __forceinline__ int xs(int c) const { return c == 0 ? xsu : xsv; }
+  __device__ __forceinline__ int xm(int c) const { return c == 0 ? xmu : xmv; }
+  // From the forms C (and, SEG, S) and the element maps, in a frame of
+  // 2^stretch = 2^(Eu - Ev).  False if the forms leave the FP32 range that the
+  // bounds are formed in, or a map is nearly singular or stretched too far.
   template <int NS, int NM, bool SEG>
-  __device__ __forceinline__ bool set(const double C[4][4], const double S[4][4]) {
-    float all = 0.0f, col = 0.0f, row = 0.0f, in_row = 0.0f, in_col[4] = {0.0f, 0.0f, 0.0f, 0.0f}, cols[4];
+  __device__ __forceinline__ bool set(const double C[4][4], const double S[4][4], const FxMap& sm, const FxMap& mm,
+                                      int stretch) {
+    float all = 0.0f, col = 0.0f, row = 0.0f, in_row = 0.0f, in_col[4] = {0.0f, 0.0f, 0.0f, 0.0f}, cols[4], rows[4];
+    rows[3] = cols[3] = 0.0f;
 #pragma unroll
     for (int j = 0; j < NM; ++j) cols[j] = 0.0f;
 #pragma unroll
@@ -84,6 +131,7 @@ struct AdjScale {
 #pragma unroll
         for (int j = 0; j < NS; ++j) r += fabsf(f32_trunc(S[i][j]));
       all += r;
+      rows[i] = r;
       if (i > 0) { row = fmaxf(row, r); in_row = fmaxf(in_row, rin); }
     }
 #pragma unroll
@@ -93,7 +141,40 @@ struct AdjScale {
     sv = max(ex(row) + 2, s11);
     s1 = max(ex(col) + 2, s11);
     s0 = max(ex(all) + 1, max(sv, s1));
-    return all < 1e37f && (all > 1e-30f || all == 0.0f);
+    if (!(all < 1e37f && (all > 1e-30f || all == 0.0f))) return false;
+    kys = fx_inverse_exponent(sm);
+    kym = fx_inverse_exponent(mm);
+    if (kys >= 20 || kym >= 20 || abs(stretch) > kMaxStretch) return false;
+    // |b| is at most the row's (column's) sum, that of xi eta added to both
+    l = 0;
+    if (abs(stretch) >= 2) {   // |b| is at most the row's (column's) sum, that of xi eta added to both
+      l = bound_y(sm, kys, rows[1] + rows[3], rows[2] + rows[3], sv);
+      l |= bound_y(mm, kym, cols[1] + cols[3], cols[2] + cols[3], s1) << 16;
+    }
+    return true;
+  }
+  // Shifts (8 bits each) that bring y = J^-T b up to 2^59 (of 2^61: the high digits
+  // of W y then add at most 2^59 to a cross sum of seven products in
+  // fx_cell_moments, whose low digits take 7 2^60), from bounds of |b|.
+  static __device__ __forceinline__ unsigned bound_y(const FxMap& m, int ky, float b0, float b1, int s) {
+    float p[2], q[2];   // |y_c| <= p[c] |b_0| + q[c] |b_1|, in units of 2^ky
+    if (m.affine) {
+      p[0] = fabsf((float)m.k1u.h) * 0x1p-29f; q[0] = fabsf((float)m.k2u.h) * 0x1p-29f;
+      p[1] = fabsf((float)m.k1v.h) * 0x1p-29f; q[1] = fabsf((float)m.k2v.h) * 0x1p-29f;
+    } else {
+      const float a3u = fabsf(m.f3u), a3v = fabsf(m.f3v);
+      const float i = __uint_as_float((unsigned)(127 + 30 - ky) << 23) / fx_smallest_det(m);
+      p[0] = (fabsf(m.f2v) + a3v) * i; q[0] = (fabsf(m.f1v) + a3v) * i;
+      p[1] = (fabsf(m.f2u) + a3u) * i; q[1] = (fabsf(m.f1u) + a3u) * i;
+    }
+    unsigned l = 0;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const float y = 1.02f * (p[c] * b0 + q[c] * b1);                 // 1.02: parameters up to 1.01, FP32 sums
+      const int e = (int)(__float_as_uint(y) >> 23) - 126 - s;         // y < 2^(e + s)
+      l |= (unsigned)min(max(-e - 2, 0), 20) << (8 * c);
+    }
+    return l;
   }
 };
 
@@ -101,19 +182,6 @@ struct AdjScale {
 __device__ __forceinline__ long long fx_down(long long v, int k) {
   k = min(max(k, 1), 62);
   return ((v >> (k - 1)) + 1) >> 1;
-}
-
-// 2^ky above |J^-T b| for |b| <= 1/2, in the frame (99: nearly singular somewhere in the element).
-// The determinant of a bilinear map is linear in xi and eta.
-__device__ __forceinline__ int fx_inverse_exponent(const FxMap& m) {
-  if (m.affine) return m.kb;
-  const float a = fmaxf(fmaxf(fabsf(m.f1u), fabsf(m.f1v)), fmaxf(fabsf(m.f2u), fabsf(m.f2v))) +
-                  fmaxf(fabsf(m.f3u), fabsf(m.f3v));
-  const float d = fabsf(m.f1u * m.f2v - m.f2u * m.f1v), d1 = fabsf(m.f1u * m.f3v - m.f3u * m.f1v),
-              d2 = fabsf(m.f3u * m.f2v - m.f2u * m.f3v);
-  const float dmin = d - 1.01f * (d1 + d2);
-  if (!(dmin > 1e-3f * d)) return 99;
-  return max(0, (int)(__float_as_uint(a / dmin) >> 23) - 126 + 30);   // f in units of 2^-30
 }
 
 // y = J^-T b 2^-ky (Q61) at xi, eta (digits of Q61), b in Q62.  Affine: B'^T b.  Bilinear: FP32 inverse Jacobian at xi, then two
@@ -288,6 +356,9 @@ __device__ __forceinline__ bool fx_cell_sweep(const FxMap& sm, const FxMap& mm, 
     long long y[4];   // J^-T b: slave u, v, master u, v
     ok &= fx_pull_back<NS>(sm, sc.kys, x1, x2, bs0, bs1, y[0], y[1]);
     ok &= fx_pull_back<NM>(mm, sc.kym, z1, z2, bm0, bm1, y[2], y[3]);
+    if (sc.l != 0u)   // stretched frames
+#pragma unroll
+      for (int k = 0; k < 4; ++k) y[k] <<= sc.shift(k);
     a.mul(om, kTri7Fx.w[q]);
     const Dg W = fx_split(a.get<4>());   // 4 omega w < 2^60
 #pragma unroll

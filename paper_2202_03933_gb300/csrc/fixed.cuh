@@ -8,9 +8,10 @@
 // are bounded -- in-plane coordinates by the pair's extent, element parameters
 // and shape functions by 1, weights by the polygon's area -- which is all that
 // fixed point needs.  Resolution: in-plane coordinates of a pair are held to
-// 2^-62 of the pair's extent (FP64 has 2^-53 of the coordinate), parameters
-// to about 2^-57; factors that stay small over a whole pair are scaled up
-// first, so that small entries keep their relative accuracy.
+// 2^-62 of the pair's extent in their direction (FP64 has 2^-53 of the
+// coordinate), parameters to about 2^-57 (2^-54 at worst, kMaxMapBits); factors
+// that stay small over a whole pair are scaled up first, so that small entries
+// keep their relative accuracy.
 //
 // A value is an int64 with a fixed number of fraction bits ("Q60" = 60).  For
 // a product it is written with balanced digits v = h 2^32 + l, l in
@@ -175,8 +176,19 @@ constexpr InvCountFx inv_count_fx() {
 }
 static __constant__ InvCountFx kInvCountFx = inv_count_fx();
 
-// One element's map in the pair's frame (in-plane coordinates times 2^-E, Q62,
-// below 1/2) and its inverse; parameters are Q61.  Affine maps: xi = B (x - c0)
+// Most bits that an element's inverse map may amplify the frame's 2^-62 by: xi
+// is then resolved to 2^-54 (FP64: 2^-53 of the element).  Elements 2^6 or so
+// smaller than the frame, and needles that lie across its axes, exceed it, and
+// the pair takes the FP64 path.  Stretched elements along the axes do not: the
+// frame has an exponent for each direction.  Parallelogram pairs (random
+// overlaps, 1.1 times as large masters, geometric mean of the block's largest
+// error over its largest entry): with one exponent for both directions and kb up
+// to 20 1.7e-16, 7.5e-16, 7e-15, 7e-14 at aspects 1, 1e3, 1e4, 1e5; FP64 2e-16
+// throughout, and this form 1.7e-16 throughout.
+constexpr int kMaxMapBits = 8;
+
+// One element's map in the pair's frame (in-plane coordinates u 2^-Eu, v 2^-Ev,
+// Q62, below 1/2) and its inverse; parameters are Q61.  Affine maps: xi = B (x - c0)
 // with B = 2^kb B', |B'| < 1 in Q61.  Bilinear maps: FP32 Newton in units of
 // 2^-30, then two steps with the residual in fixed point and the FP32
 // iteration's last Jacobian inverse G.  The last FP32 step is at most 1e-4, so
@@ -189,23 +201,26 @@ struct FxMap {
   bool affine;
   long long c0u, c0v, c1u, c1v;
   Dg k1u, k1v, k2u, k2v, k3u, k3v;   // bilinear: c1, c2, c3 (Q62); affine: the rows k1u k1v, k2u k2v of B'
-  int kb;
+  int kb;                            // 2^kb above the inverse map's entries (bilinear: at the centre)
   float f1u, f1v, f2u, f2v, f3u, f3v, b00, b01, b10, b11;
   float g00, g01, g10, g11;          // last solve's FP32 Jacobian inverse (xi per 2^-30 of the frame)
 
-  __device__ __forceinline__ void setup_bilinear(const PlaneMap& m, int E) {
+  // false if the inverse amplifies too much
+  __device__ __forceinline__ bool setup_bilinear(const PlaneMap& m, int Eu, int Ev) {
     affine = false;
-    const int kq = 62 - E;
-    c0u = fx_of_double(m.c0u, kq);
-    c0v = fx_of_double(m.c0v, kq);
-    k1u = fx_split(fx_of_double(m.c1u, kq));
-    k1v = fx_split(fx_of_double(m.c1v, kq));
-    kb = 0;
-    k2u = fx_split(fx_of_double(m.c2u, kq));
-    k2v = fx_split(fx_of_double(m.c2v, kq));
-    k3u = fx_split(fx_of_double(m.c3u, kq));
-    k3v = fx_split(fx_of_double(m.c3v, kq));
+    const int ku = 62 - Eu, kv = 62 - Ev;
+    c0u = fx_of_double(m.c0u, ku);
+    c0v = fx_of_double(m.c0v, kv);
+    k1u = fx_split(fx_of_double(m.c1u, ku));
+    k1v = fx_split(fx_of_double(m.c1v, kv));
+    k2u = fx_split(fx_of_double(m.c2u, ku));
+    k2v = fx_split(fx_of_double(m.c2v, kv));
+    k3u = fx_split(fx_of_double(m.c3u, ku));
+    k3v = fx_split(fx_of_double(m.c3v, kv));
     bilinear_floats();
+    const float b = fmaxf(fmaxf(fabsf(b00), fabsf(b01)), fmaxf(fabsf(b10), fabsf(b11)));   // xi per 2^-30
+    kb = min(max(0, (int)(__float_as_uint(b) >> 23) - 126 + 30), 31);
+    return kb <= kMaxMapBits;
   }
   // what follows from the digits
   __device__ __forceinline__ void bilinear_floats() {
@@ -217,26 +232,26 @@ struct FxMap {
     const float fd = rcp_f32(f1u * f2v - f2u * f1v);
     b00 = f2v * fd; b01 = -f2u * fd; b10 = -f1v * fd; b11 = f1u * fd;
   }
-  // i: inverse of [c1 c2] (rows); false if its scale is out of range
+  // i: inverse of [c1 c2] (rows); false if it amplifies too much
   __device__ __forceinline__ bool setup_affine(const PlaneMap& m, double i00, double i01, double i10, double i11,
-                                               int E) {
+                                               int Eu, int Ev) {
     affine = true;
-    c0u = fx_of_double(m.c0u, 62 - E);
-    c0v = fx_of_double(m.c0v, 62 - E);
-    const unsigned hi = max(max(fx_hi_abs(i00), fx_hi_abs(i01)), max(fx_hi_abs(i10), fx_hi_abs(i11)));
-    kb = max(0, fx_exponent(hi) + E);   // |B| 2^E < 2^kb
-    if (kb > 20) return false;
-    const int k = 61 + E - kb;
-    k1u = fx_split(fx_of_double(i00, k));
-    k1v = fx_split(fx_of_double(i01, k));
-    k2u = fx_split(fx_of_double(i10, k));
-    k2v = fx_split(fx_of_double(i11, k));
+    c0u = fx_of_double(m.c0u, 62 - Eu);
+    c0v = fx_of_double(m.c0v, 62 - Ev);
+    const int eu = fx_exponent(max(fx_hi_abs(i00), fx_hi_abs(i10))), ev = fx_exponent(max(fx_hi_abs(i01), fx_hi_abs(i11)));
+    kb = max(0, max(eu + Eu, ev + Ev));   // |B|, a column times 2^Eu, the other 2^Ev, < 2^kb
+    if (kb > kMaxMapBits) return false;
+    const int ku = 61 + Eu - kb, kv = 61 + Ev - kb;
+    k1u = fx_split(fx_of_double(i00, ku));
+    k1v = fx_split(fx_of_double(i01, kv));
+    k2u = fx_split(fx_of_double(i10, ku));
+    k2v = fx_split(fx_of_double(i11, kv));
     const float f = __uint_as_float((unsigned)(127 - 59 + kb) << 23);   // high words: B' 2^29, x 2^30
     b00 = (float)k1u.h * f; b01 = (float)k1v.h * f; b10 = (float)k2u.h * f; b11 = (float)k2v.h * f;
     return true;
   }
 
-  // FP32 xi of a bilinear map's point (error below 1e-6); false if the
+  // FP32 xi of a bilinear map's point (error a few 2^(kb - 24)); false if the
   // iteration did not settle.  Three Newton updates without a test settle
   // ordinary elements, and their straight code lets several points of a thread
   // overlap.
@@ -341,9 +356,9 @@ struct FxMap {
   }
 };
 
-// Left shift that brings values below `m` (> 0, with room for the FP32 error of the bound) up to 1.
-__device__ __forceinline__ int fx_room(float m) {
-  const int e = (int)(__float_as_uint(m + 1e-5f) >> 23) - 126;   // m < 2^e
+// Left shift that brings values up to `m` + err to 1 at most.
+__device__ __forceinline__ int fx_room(float m, float err) {
+  const int e = (int)(__float_as_uint(fmaxf(m, 0.0f) + err) >> 23) - 126;   // m + err < 2^e
   return min(max(-e, 0), 16);
 }
 
@@ -376,44 +391,50 @@ __device__ __forceinline__ bool fx_scales(FxMap& m, const long long* X, const lo
     s.k[0] = s.k[1] = s.k[2] = s.k[3] = 0;
     return true;
   }
+  // FP32 rounding of the parameters, whose sums' terms are up to 2^kb
+  const float err = 1e-5f + __uint_as_float((unsigned)(127 - 21 + m.kb) << 23);
   if (NEN == 4) {
-    s.k[0] = fx_room(0.5f * (1.0f - lo1)); s.k[1] = fx_room(0.5f * (1.0f + hi1));
-    s.k[2] = fx_room(0.5f * (1.0f - lo2)); s.k[3] = fx_room(0.5f * (1.0f + hi2));
+    s.k[0] = fx_room(0.5f * (1.0f - lo1), err); s.k[1] = fx_room(0.5f * (1.0f + hi1), err);
+    s.k[2] = fx_room(0.5f * (1.0f - lo2), err); s.k[3] = fx_room(0.5f * (1.0f + hi2), err);
   } else {
-    s.k[0] = fx_room(1.0f - lo3); s.k[1] = fx_room(hi1); s.k[2] = fx_room(hi2); s.k[3] = 0;
+    s.k[0] = fx_room(1.0f - lo3, err); s.k[1] = fx_room(hi1, err); s.k[2] = fx_room(hi2, err); s.k[3] = 0;
   }
   return fmaxf(fmaxf(-lo1, hi1), fmaxf(-lo2, hi2)) < 1.01f;
 }
 
-// Common frame of a pair: 2^E at least twice the largest in-plane coordinate
-// of the slave window and the largest coefficient of the master map.  Not ok
-// when one element is 2^6 or more smaller than the frame (its parameters
-// would be resolved to less than FP64 resolves them) or out of range.
+// Common frame of a pair, an exponent for each in-plane direction: 2^Eu at
+// least twice the largest u of the slave window and the largest u coefficient
+// of the master map, 2^Ev as much for v.  (The slave's first edge is along u, so
+// that stretched elements are, as a rule, along the axes.)  Not ok out of range.
 struct FxFrame {
-  int E;
+  int Eu, Ev;
   bool ok;
 };
 template <int NS, int NM>
-__device__ __forceinline__ FxFrame fx_frame(const double* __restrict__ r, const PlaneMap& s, const PlaneMap& m) {
-  unsigned hm = max(max(fx_hi_abs(m.c1u), fx_hi_abs(m.c1v)), max(fx_hi_abs(m.c2u), fx_hi_abs(m.c2v)));
-  const unsigned hs = max(max(fx_hi_abs(s.c1u), fx_hi_abs(s.c1v)), max(fx_hi_abs(s.c2u), fx_hi_abs(s.c2v)));
-  const int em = fx_exponent(hm), es = fx_exponent(hs);
-  hm = max(hm, max(fx_hi_abs(m.c0u), fx_hi_abs(m.c0v)));
-  if (NM == 4) hm = max(hm, max(fx_hi_abs(m.c3u), fx_hi_abs(m.c3v)));
+__device__ __forceinline__ FxFrame fx_frame(const double* __restrict__ r, const PlaneMap& m) {
+  unsigned hu = max(max(fx_hi_abs(m.c0u), fx_hi_abs(m.c1u)), fx_hi_abs(m.c2u));
+  unsigned hv = max(max(fx_hi_abs(m.c0v), fx_hi_abs(m.c1v)), fx_hi_abs(m.c2v));
+  if (NM == 4) {
+    hu = max(hu, fx_hi_abs(m.c3u));
+    hv = max(hv, fx_hi_abs(m.c3v));
+  }
 #pragma unroll
-  for (int k = 0; k < 2 * NS; ++k) hm = max(hm, fx_hi_abs(r[SR_PS + k]));
-  const int E = fx_exponent(hm) + 1;
-  return {E, E > -300 && E < 300 && min(em, es) > E - 7};
+  for (int k = 0; k < NS; ++k) {
+    hu = max(hu, fx_hi_abs(r[SR_PS + 2 * k]));
+    hv = max(hv, fx_hi_abs(r[SR_PS + 2 * k + 1]));
+  }
+  const int Eu = fx_exponent(hu) + 1, Ev = fx_exponent(hv) + 1;
+  return {Eu, Ev, Eu > -300 && Eu < 300 && Ev > -300 && Ev < 300};
 }
 
 // FP64 Newton from xi = 0 for a point whose fixed-point steps did not settle
 // (strongly distorted elements); false if it fails or leaves the element.
-static __device__ __noinline__ bool fx_slow_solve(PlaneMap m, int E, long long xu, long long xv, long long& xi,
-                                                  long long& eta) {
+static __device__ __noinline__ bool fx_slow_solve(PlaneMap m, int Eu, int Ev, long long xu, long long xv,
+                                                  long long& xi, long long& eta) {
   MapInverse mi;
   mi.m = m;
   double a = 0.0, b = 0.0;
-  if (!mi.newton64(fx_to_double(xu, 0, E - 62), fx_to_double(xv, 0, E - 62), a, b)) return false;
+  if (!mi.newton64(fx_to_double(xu, 0, Eu - 62), fx_to_double(xv, 0, Ev - 62), a, b)) return false;
   if (!(fabs(a) < 1.01 && fabs(b) < 1.01)) return false;
   xi = fx_of_double(a, 61);
   eta = fx_of_double(b, 61);

@@ -882,12 +882,9 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, un
               }
           }
           AdjScale sc;
-          sc.kys = fx_inverse_exponent(f.s);
-          sc.kym = fx_inverse_exponent(f.m);
           sc.eu = f.su;
           sc.ev = f.sv;
-          // out of range: multipliers beyond FP32, or nearly singular maps
-          if (sc.set<NS, NM, SEG>(C, S) && sc.kys < 20 && sc.kym < 20) {
+          if (sc.set<NS, NM, SEG>(C, S, f.s, f.m, f.Eu - f.Ev)) {
             FxRecord::store<NS, NM>(o, f, p);
             auto put = [&](int w, double v, int sc) {
               const Dg d = fx_split(fx_of_double(v, 62 - sc));
@@ -991,7 +988,7 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
     __syncthreads();
     if (ok) {
       AdjScale sc;
-      sc.load(o[32 * AdjRecord::kScales], o[32 * AdjRecord::kScales2], f.ke, f.E);
+      sc.load(o[32 * AdjRecord::kScales], o[32 * AdjRecord::kScales2], f.ke, f.Eu, f.Ev);
       ok = fx_cell_sweep<NS, NM, SEG, stride>(f.s, f.m, sc, o, weight, pts, area);
     }
     const unsigned bad = __ballot_sync(0xffffffffu, cs.cell >= 0 && !ok);
@@ -1005,7 +1002,8 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
       const long long info = o[32 * FxRecord::kInfo];
       const int nr = (int)(info & 0xff);
       AdjScale sc;
-      sc.load(o[32 * AdjRecord::kScales], o[32 * AdjRecord::kScales2], (int)(short)(info >> 32), (int)(short)(info >> 48));
+      sc.load(o[32 * AdjRecord::kScales], o[32 * AdjRecord::kScales2], FxRecord::info_ke(info), FxRecord::info_eu(info),
+              FxRecord::info_ev(info));
       // map-coefficient adjoints: minus the sums of W y (x) (1, xi, eta, xi eta), units of 2^64 of Q61 x Q61
       __syncwarp();
       if (ok) {
@@ -1034,18 +1032,19 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
         const bool neg = (a.hh - b.hh) + ((a.cr - b.cr) >> 32) < 0;
         const Dg ar2 = fx_split(neg ? -area : area);
         // one component of a vertex: the moments, and the area with the other component of an edge
-        auto part = [&](long long s, long long mv, long long e, int es, int xa, int xv) {
+        auto part = [&](int c, long long s, long long mv, long long e, int es, int xa) {
+          const int xv = c == 0 ? sc.xvu : sc.xvv;
           a.mul(ar2, fx_split(e << es));
-          return fx_down(s, xv - sc.xs) + fx_down(mv, xv - sc.xm) + fx_down(a.hh + (a.cr >> 32), xv - xa);
+          return fx_down(s, xv - sc.xs(c)) + fx_down(mv, xv - sc.xm(c)) + fx_down(a.hh + (a.cr >> 32), xv - xa);
         };
-        const long long v1u = part(r.es1[0], r.em1[0], e2v, sc.ev, sc.xav, sc.xvu);
-        const long long v1v = part(r.es1[1], r.em1[1], -e2u, sc.eu, sc.xau, sc.xvv);
-        const long long v2u = part(r.es2[0], r.em2[0], -e1v, sc.ev, sc.xav, sc.xvu);
-        const long long v2v = part(r.es2[1], r.em2[1], e1u, sc.eu, sc.xau, sc.xvv);
+        const long long v1u = part(0, r.es1[0], r.em1[0], e2v, sc.ev, sc.xav);
+        const long long v1v = part(1, r.es1[1], r.em1[1], -e2u, sc.eu, sc.xau);
+        const long long v2u = part(0, r.es2[0], r.em2[0], -e1v, sc.ev, sc.xav);
+        const long long v2v = part(1, r.es2[1], r.em2[1], e1u, sc.eu, sc.xau);
         sums[22 * stride] = v1u; sums[23 * stride] = v1v;
         sums[24 * stride] = v2u; sums[25 * stride] = v2v;
-        sums[26 * stride] = fx_down(r.s1[0], sc.xvu - sc.xs) + fx_down(r.m1[0], sc.xvu - sc.xm) - v1u - v2u;
-        sums[27 * stride] = fx_down(r.s1[1], sc.xvv - sc.xs) + fx_down(r.m1[1], sc.xvv - sc.xm) - v1v - v2v;
+        sums[26 * stride] = fx_down(r.s1[0], sc.xvu - sc.xsu) + fx_down(r.m1[0], sc.xvu - sc.xmu) - v1u - v2u;
+        sums[27 * stride] = fx_down(r.s1[1], sc.xvv - sc.xsv) + fx_down(r.m1[1], sc.xvv - sc.xmv) - v1v - v2v;
       }
       __syncwarp();
       if (ok) {
@@ -1059,7 +1058,7 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
             hh += pair[e * stride + k];
             if (!plain) cr += reinterpret_cast<const unsigned*>(pair + (16 + (i >> 1)) * stride + k)[i & 1];
           }
-          const double v = -fx_to_double(hh, cr, (plain ? 0 : 3) + (e < 8 ? sc.xs : sc.xm));
+          const double v = -fx_to_double(hh, cr, (plain ? 0 : 3) + (e < 8 ? sc.xs(e & 1) : sc.xm(e & 1)));
           o[32 * (AdjRecord::kMapS + e)] = __double_as_longlong(v);
         }
 #pragma unroll
@@ -1086,7 +1085,7 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
     {
       FxScales ss, sm;
       FxRecord::load_scales(o, ss, sm);
-      const int ke = (int)(short)(o[32 * FxRecord::kInfo] >> 32);
+      const int ke = FxRecord::info_ke(o[32 * FxRecord::kInfo]);
       FxAcc g[4][4];
       if (SEG) {
         fx_cell_products<NS, NS, true, stride>(ss, ss, weight, pts, g);

@@ -363,7 +363,7 @@ __device__ __forceinline__ void put_block(const FxAcc* __restrict__ acc, int ke,
 // Candidate pairs in chunks of kFixedPairs: 12 holds what meshes of about the
 // same size have (three by three, four by three), further chunks take the
 // points without an owner yet.  False (blocks not final) for a lane whose
-// element does not fit: degenerate, or sizes more than 2^6 apart (fx_frame).
+// element does not fit: degenerate, or a master whose map is out of range (kMaxMapBits).
 // tab: per point xi, eta, then NS products.
 template <int NS, int NM, bool SEG, bool DUAL>
 __device__ __forceinline__ bool element_fixed(bool valid, int64_t e, const int64_t* __restrict__ pair_off,
@@ -390,41 +390,40 @@ __device__ __forceinline__ bool element_fixed(bool valid, int64_t e, const int64
     int kc = ok ? (int)max((int64_t)0, min(p1 - p0, (int64_t)kFixedPairs)) : 0;
     const PlaneMap smap = kc > 0 ? slave_plane_map(r) : PlaneMap{0.0, 0.0, 1.0, 0.0, 0.0, 1.0, 0.0, 0.0};
     PlaneMap maps[kFixedPairs];
-    int E = -1000, small = 1000;
+    int Eu = -1000, Ev = -1000;
     for (int k = 0; k < kc; ++k) {
       maps[k] = master_plane_map<NM>(r, xm, conn_m, pm[p0 + k]);
-      const FxFrame f = fx_frame<NS, NM>(r, smap, maps[k]);
-      E = max(E, f.E);
-      small = min(small, fx_exponent(max(max(fx_hi_abs(maps[k].c1u), fx_hi_abs(maps[k].c1v)),
-                                         max(fx_hi_abs(maps[k].c2u), fx_hi_abs(maps[k].c2v)))));
+      const FxFrame f = fx_frame<NS, NM>(r, maps[k]);
+      Eu = max(Eu, f.Eu);
+      Ev = max(Ev, f.Ev);
     }
     __syncwarp();
-    small = min(small, fx_exponent(max(max(fx_hi_abs(smap.c1u), fx_hi_abs(smap.c1v)),
-                                       max(fx_hi_abs(smap.c2u), fx_hi_abs(smap.c2v)))));
     // det J_s = d0 + d1 xi + d2 eta, in units of 2^ED (Q61)
     const double f0 = cross2(smap.c1u, smap.c1v, smap.c2u, smap.c2v), f1 = cross2(smap.c1u, smap.c1v, smap.c3u, smap.c3v);
     const double f2 = cross2(smap.c3u, smap.c3v, smap.c2u, smap.c2v);
     const int ED = fx_exponent(fx_hi_abs(fabs(f0) + fabs(f1) + fabs(f2)));
-    if (kc > 0 && !(E > -200 && E < 200 && small > E - 7 && ED > -500 && ED < 500)) {
+    if (kc > 0 && !(Eu > -200 && Eu < 200 && Ev > -200 && Ev < 200 && ED > -500 && ED < 500)) {
       ok = false;
       kc = 0;
     }
-    if (kc == 0) E = 4;   // lanes without work run along on the unit map
+    if (kc == 0) Eu = Ev = 4;   // lanes without work run along on the unit map
     const long long d0 = fx_of_double(f0, 61 - ED);
     const Dg d1 = fx_split(fx_of_double(f1, 61 - ED)), d2 = fx_split(fx_of_double(f2, 61 - ED));
     const bool varies = NS == 4 && !(f1 == 0.0 && f2 == 0.0);
     FxMap sm;
-    sm.setup_bilinear(smap, E);
+    sm.setup_bilinear(smap, Eu, Ev);   // not inverted
     ElemCandidate cand[kFixedPairs];
     FxAcc acc[kFixedPairs][NS * NM], accD[SEG ? kFixedPairs : 1][SEG ? NS * NS : 1];
     for (int k = 0; k < kc; ++k) {
       FxMap& m = cand[k].map;
-      m.setup_bilinear(maps[k], E);   // for the box
+      const bool fits = m.setup_bilinear(maps[k], Eu, Ev);   // and for the box
       corner_range<NM>(m.c0u, m.k1u, m.k2u, m.k3u, cand[k].lo_u, cand[k].hi_u);
       corner_range<NM>(m.c0v, m.k1v, m.k2v, m.k3v, cand[k].lo_v, cand[k].hi_v);
       if (NM == 3 || map_is_affine(maps[k])) {
         const double id = 1.0 / (maps[k].c1u * maps[k].c2v - maps[k].c2u * maps[k].c1v);
-        ok &= m.setup_affine(maps[k], maps[k].c2v * id, -maps[k].c2u * id, -maps[k].c1v * id, maps[k].c1u * id, E);
+        ok &= m.setup_affine(maps[k], maps[k].c2v * id, -maps[k].c2u * id, -maps[k].c1v * id, maps[k].c1u * id, Eu, Ev);
+      } else {
+        ok &= fits;
       }
       for (int t = 0; t < NS * NM; ++t) acc[k][t].zero();
       if (SEG)
@@ -481,7 +480,7 @@ __device__ __forceinline__ bool element_fixed(bool valid, int64_t e, const int64
           bool solved = settled;
           if (NM == 3 || m.affine) m.solve_affine(xu - m.c0u, xv - m.c0v, x1, x2);
           else if (settled) solved = m.refine(xu - m.c0u, xv - m.c0v, x, y, x1, x2);
-          if (!solved) solved = fx_slow_solve(maps[k], E, xu, xv, x1, x2);
+          if (!solved) solved = fx_slow_solve(maps[k], Eu, Ev, xu, xv, x1, x2);
           constexpr long long one = 1ll << 61, tol = (long long)(kInsideTol * (double)(1ll << 61));
           const bool inside = NM == 4
               ? (x1 <= one + tol && x1 >= -(one + tol) && x2 <= one + tol && x2 >= -(one + tol))

@@ -11,7 +11,7 @@ struct FxPolygon {
   long long X[kCap], Y[kCap], A[kCap];   // vertices (Q62), cell weights omega
   long long cu, cv;                      // fan centre
   int su, sv;                            // shifts that bring the fan's edges to 2^61 .. 2^62
-  int nr, ncell, E, ke;                  // 2^ke: unit of sums of omega w N_s N_m / 2^64 with N Q61
+  int nr, ncell, Eu, Ev, ke;             // 2^ke: unit of sums of omega w N_s N_m / 2^64 with N Q61
   FxScales ss, sm;
   FxMap s, m;
 
@@ -23,9 +23,9 @@ struct FxPolygon {
   __device__ __forceinline__ int iw(int c) const { return nr > 3 ? (c + 1 == nr ? 0 : c + 1) : 2; }
 
   // From the FP64 polygon (pu, pv, n vertices).  False if the pair does not fit:
-  // elements more than 2^6 apart in size, more than 8 vertices, an element map
-  // out of range or a vertex outside its element; the caller then takes the
-  // FP64 path.  Cell areas are formed from differences scaled up to full
+  // more than 8 vertices, an element map out of range (elements about 2^6 apart
+  // in size, kMaxMapBits) or a vertex outside its element; the caller then takes
+  // the FP64 path.  Cell areas are formed from differences scaled up to full
   // width per direction (a sliver's area keeps its digits); the weights are
   // omega = area 2^t with 2^60 <= sum omega < 2^61.
   template <int NS, int NM>
@@ -36,25 +36,26 @@ struct FxPolygon {
     PlaneMap smap;
     smap.c0u = r[SR_C + 0]; smap.c0v = r[SR_C + 1]; smap.c1u = r[SR_C + 2]; smap.c1v = r[SR_C + 3];
     smap.c2u = r[SR_C + 4]; smap.c2v = r[SR_C + 5]; smap.c3u = r[SR_C + 6]; smap.c3v = r[SR_C + 7];
-    const FxFrame fr = fx_frame<NS, NM>(r, smap, mmap);
+    const FxFrame fr = fx_frame<NS, NM>(r, mmap);
     if (!fr.ok) return false;
-    E = fr.E;
+    Eu = fr.Eu;
+    Ev = fr.Ev;
     if (NM == 3 || map_is_affine(mmap)) {
       const double id = 1.0 / (mmap.c1u * mmap.c2v - mmap.c2u * mmap.c1v);
-      if (!m.setup_affine(mmap, mmap.c2v * id, -mmap.c2u * id, -mmap.c1v * id, mmap.c1u * id, E)) return false;
+      if (!m.setup_affine(mmap, mmap.c2v * id, -mmap.c2u * id, -mmap.c1v * id, mmap.c1u * id, Eu, Ev)) return false;
     } else {
-      m.setup_bilinear(mmap, E);
+      if (!m.setup_bilinear(mmap, Eu, Ev)) return false;
     }
     if (NS == 3 || r[SR_AFF] != 0.0) {
-      if (!s.setup_affine(smap, r[SR_BINV], r[SR_BINV + 1], r[SR_BINV + 2], r[SR_BINV + 3], E)) return false;
+      if (!s.setup_affine(smap, r[SR_BINV], r[SR_BINV + 1], r[SR_BINV + 2], r[SR_BINV + 3], Eu, Ev)) return false;
     } else {
-      s.setup_bilinear(smap, E);
+      if (!s.setup_bilinear(smap, Eu, Ev)) return false;
     }
     cu = 0;
     cv = 0;
     for (int k = 0; k < nr; ++k) {
-      X[k] = fx_of_double(pu[k], 62 - E);
-      Y[k] = fx_of_double(pv[k], 62 - E);
+      X[k] = fx_of_double(pu[k], 62 - Eu);
+      Y[k] = fx_of_double(pv[k], 62 - Ev);
       cu += X[k] >> 2;   // eight values below 2^61
       cv += Y[k] >> 2;
     }
@@ -91,7 +92,7 @@ struct FxPolygon {
     // sum = (total / 8) rounded down by less than 8: one more bit of room covers it
     const int t = __clzll((long long)sum) - 3 - 3 - 1;
     for (int c = 0; c < ncell; ++c) A[c] = t >= 0 ? A[c] << min(t, 62) : A[c] >> -t;
-    ke = 2 * E - 58 - t - su - sv;
+    ke = Eu + Ev - 58 - t - su - sv;
     return sum > 0 && fx_scales<NS>(s, X, Y, nr, ss) && fx_scales<NM>(m, X, Y, nr, sm);
   }
 };
@@ -126,7 +127,10 @@ struct FxRecord {
   static constexpr int kMapS = 26, kMapM = 34, kScale = 42, kPair = 43, kInfo = 44, kWords = 45;
   // words: 2k, 2k + 1: vertex k; 16 + c: weight of cell c; 24, 25: centre;
   // 26.., 34..: maps (c0, then the digits k1 k2 k3); 42: the eight factor scales; 43: pair id;
-  // 44: nr | kb_s << 8 | kb_m << 16 | affine_s << 24 | affine_m << 25 | ke << 32 | E << 48
+  // 44: nr | kb_s << 8 | kb_m << 13 | affine_s << 18 | affine_m << 19 | Ev << 20 (12 bits) | ke << 32 | Eu << 48
+  static __device__ __forceinline__ int info_ke(long long info) { return (int)(short)(info >> 32); }
+  static __device__ __forceinline__ int info_eu(long long info) { return (int)(short)(info >> 48); }
+  static __device__ __forceinline__ int info_ev(long long info) { return (int)info >> 20; }
   static __device__ __forceinline__ void store_map(long long* o, const FxMap& m, bool bilinear_possible) {
     auto put = [&](int w, Dg d) { o[32 * w] = (long long)(((unsigned long long)(unsigned)d.h << 32) | (unsigned)d.l); };
     o[0] = m.c0u;
@@ -162,10 +166,11 @@ struct FxRecord {
     o[32 * 24] = f.cu;
     o[32 * 25] = f.cv;
     o[32 * kPair] = pair;
-    o[32 * kInfo] = (long long)((unsigned long long)(unsigned)(f.nr | f.s.kb << 8 | f.m.kb << 16 | (f.s.affine ? 1 : 0) << 24 |
-                                                               (f.m.affine ? 1 : 0) << 25) |
+    o[32 * kInfo] = (long long)((unsigned long long)((unsigned)(f.nr | f.s.kb << 8 | f.m.kb << 13 |
+                                                                (f.s.affine ? 1 : 0) << 18 | (f.m.affine ? 1 : 0) << 19) |
+                                                     (unsigned)f.Ev << 20) |
                                 (unsigned long long)(unsigned short)f.ke << 32 |
-                                (unsigned long long)(unsigned short)f.E << 48);
+                                (unsigned long long)(unsigned short)f.Eu << 48);
     unsigned long long sc = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k)
@@ -181,7 +186,7 @@ struct FxRecord {
 struct FxView {
   const long long* o;
   long long cu, cv;
-  int nr, ncell, E, ke;
+  int nr, ncell, Eu, Ev, ke;
   FxScales ss, sm;
   FxMap s, m;
   __device__ __forceinline__ long long x(int k) const { return o[64 * k]; }
@@ -195,12 +200,13 @@ struct FxView {
     const long long info = o[32 * FxRecord::kInfo];
     nr = (int)(info & 0xff);
     ncell = nr > 3 ? nr : 1;
-    s.kb = (int)(info >> 8) & 0xff;
-    m.kb = (int)(info >> 16) & 0xff;
-    s.affine = (info >> 24) & 1;
-    m.affine = (info >> 25) & 1;
-    ke = (int)(short)(info >> 32);
-    E = (int)(short)(info >> 48);
+    s.kb = (int)(info >> 8) & 31;
+    m.kb = (int)(info >> 13) & 31;
+    s.affine = (info >> 18) & 1;
+    m.affine = (info >> 19) & 1;
+    ke = FxRecord::info_ke(info);
+    Eu = FxRecord::info_eu(info);
+    Ev = FxRecord::info_ev(info);
     FxRecord::load_scales(o, ss, sm);
     cu = o[32 * 24];
     cv = o[32 * 25];
@@ -251,11 +257,11 @@ __device__ __forceinline__ bool fx_back_project(F& f, int c, const double* __res
     long long xi, eta;
     long long* o = pts + (4 * q) * stride;
     if (!f.s.template solve<NS>(xu, xv, xi, eta))
-      ok &= fx_slow_solve(slave_plane_map(r), f.E, xu, xv, xi, eta);
+      ok &= fx_slow_solve(slave_plane_map(r), f.Eu, f.Ev, xu, xv, xi, eta);
     o[0] = xi;
     o[stride] = eta;
     if (!f.m.template solve<NM>(xu, xv, xi, eta))
-      ok &= fx_slow_solve(master_plane_map<NM>(r, xm, conn_m, m), f.E, xu, xv, xi, eta);
+      ok &= fx_slow_solve(master_plane_map<NM>(r, xm, conn_m, m), f.Eu, f.Ev, xu, xv, xi, eta);
     o[2 * stride] = xi;
     o[3 * stride] = eta;
   }
