@@ -258,9 +258,13 @@ __global__ void __launch_bounds__(kThreads) k_integrate_elembased(
 // element's edge, the fixed-point back-projection (2^-57 in xi) for the others
 // with the same 1e-10 tolerance.  The owner's sums stay in registers while
 // consecutive points have the same owner, and are exchanged with thread-local
-// memory when it changes.  Digits: the products' low x low terms are kept and a
-// sum holds 96 bits, so an entry's error is the table's rounding, 2^-62-boost
-// of the element's weight a product.
+// memory when it changes.  Digits: a product's size goes down to 2^-22 of the
+// largest at a rule's corners, so the table, and its products with |det J_s|,
+// have a third digit (32 more bits), the products' low terms are kept and a sum
+// holds 96 bits: an entry that only such points contribute to has all the bits
+// that FP64 gives it.  (Blocks of at most four points, n = 12, parallelograms:
+// geometric mean of the largest relative error of an entry 7e-14 with two
+// digits, 4e-15 with three, FP64 3e-15.)
 // 600x520 quad4, n = 8, dual: 5.95 ms in FP64 (FP64 pipe), 3.14 ms here, of which
 // the instructions would take half: the candidates' maps and the exchanged sums
 // (about 2 KB a thread) miss L1 in 58 % of their sectors.  Sums added in memory
@@ -317,15 +321,38 @@ __device__ __forceinline__ void exchange(FxAcc g[4][4], FxAcc* __restrict__ from
       g[a][l] = to[NC * a + l];
     }
 }
+// Three digits: d + x 2^-32 in units of the last place of d, |x| <= 2^31.
+struct Dg3 {
+  Dg d;
+  int x;
+};
 template <int NR, int NC>
-__device__ __forceinline__ void add_products(FxAcc g[4][4], const Dg* Ns, const Dg* Nc) {
+__device__ __forceinline__ void add_products(FxAcc g[4][4], const Dg3* Ns, const Dg* Nc) {
 #pragma unroll
   for (int a = 0; a < NR; ++a)
 #pragma unroll
     for (int l = 0; l < NC; ++l) {
-      g[a][l].mac(Ns[a], Nc[l]);
-      g[a][l].low(Ns[a], Nc[l]);
+      g[a][l].mac(Ns[a].d, Nc[l]);
+      g[a][l].cr += mul_hi(Ns[a].d.l, Nc[l].l) + mul_hi(Ns[a].x, Nc[l].h);   // below 2^30 + 2^29
     }
+}
+// t W / 2^61 with t of three digits, W Q61 and at most 1
+__device__ __forceinline__ Dg3 weigh(Dg t, int x, Dg W) {
+  FxAcc a;
+  a.mul(t, W);
+  const long long low = mad_wide(x, W.h, mul_wide(t.l, W.l));   // below 2^62 + 2^60
+  a.cr += low >> 32;
+  const unsigned digit = shift_in((unsigned)low, (unsigned)a.cr, 3);
+  return {fx_split(a.get<3>() + (digit >> 31)), (int)digit};
+}
+// Table entry of the product v = w N_a / sum w (at least 0, below 2^-2): digits of v 2^k, balanced.
+__device__ __forceinline__ void put_product(double v, int k, long long& t, int& x) {
+  t = fx_of_double(v, k);
+  const double up = __longlong_as_double((long long)(1023 + k) << 52);
+  const double rest = v * up - (double)t;   // exact: not zero only where t has fewer bits than v
+  const unsigned d = (unsigned)(long long)(rest * 0x1p32);
+  t += d >> 31;
+  x = (int)d;
 }
 template <int NR, int NC>
 __device__ __forceinline__ void carry_all(FxAcc g[4][4]) {
@@ -358,13 +385,25 @@ __device__ __forceinline__ void put_block(const FxAcc* __restrict__ acc, int ke,
     }
 }
 
+// The table: per point xi, eta, the NS products, and their third digits (two a word).
+template <int NS>
+constexpr int kTableWords = 2 + NS + (NS + 1) / 2;
+template <int NS>
+__device__ __forceinline__ void put_point(long long* t, double xi, double eta, double w, int boost) {
+  t[0] = fx_of_double(xi, 61);
+  t[1] = fx_of_double(eta, 61);
+  int* third = reinterpret_cast<int*>(t + 2 + NS);
+  for (int a = 0; a < NS; ++a)
+    put_product(w * (NS == 4 ? 0.25 : 2.0) * rule_shape(NS, a, xi, eta), 62 + boost, t[2 + a], third[a]);
+}
+
 // One element per lane, the warp in step (__syncwarp between the parts, which
 // lanes with another owner or candidate would otherwise run one by one).
 // Candidate pairs in chunks of kFixedPairs: 12 holds what meshes of about the
 // same size have (three by three, four by three), further chunks take the
 // points without an owner yet.  False (blocks not final) for a lane whose
 // element does not fit: degenerate, or a master whose map is out of range (kMaxMapBits).
-// tab: per point xi, eta, then NS products.
+// tab: the table (kTableWords).
 template <int NS, int NM, bool SEG, bool DUAL>
 __device__ __forceinline__ bool element_fixed(bool valid, int64_t e, const int64_t* __restrict__ pair_off,
                                               const int32_t* __restrict__ pm, const double* __restrict__ srec,
@@ -441,7 +480,7 @@ __device__ __forceinline__ bool element_fixed(bool valid, int64_t e, const int64
     unsigned got[3] = {0u, 0u, 0u};   // points of pair k in byte k (at most 144)
 #pragma unroll 1
     for (int q = 0; q < nq; ++q) {
-      const long long* t = tab + (2 + NS) * q;
+      const long long* t = tab + kTableWords<NS> * q;
       const long long xs = t[0], es = t[1];
       long long xu, xv;
       sm.residual(-sm.c0u, -sm.c0v, xs, es, xu, xv);
@@ -512,14 +551,11 @@ __device__ __forceinline__ bool element_fixed(bool valid, int64_t e, const int64
         got[1] += owner >= 4 && owner < 8 ? one : 0u;
         got[2] += owner >= 8 ? one : 0u;
         if (more) taken[q >> 5] |= 1u << (q & 31);
-        Dg Ns[4], Nc[4];
+        Dg3 Ns[4];
+        Dg Nc[4];
+        const int* third = reinterpret_cast<const int*>(t + 2 + NS);
 #pragma unroll
-        for (int i = 0; i < NS; ++i) {
-          const Dg T = fx_split(t[2 + i]);
-          a.mul(T, W);
-          a.low(T, W);
-          Ns[i] = fx_split(a.get<3>());
-        }
+        for (int i = 0; i < NS; ++i) Ns[i] = weigh(fx_split(t[2 + i]), third[i], W);
         fx_shape<NM>(none, x1, x2, Nc);
         add_products<NS, NM>(g, Ns, Nc);
         if (SEG) {
@@ -566,11 +602,7 @@ __global__ void __launch_bounds__(kThreads, SEG ? 2 : 3) k_integrate_elembased_f
     const int i = q / n, j = q - i * n;
     double xi, eta, w;
     rule_point(NS, rule, n, n * i + (i & 1 ? n - 1 - j : j), xi, eta, w);
-    long long* t = tab + (2 + NS) * q;
-    t[0] = fx_of_double(xi, 61);
-    t[1] = fx_of_double(eta, 61);
-    for (int a = 0; a < NS; ++a)
-      t[2 + a] = fx_of_double(w * (NS == 4 ? 0.25 : 2.0) * rule_shape(NS, a, xi, eta), 62 + boost);
+    put_point<NS>(tab + kTableWords<NS> * q, xi, eta, w, boost);
   }
   __syncthreads();
   unsigned long long n_live = 0, n_gp = 0;
@@ -599,7 +631,7 @@ void launch_nsnm(mortar_ctx* c, const RunParams& rp) {
   };
   auto go = [&](auto fixed, auto fp64) {
     if (boost >= 0) {
-      const size_t shm = sizeof(long long) * (2 + NS) * n * n;
+      const size_t shm = sizeof(long long) * kTableWords<NS> * n * n;
       fixed<<<grid(fixed, shm), kThreads, shm, c->stream>>>(
           c->pair_off.as<int64_t>(), c->pairs_m.as<int32_t>(), c->srec.as<double>(), c->xm.as<double>(),
           c->conn_m.as<int32_t>(), c->rule_1d.as<double>(), n, boost, c->Es, c->Mblk.as<double>(),
