@@ -14,9 +14,15 @@
 // memory, the per-point adjoints of the four seeds are accumulated side by
 // side (their map-coefficient adjoints in shared memory), and only the reverse
 // of the clip and of the projection runs once per seed.  The seeds are the
-// monomials 1, xi, eta, xi eta, of which the N_e are combinations: a seed's
+// monomials 1, x, y, x y (triangles: 1, x, y) in coordinates of the slave element
+// that are zero at its corner nearest to the pair's polygon and one at that
+// corner's neighbours (Corner), of which the N_e are combinations: a seed's
 // point adjoint is then a product or two, and the slave map's adjoints of all
-// four follow from 12 moments.  Bound by the FP64 pipe (about 75 % busy);
+// four follow from 12 moments.  Seen from that corner, N_e that are small all
+// over the pair are small seeds themselves or differences in which nothing
+// cancels, so that a row that is small keeps its digits: with a pair of 1 % of
+// the element's size at a corner, the far node's row has errors up to 3.2e-13 of
+// itself, as with the N_e as seeds, and 2.9e-12 with monomials about the centre.  Bound by the FP64 pipe (about 75 % busy);
 // 300x260 quads, dual (0.31 M pairs): 21.7 ms with the N_e as seeds, 18.7 ms
 // this way, square roots and divisions of the plane once per pair.
 //
@@ -57,10 +63,89 @@ struct TanArgs {
   int32_t watchdog_us;
 };
 
+// Corner of a slave element, and the coordinates (x, y) about it: quad4
+// x = (1 -+ xi) / 2, y = (1 -+ eta) / 2; tri3 the barycentric coordinates of the
+// two other corners.
+template <int NS>
+struct Corner {
+  bool rx = false, ry = false;   // quad4: at xi = 1, at eta = 1
+  int k = 0;                     // tri3: corner
+
+  __device__ __forceinline__ Corner(double xi, double eta) {
+    if constexpr (NS == 4) {
+      rx = xi > 0.0;
+      ry = eta > 0.0;
+    } else {
+      const double n0 = 1.0 - xi - eta;
+      k = xi > n0 ? (eta > xi ? 2 : 1) : (eta > n0 ? 2 : 0);
+    }
+  }
+  __device__ __forceinline__ void coordinates(double xi, double eta, double& x, double& y) const {
+    if constexpr (NS == 4) {
+      x = 0.5 * (rx ? 1.0 - xi : 1.0 + xi);
+      y = 0.5 * (ry ? 1.0 - eta : 1.0 + eta);
+    } else {
+      const double n0 = 1.0 - xi - eta;
+      x = k == 0 ? xi : (k == 1 ? eta : n0);
+      y = k == 0 ? eta : (k == 1 ? n0 : xi);
+    }
+  }
+  // rows of the inverse Jacobian of (xi, eta) to those of (x, y)
+  __device__ __forceinline__ void rows(double* a) const {
+    if constexpr (NS == 4) {
+      const double f = rx ? -0.5 : 0.5, g = ry ? -0.5 : 0.5;
+      a[0] *= f; a[1] *= f; a[2] *= g; a[3] *= g;
+    } else {
+      const double b0 = -a[0] - a[2], b1 = -a[1] - a[3];
+      const double x0 = k == 0 ? a[0] : (k == 1 ? a[2] : b0), x1 = k == 0 ? a[1] : (k == 1 ? a[3] : b1);
+      const double y0 = k == 0 ? a[2] : (k == 1 ? b0 : a[0]), y1 = k == 0 ? a[3] : (k == 1 ? b1 : a[1]);
+      a[0] = x0; a[1] = x1; a[2] = y0; a[3] = y1;
+    }
+  }
+  // values at the corner, its neighbours in x and y and (quad4) the opposite corner <-> in node order
+  __device__ __forceinline__ void to_nodes(double c, double x, double y, double o, double* n) const {
+    if constexpr (NS == 4) {
+      const double p = rx ? x : c, q = rx ? c : x, r = rx ? o : y, t = rx ? y : o;   // xi = -1, 1; then the far eta's
+      n[0] = ry ? r : p; n[1] = ry ? t : q; n[2] = ry ? q : t; n[3] = ry ? p : r;
+    } else {
+      n[0] = k == 0 ? c : (k == 1 ? y : x);
+      n[1] = k == 0 ? x : (k == 1 ? c : y);
+      n[2] = k == 0 ? y : (k == 1 ? x : c);
+      n[3] = 0.0;
+    }
+  }
+  // N_e of the seeds' values f: rows, and (transposed coefficients) the nodes' adjoints of a map's coefficients
+  __device__ __forceinline__ void nodal(const double* f, double* n) const {
+    if constexpr (NS == 4) {
+      const double x = f[1] - f[3], y = f[2] - f[3];
+      to_nodes((f[0] - f[1]) - y, x, y, f[3], n);
+    } else {
+      to_nodes(f[0] - f[1] - f[2], f[1], f[2], 0.0, n);
+    }
+  }
+  // coefficients in the seeds of the field with nodal values n
+  __device__ __forceinline__ void coefficients(const double* n, double* f) const {
+    if constexpr (NS == 4) {
+      const double p = ry ? n[3] : n[0], q = ry ? n[2] : n[1], r = ry ? n[0] : n[3], t = ry ? n[1] : n[2];
+      const double c = rx ? q : p, x = rx ? p : q, y = rx ? t : r, o = rx ? r : t;
+      f[0] = c;
+      f[1] = x - c;
+      f[2] = y - c;
+      f[3] = (c - x) + (o - y);
+    } else {
+      const double c = k == 0 ? n[0] : (k == 1 ? n[1] : n[2]);
+      f[0] = c;
+      f[1] = (k == 0 ? n[1] : (k == 1 ? n[2] : n[0])) - c;
+      f[2] = (k == 0 ? n[2] : (k == 1 ? n[0] : n[1])) - c;
+      f[3] = 0.0;
+    }
+  }
+};
+
 // Quadrature-point data one lane computes and the other two lanes of its
 // pair group read (shared memory), what does not depend on the component:
-// back-projections and their products, and W J_s^-1, -W J_m^-1 with the
-// seeds' scale (a quarter on quad4 slaves).
+// the seeds, the master's back-projection and its product, and W J_s^-1 (rows of
+// the corner's coordinates), -W J_m^-1.
 struct GPX {
   double s1, s2, s12, m1, m2, m12;
   double a[4], b[4];
@@ -80,10 +165,10 @@ __device__ __forceinline__ void mono_grad(const double* y, double x1, double x2,
 }
 
 // Accumulators of a thread (shared memory).  Slave side, element D: moments of
-// su_1, su_2 = W J_s^-T e_1, e_2 times Z, with (1, xi, eta, xi eta) and, on
-// quad4, (eta^2, xi eta^2) for su_1, (xi^2, xi^2 eta) for su_2, from which the
-// map adjoints of all seeds follow (grad xi eta = eta e_1 + xi e_2); segment D:
-// the map adjoints themselves.  Then the master map adjoints.
+// su_1, su_2 = W J_s^-T e_1, e_2 times Z, with (1, x, y, x y) and, on quad4,
+// (y^2, x y^2) for su_1, (x^2, x^2 y) for su_2, from which the map adjoints of
+// all seeds follow (grad x y = y e_1 + x e_2); segment D: the map adjoints
+// themselves.  Then the master map adjoints.
 template <int NS, bool SEG>
 constexpr int kSlaveSums = SEG ? 8 * NS : (NS == 4 ? 24 : 12);
 template <int NS, int NM, bool SEG>
@@ -107,10 +192,8 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
   const int32_t* cs = g.conn_s + (int64_t)NS * s;
   const int32_t* cm = g.conn_m + (int64_t)NM * m;
   double yS[4] = {0, 0, 0, 0}, yM[4] = {0, 0, 0, 0};
-  {   // monomial coefficients of the held fields
+  {   // monomial coefficients of the held field
     double y[4] = {0, 0, 0, 0};
-    for (int a = 0; a < NS; ++a) y[a] = g.ys[3 * (int64_t)cs[a] + cp];
-    if (SEG) nodal_to_mono<NS>(y, yS);
     for (int l = 0; l < NM; ++l) y[l] = g.ym[3 * (int64_t)cm[l] + cp];
     nodal_to_mono<NM>(y, yM);
   }
@@ -161,6 +244,21 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
     cv = sv * kInvCount[nr];
     ncell = nr;
   }
+  const Corner<NS> corner = [&] {   // nearest to the polygon's vertex mean (distorted elements: by the map's linear part)
+    double u = cu - smap.c0u, v = cv - smap.c0v;
+    if (nr == 3) {
+      u = (1.0 / 3.0) * (clip.u(0) + clip.u(1) + clip.u(2)) - smap.c0u;
+      v = (1.0 / 3.0) * (clip.v(0) + clip.v(1) + clip.v(2)) - smap.c0v;
+    }
+    const float fu = f32_trunc(u) * si.scf, fv = f32_trunc(v) * si.scf;
+    return si.affine ? Corner<NS>(si.i00 * u + si.i01 * v, si.i10 * u + si.i11 * v)
+                     : Corner<NS>(f64_of_f32(si.b00 * fu + si.b01 * fv), f64_of_f32(si.b10 * fu + si.b11 * fv));
+  }();
+  if (SEG) {
+    double y[4] = {0, 0, 0, 0};
+    for (int a = 0; a < NS; ++a) y[a] = g.ys[3 * (int64_t)cs[a] + cp];
+    corner.coefficients(y, yS);
+  }
   if (!live) ncell = 0;
   constexpr int KS = kSlaveSums<NS, SEG>, KM = NM == 4 ? 8 : 6;   // master sums per seed
   for (int i = 0; i < KS + KM * NS; ++i) acc[i * kTanThreads] = 0.0;
@@ -194,7 +292,6 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
       if (cell_ok && qo < 7) {
         double l1, l2, w;
         tri7_point(qo, l1, l2, w);
-        if (NS == 4) w *= 0.25;
         const double W = w * area;
         const double xu = au + l1 * e1u + l2 * e2u;
         const double xv = av + l1 * e1v + l2 * e2v;
@@ -202,15 +299,18 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
         double xs1, xs2, xm1, xm2, a00, a01, a10, a11;
         if (!si.solve(xu, xv, xs1, xs2)) newton_fail++;
         if (!mi.solve(xu, xv, xm1, xm2)) newton_fail++;
-        o.s1 = xs1; o.s2 = xs2; o.s12 = xs1 * xs2;
+        double x, y;
+        corner.coordinates(xs1, xs2, x, y);
+        o.s1 = x; o.s2 = y; o.s12 = x * y;
         o.m1 = xm1; o.m2 = xm2; o.m12 = xm1 * xm2;
         si.jinv(xs1, xs2, a00, a01, a10, a11);
         o.a[0] = W * a00; o.a[1] = W * a01; o.a[2] = W * a10; o.a[3] = W * a11;
+        corner.rows(o.a);
         mi.jinv(xm1, xm2, a00, a01, a10, a11);
         o.b[0] = -W * a00; o.b[1] = -W * a01; o.b[2] = -W * a10; o.b[3] = -W * a11;
         if (NS == 4 && !SEG) {
-          o.s11 = xs1 * xs1; o.s22 = xs2 * xs2;
-          o.s122 = o.s12 * xs2; o.s112 = o.s12 * xs1;
+          o.s11 = x * x; o.s22 = y * y;
+          o.s122 = o.s12 * y; o.s112 = o.s12 * x;
         }
       }
       __syncwarp();
@@ -224,7 +324,7 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
         const double s1 = x.s1, s2 = x.s2, s12 = x.s12, m1 = x.m1, m2 = x.m2, m12 = x.m12;
         double Z = -mono_value<NM>(yM, m1, m2, m12);
         if (SEG) Z += mono_value<NS>(yS, s1, s2, s12);
-        const double wZ = (NS == 4 ? 0.25 * w : w) * Z;
+        const double wZ = w * Z;
         arb[0] += wZ;
         arb[1] = fma(wZ, s1, arb[1]);
         arb[2] = fma(wZ, s2, arb[2]);
@@ -232,7 +332,7 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
         // J_m^-T (adjoint of xi_m) of the seed 1
         double g0, g1;
         mono_grad<NM>(yM, m1, m2, g0, g1);
-        double tu[4], tv[4], su[4], sv[4];   // master and slave point adjoints of the seeds 1, xi, eta, xi eta
+        double tu[4], tv[4], su[4], sv[4];   // master and slave point adjoints of the seeds 1, x, y, x y
         tu[0] = fma(x.b[0], g0, x.b[2] * g1);
         tv[0] = fma(x.b[1], g0, x.b[3] * g1);
         tu[1] = s1 * tu[0]; tv[1] = s1 * tv[0];
@@ -339,7 +439,7 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
     Y[l] = v3(g.xm[3 * n], g.xm[3 * n + 1], g.xm[3 * n + 2]);
   }
   const PlaneBasis<NS> basis(X, t1, t2, n0);
-  double Ks[NS][24];   // rows of the seeds 1, xi, eta, xi eta (a quarter of them on quad4)
+  double Ks[NS][24];   // rows of the seeds
 #pragma unroll 1
   for (int e = 0; e < NS; ++e) {
     double sbu[4] = {0, 0, 0, 0}, sbv[4] = {0, 0, 0, 0}, mbu[4] = {0, 0, 0, 0}, mbv[4] = {0, 0, 0, 0};
@@ -355,13 +455,20 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
       } else {
         if (e == 0) smb[k] = 0.0;
         else if (e < 3) smb[k] = -sum(12 * (e - 1) + k);
-        else   // eta su_1 + xi su_2 with 1, xi, eta, xi eta
+        else   // y su_1 + x su_2 with 1, x, y, x y
           smb[k] = -(sum((k < 2 ? 4 : (k < 4 ? 6 : (k < 6 ? 8 : 10))) + c) +
                      sum(12 + (k < 2 ? 2 : (k < 4 ? 8 : (k < 6 ? 6 : 10))) + c));
       }
       mmb[k] = k < KM ? -sum(KS + KM * e + k) : 0.0;
     }
-    map_coeff_reverse<NS>(smb, sbu, sbv);
+    {
+      const double cbu_e[4] = {smb[0], smb[2], smb[4], smb[6]}, cbv_e[4] = {smb[1], smb[3], smb[5], smb[7]};
+      double n[4];
+      corner.nodal(cbu_e, n);
+      for (int a = 0; a < NS; ++a) sbu[a] += n[a];
+      corner.nodal(cbv_e, n);
+      for (int a = 0; a < NS; ++a) sbv[a] += n[a];
+    }
     map_coeff_reverse<NM>(mmb, mbu, mbv);
     double gX[4][3], gY[4][3];
     for (int a = 0; a < 4; ++a)
@@ -376,21 +483,12 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
         Ks[e][12 + 3 * a + d] = gY[a][d];
       }
   }
-  // N_e from the seeds: corners (-1,-1), (1,-1), (1,1), (-1,1) of quad4; (1 - xi - eta, xi, eta) of tri3
-  auto nodal = [&](const double* f, double* out) {
-    if constexpr (NS == 4) {
-      const double a = f[0] - f[2], b = f[1] - f[3], d = f[0] + f[2], e = f[1] + f[3];
-      out[0] = a - b; out[1] = a + b; out[2] = d + e; out[3] = d - e;
-    } else {
-      out[0] = f[0] - f[1] - f[2]; out[1] = f[1]; out[2] = f[2]; out[3] = 0.0;
-    }
-  };
   double AT[4][4];   // dual: rows of A in the seeds
   if (DUAL)
     for (int a = 0; a < NS; ++a) {
       double v[4];
-      for (int e = 0; e < NS; ++e) v[e] = (NS == 4 ? 4.0 : 1.0) * r[SR_A + 4 * a + e];
-      nodal_to_mono<NS>(v, AT[a]);
+      for (int e = 0; e < NS; ++e) v[e] = r[SR_A + 4 * a + e];
+      corner.coefficients(v, AT[a]);
     }
   for (int k = 0; k < 24; ++k) {
     double f[4], row[4];
@@ -402,13 +500,13 @@ __device__ void tangent_pair(const TanArgs& g, int64_t p, int cp, bool live, dou
         row[a] = v;
       }
     } else {
-      nodal(f, row);
+      corner.nodal(f, row);
     }
     for (int a = 0; a < 4; ++a) __stcs(kout + 72 * a + k, a < NS ? row[a] : 0.0);
   }
   if (DUAL) {
     double On[4];
-    nodal(O, On);
+    corner.nodal(O, On);
     for (int e = 0; e < 4; ++e) __stcs(g.Op + 12 * p + 3 * e + cp, e < NS ? On[e] : 0.0);
   }
 }
