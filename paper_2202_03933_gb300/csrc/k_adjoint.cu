@@ -469,9 +469,10 @@ __device__ __forceinline__ void adjoint_empty(int64_t p, const FwdOut& fo) {
 //    Newton + one Newton step on the FP64 residual), and the
 //    implicit-function step applies the FP64 inverse Jacobian at the
 //    converged xi (MapInverse::jinvT);
-//  * the clip is recorded as a compact vertex pool (ClipPool).
+//  * the clip is the record's vertex pool (ClipPool).
 template <int NS, int NM, bool SEG, bool DUAL>
-__device__ __noinline__ void adjoint_pair_fast(int64_t p, const int32_t* __restrict__ ps, const int32_t* __restrict__ pm,
+__device__ __noinline__ void adjoint_pair_fast(int64_t p, const ClipPool<NS, NM>& cp, bool mrev,
+                                  const int32_t* __restrict__ ps, const int32_t* __restrict__ pm,
                                   const double* __restrict__ srec, const double* __restrict__ xs,
                                   const double* __restrict__ xm, const int32_t* __restrict__ conn_s,
                                   const int32_t* __restrict__ conn_m, const double* __restrict__ lambda,
@@ -499,12 +500,8 @@ __device__ __noinline__ void adjoint_pair_fast(int64_t p, const int32_t* __restr
   PlaneMap smap;
   smap.c0u = r[SR_C + 0]; smap.c0v = r[SR_C + 1]; smap.c1u = r[SR_C + 2]; smap.c1v = r[SR_C + 3];
   smap.c2u = r[SR_C + 4]; smap.c2v = r[SR_C + 5]; smap.c3u = r[SR_C + 6]; smap.c3v = r[SR_C + 7];
-  const bool mrev = polygon_reversed<NM>(mu, mv);
-  // ---- forward clip recorded as a vertex pool, and merge (same decisions as clip_polygon)
-  ClipPool<NS, NM> cp;
-  const bool nonempty = cp.run(r, mu, mv, mrev, ctr.clip_over);
   const int nr = cp.nr;
-  if (nonempty) {
+  {
     // monomial coefficients and the pair's bilinear forms
     {
       V3 X[4], Y[4], lam[4], Lam[4], LM[4], YM[4];
@@ -715,8 +712,6 @@ ctr.cells++; ctr.gp += 7;
     adjoint_blocks<NS, NM, SEG, DUAL>(p, r, G, H, fo);
     adjoint_finish<NS, NM, SEG>(p, cs, cm, r, xs, xm, Lam, cp, Bu, Bv, mrev, smb, mmb, G, H, sl_out, gm_out);
     ctr.nonempty++;
-  } else {
-    adjoint_empty<SEG>(p, fo);
   }
 }
 
@@ -952,24 +947,30 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
   int64_t r0 = 0;
   int records = 0, w = 0;
   bool more = true;
-  for (;;) {   // bounded: the shared counter only grows
-    if (w >= records && more) {
-      unsigned long long g0 = ~0ull >> 1;
-      if (!wd.expired(&st->timeout)) {
-        if (lane == 0) g0 = atomicAdd(&st->pair_ctr[2], (unsigned long long)turn);
-        g0 = __shfl_sync(0xffffffffu, g0, 0);
+  for (;;) {
+    int ncell = 0;
+    for (;;) {   // to the next records with cells; bounded: the shared counter only grows
+      if (w >= records) {
+        if (!more) break;
+        unsigned long long g0 = ~0ull >> 1;
+        if (!wd.expired(&st->timeout)) {
+          if (lane == 0) g0 = atomicAdd(&st->pair_ctr[2], (unsigned long long)turn);
+          g0 = __shfl_sync(0xffffffffu, g0, 0);
+        }
+        more = (int64_t)g0 < n;
+        r0 = (int64_t)g0;
+        records = more ? (int)min((int64_t)turn, n - r0) : 0;
+        w = 0;
+        continue;
       }
-      more = (int64_t)g0 < n;
-      r0 = (int64_t)g0;
-      records = more ? (int)min((int64_t)turn, n - r0) : 0;
-      w = 0;
+      if (w + lane < records) {
+        const int64_t i = r0 + w + lane;
+        ncell = record_cells(ar.rec[((i >> 5) * W + FxRecord::kInfo) * 32 + (i & 31)]);
+      }
+      if (__any_sync(0xffffffffu, ncell > 0)) break;
+      w += 32;
     }
     if (!__syncthreads_or(w < records)) break;
-    int ncell = 0;
-    if (w + lane < records) {
-      const int64_t i = r0 + w + lane;
-      ncell = record_cells(ar.rec[((i >> 5) * W + FxRecord::kInfo) * 32 + (i & 31)]);
-    }
     const CellSlot cs = assign_cells(ncell);
     const int64_t i = w < records ? r0 + w + cs.rec : 0;
     w += cs.taken;
@@ -1122,7 +1123,9 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_finish(AdjArgs g) 
     const long long* o = g.rec + grp * (32 * W) + (threadIdx.x & 31);
     const int nr = (int)(o[32 * FxRecord::kInfo] & 0xff);
     if (nr == kSlowPair || nr == kSlowCounted) {
-      adjoint_pair_fast<NS, NM, SEG, DUAL>(o[32 * FxRecord::kPair], g.ps, g.pm, g.srec, g.xs, g.xm, g.conn_s, g.conn_m,
+      ClipPool<NS, NM> cp;
+      const bool mrev = load_pool(o, cp);
+      adjoint_pair_fast<NS, NM, SEG, DUAL>(o[32 * FxRecord::kPair], cp, mrev, g.ps, g.pm, g.srec, g.xs, g.xm, g.conn_s, g.conn_m,
                                            g.lambda, g.sl, g.gm, g.fo, nr == kSlowPair ? ctr : counted);
     } else if (nr != 0) {
       const int64_t p = o[32 * FxRecord::kPair];

@@ -229,24 +229,15 @@ constexpr int kQuadThreads = 128;   // of the quadrature kernel's blocks
 template <bool SEG>
 constexpr int kPtsBytes = (SEG ? 52 : 28) * 8;
 
-// One pair in FP64 (pairs whose geometry does not fit the fixed-point frame): FP64 clip, then the 7-point rule on the
-// centroid fan with the map inversions of MapInverse.
+// The clip polygon (pu, pv, nr vertices) of pair p in FP64, for pairs whose
+// geometry does not fit the fixed-point frame: the 7-point rule on the centroid
+// fan with the map inversions of MapInverse.
 template <int NS, int NM, bool SEG>
-__device__ __noinline__ void integrate_pair_fp64(int64_t p, const int32_t* __restrict__ ps,
-                                                      const int32_t* __restrict__ pm,
-                                                      const double* __restrict__ srec, const double* __restrict__ xm,
-                                                      const int32_t* __restrict__ conn_m, const RunParams& rp,
-                                                      double* __restrict__ Mblk, double* __restrict__ Dblk,
-                                                      uint8_t* __restrict__ flag, PairCounters& ctr) {
-  const double* r = srec + (int64_t)SR_STRIDE * ps[p];
-  PlaneMap mmap;
-  double pu[kPolyS], pv[kPolyS];
-  const int nr = clip_polygon_pool<NS, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
-  if (nr == 0) {
-    write_zero_blocks(p, SEG, Mblk, Dblk);
-    flag[p] = 0;
-    return;
-  }
+__device__ __noinline__ void integrate_polygon_fp64(int64_t p, const double* __restrict__ r, const PlaneMap& mmap,
+                                                    const double* __restrict__ pu, const double* __restrict__ pv, int nr,
+                                                    const RunParams& rp, double* __restrict__ Mblk,
+                                                    double* __restrict__ Dblk, uint8_t* __restrict__ flag,
+                                                    PairCounters& ctr) {
   MapInverse mi;
   mi.setup(mmap, NM == 3 || map_is_affine(mmap));
   MapInverse si;
@@ -334,6 +325,25 @@ __device__ __noinline__ void integrate_pair_fp64(int64_t p, const int32_t* __res
   flag[p] = 1;
 }
 
+// One pair in FP64 from its clip on (pairs that the cell kernel hands back).
+template <int NS, int NM, bool SEG>
+__device__ __noinline__ void integrate_pair_fp64(int64_t p, const int32_t* __restrict__ ps,
+                                                 const int32_t* __restrict__ pm, const double* __restrict__ srec,
+                                                 const double* __restrict__ xm, const int32_t* __restrict__ conn_m,
+                                                 const RunParams& rp, double* __restrict__ Mblk,
+                                                 double* __restrict__ Dblk, uint8_t* __restrict__ flag,
+                                                 PairCounters& ctr) {
+  const double* r = srec + (int64_t)SR_STRIDE * ps[p];
+  PlaneMap mmap;
+  double pu[kPolyS], pv[kPolyS];
+  const int nr = clip_polygon_pool<NS, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
+  if (nr > 0) {
+    integrate_polygon_fp64<NS, NM, SEG>(p, r, mmap, pu, pv, nr, rp, Mblk, Dblk, flag, ctr);
+  } else {
+    write_zero_blocks(p, SEG, Mblk, Dblk);
+    flag[p] = 0;
+  }
+}
 
 // FP64 clip of pair p, and its record at o (word w at o[32 w]).  Empty pairs
 // get zero blocks; pairs that do not fit the fixed-point frame are integrated
@@ -363,7 +373,7 @@ __device__ __forceinline__ void clip_record(bool has, int64_t p, const int32_t* 
         ctr.gp += 7 * f.ncell;
         ctr.nonempty++;
       } else {
-        integrate_pair_fp64<NS, NM, SEG>(p, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, ctr);
+        integrate_polygon_fp64<NS, NM, SEG>(p, r, mmap, pu, pv, nr, rp, Mblk, Dblk, flag, ctr);
       }
     }
   }
@@ -535,6 +545,10 @@ __global__ void __launch_bounds__(kQuadThreads, 4) k_pair_quadrature(
       if (w + lane < records) {
         const int64_t i = r0 + w + lane;
         ncell = record_cells(rec[((i >> 5) * FxRecord::kWords + FxRecord::kInfo) * 32 + (i & 31)]);
+      }
+      if (!__any_sync(0xffffffffu, ncell > 0)) {   // empty pairs, or pairs done in FP64
+        w += 32;
+        continue;
       }
       const CellSlot cs = assign_cells(ncell);
       const int64_t i = r0 + w + cs.rec;

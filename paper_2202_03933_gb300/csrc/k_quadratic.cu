@@ -41,28 +41,15 @@ struct QCounters {
   unsigned long long gp = 0, cells = 0, newton_fail = 0, clip_over = 0;
 };
 
-// One unit in FP64, for those that do not fit the fixed-point frame:
-// sub-element k of pair p.  Writes the unit's 8 x 4 block and flag.
+// The clip polygon (Pu, Pv, nr vertices) of unit u in FP64, for units that do
+// not fit the fixed-point frame.  Writes the unit's 8 x 4 block and flag.
 template <int NP, int NM>
-__device__ __noinline__ void integrate_unit(int64_t u, const int32_t* __restrict__ ps, const int32_t* __restrict__ pm,
-                               const double* __restrict__ srec, const double* __restrict__ xm,
-                               const int32_t* __restrict__ conn_m, double* __restrict__ U,
-                               uint8_t* __restrict__ uflag, QCounters& ctr) {
-  constexpr int NSUB = NP == 8 ? 4 : 3;
-  const int64_t p = u >> 2;
+__device__ __noinline__ void integrate_unit_polygon(int64_t u, const double* __restrict__ r, const PlaneMap& mmap,
+                                                    const double* __restrict__ Pu, const double* __restrict__ Pv, int nr,
+                                                    double* __restrict__ U, uint8_t* __restrict__ uflag,
+                                                    QCounters& ctr) {
   const int k = (int)(u & 3);
-  const int32_t s = ps[p], m = pm[p];
-  const double* r = srec + (int64_t)SR_STRIDE * (4 * (int64_t)s + k);
   double2* out = reinterpret_cast<double2*>(U + 32 * u);
-  PlaneMap mmap;
-  double Pu[kPolyS], Pv[kPolyS];
-  const int nr = clip_polygon_pool<NSUB, NM, kPolyS>(r, xm, conn_m, m, mmap, Pu, Pv, ctr.clip_over);
-  if (nr == 0) {
-#pragma unroll
-    for (int i = 0; i < 16; ++i) __stcs(out + i, make_double2(0.0, 0.0));
-    uflag[u] = 0;
-    return;
-  }
   double Mq[8][4];
 #pragma unroll
   for (int a = 0; a < 8; ++a)
@@ -132,6 +119,21 @@ __device__ __noinline__ void integrate_unit(int64_t u, const int32_t* __restrict
     __stcs(out + 2 * a + 1, make_double2(Mq[a][2], NM == 4 ? Mq[a][3] : 0.0));
   }
   uflag[u] = 1;
+}
+
+// One unit in FP64 from its clip on (units that the cell kernel hands back).
+template <int NP, int NM>
+__device__ __noinline__ void integrate_unit(int64_t u, const int32_t* __restrict__ ps, const int32_t* __restrict__ pm,
+                                            const double* __restrict__ srec, const double* __restrict__ xm,
+                                            const int32_t* __restrict__ conn_m, double* __restrict__ U,
+                                            uint8_t* __restrict__ uflag, QCounters& ctr) {
+  const int64_t p = u >> 2;
+  const double* r = srec + (int64_t)SR_STRIDE * (4 * (int64_t)ps[p] + (u & 3));
+  PlaneMap mmap;
+  double Pu[kPolyS], Pv[kPolyS];
+  const int nr = clip_polygon_pool<NP == 8 ? 4 : 3, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, Pu, Pv, ctr.clip_over);
+  if (nr > 0) integrate_unit_polygon<NP, NM>(u, r, mmap, Pu, Pv, nr, U, uflag, ctr);
+  else uflag[u] = 0;
 }
 
 // Half of a quadratic element's shape functions in Q61 (HALF 0: corners, 1:
@@ -247,12 +249,16 @@ __global__ void __launch_bounds__(kQThreads, 4) k_quadratic_clip(
     if (32 * (int64_t)g >= n) break;
     long long* o = rec + (int64_t)g * (32 * FxRecord::kWords) + lane;
     bool stored = false;
+    int nr = 0;
+    int64_t u = 0;
+    const double* r = srec;
+    PlaneMap mmap;
+    double pu[kPolyS], pv[kPolyS];
     if (i < n) {
-      const int64_t u = 4 * first + order[i], p = u >> 2;
-      const double* r = srec + (int64_t)SR_STRIDE * (4 * (int64_t)ps[p] + (u & 3));
-      PlaneMap mmap;
-      double pu[kPolyS], pv[kPolyS];
-      const int nr = clip_polygon_pool<NSUB, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
+      u = 4 * first + order[i];
+      const int64_t p = u >> 2;
+      r = srec + (int64_t)SR_STRIDE * (4 * (int64_t)ps[p] + (u & 3));
+      nr = clip_polygon_pool<NSUB, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
       if (nr == 0) {
         uflag[u] = 0;
       } else {
@@ -262,11 +268,11 @@ __global__ void __launch_bounds__(kQThreads, 4) k_quadratic_clip(
           FxRecord::store<NSUB, NM>(o, f, u);
           ctr.cells += f.ncell;
           ctr.gp += 7 * f.ncell;
-        } else {
-          integrate_unit<NP, NM>(u, ps, pm, srec, xm, conn_m, U, uflag, ctr);
         }
       }
     }
+    __syncwarp();   // lanes leave setup in several places; those for FP64 run together
+    if (nr > 0 && !stored) integrate_unit_polygon<NP, NM>(u, r, mmap, pu, pv, nr, U, uflag, ctr);
     if (!stored) o[32 * FxRecord::kInfo] = 0;   // nr = 0: nothing left for the cell kernel
     __syncwarp();
   }
@@ -305,6 +311,10 @@ __global__ void __launch_bounds__(kQThreads, 4) k_quadratic_cells(
       if (w + lane < records) {
         const int64_t i = r0 + w + lane;
         ncell = record_cells(rec[((i >> 5) * FxRecord::kWords + FxRecord::kInfo) * 32 + (i & 31)]);
+      }
+      if (!__any_sync(0xffffffffu, ncell > 0)) {   // empty units, or units done in FP64
+        w += 32;
+        continue;
       }
       const CellSlot cs = assign_cells(ncell);
       const int64_t i = r0 + w + cs.rec;

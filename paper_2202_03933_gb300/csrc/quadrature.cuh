@@ -32,25 +32,25 @@ struct FxPolygon {
   __device__ __forceinline__ bool setup(const double* __restrict__ r, const PlaneMap& mmap, const double* pu,
                                         const double* pv, int n) {
     nr = n;
-    if (n > kCap) return false;
     PlaneMap smap;
     smap.c0u = r[SR_C + 0]; smap.c0v = r[SR_C + 1]; smap.c1u = r[SR_C + 2]; smap.c1v = r[SR_C + 3];
     smap.c2u = r[SR_C + 4]; smap.c2v = r[SR_C + 5]; smap.c3u = r[SR_C + 6]; smap.c3v = r[SR_C + 7];
     const FxFrame fr = fx_frame<NS, NM>(r, mmap);
-    if (!fr.ok) return false;
+    bool ok = fr.ok && n <= kCap;   // one exit, so that the lanes that take the FP64 path run it together
     Eu = fr.Eu;
     Ev = fr.Ev;
     if (NM == 3 || map_is_affine(mmap)) {
       const double id = 1.0 / (mmap.c1u * mmap.c2v - mmap.c2u * mmap.c1v);
-      if (!m.setup_affine(mmap, mmap.c2v * id, -mmap.c2u * id, -mmap.c1v * id, mmap.c1u * id, Eu, Ev)) return false;
+      ok &= m.setup_affine(mmap, mmap.c2v * id, -mmap.c2u * id, -mmap.c1v * id, mmap.c1u * id, Eu, Ev);
     } else {
-      if (!m.setup_bilinear(mmap, Eu, Ev)) return false;
+      ok &= m.setup_bilinear(mmap, Eu, Ev);
     }
     if (NS == 3 || r[SR_AFF] != 0.0) {
-      if (!s.setup_affine(smap, r[SR_BINV], r[SR_BINV + 1], r[SR_BINV + 2], r[SR_BINV + 3], Eu, Ev)) return false;
+      ok &= s.setup_affine(smap, r[SR_BINV], r[SR_BINV + 1], r[SR_BINV + 2], r[SR_BINV + 3], Eu, Ev);
     } else {
-      if (!s.setup_bilinear(smap, Eu, Ev)) return false;
+      ok &= s.setup_bilinear(smap, Eu, Ev);
     }
+    if (!ok) return false;
     cu = 0;
     cv = 0;
     for (int k = 0; k < nr; ++k) {
