@@ -115,6 +115,7 @@ struct AdjScale {
                                       int stretch) {
     float all = 0.0f, col = 0.0f, row = 0.0f, in_row = 0.0f, in_col[4] = {0.0f, 0.0f, 0.0f, 0.0f}, cols[4], rows[4];
     rows[3] = cols[3] = 0.0f;
+    unsigned long long any = 0;   // of the forms' bits but the sign
 #pragma unroll
     for (int j = 0; j < NM; ++j) cols[j] = 0.0f;
 #pragma unroll
@@ -123,13 +124,17 @@ struct AdjScale {
 #pragma unroll
       for (int j = 0; j < NM; ++j) {
         const float c = fabsf(f32_trunc(C[i][j]));
+        any |= (unsigned long long)__double_as_longlong(C[i][j]) << 1;
         r += c;
         cols[j] += c;
         if (i > 0 && j > 0) { rin += c; in_col[j] += c; }
       }
       if (SEG)
 #pragma unroll
-        for (int j = 0; j < NS; ++j) r += fabsf(f32_trunc(S[i][j]));
+        for (int j = 0; j < NS; ++j) {
+          r += fabsf(f32_trunc(S[i][j]));
+          any |= (unsigned long long)__double_as_longlong(S[i][j]) << 1;
+        }
       all += r;
       rows[i] = r;
       if (i > 0) { row = fmaxf(row, r); in_row = fmaxf(in_row, rin); }
@@ -141,11 +146,10 @@ struct AdjScale {
     sv = max(ex(row) + 2, s11);
     s1 = max(ex(col) + 2, s11);
     s0 = max(ex(all) + 1, max(sv, s1));
-    if (!(all < 1e37f && (all > 1e-30f || all == 0.0f))) return false;
+    if (!(all < 1e37f && (all > 1e-30f || any == 0))) return false;   // no multipliers at all: zero forms
     kys = fx_inverse_exponent(sm);
     kym = fx_inverse_exponent(mm);
     if (kys >= 20 || kym >= 20 || abs(stretch) > kMaxStretch) return false;
-    // |b| is at most the row's (column's) sum, that of xi eta added to both
     l = 0;
     if (abs(stretch) >= 2) {   // |b| is at most the row's (column's) sum, that of xi eta added to both
       l = bound_y(sm, kys, rows[1] + rows[3], rows[2] + rows[3], sv);
