@@ -232,15 +232,6 @@ struct ClipRec {
   }
 };
 
-// Compact clip record: the same Sutherland-Hodgman clip and merge as
-// ClipRec (identical decisions, quotients to an ulp), recorded as a pool of
-// vertices instead of whole stages.  Pool slots [0, NM) are the master
-// polygon's vertices (counter-clockwise), every later slot is an edge
-// intersection x = p + t (q - p) made at stage i from pool slots p and q; a
-// copied vertex keeps its slot.  The working polygon of a stage is a list of
-// 4-bit slot ids packed into 64 bits.  Reverse: slots are visited from the
-// last intersection down, so that each slot's adjoint is complete before it
-// is passed on to its two parents and to the clip edge.
 // Orientation of the projected master polygon: true if clockwise.  In FP32
 // where the area is above 1e-4 of its terms.
 template <int NM>
@@ -261,6 +252,15 @@ __device__ __forceinline__ bool polygon_reversed(const double* mu, const double*
   return ma2 < 0.0;
 }
 
+// Compact clip record: the same Sutherland-Hodgman clip and merge as
+// ClipRec (identical decisions, quotients to an ulp), recorded as a pool of
+// vertices instead of whole stages.  Pool slots [0, NM) are the master
+// polygon's vertices (counter-clockwise), every later slot is an edge
+// intersection x = p + t (q - p) made at stage i from pool slots p and q; a
+// copied vertex keeps its slot.  The working polygon of a stage is a list of
+// 4-bit slot ids packed into 64 bits.  Reverse: slots are visited from the
+// last intersection down, so that each slot's adjoint is complete before it
+// is passed on to its two parents and to the clip edge.
 template <int NS, int NM>
 struct ClipPool {
   static constexpr int kSlots = 12;   // master vertices + intersections (convex quads: <= 4 + 8)
@@ -280,7 +280,8 @@ struct ClipPool {
   __device__ __forceinline__ bool close(int a, int b, double em2) const {
     const float ua = f32_trunc(pu[a]), va = f32_trunc(pv[a]), ub = f32_trunc(pu[b]), vb = f32_trunc(pv[b]);
     const float d = fabsf(ua - ub) + fabsf(va - vb);
-    if (d > 1e-5f * (fabsf(ua) + fabsf(va) + fabsf(ub) + fabsf(vb)) && 0.25f * d * d > f32_trunc(em2)) return false;
+    const float e = f32_trunc(em2);   // 0: none, or below FP32's range
+    if (e > 0.0f && d > 1e-5f * (fabsf(ua) + fabsf(va) + fabsf(ub) + fabsf(vb)) && 0.25f * d * d > e) return false;
     const double du = pu[a] - pu[b], dv = pv[a] - pv[b];
     return du * du + dv * dv < em2;
   }
@@ -386,7 +387,8 @@ struct ClipPool {
       fa += x - y;
       fs += fabsf(x) + fabsf(y);
     }
-    if (fabsf(fa) > 1e-4f * fs && 0.25f * fabsf(fa) > f32_trunc(r[SR_EPSA])) return true;
+    const float ea = f32_trunc(r[SR_EPSA]);   // 0: none, or below FP32's range
+    if (ea > 0.0f && fabsf(fa) > 1e-4f * fs && 0.25f * fabsf(fa) > ea) return true;
     double pa2 = 0.0;
     for (int k = 0; k < nr; ++k) {
       const int a = id(k), b = id(k + 1 == nr ? 0 : k + 1);
