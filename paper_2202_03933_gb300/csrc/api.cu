@@ -182,7 +182,7 @@ void enqueue_run(mortar_ctx* c, const Phases& ph) {
   const bool fused = ph.adjoint && ph.integrate && adjoint_fuses_forward(c);
   {
     NvtxRange nv(fused ? "mortar:pairs(forward+adjoint)" : "mortar:pairs(forward)");
-    if (fused) launch_adjoint_pairs(c, rp, true);
+    if (fused) launch_adjoint_pairs(c, rp);
     else if (ph.integrate) launch_integrate(c, rp);
   }
   if (c->timing) record_event(c->ev[2], st);
@@ -194,7 +194,7 @@ void enqueue_run(mortar_ctx* c, const Phases& ph) {
   if (c->timing) record_event(c->ev[3], st);
   if (ph.adjoint) {
     NvtxRange nv("mortar:adjoint");
-    if (!fused) launch_adjoint_pairs(c, rp, false);
+    if (!fused) launch_adjoint_pairs(c, rp);
     if (c->timing) record_event(c->ev[5], st);
     launch_adjoint_rest(c, rp);
   }

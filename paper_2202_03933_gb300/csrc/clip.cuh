@@ -11,6 +11,19 @@ namespace mortar {
 
 constexpr int kPolyS = 10;   // stored clip-polygon vertices (convex quad vs quad: <= 8)
 
+// In-plane coordinates, in the plane of slave record r, of the master element with the nodes conn.
+template <int NM>
+__device__ __forceinline__ void project_master(const double* __restrict__ r, const double* __restrict__ xm,
+                                               const int32_t* __restrict__ conn, double* mu, double* mv) {
+#pragma unroll
+  for (int l = 0; l < NM; ++l) {
+    const int64_t n = conn[l];
+    const double dx = xm[3 * n] - r[SR_X0], dy = xm[3 * n + 1] - r[SR_X0 + 1], dz = xm[3 * n + 2] - r[SR_X0 + 2];
+    mu[l] = dx * r[SR_T1] + dy * r[SR_T1 + 1] + dz * r[SR_T1 + 2];
+    mv[l] = dx * r[SR_T2] + dy * r[SR_T2 + 1] + dz * r[SR_T2 + 2];
+  }
+}
+
 // Projection of the master element, its map, and the clipped, merged polygon
 // (Pu, Pv, nr vertices; nr = 0 when the pair contributes nothing).
 template <int NS, int NM, int CAP>
@@ -21,17 +34,8 @@ __device__ __forceinline__ int clip_polygon(const double* __restrict__ r, const 
   const double eps_in = r[SR_EPSIN];
   if (!(eps_in >= 0.0)) return 0;
   const long long eps_bits = __double_as_longlong(eps_in);
-  const double x0x = r[SR_X0], x0y = r[SR_X0 + 1], x0z = r[SR_X0 + 2];
-  const double t1x = r[SR_T1], t1y = r[SR_T1 + 1], t1z = r[SR_T1 + 2];
-  const double t2x = r[SR_T2], t2y = r[SR_T2 + 1], t2z = r[SR_T2 + 2];
   double mu[4], mv[4];
-#pragma unroll
-  for (int l = 0; l < NM; ++l) {
-    const int64_t n = conn_m[(int64_t)NM * m + l];
-    const double dx = xm[3 * n] - x0x, dy = xm[3 * n + 1] - x0y, dz = xm[3 * n + 2] - x0z;
-    mu[l] = dx * t1x + dy * t1y + dz * t1z;
-    mv[l] = dx * t2x + dy * t2y + dz * t2z;
-  }
+  project_master<NM>(r, xm, conn_m + (int64_t)NM * m, mu, mv);
   mmap = plane_map<NM>(mu, mv);
   double ma2 = 0.0;
 #pragma unroll
@@ -364,35 +368,6 @@ struct MapInverse {
     if (!coarse(xu, xv, xi, eta, ci)) return newton64(xu, xv, xi, eta);
     polish(xu, xv, xi, eta, ci);
     return true;
-  }
-};
-
-// Shape functions and the pull-back of a shape-function adjoint to xi:
-// quad4 with a = 1 - xi, b = 1 + xi, c = 1 - eta, d = 1 + eta:
-//   N = (a c, b c, b d, a d) / 4,  dN/dxi = (-c, c, d, -d) / 4,  dN/deta = (-a, -b, b, a) / 4.
-template <int NEN>
-struct ShapeAD {
-  double N[4];
-  double qa, qb, qc, qd;
-  __device__ __forceinline__ void eval(double xi, double eta) {
-    if constexpr (NEN == 4) {
-      qa = 0.25 * (1.0 - xi); qb = 0.25 * (1.0 + xi);
-      const double c = 1.0 - eta, d = 1.0 + eta;
-      qc = 0.25 * c; qd = 0.25 * d;
-      N[0] = qa * c; N[1] = qb * c; N[2] = qb * d; N[3] = qa * d;
-    } else {
-      N[0] = 1.0 - xi - eta; N[1] = xi; N[2] = eta; N[3] = 0.0;
-    }
-  }
-  // (dxi, deta) += sum_k Nb[k] grad N_k
-  __device__ __forceinline__ void pull(const double* Nb, double& g0, double& g1) const {
-    if constexpr (NEN == 4) {
-      g0 = fma(qc, Nb[1] - Nb[0], qd * (Nb[2] - Nb[3]));
-      g1 = fma(qa, Nb[3] - Nb[0], qb * (Nb[2] - Nb[1]));
-    } else {
-      g0 = Nb[1] - Nb[0];
-      g1 = Nb[2] - Nb[0];
-    }
   }
 };
 

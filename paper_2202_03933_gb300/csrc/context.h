@@ -143,7 +143,6 @@ void launch_candidates(mortar_ctx* c);
 // k_integrate.cu
 void launch_integrate(mortar_ctx* c, const RunParams& rp);
 bool integrate_batched_fits(int rounds, int block);   // shared memory of the sort kernel's batches fits
-int integrate_rounds(int rounds, int block);          // rounds the integration kernel uses for a setting
 
 // k_contact.cu
 void launch_contact_terms(mortar_ctx* c, bool with_ncp, double cpen);   // normals, gap (+ active, ncp)
@@ -160,7 +159,7 @@ void launch_finalize_status(mortar_ctx* c);
 // k_adjoint.cu
 int prepare_adjoint_buffers(mortar_ctx* c);   // sizes per-pair adjoint buffers from n_pairs
 bool adjoint_fuses_forward(const mortar_ctx* c);   // the adjoint pair kernel also writes M/D blocks
-void launch_adjoint_pairs(mortar_ctx* c, const RunParams& rp, bool fused);
+void launch_adjoint_pairs(mortar_ctx* c, const RunParams& rp);
 void launch_adjoint_rest(mortar_ctx* c, const RunParams& rp);   // element adjoint, gathers, J
 
 // k_tangent.cu
@@ -187,7 +186,7 @@ template <int NS, int NM>
 void integrate_nsnm(const IntegrateArgs& a, const RunParams& rp, int n_sm, int variant, int block, int chunk,
                     int rounds);
 template <int NS, int NM>
-void adjoint_pairs_nsnm(mortar_ctx* c, const RunParams& rp, unsigned grid, unsigned block, int32_t chunk, bool fused);
+void adjoint_pairs_nsnm(mortar_ctx* c, const RunParams& rp, unsigned grid, unsigned block, int32_t chunk);
 template <int NS, int NM>
 void tangent_pairs_nsnm(mortar_ctx* c, const RunParams& rp);
 template <int NS, int NM>

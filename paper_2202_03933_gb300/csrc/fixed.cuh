@@ -450,12 +450,7 @@ template <int NM>
 __device__ __noinline__ PlaneMap master_plane_map(const double* __restrict__ r, const double* __restrict__ xm,
                                                   const int32_t* __restrict__ conn_m, int32_t m) {
   double mu[4], mv[4];
-  for (int l = 0; l < NM; ++l) {
-    const int64_t n = conn_m[(int64_t)NM * m + l];
-    const double dx = xm[3 * n] - r[SR_X0], dy = xm[3 * n + 1] - r[SR_X0 + 1], dz = xm[3 * n + 2] - r[SR_X0 + 2];
-    mu[l] = dx * r[SR_T1] + dy * r[SR_T1 + 1] + dz * r[SR_T1 + 2];
-    mv[l] = dx * r[SR_T2] + dy * r[SR_T2 + 1] + dz * r[SR_T2 + 2];
-  }
+  project_master<NM>(r, xm, conn_m + (int64_t)NM * m, mu, mv);
   return plane_map<NM>(mu, mv);
 }
 

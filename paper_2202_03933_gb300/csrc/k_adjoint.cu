@@ -486,16 +486,8 @@ __device__ __noinline__ void adjoint_pair_fast(int64_t p, const ClipPool<NS, NM>
   const double* r = srec + (int64_t)SR_STRIDE * s;
   const int32_t* cs = conn_s + (int64_t)NS * s;
   const int32_t* cm = conn_m + (int64_t)NM * m;
-  const V3 x0 = v3(r[SR_X0], r[SR_X0 + 1], r[SR_X0 + 2]);
-  const V3 t1 = v3(r[SR_T1], r[SR_T1 + 1], r[SR_T1 + 2]);
-  const V3 t2 = v3(r[SR_T2], r[SR_T2 + 1], r[SR_T2 + 2]);
   double mu[4], mv[4];
-  for (int l = 0; l < NM; ++l) {
-    const int64_t n = cm[l];
-    const double dx = xm[3 * n] - x0.x, dy = xm[3 * n + 1] - x0.y, dz = xm[3 * n + 2] - x0.z;
-    mu[l] = dx * t1.x + dy * t1.y + dz * t1.z;
-    mv[l] = dx * t2.x + dy * t2.y + dz * t2.z;
-  }
+  project_master<NM>(r, xm, cm, mu, mv);
   const PlaneMap mmap = plane_map<NM>(mu, mv);
   PlaneMap smap;
   smap.c0u = r[SR_C + 0]; smap.c0v = r[SR_C + 1]; smap.c1u = r[SR_C + 2]; smap.c1v = r[SR_C + 3];
@@ -569,7 +561,8 @@ __device__ __noinline__ void adjoint_pair_fast(int64_t p, const ClipPool<NS, NM>
       const double cr = cross2(e1u, e1v, e2u, e2v);
       const double area = 0.5 * fabs(cr);
       double area_b = 0.0, e1bu = 0.0, e1bv = 0.0, e2bu = 0.0, e2bv = 0.0, abu = 0.0, abv = 0.0;
-ctr.cells++; ctr.gp += 7;
+      ctr.cells++;
+      ctr.gp += 7;
 #pragma unroll 1
       for (int q = 0; q < 7; ++q) {
         double l1, l2, w;
@@ -792,7 +785,7 @@ __device__ __forceinline__ bool next_group(unsigned long long* ctr, int64_t n, i
 // forward integration, where the work's character changes: k_pair_sort,
 // k_adjoint_clip, k_adjoint_cells, k_adjoint_finish, with a record per pair in
 // between (832 B, 960 B with segment D).  planar 600x520, dual (1.35 M pairs):
-// 0.25 + 1.1 + 4.3 + 1.2 ms against 14.5 to 16.8 ms (by batch size) of one FP64
+// 0.20 + 1.35 + 4.3 + 1.36 ms against 14.5 to 16.8 ms (by batch size) of one FP64
 // kernel with the same sweep.
 //
 // First kernel: FP64 clip with its record, the pair's bilinear forms CY [and
@@ -818,13 +811,7 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_clip(AdjArgs g, un
       const int32_t* cm = g.conn_m + (int64_t)NM * m;
       o[32 * FxRecord::kPair] = p;
       double mu[4], mv[4];
-      for (int l = 0; l < NM; ++l) {
-        const int64_t nd = cm[l];
-        const double dx = g.xm[3 * nd] - r[SR_X0], dy = g.xm[3 * nd + 1] - r[SR_X0 + 1],
-                     dz = g.xm[3 * nd + 2] - r[SR_X0 + 2];
-        mu[l] = dx * r[SR_T1] + dy * r[SR_T1 + 1] + dz * r[SR_T1 + 2];
-        mv[l] = dx * r[SR_T2] + dy * r[SR_T2 + 1] + dz * r[SR_T2 + 2];
-      }
+      project_master<NM>(r, g.xm, cm, mu, mv);
       const PlaneMap mmap = plane_map<NM>(mu, mv);
       const bool mrev = polygon_reversed<NM>(mu, mv);
       ClipPool<NS, NM> cp;
@@ -1110,7 +1097,7 @@ __global__ void __maxnreg__(168) k_adjoint_cells(AdjArgs ar) {
 // blocks M = A G belong here: inside the cell kernel they cost 0.8 ms more at
 // 600x520 (4.5 -> 5.3) than they save.  What depends on the slave element alone
 // (the plane's reverse) is done once per element (k_adjoint_elems): pairs
-// leave 30 words, 42 with dual LMs.
+// leave 30 words, 42 with segment D.
 template <int NS, int NM, bool SEG, bool DUAL>
 __global__ void __launch_bounds__(kMaxPairBlock, 2) k_adjoint_finish(AdjArgs g) {
   constexpr int W = SEG ? AdjRecord::kWordsSeg : AdjRecord::kWords;
@@ -1663,8 +1650,7 @@ void launch_fixed(mortar_ctx* c, const RunParams& rp, int block, int rounds) {
 }  // namespace
 
 template <int NS, int NM>
-void adjoint_pairs_nsnm(mortar_ctx* c, const RunParams& rp, unsigned grid, unsigned block, int32_t chunk,
-                        bool fused) {
+void adjoint_pairs_nsnm(mortar_ctx* c, const RunParams& rp, unsigned grid, unsigned block, int32_t chunk) {
   const bool seg = rp.d_domain == 1, dual = rp.lm == 1;
   if (c->variant == 1) {
     if (seg && dual) launch_pairs_t<NS, NM, true, true>(c, rp, grid, block, chunk);
@@ -1673,7 +1659,6 @@ void adjoint_pairs_nsnm(mortar_ctx* c, const RunParams& rp, unsigned grid, unsig
     else launch_pairs_t<NS, NM, false, false>(c, rp, grid, block, chunk);
     return;
   }
-  (void)fused;
   const int rounds = c->rounds > 0 ? c->rounds : kSortBatch / 32;
   if (seg && dual) launch_fixed<NS, NM, true, true>(c, rp, (int)block, rounds);
   else if (seg) launch_fixed<NS, NM, true, false>(c, rp, (int)block, rounds);
@@ -1681,7 +1666,7 @@ void adjoint_pairs_nsnm(mortar_ctx* c, const RunParams& rp, unsigned grid, unsig
   else launch_fixed<NS, NM, false, false>(c, rp, (int)block, rounds);
 }
 template void adjoint_pairs_nsnm<MORTAR_PAIR_NS, MORTAR_PAIR_NM>(mortar_ctx*, const RunParams&, unsigned, unsigned,
-                                                                  int32_t, bool);
+                                                                  int32_t);
 #else   // the main part: element adjoint, gathers, J, dispatch
 
 template <int NS>
@@ -1733,14 +1718,14 @@ int prepare_adjoint_buffers(mortar_ctx* c) {
 
 bool adjoint_fuses_forward(const mortar_ctx* c) { return c->variant == 0; }
 
-void launch_adjoint_pairs(mortar_ctx* c, const RunParams& rp, bool fused) {
+void launch_adjoint_pairs(mortar_ctx* c, const RunParams& rp) {
   const unsigned block = c->block_size > 0 ? (unsigned)c->block_size : 128u;
   const int32_t chunk = c->chunk_pairs > 0 ? c->chunk_pairs : 32;
   const unsigned grid = 0;   // the one-pair-per-thread kernels size their own grid
-  if (c->nen_s == 4 && c->nen_m == 4) adjoint_pairs_nsnm<4, 4>(c, rp, grid, block, chunk, fused);
-  else if (c->nen_s == 4 && c->nen_m == 3) adjoint_pairs_nsnm<4, 3>(c, rp, grid, block, chunk, fused);
-  else if (c->nen_s == 3 && c->nen_m == 4) adjoint_pairs_nsnm<3, 4>(c, rp, grid, block, chunk, fused);
-  else adjoint_pairs_nsnm<3, 3>(c, rp, grid, block, chunk, fused);
+  if (c->nen_s == 4 && c->nen_m == 4) adjoint_pairs_nsnm<4, 4>(c, rp, grid, block, chunk);
+  else if (c->nen_s == 4 && c->nen_m == 3) adjoint_pairs_nsnm<4, 3>(c, rp, grid, block, chunk);
+  else if (c->nen_s == 3 && c->nen_m == 4) adjoint_pairs_nsnm<3, 4>(c, rp, grid, block, chunk);
+  else adjoint_pairs_nsnm<3, 3>(c, rp, grid, block, chunk);
 }
 
 void launch_adjoint_rest(mortar_ctx* c, const RunParams& rp) {

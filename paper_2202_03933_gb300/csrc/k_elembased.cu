@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kThreads) k_integrate_elembased(
 // that FP64 gives it.  (Blocks of at most four points, n = 12, parallelograms:
 // geometric mean of the largest relative error of an entry 7e-14 with two
 // digits, 4e-15 with three, FP64 3e-15.)
-// 600x520 quad4, n = 8, dual: 5.95 ms in FP64 (FP64 pipe), 3.14 ms here, of which
+// 600x520 quad4, n = 8, dual: 5.95 ms in FP64 (FP64 pipe), 3.2 ms here, of which
 // the instructions would take half: the candidates' maps and the exchanged sums
 // (about 2 KB a thread) miss L1 in 58 % of their sectors.  Sums added in memory
 // point by point: 4.07 ms; without the warp in step: 9.0 ms; 2 or 4 blocks per SM

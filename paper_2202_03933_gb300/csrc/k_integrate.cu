@@ -21,7 +21,7 @@
 //    element maps and the cell weights into a fixed-point record;
 //    k_pair_quadrature integrates the records on the integer pipe, one cell of
 //    a pair per lane (fixed.cuh, quadrature.cuh).
-//    planar_600x520 (1.35 M pairs, dual LMs): 0.24 + 1.0 + 1.65 ms, against
+//    planar_600x520 (1.35 M pairs, dual LMs): 0.20 + 0.95 + 1.63 ms, against
 //    6.2 ms (batches of 64 pairs, the former default) and 5.6 ms (1024) of the
 //    one-kernel FP64 form.  The clip kernel is bound by the FP64 pipe (50 %
 //    busy, 400 instructions a pair) and instruction fetch, the quadrature
@@ -30,7 +30,7 @@
 //  * one kernel (k_integrate_fused): for callers without workspace.  Clip
 //    records in shared memory, then the same quadrature.
 //  * pairs that do not fit the fixed-point frame are integrated in FP64 in
-//    either form (integrate_pair_fp64): affine maps are inverted with one
+//    either form (integrate_polygon_fp64): affine maps are inverted with one
 //    precomputed 2x2 inverse, bilinear ones by Newton in FP32, then one step
 //    with an FP64 residual (MapInverse in clip.cuh).
 //  * variant 1: one pair per thread, FP64 Newton from xi = 0 at every point
@@ -640,12 +640,8 @@ void launch_dispatch(const IntegrateArgs& a, const RunParams& rp, int nen_s, int
 }  // namespace
 
 bool integrate_batched_fits(int rounds, int block) {
-  return block >= 32 && block <= kMaxPairBlock && (size_t)(block / 32) * batch_smem_bytes(32 * rounds) <= kMaxDynSmem;
-}
-
-int integrate_rounds(int rounds, int block) {
-  (void)block;
-  return rounds <= 1 ? 1 : (rounds >= 32 ? 32 : rounds);
+  return block >= 32 && block <= kMaxPairBlock &&
+         (size_t)(kSortThreads / 32) * batch_smem_bytes(32 * rounds) <= kMaxDynSmem;
 }
 
 void launch_integrate_raw(const IntegrateArgs& a, const RunParams& rp, int nen_s, int nen_m, int n_sm) {
@@ -674,7 +670,7 @@ void launch_integrate(mortar_ctx* c, const RunParams& rp) {
   }
   const int block = c->block_size > 0 ? c->block_size : 128;
   const int chunk = c->chunk_pairs > 0 ? c->chunk_pairs : 32;
-  const int rounds = integrate_rounds(c->rounds > 0 ? c->rounds : kSortBatch / 32, block);
+  const int rounds = c->rounds > 0 ? c->rounds : kSortBatch / 32;
   launch_dispatch(a, rp, c->nen_s, c->nen_m, c->n_sm, c->variant, block, chunk, rounds);
 }
 #endif  // MORTAR_PAIR_NS

@@ -20,8 +20,8 @@
 // (k_quadratic_clip), and integrated on the integer pipe with one cell of a unit
 // per lane (k_quadratic_cells).  A last kernel sums the non-empty unit blocks
 // of every pair in the fixed order k = 0..3 (bitwise reproducible) into the pair
-// block and its flag.  quad8 450x390 (0.71 M pairs, 2.8 M units): 0.5 + 2.3 + 4.9 +
-// 0.2 ms against 14.7 ms of one FP64 kernel; the clip is bound by the FP64 pipe
+// block and its flag.  quad8 450x390 (0.71 M pairs, 2.8 M units): 0.43 + 2.06 +
+// 4.55 + 0.19 ms against 14.7 ms of one FP64 kernel; the clip is bound by the FP64 pipe
 // (most units are empty), the cells by issue over the integer pipes.
 #include "clip.cuh"
 #include "context.h"

@@ -22,9 +22,10 @@
 // over the pair are small seeds themselves or differences in which nothing
 // cancels, so that a row that is small keeps its digits: with a pair of 1 % of
 // the element's size at a corner, the far node's row has errors up to 3.2e-13 of
-// itself, as with the N_e as seeds, and 2.9e-12 with monomials about the centre.  Bound by the FP64 pipe (about 75 % busy);
-// 300x260 quads, dual (0.31 M pairs): 21.7 ms with the N_e as seeds, 18.7 ms
-// this way, square roots and divisions of the plane once per pair.
+// itself, as with the N_e as seeds, and 2.9e-12 with monomials about the centre.
+// Bound by the FP64 pipe (about 75 % busy); 300x260 quads, dual (0.31 M pairs):
+// 21.8 ms with the N_e as seeds, 18.9 ms this way (18.7 about the centre), square
+// roots and divisions of the plane once per pair.
 //
 // The derivatives through A (dual LMs) and of the element-domain D depend on
 // the slave element alone: a per-element kernel pushes the pair sums of O and

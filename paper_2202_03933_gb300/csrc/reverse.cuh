@@ -475,13 +475,7 @@ __device__ __forceinline__ int clip_polygon_pool(const double* __restrict__ r, c
                                                  double* Pu, double* Pv, unsigned long long& clip_over) {
   if (!(r[SR_EPSIN] >= 0.0)) return 0;
   double mu[4], mv[4];
-#pragma unroll
-  for (int l = 0; l < NM; ++l) {
-    const int64_t n = conn_m[(int64_t)NM * m + l];
-    const double dx = xm[3 * n] - r[SR_X0], dy = xm[3 * n + 1] - r[SR_X0 + 1], dz = xm[3 * n + 2] - r[SR_X0 + 2];
-    mu[l] = dx * r[SR_T1] + dy * r[SR_T1 + 1] + dz * r[SR_T1 + 2];
-    mv[l] = dx * r[SR_T2] + dy * r[SR_T2 + 1] + dz * r[SR_T2 + 2];
-  }
+  project_master<NM>(r, xm, conn_m + (int64_t)NM * m, mu, mv);
   mmap = plane_map<NM>(mu, mv);
   ClipPool<NS, NM> cp;
   unsigned long long over = 0;
