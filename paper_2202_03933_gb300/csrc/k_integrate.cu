@@ -233,11 +233,10 @@ constexpr int kPtsBytes = (SEG ? 52 : 28) * 8;
 // geometry does not fit the fixed-point frame: the 7-point rule on the centroid
 // fan with the map inversions of MapInverse.
 template <int NS, int NM, bool SEG>
-__device__ __noinline__ void integrate_polygon_fp64(int64_t p, const double* __restrict__ r, const PlaneMap& mmap,
-                                                    const double* __restrict__ pu, const double* __restrict__ pv, int nr,
-                                                    const RunParams& rp, double* __restrict__ Mblk,
-                                                    double* __restrict__ Dblk, uint8_t* __restrict__ flag,
-                                                    PairCounters& ctr) {
+__device__ __forceinline__ void polygon_fp64(int64_t p, const double* __restrict__ r, const PlaneMap& mmap,
+                                             const double* pu, const double* pv, int nr, const RunParams& rp,
+                                             double* __restrict__ Mblk, double* __restrict__ Dblk,
+                                             uint8_t* __restrict__ flag, PairCounters& ctr) {
   MapInverse mi;
   mi.setup(mmap, NM == 3 || map_is_affine(mmap));
   MapInverse si;
@@ -325,7 +324,17 @@ __device__ __noinline__ void integrate_polygon_fp64(int64_t p, const double* __r
   flag[p] = 1;
 }
 
-// One pair in FP64 from its clip on (pairs that the cell kernel hands back).
+template <int NS, int NM, bool SEG>
+__device__ __noinline__ void integrate_polygon_fp64(int64_t p, const double* __restrict__ r, const PlaneMap& mmap,
+                                                    const double* __restrict__ pu, const double* __restrict__ pv, int nr,
+                                                    const RunParams& rp, double* __restrict__ Mblk,
+                                                    double* __restrict__ Dblk, uint8_t* __restrict__ flag,
+                                                    PairCounters& ctr) {
+  polygon_fp64<NS, NM, SEG>(p, r, mmap, pu, pv, nr, rp, Mblk, Dblk, flag, ctr);
+}
+
+// One pair in FP64 from its clip on (pairs that the cell kernel hands back; in
+// the one-kernel form, whose code is short of room, all of them).
 template <int NS, int NM, bool SEG>
 __device__ __noinline__ void integrate_pair_fp64(int64_t p, const int32_t* __restrict__ ps,
                                                  const int32_t* __restrict__ pm, const double* __restrict__ srec,
@@ -338,7 +347,7 @@ __device__ __noinline__ void integrate_pair_fp64(int64_t p, const int32_t* __res
   double pu[kPolyS], pv[kPolyS];
   const int nr = clip_polygon_pool<NS, NM, kPolyS>(r, xm, conn_m, pm[p], mmap, pu, pv, ctr.clip_over);
   if (nr > 0) {
-    integrate_polygon_fp64<NS, NM, SEG>(p, r, mmap, pu, pv, nr, rp, Mblk, Dblk, flag, ctr);
+    polygon_fp64<NS, NM, SEG>(p, r, mmap, pu, pv, nr, rp, Mblk, Dblk, flag, ctr);
   } else {
     write_zero_blocks(p, SEG, Mblk, Dblk);
     flag[p] = 0;
@@ -348,7 +357,8 @@ __device__ __noinline__ void integrate_pair_fp64(int64_t p, const int32_t* __res
 // FP64 clip of pair p, and its record at o (word w at o[32 w]).  Empty pairs
 // get zero blocks; pairs that do not fit the fixed-point frame are integrated
 // in FP64 here.  Either way the record says that no cells are left.
-template <int NS, int NM, bool SEG>
+// AGAIN: such pairs are clipped again rather than their polygon passed on.
+template <int NS, int NM, bool SEG, bool AGAIN>
 __device__ __forceinline__ void clip_record(bool has, int64_t p, const int32_t* __restrict__ ps,
                                             const int32_t* __restrict__ pm, const double* __restrict__ srec,
                                             const double* __restrict__ xm, const int32_t* __restrict__ conn_m,
@@ -372,6 +382,8 @@ __device__ __forceinline__ void clip_record(bool has, int64_t p, const int32_t* 
         ctr.cells += f.ncell;
         ctr.gp += 7 * f.ncell;
         ctr.nonempty++;
+      } else if (AGAIN) {
+        integrate_pair_fp64<NS, NM, SEG>(p, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, ctr);
       } else {
         integrate_polygon_fp64<NS, NM, SEG>(p, r, mmap, pu, pv, nr, rp, Mblk, Dblk, flag, ctr);
       }
@@ -435,7 +447,7 @@ __device__ __forceinline__ void integrate_cells(const CellSlot& cs, const long l
 // as spreads the list over all warps, 8 pairs (about a warp full of cells) to 32.
 // 14,400 pairs of quad4 elements through the no-allocation entry point: 251 us a
 // call with the former FP64 kernel (one pair per lane, all of it in one round
-// of 450 warps), 170 us with this one.
+// of 450 warps), 158 us with this one.
 constexpr int kFusedThreads = 128;
 template <bool SEG>
 constexpr size_t kFusedSmem = (size_t)kFusedThreads * (kPtsBytes<SEG> + FxRecord::kWords * 8);
@@ -463,7 +475,7 @@ __global__ void __launch_bounds__(kFusedThreads, 3) k_integrate_fused(
     const int64_t p0 = (int64_t)__shfl_sync(0xffffffffu, g0, 0);
     if (p0 >= n) break;
     const int pairs = (int)min((int64_t)turn, n - p0);
-    clip_record<NS, NM, SEG>(lane < pairs, p0 + lane, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, rec + lane, ctr);
+    clip_record<NS, NM, SEG, true>(lane < pairs, p0 + lane, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag, rec + lane, ctr);
     __syncwarp();
     for (int w = 0; w < pairs;) {
       int ncell = 0;
@@ -509,7 +521,7 @@ __global__ void __launch_bounds__(kMaxPairBlock, 2) k_pair_clip(
     g = __shfl_sync(0xffffffffu, g, 0);
     const int64_t i = 32 * (int64_t)g + lane;
     if (32 * (int64_t)g >= n) break;
-    clip_record<NS, NM, SEG>(i < n, i < n ? first + order[i] : 0, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag,
+    clip_record<NS, NM, SEG, false>(i < n, i < n ? first + order[i] : 0, ps, pm, srec, xm, conn_m, rp, Mblk, Dblk, flag,
                              rec + (int64_t)g * (32 * FxRecord::kWords) + lane, ctr);
     __syncwarp();
   }
