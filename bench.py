@@ -55,8 +55,8 @@ UNIT = "pairs/s"
 # profiles/.  The quadrature is 64-bit fixed point on the integer pipes, so the
 # kernels' common roofline is the issue rate.
 EXEC_PER_PAIR = {
-    "fused": {"warp_inst": 2056.0, "flops": 1084.4, "dram_bytes": 4109.0, "fp64_form": 8492.3},
-    "integrate": {"warp_inst": 1061.2, "flops": 381.4, "dram_bytes": 1584.0, "fp64_form": 2994.6},
+    "fused": {"warp_inst": 2069.5, "flops": 1084.4, "dram_bytes": 4146.5, "fp64_form": 8492.3},
+    "integrate": {"warp_inst": 1062.0, "flops": 381.5, "dram_bytes": 1632.4, "fp64_form": 2994.6},
 }
 # fp64_form: executed FP64 flops per pair of the same integration with the
 # quadrature on the FP64 pipe (this library's former kernels).
