@@ -111,8 +111,8 @@ typedef struct mortar_options {
   int32_t watchdog_us;      /* time budget of a persistent pair kernel in microseconds, 0 = none (0): a
                                kernel whose thread blocks run longer stops taking work, the pair kernels
                                after it take none, and the call returns MORTAR_ERR_TIMEOUT (results not
-                               valid; the context stays usable).  The budget is of each kernel: a run
-                               has up to four for every 4 M pairs */
+                               valid; the context stays usable).  The budget is of each kernel, of
+                               which a run has up to four for every 1 to 4 M pairs */
 } mortar_options;
 
 typedef struct mortar_stats {

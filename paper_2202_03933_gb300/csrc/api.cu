@@ -653,12 +653,14 @@ int mortar_tangent(mortar_ctx* c, const double* ys, const double* ym, int32_t ad
   const RunParams rp = run_params(c);
   DevStatus* dst = c->dstat.as<DevStatus>();
   cudaMemsetAsync(&dst->work_ctr3, 0, 3 * sizeof(unsigned long long), c->stream);   // work_ctr3, nnzb_K, over_K
+  cudaMemsetAsync(&dst->timeout, 0, sizeof(dst->timeout), c->stream);
   if (c->timing) record_event(c->ev[6], c->stream);
   launch_tangent_blocks(c, rp);
   launch_tangent_rows(c, rp, 0);
   cudaMemcpyAsync(c->hstat, c->dstat.p, sizeof(DevStatus), cudaMemcpyDeviceToHost, c->stream);
   MORTAR_TRY(cuda_status(cudaStreamSynchronize(c->stream)));
   MORTAR_TRY(check_cuda());
+  if (c->hstat->timeout) return MORTAR_ERR_TIMEOUT;   // pairs without their blocks
   const int64_t need = (int64_t)c->hstat->nnzb_K;
   if (need > c->tan_nnzb_cap) {
     const int64_t cap = need + need / 16 + 64;

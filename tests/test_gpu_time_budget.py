@@ -86,3 +86,18 @@ def test_budget_of_a_captured_run(mt):
     for _ in range(2):
         m.run_graph(lam)
         assert _same(list(m.gradient()[1:]) + [m.scipy(w).data for w in (mt.MATRIX_D, mt.MATRIX_M)], ref)
+
+
+def test_budget_of_the_linearisation(mt):
+    itf = inputs.planar_noisy(120, 104, 1, 89, "tbt")
+    rng = np.random.default_rng(10)
+    ys, ym = rng.uniform(-1, 1, itf.xs.shape), rng.uniform(-1, 1, itf.xm.shape)
+    m = mt.Mortar(lm=1, delta=itf.delta)
+    m.set_interface(itf.xs, itf.conn_s, itf.xm, itf.conn_m)
+    m.evaluate()
+    ref = m.tangent(ys, ym)
+    m.set_watchdog(20)
+    with pytest.raises(mt._native.MortarError, match="TIMEOUT"):
+        m.tangent(ys, ym)
+    m.set_watchdog(0)
+    assert _same(m.tangent(ys, ym), ref)
